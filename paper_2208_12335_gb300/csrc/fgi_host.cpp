@@ -629,7 +629,7 @@ int build_plan(fgi_ctx *c, const char *tune_path)
     // species whose shells share one knot grid also get their coefficients
     // interleaved by interval, so that one point's shells read neighbouring
     // cache lines
-    std::vector<float> scoef, scoefn;
+    std::vector<float> scoef, scoefn, sbound;
     std::vector<int> shell_fn0, shell_by_l;     // per species slot: first function, radial (grouped by l)
     for (const SpeciesH &s : c->species) {
         DevSpecies d{};
@@ -673,6 +673,16 @@ int build_plan(fgi_ctx *c, const char *tune_path)
                     const size_t src = 8 * ((size_t)drad[s.shells[i]].coef_off + k);
                     scoefn.insert(scoefn.end(), coef_ddn.begin() + src, coef_ddn.begin() + src + 8);
                 }
+            if (r0.nk < 65536) {
+                const size_t ns = s.shells.size();
+                d.sbound_stride = (int)((ns + 3) / 4 * 4);
+                d.sbound_off = (long long)sbound.size();
+                sbound.resize(sbound.size() + (size_t)d.sbound_stride * (r0.nk - 1), 0.f);
+                float *dst = sbound.data() + d.sbound_off;
+                for (int k = 0; k < r0.nk - 1; k++)
+                    for (size_t i = 0; i < ns; i++)
+                        dst[(size_t)k * d.sbound_stride + i] = rbound[drad[s.shells[lord[i]]].bound_off + k];
+            }
         }
         shell_rad.insert(shell_rad.end(), s.shells.begin(), s.shells.end());
         for (int i : lord) {
@@ -699,6 +709,7 @@ int build_plan(fgi_ctx *c, const char *tune_path)
     }
     if (scoef.empty()) scoef.assign(8, 0.f);
     if (scoefn.empty()) scoefn.assign(8, 0.f);
+    if (sbound.empty()) sbound.assign(4, 0.f);
     BigVec<double> px(c->n_pts), py(c->n_pts), pz(c->n_pts);
 #pragma omp parallel for schedule(static)
     for (int64_t p = 0; p < c->n_pts; p++) {
@@ -762,7 +773,7 @@ int build_plan(fgi_ctx *c, const char *tune_path)
            i_sv0 = add(sys_val0.data(), sys_val0.size() * 8), i_sf0 = add(sys_fn0.data(), sys_fn0.size() * 8),
            i_fsys = add(c->fn_sys.data(), c->fn_sys.size() * 4), i_status = add(nullptr, 64),
            i_snnz = add(sys_nnz.data(), sys_nnz.size() * 8), i_colg = add(col_glob.data(), col_glob.size() * 4),
-           i_rbnd = add(rbound.data(), rbound.size() * 4);
+           i_rbnd = add(rbound.data(), rbound.size() * 4), i_sbnd = add(sbound.data(), sbound.size() * 4);
     cudaError_t e = cudaMalloc((void **)&c->d_arena, total);
     if (e != cudaSuccess) {
         c->d_arena = nullptr;
@@ -810,6 +821,7 @@ int build_plan(fgi_ctx *c, const char *tune_path)
     c->d_sys_nnz = (long long *)at(i_snnz);
     P.col_glob = (const int *)at(i_colg);
     P.rbound = (const float *)at(i_rbnd);
+    P.sbound = (const float *)at(i_sbnd);
     c->d_status = (int *)at(i_status);
 
     // tensor-core path plan (operand images, tiles, waves)

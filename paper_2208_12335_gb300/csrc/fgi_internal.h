@@ -36,6 +36,8 @@ struct DevSpecies {
     int nk;               // shared grid: knots
     float inv_h_hi, inv_h_lo;   // shared grid: 1/h as a double-float
     int lmax;             // largest angular momentum of its shells
+    int sbound_stride;    // floats per interval of its interleaved bounds (0: none, see DevPlan::sbound)
+    long long sbound_off; // first of them in DevPlan::sbound
     int nl[4];            // shells of each l (DevPlan::shells holds them grouped by l)
 };
 
@@ -115,6 +117,10 @@ struct DevPlan {
     // [16] max |Y_lm| (index l*l + l + m), then per radial, per knot
     // interval k, a bound of |u(r)/r| over r >= k h
     const float *rbound;
+    // the same bounds for species on one knot grid of fewer than 65536 knots,
+    // interleaved by interval in the order of DevPlan::shells and padded with
+    // zeros to four shells, so that one 16-byte load serves four shells
+    const float *sbound;
 };
 
 // ---- launchers (return the launch status) ----

@@ -196,11 +196,15 @@ __device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 lo, __nv_bfloat16 hi
     return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
 }
 
-// byte offset of the 16-byte unit (row r, 8-column group g) inside chunk (blk, c)
+// byte offset (plane 0) of the 16-byte unit (row r, 8-column group g) inside
+// chunk (blk, c); a chunk's three planes follow each other
 __device__ __forceinline__ long long unit_offset(int blk, int nchunk, int c, int r, int g)
 {
-    return ((long long)(blk * nchunk + c) * 16 + (r >> 3)) * 1024 + (r & 7) * 128 + ((g ^ (r & 7)) << 4);
+    return (long long)(blk * nchunk + c) * kChunkStride + r * 128 + ((g ^ (r & 7)) << 4);
 }
+
+// Adding and subtracting it rounds |x| < 2^22 to the nearest integer (ties to even)
+constexpr float kRoundMagic = 12582912.f;            // 1.5 * 2^23
 
 // Normalisation constants of the real spherical harmonics as double-floats.
 #define FGI_DF_CONST(c) {(float)(c), (float)((c) - (double)(float)(c))}
@@ -248,7 +252,7 @@ __device__ __forceinline__ void split3_df(df x, __nv_bfloat16 &a, __nv_bfloat16 
     c = __float2bfloat16_rn(r);
 }
 
-__device__ __forceinline__ void store_split8_df(uint8_t *dst, long long plane, const df *x, int n_split)
+__device__ __forceinline__ void store_split8_df(uint8_t *dst, const df *x, int n_split)
 {
     uint32_t w0[4], w1[4], w2[4];
 #pragma unroll
@@ -261,8 +265,8 @@ __device__ __forceinline__ void store_split8_df(uint8_t *dst, long long plane, c
         w2[q] = pack_bf16(a2, b2);
     }
     *reinterpret_cast<uint4 *>(dst) = make_uint4(w0[0], w0[1], w0[2], w0[3]);
-    if (n_split > 1) *reinterpret_cast<uint4 *>(dst + plane) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
-    if (n_split > 2) *reinterpret_cast<uint4 *>(dst + 2 * plane) = make_uint4(w2[0], w2[1], w2[2], w2[3]);
+    if (n_split > 1) *reinterpret_cast<uint4 *>(dst + kChunkBytes) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
+    if (n_split > 2) *reinterpret_cast<uint4 *>(dst + 2 * kChunkBytes) = make_uint4(w2[0], w2[1], w2[2], w2[3]);
 }
 
 // Split with a fixed-point leading term: x0 = m * unit, m = rint(x / unit),
@@ -283,7 +287,7 @@ __device__ __forceinline__ void split_fixed(df x, float scale, float unit, __nv_
     c = __float2bfloat16_rn((d - __bfloat162float(b)) + x.lo);
 }
 
-__device__ __forceinline__ void store_fixed8(uint8_t *dst, long long plane, const df *x, float scale, float unit)
+__device__ __forceinline__ void store_fixed8(uint8_t *dst, const df *x, float scale, float unit)
 {
     uint32_t w0[4], w1[4], w2[4];
 #pragma unroll
@@ -296,8 +300,8 @@ __device__ __forceinline__ void store_fixed8(uint8_t *dst, long long plane, cons
         w2[q] = pack_bf16(a2, b2);
     }
     *reinterpret_cast<uint4 *>(dst) = make_uint4(w0[0], w0[1], w0[2], w0[3]);
-    *reinterpret_cast<uint4 *>(dst + plane) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
-    *reinterpret_cast<uint4 *>(dst + 2 * plane) = make_uint4(w2[0], w2[1], w2[2], w2[3]);
+    *reinterpret_cast<uint4 *>(dst + kChunkBytes) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
+    *reinterpret_cast<uint4 *>(dst + 2 * kChunkBytes) = make_uint4(w2[0], w2[1], w2[2], w2[3]);
 }
 
 // Power-of-two scale 2^(b-e) and unit 2^(e-b) for a row whose largest |x|
@@ -350,8 +354,6 @@ __device__ __forceinline__ float radial_over_d_f32(const DevRadial &R, const flo
     return u * ip;
 }
 
-constexpr int kPhiValStride = 33;   // float2 per row of phi_smem (32 points + padding)
-
 // Interval-0 entry of shell sh's spline and the distance between interval
 // entries: the species' interleaved table when its shells share one grid.
 __device__ __forceinline__ const float4 *spline_tab(const DevPlan &P, const DevSpecies &S, const DevRadial &R, int sh,
@@ -377,37 +379,33 @@ __device__ __forceinline__ const float4 *spline_tab(const DevPlan &P, const DevS
 // slower: the doubled per-lane state costs occupancy or spills, and these
 // kernels wait mostly on their loads.)
 
-// byte offset of element (row r, point p) in the image chunk grid of block I
-// (below 2^31: a batch's image plane is at most 64 blocks x 16 chunks x 16 KB)
-__device__ __forceinline__ int elem_offset(int I, int nc_alloc, int r, int p)
-{
-    const int g = (p >> 3) & 7;
-    return ((I * nc_alloc + (p >> 6)) * 16 + (r >> 3)) * 1024 + (r & 7) * 128 + ((g ^ (r & 7)) << 4) + (p & 7) * 2;
-}
-
 // One value split on its row's or point's grid (split_fixed; NSPLIT 1:
 // plain BF16) and stored as one 16-bit BF16 per plane
 template <int NSPLIT>
-__device__ __forceinline__ void store_value(uint8_t *dst, long long plane, df x, float scale, float unit)
+__device__ __forceinline__ void store_value(uint8_t *dst, df x, float scale, float unit)
 {
     if (NSPLIT == 3) {
-        __nv_bfloat16 a, b, c;
-        split_fixed(x, scale, unit, a, b, c);
-        *reinterpret_cast<unsigned short *>(dst) = __bfloat16_as_ushort(a);
-        *reinterpret_cast<unsigned short *>(dst + plane) = __bfloat16_as_ushort(b);
-        *reinterpret_cast<unsigned short *>(dst + 2 * plane) = __bfloat16_as_ushort(c);
+        // split_fixed with the rounding to an integer as an addition (the FRND
+        // unit has a sixteenth of the FADD rate): |x scale| <= 2^8, far inside
+        // 2^22.  x0 has at most 9 significant bits, 8 below a power of two: its
+        // BF16 form is the upper half of the word.
+        const float x0 = (fmaf(x.hi, scale, kRoundMagic) - kRoundMagic) * unit;
+        const float d = x.hi - x0;
+        const __nv_bfloat16 b = __float2bfloat16_rn(d);
+        const __nv_bfloat16 c = __float2bfloat16_rn((d - __bfloat162float(b)) + x.lo);
+        *reinterpret_cast<unsigned short *>(dst) = (unsigned short)(__float_as_uint(x0) >> 16);
+        *reinterpret_cast<unsigned short *>(dst + kChunkBytes) = __bfloat16_as_ushort(b);
+        *reinterpret_cast<unsigned short *>(dst + 2 * kChunkBytes) = __bfloat16_as_ushort(c);
     } else {
         *reinterpret_cast<unsigned short *>(dst) = __bfloat16_as_ushort(__float2bfloat16_rn(x.hi));
     }
 }
 
-__device__ __forceinline__ void store_zero(uint8_t *dst, long long plane, int nsplit)
+template <int NSPLIT>
+__device__ __forceinline__ void store_zero(uint8_t *dst)
 {
-    *reinterpret_cast<unsigned short *>(dst) = 0;
-    if (nsplit > 1) {
-        *reinterpret_cast<unsigned short *>(dst + plane) = 0;
-        *reinterpret_cast<unsigned short *>(dst + 2 * plane) = 0;
-    }
+#pragma unroll
+    for (int pl = 0; pl < NSPLIT; pl++) *reinterpret_cast<unsigned short *>(dst + pl * kChunkBytes) = 0;
 }
 
 // Ratios of the other normalisation constants of an l shell to its first
@@ -456,6 +454,10 @@ __device__ __forceinline__ void emit_shell_lane(const df *rk, float x, float y, 
     constexpr int NM = 2 * L + 1;
     constexpr int NG = L < 2 ? 1 : (L == 2 ? 2 : 4);
     constexpr int G0 = L == 2 ? 0 : 1;               // first kYlmRatio entry of groups 1..
+    if constexpr (L == 0) {                          // the angular factor is 1
+        if (f0 >= f_lo && f0 < f_hi) emit(f0, rk);
+        return;
+    }
     float Q[NM];
     int gi[7];
     ylm_poly_unit<L>(x, y, z, Q, gi);
@@ -479,46 +481,75 @@ __device__ __forceinline__ void emit_shell_lane(const df *rk, float x, float y, 
     }
 }
 
+// a point's or an atom's coordinates as double-floats (24 bytes, 8-byte aligned)
+struct Dd3 {
+    float2 x, y, z;
+};
+__device__ __forceinline__ Dd3 load_dd3(const float *p)
+{
+    const float2 *q = reinterpret_cast<const float2 *>(p);
+    return Dd3{__ldg(q), __ldg(q + 1), __ldg(q + 2)};
+}
+
+// FP32 difference of two positions (from the double-floats)
+__device__ __forceinline__ float3 offset_f32(const Dd3 &p, const Dd3 &a)
+{
+    return make_float3((p.x.x - a.x.x) + (p.x.y - a.x.y), (p.y.x - a.y.x) + (p.y.y - a.y.y),
+                       (p.z.x - a.z.x) + (p.z.y - a.z.y));
+}
+
+// One interval of a shell's spline: c0..c3 and the low parts of c0 and c1.
+// The 32-byte entry in one load: the lanes' intervals differ, so a load costs
+// the L1 one tag look-up per lane, and two 16-byte loads cost two.  (These
+// look-ups, with those of the bounds below, kept the L1 60 % busy beside an
+// issue rate of 64 %.  One load an entry, one for four shells' bounds and the
+// lanes without divergence: 64-atom Si cluster, 1.11 M points, H images 3.75
+// -> 2.68 ms, density images 2.62 -> 1.84 ms; 75-atom cluster with f shells,
+// two images a batch, 6.57 -> 3.72 ms.)
+struct SplineEntry {
+    float4 h;
+    float2 l;
+};
+__device__ __forceinline__ SplineEntry load_entry(const float4 *p)
+{
+    SplineEntry e;
+    asm("{\n\t.reg .f32 u0, u1;\n\t"
+        "ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,u0,u1}, [%6];\n\t}"
+        : "=f"(e.h.x), "=f"(e.h.y), "=f"(e.h.z), "=f"(e.h.w), "=f"(e.l.x), "=f"(e.l.y)
+        : "l"(p));
+    return e;
+}
+
+// u = c0 + t c1 + t^2 (c2 + t c3) at t + tl: c0 + t c1 in double-float
+__device__ __forceinline__ df spline_value(const SplineEntry &e, float t, float tl)
+{
+    const df lin = df_two_prod(t, e.h.y);
+    const float lin_lo = fmaf(t, e.l.y, fmaf(tl, e.h.y, lin.lo));
+    const float quad = (t * t) * fmaf(t, e.h.w, e.h.z);
+    const df uu = df_two_sum(e.h.x, lin.hi);
+    return df_two_sum(uu.hi, uu.lo + ((e.l.x + lin_lo) + quad));
+}
+
 // Every function [f_lo, f_hi) of atom `atom` (species S, shell table sh_tab
-// indexed from S.shell0) at the point whose double-float coordinates pp
-// holds (nullptr: no point).  emit(f, val[NIMG]) receives phi times the
-// image's scale (SCALED false: image 0 unscaled); emit0(f) a value that is
-// zero in every image (beyond the species' cutoff, or no point); zero_all()
-// is called by all 32 lanes of the warp, instead of emit0, when every lane
-// is beyond the cutoff or has no point (the warp's part of the image is then
-// cleared with 16-byte stores).  The per-point scales are folded into the
-// powers 1/d^(l+1) once per (point, atom).  All 32 lanes of the warp call
-// this together, for the same atom.
-template <int NIMG, bool SCALED, class Emit, class Emit0, class Zero>
-__device__ __forceinline__ void eval_atom_lane(const DevPlan &P, const DevSpecies &S, const DevShell *sh_tab,
-                                               int atom, const float *pp, int f_lo, int f_hi, const df *scale,
-                                               Emit &emit, Emit0 &emit0, Zero &zero_all)
+// indexed from S.shell0) at the point pp (has: there is one), for any
+// species and any point: each shell's own knots, and the point at the
+// nucleus.  emit(f, val[NIMG]) receives phi times the image's scale (SCALED
+// false: image 0 unscaled); emit0(f) a value that is zero in every image.
+template <int NIMG, bool SCALED, class Emit, class Emit0>
+__device__ __forceinline__ void eval_atom_general(const DevPlan &P, const DevSpecies &S, const DevShell *sh_tab,
+                                                  const Dd3 &aa, const Dd3 &pp, bool has, int f_lo, int f_hi,
+                                                  const df *scale, Emit &emit, Emit0 &emit0)
 {
     const df zero{0.f, 0.f};
-    bool none = pp == nullptr;
-    const float *aa = P.atom_dd + 6 * atom;
-    if (!none) {
-        // beyond the species' largest cutoff every value is zero (FP32
-        // distance, relative error ~1e-7, against the cutoff with a 1e-5 margin)
-        const float xf = (pp[0] - aa[0]) + (pp[1] - aa[1]);
-        const float yf = (pp[2] - aa[2]) + (pp[3] - aa[3]);
-        const float zf = (pp[4] - aa[4]) + (pp[5] - aa[5]);
-        const float rcs = (float)S.rcut * 1.00001f;
-        none = xf * xf + yf * yf + zf * zf > rcs * rcs;
-    }
-    if (__all_sync(0xffffffffu, none)) {
-        zero_all();
-        return;
-    }
-    if (none) {
+    const float3 o = offset_f32(pp, aa);
+    const float rcs = (float)S.rcut * 1.00001f;
+    if (!has || o.x * o.x + o.y * o.y + o.z * o.z > rcs * rcs) {
         for (int f = f_lo; f < f_hi; f++) emit0(f);
         return;
     }
-    // offset from the atom (the rounding of the low parts differs from point
-    // to point), d^2 (terms of one sign), 1/d from a refined rsqrtf, d = d^2/d
-    const df x = df_sub_sloppy(df{pp[0], pp[1]}, df{aa[0], aa[1]});
-    const df y = df_sub_sloppy(df{pp[2], pp[3]}, df{aa[2], aa[3]});
-    const df z = df_sub_sloppy(df{pp[4], pp[5]}, df{aa[4], aa[5]});
+    const df x = df_sub_sloppy(df{pp.x.x, pp.x.y}, df{aa.x.x, aa.x.y});
+    const df y = df_sub_sloppy(df{pp.y.x, pp.y.y}, df{aa.y.x, aa.y.y});
+    const df z = df_sub_sloppy(df{pp.z.x, pp.z.y}, df{aa.z.x, aa.z.y});
     const df d2 = df_add_sloppy(df_add_sloppy(df_mul(x, x), df_mul(y, y)), df_mul(z, z));
     const bool origin = d2.hi < 1e-24f;                 // d < 1e-12
     df d = zero, i0 = zero;
@@ -526,88 +557,116 @@ __device__ __forceinline__ void eval_atom_lane(const DevPlan &P, const DevSpecie
         i0 = df_rsqrt(d2);
         d = df_mul(d2, i0);
     }
-    // 1/d^(l+1) for l <= lmax, times each image's scale
-    df ip[NIMG][4];
-    {
-        df pw[4];
-        pw[0] = i0;
-        pw[1] = S.lmax >= 1 ? df_mul(i0, i0) : zero;
-        pw[2] = S.lmax >= 2 ? df_mul(pw[1], i0) : zero;
-        pw[3] = S.lmax >= 3 ? df_mul(pw[2], i0) : zero;
-#pragma unroll
-        for (int k = 0; k < NIMG; k++) {
-            const bool sc = SCALED || k > 0;
-#pragma unroll
-            for (int q = 0; q < 4; q++) ip[k][q] = (sc && q <= S.lmax) ? df_mul(pw[q], scale[k]) : pw[q];
-        }
-    }
     float grid_hi = -1.f, grid_lo = 0.f, t = 0.f, tl = 0.f;
-    int grid_nk = -1, kk = 0;
-    const float4 *sc = nullptr;
-    if (S.shared_grid && !origin) {
-        const df sd = df_mul(d, df{S.inv_h_hi, S.inv_h_lo});
-        kk = (int)floorf(sd.hi);
-        kk = max(0, min(kk, S.nk - 2));
-        t = sd.hi - (float)kk;
-        tl = sd.lo;
-        sc = P.scoefn + S.scoef_off + 2 * ((long long)kk * S.n_shell);
-    }
-    // the shells grouped by l: the power 1/d^(l+1) and the angular
-    // polynomial's form are fixed within a group
-    int sh = 0;
+    int grid_nk = -1, kk = 0, sh = 0;
+    df pw = i0;
     auto shells_of_l = [&](auto lc) {
         constexpr int L = decltype(lc)::value;
         constexpr int NM = 2 * L + 1;
         const int end = sh + S.nl[L];
+        if (L > 0) pw = df_mul(pw, i0);
         for (; sh < end; sh++) {
             const DevShell R = sh_tab[S.shell0 + sh];
             const int f = R.fn0;
             if (f + NM <= f_lo || f >= f_hi) continue;
-            df uu = zero;                               // C_l u(d), or its limit C_0 u'(0) d at the origin
-            bool live = d.hi < R.rcut_f;
-            if (live) {
-                if (origin) {
-                    live = L == 0;
-                    if (live) {
-                        const float4 ch = __ldg(P.coef_ddn + 2 * R.coef_off), cl = __ldg(P.coef_ddn + 2 * R.coef_off + 1);
-                        uu = df_mul(df{ch.y, cl.y}, df{R.inv_h_hi, R.inv_h_lo});   // the l = 0 limit C_0 c1/h
-                    }
-                } else {
-                    const float4 *ce;
-                    if (sc) {
-                        ce = sc + 2 * sh;
-                    } else {
-                        if (R.inv_h_hi != grid_hi || R.inv_h_lo != grid_lo || R.nk != grid_nk) {
-                            grid_hi = R.inv_h_hi;
-                            grid_lo = R.inv_h_lo;
-                            grid_nk = R.nk;
-                            const df s2 = df_mul(d, df{R.inv_h_hi, R.inv_h_lo});
-                            kk = (int)floorf(s2.hi);
-                            kk = max(0, min(kk, R.nk - 2));
-                            t = s2.hi - (float)kk;
-                            tl = s2.lo;
-                        }
-                        ce = P.coef_ddn + 2 * (R.coef_off + kk);
-                    }
-                    // u = c0 + t c1 + t^2 (c2 + t c3): c0 + t c1 in double-float
-                    const float4 ch = __ldg(ce);
-                    const float4 cl = __ldg(ce + 1);
-                    const df lin = df_two_prod(t, ch.y);
-                    const float lin_lo = fmaf(t, cl.y, fmaf(tl, ch.y, lin.lo));
-                    const float quad = (t * t) * fmaf(t, ch.w, ch.z);
-                    uu = df_two_sum(ch.x, lin.hi);
-                    uu = df_two_sum(uu.hi, uu.lo + ((cl.x + lin_lo) + quad));
-                }
-            }
-            if (!live) {
+            if (!(d.hi < R.rcut_f) || (origin && L > 0)) {
                 const int m0 = max(f, f_lo), m1 = min(f + NM, f_hi);
                 for (int m = m0; m < m1; m++) emit0(m);
                 continue;
             }
             df rk[NIMG];
+            if (origin) {                               // the l = 0 limit C_0 c1/h
+                const SplineEntry e = load_entry(P.coef_ddn + 2 * R.coef_off);
+                const df u = df_mul(df{e.h.y, e.l.y}, df{R.inv_h_hi, R.inv_h_lo});
 #pragma unroll
-            for (int k = 0; k < NIMG; k++)
-                rk[k] = origin ? ((SCALED || k > 0) ? df_mul(uu, scale[k]) : uu) : df_mul(uu, ip[k][L]);
+                for (int k = 0; k < NIMG; k++) rk[k] = (SCALED || k > 0) ? df_mul(u, scale[k]) : u;
+            } else {
+                if (R.inv_h_hi != grid_hi || R.inv_h_lo != grid_lo || R.nk != grid_nk) {
+                    grid_hi = R.inv_h_hi;
+                    grid_lo = R.inv_h_lo;
+                    grid_nk = R.nk;
+                    const df s2 = df_mul(d, df{R.inv_h_hi, R.inv_h_lo});
+                    kk = (int)floorf(s2.hi);
+                    kk = max(0, min(kk, R.nk - 2));
+                    t = s2.hi - (float)kk;
+                    tl = s2.lo;
+                }
+                const df u = spline_value(load_entry(P.coef_ddn + 2 * (R.coef_off + kk)), t, tl);
+#pragma unroll
+                for (int k = 0; k < NIMG; k++) rk[k] = df_mul(u, (SCALED || k > 0) ? df_mul(pw, scale[k]) : pw);
+            }
+            emit_shell_lane<L, NIMG>(rk, x.hi, y.hi, z.hi, f, f_lo, f_hi, emit);
+        }
+    };
+    shells_of_l(std::integral_constant<int, 0>{});
+    if (S.lmax >= 1) shells_of_l(std::integral_constant<int, 1>{});
+    if (S.lmax >= 2) shells_of_l(std::integral_constant<int, 2>{});
+    if (S.lmax >= 3) shells_of_l(std::integral_constant<int, 3>{});
+}
+
+// The same for the 32 lanes of a warp together (one atom, a point each).
+// Warps whose lanes are all beyond the species' cutoff call zero_all() and
+// clear their part of the image with 16-byte stores.  Where the species'
+// shells share one knot grid (and no lane sits on the nucleus) the lanes run
+// one path without divergence: a lane beyond the cutoff or without a point
+// multiplies by zero instead of branching, the interval and its fraction are
+// found once, and the next shell's coefficients load while the present ones
+// are used.  The order of operations of a value is that of the general path.
+template <int NIMG, bool SCALED, class Emit, class Emit0, class Zero>
+__device__ __forceinline__ void eval_atom_warp(const DevPlan &P, const DevSpecies &S, const DevShell *sh_tab,
+                                               const Dd3 &aa, const Dd3 &pp, bool has, int f_lo, int f_hi,
+                                               const df *scale, Emit &emit, Emit0 &emit0, Zero &zero_all)
+{
+    const df zero{0.f, 0.f};
+    // beyond the species' largest cutoff every value is zero (FP32 distance,
+    // relative error ~1e-7, against the cutoff with a 1e-5 margin)
+    const float3 o = offset_f32(pp, aa);
+    const float rcs = (float)S.rcut * 1.00001f;
+    bool none = !has || o.x * o.x + o.y * o.y + o.z * o.z > rcs * rcs;
+    if (__all_sync(0xffffffffu, none)) {
+        zero_all();
+        return;
+    }
+    // offset from the atom (the rounding of the low parts differs from point
+    // to point), d^2 (terms of one sign), 1/d from a refined rsqrtf, d = d^2/d
+    const df x = df_sub_sloppy(df{pp.x.x, pp.x.y}, df{aa.x.x, aa.x.y});
+    const df y = df_sub_sloppy(df{pp.y.x, pp.y.y}, df{aa.y.x, aa.y.y});
+    const df z = df_sub_sloppy(df{pp.z.x, pp.z.y}, df{aa.z.x, aa.z.y});
+    const df d2 = df_add_sloppy(df_add_sloppy(df_mul(x, x), df_mul(y, y)), df_mul(z, z));
+    if (!S.shared_grid || __any_sync(0xffffffffu, !none && d2.hi < 1e-24f)) {
+        eval_atom_general<NIMG, SCALED>(P, S, sh_tab, aa, pp, has, f_lo, f_hi, scale, emit, emit0);
+        return;
+    }
+    const df i0 = df_rsqrt(d2);
+    const df d = df_mul(d2, i0);
+    const bool live = !none && d.hi < sh_tab[S.shell0].rcut_f;
+    const df sd = df_mul(d, df{S.inv_h_hi, S.inv_h_lo});
+    const int kk = live ? max(0, min((int)floorf(sd.hi), S.nk - 2)) : 0;
+    const float t = sd.hi - (float)kk, tl = sd.lo;
+    const float4 *ce = P.scoefn + S.scoef_off + 2 * ((long long)kk * S.n_shell);
+    SplineEntry next = load_entry(ce);
+    int sh = 0;
+    df pw = i0;                                         // 1/d^(l+1)
+    auto shells_of_l = [&](auto lc) {
+        constexpr int L = decltype(lc)::value;
+        constexpr int NM = 2 * L + 1;
+        const int end = sh + S.nl[L];
+        if (L > 0) pw = df_mul(pw, i0);
+        df ip[NIMG];                                    // times each image's scale
+#pragma unroll
+        for (int k = 0; k < NIMG; k++) ip[k] = (SCALED || k > 0) ? df_mul(pw, scale[k]) : pw;
+        for (; sh < end; sh++) {
+            const SplineEntry e = next;
+            if (sh + 1 < S.n_shell) next = load_entry(ce + 2 * (sh + 1));
+            const int f = sh_tab[S.shell0 + sh].fn0;
+            if (f + NM <= f_lo || f >= f_hi) continue;
+            const df u = spline_value(e, t, tl);
+            df rk[NIMG];
+#pragma unroll
+            for (int k = 0; k < NIMG; k++) {
+                rk[k] = df_mul(u, ip[k]);
+                if (!live) rk[k] = zero;
+            }
             emit_shell_lane<L, NIMG>(rk, x.hi, y.hi, z.hi, f, f_lo, f_hi, emit);
         }
     };
@@ -626,6 +685,9 @@ __device__ __forceinline__ const DevShell *stage_shells(const DevPlan &P, DevShe
     return smem;                                    // valid after the caller's next __syncthreads
 }
 
+// swizzled place of point column group g16 = g << 4 in row r of a chunk
+__device__ __forceinline__ uint32_t row_offset(uint32_t r, uint32_t g16) { return r * 128u + (((r << 4) ^ g16) & 0x70u); }
+
 // H images of one 128-row block: warp tasks (atom of the block, 32-point
 // group), lane = point.  NIMG 1: psi = phi sqrt|w v| on the second grid set;
 // NIMG 2: phi (first set) and w v phi (second set) into two images.
@@ -633,7 +695,7 @@ template <int NIMG, int NSPLIT>
 __device__ __forceinline__ void h_image_lanes(const DevPlan &P, const DevBatch &B, const TcBatch &T,
                                               const DevAct *act, const DevShell *sh_tab, int I, int e0, int ne,
                                               uint8_t *img0, uint8_t *img1, const float2 *wvs,
-                                              const float (*fsc)[128][2])
+                                              const float2 (*fsc)[128])
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
     const int r0 = I * 128;
@@ -644,52 +706,54 @@ __device__ __forceinline__ void h_image_lanes(const DevPlan &P, const DevBatch &
         const DevSpecies S = P.species[P.atom_species[A.atom]];
         const int f_lo = max(0, r0 - A.fn_loc), f_hi = min(S.n_fn, r0 + 128 - A.fn_loc);
         const int p = q * 32 + lane;
-        const bool live = p < B.np;
-        const float *pp = live ? P.pts_dd + 6 * (B.pt0 + p) : nullptr;
+        const bool has = p < B.np;
+        const Dd3 pp = load_dd3(P.pts_dd + 6 * (B.pt0 + (has ? p : 0)));
+        const Dd3 aa = load_dd3(P.atom_dd + 6 * A.atom);
         df scale[NIMG];
-        const float2 s2 = live ? wvs[p] : make_float2(0.f, 0.f);
+        const float2 s2 = has ? wvs[p] : make_float2(0.f, 0.f);
 #pragma unroll
         for (int k = 0; k < NIMG; k++) scale[k] = df{s2.x, s2.y};
         const int rb = A.fn_loc - r0;
+        uint8_t *const c0 = img0 + (long long)(I * T.nc_alloc + (q >> 1)) * kChunkStride;
+        uint8_t *const c1 = img1 + (long long)(I * T.nc_alloc + (q >> 1)) * kChunkStride;
+        const uint32_t g16 = (uint32_t)((p >> 3) & 7) << 4, pb = (uint32_t)(p & 7) * 2u;
         auto emit = [&](int f, const df *val) {
             const int r = rb + f;
-            const int off = elem_offset(I, T.nc_alloc, r, p);
+            const uint32_t off = row_offset((uint32_t)r, g16) + pb;
 #pragma unroll
             for (int k = 0; k < NIMG; k++) {
-                const int set = NIMG == 1 ? 1 : k;
-                store_value<NSPLIT>((k == 0 ? img0 : img1) + off, T.plane_phi, val[k], fsc[set][r][0],
-                                    fsc[set][r][1]);
+                const float2 su = fsc[NIMG == 1 ? 1 : k][r];
+                store_value<NSPLIT>((k == 0 ? c0 : c1) + off, val[k], su.x, su.y);
             }
         };
         auto emit0 = [&](int f) {
-            const int off = elem_offset(I, T.nc_alloc, rb + f, p);
+            const uint32_t off = row_offset((uint32_t)(rb + f), g16) + pb;
 #pragma unroll
-            for (int k = 0; k < NIMG; k++) store_zero((k == 0 ? img0 : img1) + off, T.plane_phi, NSPLIT);
+            for (int k = 0; k < NIMG; k++) store_zero<NSPLIT>((k == 0 ? c0 : c1) + off);
         };
         // the warp's 32 columns of rows rb + [f_lo, f_hi): four 16-byte units
         // per row and plane
         auto zero_all = [&]() {
-            const int pc = q * 32;
             for (int u = lane; u < (f_hi - f_lo) * 4; u += 32) {
-                const int off = elem_offset(I, T.nc_alloc, rb + f_lo + (u >> 2), pc + (u & 3) * 8);
+                const uint32_t off = row_offset((uint32_t)(rb + f_lo + (u >> 2)),
+                                                (uint32_t)((q & 1) * 4 + (u & 3)) << 4);
 #pragma unroll
                 for (int k = 0; k < NIMG; k++)
 #pragma unroll
                     for (int pl = 0; pl < NSPLIT; pl++)
-                        *reinterpret_cast<uint4 *>((k == 0 ? img0 : img1) + off + pl * T.plane_phi) =
+                        *reinterpret_cast<uint4 *>((k == 0 ? c0 : c1) + off + pl * kChunkBytes) =
                             make_uint4(0u, 0u, 0u, 0u);
             }
         };
-        eval_atom_lane<NIMG, NIMG == 1>(P, S, sh_tab, A.atom, pp, f_lo, f_hi, scale, emit, emit0, zero_all);
+        eval_atom_warp<NIMG, NIMG == 1>(P, S, sh_tab, aa, pp, has, f_lo, f_hi, scale, emit, emit0, zero_all);
     }
 }
 
 // -------------------------------------------- basis -> operand images (K1)
-// CTA per (batch, 128-row block).  A first FP32 pass takes the rows' maxima
-// and sums for the fixed-point grids; then, for each 32-point half chunk,
-// phi of the block's rows is evaluated into shared memory and the split
-// planes of psi = phi sqrt|w v| (batches where w v has one sign) or of phi
-// and w v phi (mixed signs) are written as swizzled 16-byte units.
+// CTA per (batch, 128-row block).  A first pass takes bounds of the rows'
+// maxima and sums for the fixed-point grids; then every function is evaluated
+// lane per point and the split planes of psi = phi sqrt|w v| (batches where
+// w v has one sign) or of phi and w v phi (mixed signs) are written.
 //
 // The radial factor N_lm u(d)/d^(l+1) -- shared by all angular points of a
 // radial shell, so its rounding would be systematic -- is evaluated in
@@ -698,30 +762,105 @@ __device__ __forceinline__ void h_image_lanes(const DevPlan &P, const DevBatch &
 // rounding varies from point to point).
 
 constexpr int kPhiThreads = 256;
-constexpr int kDistCacheFloats = 128 * kPhiValStride * 2;     // the dynamic buffer, as floats
+constexpr int kKnotCache = 8448;                      // (atom, point) knots of the bound pass kept in shared memory
+constexpr int kGeoCache = 128 * 33 / 2;               // float4 slots of the pass over the points
 
 // FP32 distance from atom `atom` to point `pt` (from the double-float
 // coordinates), for the bounds of the digit grids
 __device__ __forceinline__ float point_atom_dist_f32(const DevPlan &P, int atom, long long pt)
 {
-    const float *aa = P.atom_dd + 6 * atom;
-    const float *pp = P.pts_dd + 6 * pt;
-    const float x = (pp[0] - aa[0]) + (pp[1] - aa[1]);
-    const float y = (pp[2] - aa[2]) + (pp[3] - aa[3]);
-    const float z = (pp[4] - aa[4]) + (pp[5] - aa[5]);
-    return sqrtf(x * x + y * y + z * z);
+    const float3 o = offset_f32(load_dd3(P.pts_dd + 6 * pt), load_dd3(P.atom_dd + 6 * atom));
+    return sqrtf(o.x * o.x + o.y * o.y + o.z * o.z);
+}
+
+// Knot interval of distance d from below (against FP32 rounding of d) for the
+// suffix bounds of |u(r)/r|, or kNoKnot beyond the cutoff
+constexpr int kNoKnot = 0xFFFF;
+__device__ __forceinline__ int knot_below(float d, float rcut_f, float inv_h, int nk)
+{
+    if (!(d < rcut_f * 1.00001f)) return kNoKnot;
+    return min(max((int)(d * 0.999999f * inv_h), 0), nk - 2);
+}
+
+// lane m folds function m of a shell (first function f1 of its atom, 2l+1 of
+// them) into its row: the bound of the radial factor times max |Y_lm|
+__device__ __forceinline__ void fold_row(const DevPlan &P, const DevShell &R, int fn_loc, int r0, int f_lo, int f_hi,
+                                         int lane, float m, float s, unsigned int *rowmax, float *rowsum)
+{
+    const int fr = R.fn0 + lane;
+    if (lane < 2 * R.l + 1 && m > 0.f && fr >= f_lo && fr < f_hi) {
+        const int row = fn_loc + fr - r0;
+        const float yl = __ldg(P.rbound + R.l * R.l + lane);
+        rowmax[row] = __float_as_uint(fminf(m * yl, 1.0e30f));
+        rowsum[row] = fminf(s * 1.0001f * yl, 1.0e30f);       // 1.0001: FP32 sums
+    }
+}
+
+__device__ __forceinline__ float warp_sum(float s)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+// Row bounds of one atom's functions from the interleaved table of its
+// species: four shells per task, one 16-byte look-up per point for all four.
+// MIXED: also the bounds of |phi| itself (set 0), which only batches with
+// both signs use.
+template <bool MIXED>
+__device__ __forceinline__ void row_bounds_quad(const DevPlan &P, const DevBatch &B, const DevAct &A,
+                                                const DevSpecies &S, const DevShell *sh_tab, int quad, int r0, int f_lo,
+                                                int f_hi, const unsigned short *kc, const float *wvf,
+                                                unsigned int (*rowmax)[128], float (*rowsum)[128])
+{
+    const int lane = threadIdx.x & 31;
+    const float *bt = P.sbound + S.sbound_off + 4 * quad;
+    float m0[4] = {}, m1[4] = {}, s0[4] = {}, s1[4] = {};
+    for (int p = lane; p < B.np; p += 32) {
+        const int ki = kc ? (int)kc[p]
+                          : knot_below(point_atom_dist_f32(P, A.atom, B.pt0 + p), sh_tab[S.shell0].rcut_f, S.inv_h_hi, S.nk);
+        if (ki != kNoKnot) {
+            const float4 t4 = __ldg(reinterpret_cast<const float4 *>(bt + (long long)ki * S.sbound_stride));
+            const float t[4] = {t4.x, t4.y, t4.z, t4.w};
+            const float w = wvf[p];
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const float tw = t[j] * w;
+                m1[j] = fmaxf(m1[j], tw);
+                s1[j] += tw;
+                if (MIXED) {
+                    m0[j] = fmaxf(m0[j], t[j]);
+                    s0[j] += t[j];
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        const int sh = 4 * quad + j;
+        if (sh >= S.n_shell) break;
+        const DevShell R = sh_tab[S.shell0 + sh];
+        if (R.fn0 + 2 * R.l + 1 <= f_lo || R.fn0 >= f_hi) continue;
+        const float a1 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m1[j]))), b1 = warp_sum(s1[j]);
+        fold_row(P, R, A.fn_loc, r0, f_lo, f_hi, lane, a1, b1, rowmax[1], rowsum[1]);
+        if (MIXED) {
+            const float a0 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m0[j])));
+            const float b0 = warp_sum(s0[j]);
+            fold_row(P, R, A.fn_loc, r0, f_lo, f_hi, lane, a0, b0, rowmax[0], rowsum[0]);
+        }
+    }
 }
 
 __global__ void __launch_bounds__(kPhiThreads, 4) k_tc_phi(DevPlan P, const TcBatch *tb, const WorkItem *items,
                                                 uint8_t *ws, const double *v, int n_split, int fixed,
                                                 int *bsign, int bound)
 {
-    extern __shared__ float2 phi_smem[];             // [128][kPhiValStride] double-float values
+    extern __shared__ float4 phi_smem[];            // knots of the bound pass, or offsets of the pass over the points
     __shared__ float2 wvs[kMaxBatchPoints];         // per-point image scale (double-float)
     __shared__ DevShell shs[kMaxShellsSmem];
     __shared__ unsigned int rowmax[2][128];          // |phi|, |w v phi| maxima (float bits)
     __shared__ float rowsum[2][128];                 // sums of |phi|, |w v phi| over the points
-    __shared__ float fsc[2][128][2];                 // per row: scale, unit
+    __shared__ float2 fsc[2][128];                   // per row: scale, unit
     __shared__ float wvf[kMaxBatchPoints];           // |w v| per point (FP32), first pass
     const WorkItem it = items[blockIdx.x];
     const DevBatch B = P.batches[it.batch];
@@ -765,20 +904,23 @@ __global__ void __launch_bounds__(kPhiThreads, 4) k_tc_phi(DevPlan P, const TcBa
             const float a = fabsf((float)(P.pw[B.pt0 + p] * v[B.pt0 + p])) * (1.f + 1.f / 1048576.f);
             wvf[p] = fminf(sgn != 0 ? sqrtf(a) * (1.f + 1.f / 1048576.f) : a, 1.0e30f);
         }
-        // distances of the block's atoms to the batch's points (FP32), once,
-        // in the dynamic buffer when they fit
-        float *dcache = reinterpret_cast<float *>(phi_smem);
-        const bool dcached = ne * B.np <= kDistCacheFloats;
-        if (dcached) {
+        // knots of the points on the block's atoms' grids, once, when they fit
+        unsigned short *kcache = reinterpret_cast<unsigned short *>(phi_smem);
+        const bool cached = ne * B.np <= kKnotCache;
+        if (cached) {
             for (int q = threadIdx.x; q < ne * B.np; q += blockDim.x) {
                 const int eq = q / B.np, p = q - eq * B.np;
-                dcache[q] = point_atom_dist_f32(P, act[e0 + eq].atom, B.pt0 + p);
+                const int atom = act[e0 + eq].atom;
+                const DevSpecies &S = P.species[P.atom_species[atom]];
+                if (S.sbound_stride > 0)
+                    kcache[q] = (unsigned short)knot_below(point_atom_dist_f32(P, atom, B.pt0 + p),
+                                                           sh_tab[S.shell0].rcut_f, S.inv_h_hi, S.nk);
             }
         }
         __syncthreads();
-        // warp tasks (atom of the block, shell): the lanes stride over the
-        // batch's points, one lookup per point, and keep the maxima and sums in
-        // registers; one warp reduction per task, whose rows it alone writes
+        // warp tasks (atom of the block, four of its shells): the lanes stride
+        // over the batch's points and keep the maxima and sums in registers;
+        // one warp reduction per shell, whose rows the warp alone writes
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
         int job0 = 0;
         for (int e = e0; e <= e1; e++) {
@@ -786,18 +928,29 @@ __global__ void __launch_bounds__(kPhiThreads, 4) k_tc_phi(DevPlan P, const TcBa
             const DevSpecies S = P.species[P.atom_species[A.atom]];
             const int f_lo = max(0, r0 - A.fn_loc), f_hi = min(S.n_fn, r0 + 128 - A.fn_loc);
             const int first = ((warp - job0) % nwarp + nwarp) % nwarp;
+            if (S.sbound_stride > 0) {
+                const int nq = (S.n_shell + 3) >> 2;
+                job0 += nq;
+                const unsigned short *kc = cached ? kcache + (e - e0) * B.np : nullptr;
+                for (int qd = first; qd < nq; qd += nwarp) {
+                    if (sgn != 0)
+                        row_bounds_quad<false>(P, B, A, S, sh_tab, qd, r0, f_lo, f_hi, kc, wvf, rowmax, rowsum);
+                    else
+                        row_bounds_quad<true>(P, B, A, S, sh_tab, qd, r0, f_lo, f_hi, kc, wvf, rowmax, rowsum);
+                }
+                continue;
+            }
+            // shells on knot grids of their own (or too long for the cache's index)
             job0 += S.n_shell;
             for (int sh = first; sh < S.n_shell; sh += nwarp) {
                 const DevShell R = sh_tab[S.shell0 + sh];
-                const int nm = 2 * R.l + 1, f1 = R.fn0;
-                if (f1 + nm <= f_lo || f1 >= f_hi) continue;
+                if (R.fn0 + 2 * R.l + 1 <= f_lo || R.fn0 >= f_hi) continue;
                 const float rcl = R.rcut_f * 1.00001f;
                 const float *bt = P.rbound + R.bound_off;
                 float m0 = 0.f, m1 = 0.f, s0 = 0.f, s1 = 0.f;
                 for (int p = lane; p < B.np; p += 32) {
-                    const float d = dcached ? dcache[(e - e0) * B.np + p] : point_atom_dist_f32(P, A.atom, B.pt0 + p);
+                    const float d = point_atom_dist_f32(P, A.atom, B.pt0 + p);
                     if (d < rcl) {
-                        // knot index taken from below against FP32 rounding of d
                         const int ki = min(max((int)(d * 0.999999f * R.inv_h_hi), 0), R.nk - 2);
                         const float t = __ldg(bt + ki);
                         const float tw = t * wvf[p];
@@ -809,21 +962,10 @@ __global__ void __launch_bounds__(kPhiThreads, 4) k_tc_phi(DevPlan P, const TcBa
                 }
                 m0 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m0)));
                 m1 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m1)));
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-                    s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-                }
-                // lane m folds function m of the shell into its row
-                const int fr = f1 + lane;
-                if (lane < nm && m0 > 0.f && fr >= f_lo && fr < f_hi) {
-                    const int row = A.fn_loc + fr - r0;
-                    const float yl = __ldg(P.rbound + R.l * R.l + lane);
-                    rowmax[0][row] = __float_as_uint(fminf(m0 * yl, 1.0e30f));
-                    rowmax[1][row] = __float_as_uint(fminf(m1 * yl, 1.0e30f));
-                    rowsum[0][row] = fminf(s0 * 1.0001f * yl, 1.0e30f);   // 1.0001: FP32 sums
-                    rowsum[1][row] = fminf(s1 * 1.0001f * yl, 1.0e30f);
-                }
+                s0 = warp_sum(s0);
+                s1 = warp_sum(s1);
+                fold_row(P, R, A.fn_loc, r0, f_lo, f_hi, lane, m0, s0, rowmax[0], rowsum[0]);
+                fold_row(P, R, A.fn_loc, r0, f_lo, f_hi, lane, m1, s1, rowmax[1], rowsum[1]);
             }
         }
         __syncthreads();
@@ -831,8 +973,7 @@ __global__ void __launch_bounds__(kPhiThreads, 4) k_tc_phi(DevPlan P, const TcBa
             const int which = q >> 7, r = q & 127;
             float sc, un;
             fixed_scale_adaptive(__uint_as_float(rowmax[which][r]), rowsum[which][r], T.nc * 64, sc, un);
-            fsc[which][r][0] = sc;
-            fsc[which][r][1] = un;
+            fsc[which][r] = make_float2(sc, un);
         }
         __syncthreads();
     } else if (fixed) {
@@ -851,8 +992,8 @@ __global__ void __launch_bounds__(kPhiThreads, 4) k_tc_phi(DevPlan P, const TcBa
         // FP32 offsets and distances of the block's atoms to the batch's points,
         // once, in the (not yet used) value buffer when they fit: every shell
         // job of an atom reads them instead of recomputing them
-        float4 *geo = reinterpret_cast<float4 *>(phi_smem);
-        const bool geo_cached = ne * B.np <= 128 * kPhiValStride / 2;    // float4 slots of the buffer
+        float4 *geo = phi_smem;
+        const bool geo_cached = ne * B.np <= kGeoCache;
         if (geo_cached) {
             for (int q = threadIdx.x; q < ne * B.np; q += blockDim.x) {
                 const int eq = q / B.np, p = q - eq * B.np;
@@ -945,8 +1086,7 @@ __global__ void __launch_bounds__(kPhiThreads, 4) k_tc_phi(DevPlan P, const TcBa
             const int which = q >> 7, r = q & 127;
             float sc, un;
             fixed_scale_adaptive(__uint_as_float(rowmax[which][r]), rowsum[which][r], T.nc * 64, sc, un);
-            fsc[which][r][0] = sc;
-            fsc[which][r][1] = un;
+            fsc[which][r] = make_float2(sc, un);
         }
         __syncthreads();
     }
@@ -975,9 +1115,48 @@ __global__ void __launch_bounds__(kPhiThreads, 4) k_tc_phi(DevPlan P, const TcBa
         const int r = nlive + u / (T.nc * 8), cg = u % (T.nc * 8);
         const long long off = unit_offset(I, T.nc_alloc, cg >> 3, r, cg & 7);
         for (int pl = 0; pl < nplanes; pl++) {
-            *reinterpret_cast<uint4 *>(phi_img + off + pl * T.plane_phi) = make_uint4(0u, 0u, 0u, 0u);
-            if (sgn == 0) *reinterpret_cast<uint4 *>(a_img + off + pl * T.plane_phi) = make_uint4(0u, 0u, 0u, 0u);
+            *reinterpret_cast<uint4 *>(phi_img + off + pl * kChunkBytes) = make_uint4(0u, 0u, 0u, 0u);
+            if (sgn == 0) *reinterpret_cast<uint4 *>(a_img + off + pl * kChunkBytes) = make_uint4(0u, 0u, 0u, 0u);
         }
+    }
+}
+
+// The density's image of one 64-point chunk: warp tasks (active atom, 32-point
+// half of the chunk), lane = point (the same point for all of a warp's
+// tasks), every function of the atom, split on the point's grid.
+template <int NSPLIT>
+__device__ __forceinline__ void density_image_lanes(const DevPlan &P, const DevBatch &B, const TcBatch &T,
+                                                    const DevAct *act, const DevShell *sh_tab, int c, uint8_t *phi_img,
+                                                    const float2 *csc)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;   // nwarp even
+    const int half = warp & 1, k = half * 32 + lane, p = c * 64 + k;
+    const bool has = p < B.np;
+    const Dd3 pp = load_dd3(P.pts_dd + 6 * (B.pt0 + (has ? p : 0)));
+    const float2 su = NSPLIT == 3 ? csc[k] : make_float2(0.f, 0.f);
+    uint8_t *const img = phi_img + (long long)c * kChunkStride;
+    const uint32_t g16 = (uint32_t)(k >> 3) << 4, pb = (uint32_t)(k & 7) * 2u;
+    const uint32_t blk = (uint32_t)T.nc_alloc * kChunkStride - 128u * 128u;   // a row block, less its rows' offsets
+    for (int e = warp >> 1; e < B.n_act; e += nwarp >> 1) {
+        const DevAct A = act[e];
+        const DevSpecies S = P.species[P.atom_species[A.atom]];
+        const Dd3 aa = load_dd3(P.atom_dd + 6 * A.atom);
+        auto place = [&](int f, uint32_t g) {
+            const uint32_t rg = (uint32_t)(A.fn_loc + f);
+            return (rg >> 7) * blk + row_offset(rg, g);
+        };
+        auto emit = [&](int f, const df *val) { store_value<NSPLIT>(img + place(f, g16) + pb, val[0], su.x, su.y); };
+        auto emit0 = [&](int f) { store_zero<NSPLIT>(img + place(f, g16) + pb); };
+        // the warp's 32 columns of the atom's rows: four 16-byte units per row and plane
+        auto zero_all = [&]() {
+            for (int u = lane; u < S.n_fn * 4; u += 32) {
+                const uint32_t off = place(u >> 2, (uint32_t)(half * 4 + (u & 3)) << 4);
+#pragma unroll
+                for (int pl = 0; pl < NSPLIT; pl++)
+                    *reinterpret_cast<uint4 *>(img + off + pl * kChunkBytes) = make_uint4(0u, 0u, 0u, 0u);
+            }
+        };
+        eval_atom_warp<1, false>(P, S, sh_tab, aa, pp, has, 0, S.n_fn, nullptr, emit, emit0, zero_all);
     }
 }
 
@@ -988,10 +1167,9 @@ __global__ void __launch_bounds__(kPhiThreads, 4) k_tc_phi(DevPlan P, const TcBa
 __global__ void __launch_bounds__(kPhiThreads, 5) k_tc_phi_cols(DevPlan P, const TcBatch *tb, const WorkItem *items,
                                                      uint8_t *ws, int n_split, int bound)
 {
-    __shared__ unsigned int colmax[64];
-    __shared__ float colsum[64];
-    __shared__ float csc[2][64];
-    __shared__ float ymax[kMaxL + 1];                // max over m of max |Y_lm|, per l
+    __shared__ float colmax[kPhiThreads / 64][64], colsum[kPhiThreads / 64][64];
+    __shared__ float2 csc[64];                       // per point: scale, unit
+    __shared__ float2 ylim[kMaxL + 1];               // per l: max over m of max |Y_lm|, bound of the sum over m
     __shared__ DevShell shs[kMaxShellsSmem];
     const WorkItem it = items[blockIdx.x];
     const DevBatch B = P.batches[it.batch];
@@ -1003,121 +1181,104 @@ __global__ void __launch_bounds__(kPhiThreads, 5) k_tc_phi_cols(DevPlan P, const
     const DevShell *sh_tab = stage_shells(P, shs);
     __syncthreads();
     if (fixed) {
-        if (threadIdx.x < 64) {
-            colmax[threadIdx.x] = 0u;
-            colsum[threadIdx.x] = 0.f;
-        }
         if (bound && threadIdx.x <= kMaxL) {
             const int l = threadIdx.x;
             float y = 0.f;
             for (int m = 0; m <= 2 * l; m++) y = fmaxf(y, __ldg(P.rbound + l * l + m));
-            ymax[l] = y;
+            // sum over m of |Y_lm| <= (2l+1)/sqrt(4 pi): Cauchy-Schwarz with
+            // sum_m Y_lm^2 = (2l+1)/(4 pi) (Unsold's theorem)
+            ylim[l] = make_float2(y, (float)(2 * l + 1) * (0.28209479f * 1.000001f));
         }
         __syncthreads();
-        for (int u = threadIdx.x; u < B.n_act * 64; u += blockDim.x) {
-            const int e = u >> 6, k = u & 63, p = c * 64 + k;
-            if (p >= B.np) continue;
-            const DevAct A = act[e];
-            const DevSpecies S = P.species[P.atom_species[A.atom]];
-            const float *pp = P.pts_dd + 6 * (B.pt0 + p);
-            const float *aa = P.atom_dd + 6 * A.atom;
-            const float x = (pp[0] - aa[0]) + (pp[1] - aa[1]);
-            const float y = (pp[2] - aa[2]) + (pp[3] - aa[3]);
-            const float z = (pp[4] - aa[4]) + (pp[5] - aa[5]);
-            const float d = sqrtf(x * x + y * y + z * z);
-            if (d > (float)S.rcut * 1.00001f) continue;        // every shell is zero here
-            float mx = 0.f, sm = 0.f;
-            if (bound) {
-                // table bounds: one lookup per shell, the knot index taken
-                // from below against FP32 rounding of d
-                const float dl = d * 0.999999f;
-                for (int sh = 0; sh < S.n_shell; sh++) {
-                    const DevShell R = sh_tab[S.shell0 + sh];
-                    if (d >= R.rcut_f * 1.00001f) continue;
-                    const int ki = min(max((int)(dl * R.inv_h_hi), 0), R.nk - 2);
-                    const float tb = __ldg(P.rbound + R.bound_off + ki);
-                    mx = fmaxf(mx, fminf(tb * ymax[R.l], 1.0e30f));
-                    // sum over m of |Y_lm| <= (2l+1)/sqrt(4 pi): Cauchy-Schwarz with
-                    // sum_m Y_lm^2 = (2l+1)/(4 pi) (Unsold's theorem)
-                    sm += fminf(tb * (float)(2 * R.l + 1) * (0.28209479f * 1.000001f), 1.0e30f);
+        // one column of the chunk and every fourth active atom per thread: the
+        // column's coordinates load once and its maximum and sum stay in
+        // registers
+        const int k = threadIdx.x & 63, part = threadIdx.x >> 6, p = c * 64 + k;
+        float mxc = 0.f, smc = 0.f;
+        if (p < B.np) {
+            const Dd3 pp = load_dd3(P.pts_dd + 6 * (B.pt0 + p));
+            for (int e = part; e < B.n_act; e += kPhiThreads / 64) {
+                const DevAct A = act[e];
+                const DevSpecies &S = P.species[P.atom_species[A.atom]];
+                const float3 o = offset_f32(pp, load_dd3(P.atom_dd + 6 * A.atom));
+                const float d = sqrtf(o.x * o.x + o.y * o.y + o.z * o.z);
+                if (d > (float)S.rcut * 1.00001f) continue;        // every shell is zero here
+                float mx = 0.f, sm = 0.f;
+                if (bound && S.sbound_stride > 0) {
+                    // table bounds, four shells a look-up
+                    const int ki = knot_below(d, sh_tab[S.shell0].rcut_f, S.inv_h_hi, S.nk);
+                    if (ki == kNoKnot) continue;
+                    const float4 *bt = reinterpret_cast<const float4 *>(P.sbound + S.sbound_off +
+                                                                        (long long)ki * S.sbound_stride);
+                    for (int q = 0; 4 * q < S.n_shell; q++) {
+                        const float4 t4 = __ldg(bt + q);
+                        const float t[4] = {t4.x, t4.y, t4.z, t4.w};
+#pragma unroll
+                        for (int j = 0; j < 4; j++) {
+                            // entries past the species' shells are zero bounds
+                            const float2 yl = ylim[sh_tab[S.shell0 + min(4 * q + j, S.n_shell - 1)].l];
+                            mx = fmaxf(mx, fminf(t[j] * yl.x, 1.0e30f));
+                            sm += fminf(t[j] * yl.y, 1.0e30f);
+                        }
+                    }
+                } else if (bound) {
+                    // table bounds: one lookup per shell, the knot index taken
+                    // from below against FP32 rounding of d
+                    const float dl = d * 0.999999f;
+                    for (int sh = 0; sh < S.n_shell; sh++) {
+                        const DevShell R = sh_tab[S.shell0 + sh];
+                        if (d >= R.rcut_f * 1.00001f) continue;
+                        const int ki = min(max((int)(dl * R.inv_h_hi), 0), R.nk - 2);
+                        const float tb = __ldg(P.rbound + R.bound_off + ki);
+                        mx = fmaxf(mx, fminf(tb * ylim[R.l].x, 1.0e30f));
+                        sm += fminf(tb * ylim[R.l].y, 1.0e30f);
+                    }
+                } else {
+                    const float inv_d = __frcp_rn(d);
+                    for (int sh = 0; sh < S.n_shell; sh++) {
+                        const DevRadial R = P.radials[P.shell_rad[S.shell0 + sh]];
+                        int tstep;
+                        const float4 *tab = spline_tab(P, S, R, sh, tstep);
+                        const float rad = radial_over_d_f32(R, tab, tstep, d, inv_d);
+                        float Q[7];
+                        int ci[7];
+                        ylm_poly_f32(R.l, o.x, o.y, o.z, Q, ci);
+#pragma unroll
+                        for (int m = 0; m < 7; m++) {
+                            if (m >= 2 * R.l + 1) break;
+                            const float a = fabsf(rad * kYlmC[ci[m]].x * Q[m]);
+                            mx = fmaxf(mx, a);
+                            sm += a;
+                        }
+                    }
+                    if (!(mx < 1.0e30f)) mx = 1.0e30f;
                 }
                 if (!(sm < 1.0e30f)) sm = 1.0e30f;
-                atomicMax(&colmax[k], __float_as_uint(mx));
-                atomicAdd(&colsum[k], sm);
-                continue;
+                mxc = fmaxf(mxc, mx);
+                smc += sm;
             }
-            const float inv_d = __frcp_rn(d);
-            for (int sh = 0; sh < S.n_shell; sh++) {
-                const DevRadial R = P.radials[P.shell_rad[S.shell0 + sh]];
-                int tstep;
-                const float4 *tab = spline_tab(P, S, R, sh, tstep);
-                const float rad = radial_over_d_f32(R, tab, tstep, d, inv_d);
-                float Q[7];
-                int ci[7];
-                ylm_poly_f32(R.l, x, y, z, Q, ci);
-#pragma unroll
-                for (int m = 0; m < 7; m++) {
-                    if (m >= 2 * R.l + 1) break;
-                    const float a = fabsf(rad * kYlmC[ci[m]].x * Q[m]);
-                    mx = fmaxf(mx, a);
-                    sm += a;
-                }
-            }
-            if (!(mx < 1.0e30f)) mx = 1.0e30f;
-            if (!(sm < 1.0e30f)) sm = 1.0e30f;
-            atomicMax(&colmax[k], __float_as_uint(mx));
-            atomicAdd(&colsum[k], sm);
         }
+        colmax[part][k] = mxc;
+        colsum[part][k] = smc;
         __syncthreads();
         if (threadIdx.x < 64) {
             float sc, un;
-            fixed_scale_adaptive(__uint_as_float(colmax[threadIdx.x]), colsum[threadIdx.x], T.nkc * 64, sc, un);
-            csc[0][threadIdx.x] = sc;
-            csc[1][threadIdx.x] = un;
+            const float mx = fmaxf(fmaxf(colmax[0][k], colmax[1][k]), fmaxf(colmax[2][k], colmax[3][k]));
+            const float sm = (colsum[0][k] + colsum[1][k]) + (colsum[2][k] + colsum[3][k]);
+            fixed_scale_adaptive(mx, sm, T.nkc * 64, sc, un);
+            csc[k] = make_float2(sc, un);
         }
         __syncthreads();
     }
-    // warp tasks (active atom, 32-point half of the chunk), lane = point:
-    // every function of the atom at the lane's point, split on the point's grid
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-    const int nsplit = fixed ? 3 : 1;
-    for (int task = warp; task < B.n_act * 2; task += nwarp) {
-        const DevAct A = act[task >> 1];
-        const DevSpecies S = P.species[P.atom_species[A.atom]];
-        const int k = (task & 1) * 32 + lane, p = c * 64 + k;
-        const float *pp = p < B.np ? P.pts_dd + 6 * (B.pt0 + p) : nullptr;
-        const float sc = fixed ? csc[0][k] : 0.f, un = fixed ? csc[1][k] : 0.f;
-        auto emit = [&](int f, const df *val) {
-            const int rg = A.fn_loc + f;
-            const int off = elem_offset(rg >> 7, T.nc_alloc, rg & 127, p);
-            if (fixed)
-                store_value<3>(phi_img + off, T.plane_phi, val[0], sc, un);
-            else
-                store_value<1>(phi_img + off, T.plane_phi, val[0], sc, un);
-        };
-        auto emit0 = [&](int f) {
-            const int rg = A.fn_loc + f;
-            store_zero(phi_img + elem_offset(rg >> 7, T.nc_alloc, rg & 127, p), T.plane_phi, nsplit);
-        };
-        // the warp's 32 columns of the atom's rows: four 16-byte units per row and plane
-        auto zero_all = [&]() {
-            const int pc = c * 64 + (task & 1) * 32;
-            for (int u = lane; u < S.n_fn * 4; u += 32) {
-                const int rg = A.fn_loc + (u >> 2);
-                const int off = elem_offset(rg >> 7, T.nc_alloc, rg & 127, pc + (u & 3) * 8);
-                for (int pl = 0; pl < nsplit; pl++)
-                    *reinterpret_cast<uint4 *>(phi_img + off + pl * T.plane_phi) = make_uint4(0u, 0u, 0u, 0u);
-            }
-        };
-        eval_atom_lane<1, false>(P, S, sh_tab, A.atom, pp, 0, S.n_fn, nullptr, emit, emit0, zero_all);
-    }
+    if (fixed) density_image_lanes<3>(P, B, T, act, sh_tab, c, phi_img, csc);
+    else density_image_lanes<1>(P, B, T, act, sh_tab, c, phi_img, csc);
     // rows [n_b, 64 nkc) of the contraction's last function chunk: zeros
     const int nplanes = fixed ? 3 : 1;
     for (int u = threadIdx.x; u < (T.nkc * 64 - B.nfn) * 8; u += blockDim.x) {
         const int rg = B.nfn + (u >> 3), g = u & 7;
         const long long off = unit_offset(rg >> 7, T.nc_alloc, c, rg & 127, g);
         for (int pl = 0; pl < nplanes; pl++)
-            *reinterpret_cast<uint4 *>(phi_img + off + pl * T.plane_phi) = make_uint4(0u, 0u, 0u, 0u);
+            *reinterpret_cast<uint4 *>(phi_img + off + pl * kChunkBytes) = make_uint4(0u, 0u, 0u, 0u);
     }
 }
 
@@ -1297,14 +1458,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_h(DevPlan P, const TcBatch
                     }
                     uint8_t *a_sm = sm + st * kStageBytes, *b_sm = a_sm + 3 * kChunkBytes;
                     mbar_expect_tx(&S->full[st], 2 * chunk);
-                    for (int s = 0; s < n_split; s++) {
-                        bulk_g2s(a_sm + s * kChunkBytes,
-                                 a_img + s * T.plane_phi + (long long)(it.tj * T.nc_alloc + c) * kChunkBytes,
-                                 kChunkBytes, &S->full[st]);
-                        bulk_g2s(b_sm + s * kChunkBytes,
-                                 b_img + s * T.plane_phi + (long long)(it.ti * T.nc_alloc + c) * kChunkBytes,
-                                 kChunkBytes, &S->full[st]);
-                    }
+                    bulk_g2s(a_sm, a_img + (long long)(it.tj * T.nc_alloc + c) * kChunkStride, chunk, &S->full[st]);
+                    bulk_g2s(b_sm, b_img + (long long)(it.ti * T.nc_alloc + c) * kChunkStride, chunk, &S->full[st]);
                 }
             }
             // do not leave while a copy may still be landing
@@ -1622,9 +1777,9 @@ __global__ void __launch_bounds__(256) k_tc_gather_d(DevPlan P, const TcBatch *t
             }
             uint8_t *dst = img + unit_offset(J, T.nkc, kc, r, g);
             if (fixed)
-                store_fixed8(dst, T.plane_d, x, rsc[0][r], rsc[1][r]);
+                store_fixed8(dst, x, rsc[0][r], rsc[1][r]);
             else
-                store_split8_df(dst, T.plane_d, x, n_split);
+                store_split8_df(dst, x, n_split);
         }
     }
 }
@@ -1685,16 +1840,13 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_density(DevPlan P, const T
                     uint8_t *a_sm = sm + st * kStageBytes, *b_sm = a_sm + 3 * kChunkBytes;
                     mbar_expect_tx(&S->full[st], 2 * chunk);
                     const int I = kc >> 1, half = kc & 1;
-                    for (int s = 0; s < n_split; s++) {
-                        bulk_g2s(a_sm + s * kChunkBytes,
-                                 d_img + s * T.plane_d + (long long)(J * T.nkc + kc) * kChunkBytes, kChunkBytes,
-                                 &S->full[st]);
+                    bulk_g2s(a_sm, d_img + (long long)(J * T.nkc + kc) * kChunkStride, chunk, &S->full[st]);
+                    for (int s = 0; s < n_split; s++)
                         for (int c2 = 0; c2 < 2; c2++)
                             bulk_g2s(b_sm + s * kChunkBytes + c2 * 8192,
-                                     phi_img + s * T.plane_phi +
-                                         ((long long)(I * T.nc_alloc + 2 * m + c2) * 16 + 8 * half) * 1024,
+                                     phi_img + (long long)(I * T.nc_alloc + 2 * m + c2) * kChunkStride +
+                                         s * kChunkBytes + half * 8192,
                                      8192, &S->full[st]);
-                    }
                 }
             }
             for (long long q = (n > kStages ? n - kStages : 0); q < n; q++)
@@ -1763,7 +1915,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_density(DevPlan P, const T
                     const long long off = unit_offset(J, T.nc_alloc, c, r, (cc & 1) * 4 + gg);
 #pragma unroll
                     for (int sp = 0; sp < 3; sp++)
-                        pre[sp][gg] = sp < n_split ? *reinterpret_cast<const uint4 *>(phi_img + off + sp * T.plane_phi)
+                        pre[sp][gg] = sp < n_split ? *reinterpret_cast<const uint4 *>(phi_img + off + sp * kChunkBytes)
                                                    : make_uint4(0u, 0u, 0u, 0u);
                 }
             }
@@ -1808,7 +1960,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_density(DevPlan P, const T
                         if (cq == 0)
                             uu = pre[sp][gg];
                         else
-                            uu = sp < n_split ? *reinterpret_cast<const uint4 *>(phi_img + off + sp * T.plane_phi)
+                            uu = sp < n_split ? *reinterpret_cast<const uint4 *>(phi_img + off + sp * kChunkBytes)
                                               : make_uint4(0u, 0u, 0u, 0u);
                         w[sp][0] = uu.x; w[sp][1] = uu.y; w[sp][2] = uu.z; w[sp][3] = uu.w;
                     }
@@ -1980,7 +2132,8 @@ size_t smem_tc(int n_split)
     return 1024 + (size_t)kStages * kStageBytes + sizeof(TcRing);
 }
 
-size_t smem_phi() { return 128 * kPhiValStride * sizeof(float2); }
+// the bound pass keeps knots (bound_grids 2), the pass over the points offsets
+size_t smem_phi(bool bound) { return bound ? kKnotCache * sizeof(unsigned short) : kGeoCache * sizeof(float4); }
 
 size_t smem_tc_h() { return smem_tc(3) + sizeof(HPairTab) + 16; }
 
@@ -1995,7 +2148,7 @@ cudaError_t set_attrs()
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_tc_density<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_tc(3));
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_tc_phi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_phi());
+    e = cudaFuncSetAttribute(k_tc_phi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_phi(false));
     if (e != cudaSuccess) return e;
     attrs_set = true;
     return cudaSuccess;
@@ -2251,9 +2404,7 @@ cudaError_t tc_launch_phi(const TcPlan &t, const DevPlan &P, const TcWave &w, co
     if (w.nphi <= 0) return cudaSuccess;
     // the H images (v given) of the split mode use the fixed-point leading term
     const int fixed = (v != nullptr && n_split == 3) ? 1 : 0;
-    // the dynamic buffer caches geometry for the FP32 pass over the points
-    // (bound_grids 0 and 1), or the point-atom distances of the table-bound pass
-    const size_t dyn = smem_phi();
+    const size_t dyn = smem_phi(t.bound_grids >= 2);
     k_tc_phi<<<(unsigned)w.nphi, kPhiThreads, dyn, s>>>(P, t.d_batches, t.d_items + w.phi0,
                                                        (uint8_t *)ws + t.img_base, v, n_split, fixed,
                                                        reinterpret_cast<int *>((uint8_t *)ws + t.sign_off),

@@ -17,12 +17,14 @@
 namespace fgi {
 
 constexpr int kChunkBytes = 16384;       // 128 rows x 64 columns x 2 bytes
+constexpr int kChunkStride = 3 * kChunkBytes;   // the three planes of a chunk are adjacent: one bulk copy
+                                                // moves them, and a value's planes are one address apart
 
 struct TcBatch {
     long long img_phi;     // byte offset (in the wave's workspace) of the phi image
     long long img_aux;     // byte offset of the w v phi image (H) or the D image (density)
-    long long plane_phi;   // bytes per plane of the phi / w v phi images
-    long long plane_d;     // bytes per plane of the D image
+    long long plane_phi;   // bytes of one plane of the phi / w v phi images (a third of the image)
+    long long plane_d;     // the same for the D image
     int nrb;               // 128-row blocks (functions)
     int nc;                // 64-point chunks holding points
     int nc_alloc;          // allocated 64-point chunks (even)

@@ -1,0 +1,67 @@
+"""The basis kernels' path for species whose shells share one knot grid against
+the general path, over the forms the first accepts: thirteen shells (four a
+bound look-up, a remainder of one), points on the nuclei and beyond every
+cutoff, batches at the edges of a warp and of a 64-point chunk, potentials of
+one sign (one image) and of both (two).
+
+The general path is taken for the same functions by padding one shell's spline
+with an interval of zeros: the knot grids then differ, the functions do not.
+Both paths do the same operations in the same order, and the contractions sum
+in fixed order: H and the density are equal bit by bit.
+"""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def molecule():
+    rc = 4.0 * W.BOHR_PER_ANG
+    ls = [0, 0, 0, 0, 1, 1, 1, 1, 2, 2, 2, 3, 3]
+    radials = [W.make_radial(W.RadialSpec(l, (0.4 + 0.11 * i, 1.9), (1.0, -0.2), rc, rc - W.BOHR_PER_ANG, 1700))
+               for i, l in enumerate(ls)]
+    species = [W.Species("A", 6.0, list(range(13))), W.Species("B", 3.0, [8, 0, 4])]
+    xyz = np.array([[0.0, 0.0, 0.0], [2.4, 0.3, -0.2], [-0.7, 2.2, 1.0], [1.1, -1.9, 1.7], [-2.0, -1.2, -1.4]])
+    sp = np.array([0, 1, 0, 1, 0], dtype=np.int32)
+    prob = W.build_problem("paths", radials, species, [(sp, xyz)], lambda k: (14, 38), 9, (200, 50, None))
+    pts = np.concatenate([prob.pts, xyz, [[30.0, 1.0, 0.0], [5.0, 6.5, 3.0]]])
+    w = np.concatenate([prob.w, np.full(len(xyz) + 2, 1e-3)])
+    v = np.concatenate([prob.v, np.full(len(xyz) + 2, -0.3)])
+    # batches of 1, 31, 32, 33, 64, 65 points, then of 199
+    off = np.cumsum([0, 1, 31, 32, 33, 64, 65])
+    off = np.concatenate([off, np.arange(off[-1] + 199, len(w), 199), [len(w)]]).astype(np.int64)
+    return W.Problem("paths", radials, species, prob.atom_off, prob.atom_species, prob.atom_xyz, pts, w, off,
+                     np.zeros(len(off) - 1, dtype=np.int32), v)
+
+
+@pytest.mark.parametrize("precision", ["split_bf16", "bf16"])
+@pytest.mark.parametrize("both_signs", [False, True])
+@pytest.mark.parametrize("points", [0, 512])                      # batches as given, and merged
+def test_shared_knots_equal_general_path(molecule, both_signs, points, precision, tmp_path):
+    import paper_2208_12335_gb300 as fgi
+    v = molecule.v + (0.4 if both_signs else 0.0)
+    assert (v.max() > 0) == both_signs
+    tune = tmp_path / "tune.txt"
+    tune.write_text("h_sb_points %d\ndensity_sb_points %d\n" % (points, points))
+    padded = list(molecule.radials)
+    for i in (8, 12):                                             # a shell of each species
+        r = padded[i]
+        padded[i] = W.Radial(r.l, r.h, np.concatenate([r.coef, np.zeros((1, 4))]), r.spec, r.norm)
+    out = []
+    for radials in (molecule.radials, padded):
+        ctx = fgi.Context(0).load(dataclasses.replace(molecule, radials=radials), precision, tune_path=str(tune))
+        d = torch.from_numpy(np.random.default_rng(5).standard_normal(ctx.sizes()[1])).cuda()
+        h = ctx.integrate_h(torch.from_numpy(v).cuda())
+        n = ctx.density(d)[0]
+        ctx.sync()
+        out.append((ctx.batch_work()[1], h.cpu().numpy(), n.cpu().numpy()))
+    (a, h0, n0), (b, h1, n1) = out
+    assert np.array_equal(a, b)                                   # the same active functions
+    assert np.abs(h0).max() > 0 and np.array_equal(h0, h1)
+    assert np.abs(n0).max() > 0 and np.array_equal(n0, n1)
