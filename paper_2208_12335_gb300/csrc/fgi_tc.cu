@@ -191,11 +191,6 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool a_mn, bool 
 }
 
 // --------------------------------------------------------------- splitting
-__device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 lo, __nv_bfloat16 hi)
-{
-    return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-}
-
 // byte offset (plane 0) of the 16-byte unit (row r, 8-column group g) inside
 // chunk (blk, c); a chunk's three planes follow each other
 __device__ __forceinline__ long long unit_offset(int blk, int nchunk, int c, int r, int g)
@@ -242,31 +237,11 @@ __device__ __forceinline__ void ylm_poly_f32(int l, float x, float y, float z, f
     }
 }
 
-// 3-term BF16 split of a double-float value
-__device__ __forceinline__ void split3_df(df x, __nv_bfloat16 &a, __nv_bfloat16 &b, __nv_bfloat16 &c)
+// two FP32 values rounded to BF16, lo in the low half
+__device__ __forceinline__ uint32_t pack2_bf16(float lo, float hi)
 {
-    a = __float2bfloat16_rn(x.hi);
-    float r = (x.hi - __bfloat162float(a)) + x.lo;
-    b = __float2bfloat16_rn(r);
-    r -= __bfloat162float(b);
-    c = __float2bfloat16_rn(r);
-}
-
-__device__ __forceinline__ void store_split8_df(uint8_t *dst, const df *x, int n_split)
-{
-    uint32_t w0[4], w1[4], w2[4];
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-        __nv_bfloat16 a0, a1, a2, b0, b1, b2;
-        split3_df(x[2 * q], a0, a1, a2);
-        split3_df(x[2 * q + 1], b0, b1, b2);
-        w0[q] = pack_bf16(a0, b0);
-        w1[q] = pack_bf16(a1, b1);
-        w2[q] = pack_bf16(a2, b2);
-    }
-    *reinterpret_cast<uint4 *>(dst) = make_uint4(w0[0], w0[1], w0[2], w0[3]);
-    if (n_split > 1) *reinterpret_cast<uint4 *>(dst + kChunkBytes) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
-    if (n_split > 2) *reinterpret_cast<uint4 *>(dst + 2 * kChunkBytes) = make_uint4(w2[0], w2[1], w2[2], w2[3]);
+    const __nv_bfloat162 w = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&w);
 }
 
 // Split with a fixed-point leading term: x0 = m * unit, m = rint(x / unit),
@@ -274,35 +249,9 @@ __device__ __forceinline__ void store_split8_df(uint8_t *dst, const df *x, int n
 // product x0*y0 of a row pair is an integer multiple of unit_x*unit_y not
 // exceeding 2^14 in units; a sum of up to 1024 of them (a batch) is exact in
 // FP32 whatever the accumulator's rounding.  The remainder x - x0 is split
-// relative to itself into two BF16 terms.
-__device__ __forceinline__ void split_fixed(df x, float scale, float unit, __nv_bfloat16 &a,
-                                            __nv_bfloat16 &b, __nv_bfloat16 &c)
-{
-    const float x0 = rintf(x.hi * scale) * unit;
-    // x.hi - x0 is exact: x0 is a multiple of unit, and unit >= ulp(x.hi)
-    // because |x.hi| <= 2^e (1 + 2^-12) and unit = 2^(e - bits), bits <= 8
-    const float d = x.hi - x0;
-    a = __float2bfloat16_rn(x0);
-    b = __float2bfloat16_rn(d);
-    c = __float2bfloat16_rn((d - __bfloat162float(b)) + x.lo);
-}
-
-__device__ __forceinline__ void store_fixed8(uint8_t *dst, const df *x, float scale, float unit)
-{
-    uint32_t w0[4], w1[4], w2[4];
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-        __nv_bfloat16 a0, a1, a2, b0, b1, b2;
-        split_fixed(x[2 * q], scale, unit, a0, a1, a2);
-        split_fixed(x[2 * q + 1], scale, unit, b0, b1, b2);
-        w0[q] = pack_bf16(a0, b0);
-        w1[q] = pack_bf16(a1, b1);
-        w2[q] = pack_bf16(a2, b2);
-    }
-    *reinterpret_cast<uint4 *>(dst) = make_uint4(w0[0], w0[1], w0[2], w0[3]);
-    *reinterpret_cast<uint4 *>(dst + kChunkBytes) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
-    *reinterpret_cast<uint4 *>(dst + 2 * kChunkBytes) = make_uint4(w2[0], w2[1], w2[2], w2[3]);
-}
+// relative to itself into two BF16 terms.  x.hi - x0 is exact: x0 is a
+// multiple of unit, and unit >= ulp(x.hi) because |x.hi| <= 2^e (1 + 2^-12)
+// and unit = 2^(e - bits), bits <= 8.
 
 // Power-of-two scale 2^(b-e) and unit 2^(e-b) for a row whose largest |x|
 // is mx: |x| * scale <= 2^b.  b digit bits keep the exact sum: 2^(2b) times
@@ -379,13 +328,13 @@ __device__ __forceinline__ const float4 *spline_tab(const DevPlan &P, const DevS
 // slower: the doubled per-lane state costs occupancy or spills, and these
 // kernels wait mostly on their loads.)
 
-// One value split on its row's or point's grid (split_fixed; NSPLIT 1:
+// One value split on its row's or point's grid (as above; NSPLIT 1:
 // plain BF16) and stored as one 16-bit BF16 per plane
 template <int NSPLIT>
 __device__ __forceinline__ void store_value(uint8_t *dst, df x, float scale, float unit)
 {
     if (NSPLIT == 3) {
-        // split_fixed with the rounding to an integer as an addition (the FRND
+        // the rounding to an integer as an addition (the FRND
         // unit has a sixteenth of the FADD rate): |x scale| <= 2^8, far inside
         // 2^22.  x0 has at most 9 significant bits, 8 below a power of two: its
         // BF16 form is the upper half of the word.
@@ -1668,23 +1617,38 @@ __global__ void k_d_colbounds(const float2 *v, const int *col_of, long long nnz,
     }
 }
 
+// Row j of the gather: with li_j its index in its atom, `base` = (first stored
+// value of row j) - li_j.  A stored value (j, i) with i >= j lies at base +
+// [start of atom(i)'s run in the row, 0 for j's own atom] + li_i; one with
+// i < j in row i at (row i's base) + [start of atom(j)'s run] + li_j.
+struct GatherRow {
+    long long base;
+    int atom, loc, li, pad;
+};
+
+// Bound by the latency and sectors of the loads of D.  One warp walks 16 rows,
+// a lane owns two neighbouring columns of the 64-column chunk: a row's loads
+// are the consecutive stored values of its runs, and its three stores are
+// whole 128-byte rows of the image.  The offset of a (row atom, column) pair
+// is looked up once per row atom; four rows' loads are in flight together.
+// (Eight values a thread, its loads 64 bytes apart and a table search a value,
+// took 300 issue slots a value: 64-atom Si cluster, 1368 super-batches, 3.2 ms;
+// now 0.8 ms, the full G of the adjoint 5.2 -> 1.5 ms.)
+template <int NSPLIT>
 __global__ void __launch_bounds__(256) k_tc_gather_d(DevPlan P, const TcBatch *tb, const WorkItem *items,
                                                      uint8_t *ws, const float2 *ddv, const unsigned int *gmax,
-                                                     const float *gsum, float offdiag_scale, int n_split, int full)
+                                                     const float *gsum, float offdiag_scale, int full)
 {
     const WorkItem it = items[blockIdx.x];
     const DevBatch B = P.batches[it.batch];
     const TcBatch T = tb[it.batch];
     const int J = it.ti;
-    __shared__ FnRef rref[128], cref[64];
-    __shared__ float rsc[2][128];
+    __shared__ GatherRow row[128];
+    __shared__ float2 rsc[128];                      // per row: scale, unit
     __shared__ int4 sact[kGatherActSmem];            // per active atom: fn_loc, atom, loc, first global fn
     const DevAct *act = P.act + B.act0;
-    const bool fixed = n_split == 3;
     const int *pp_sys = P.pairpos + P.sys_pair_off[B.sys];
-    const int nat = P.sys_nat[B.sys];
-    // the batch's active atoms in shared memory, so that each column's
-    // reference costs one search there and one global load (its row start)
+    const long long nat = P.sys_nat[B.sys];
     const bool staged = B.n_act <= kGatherActSmem;
     if (staged) {
         for (int e = threadIdx.x; e < B.n_act; e += blockDim.x) {
@@ -1693,93 +1657,120 @@ __global__ void __launch_bounds__(256) k_tc_gather_d(DevPlan P, const TcBatch *t
         }
     }
     __syncthreads();
-    auto ref_of = [&](int l) -> FnRef {
-        if (!staged) return fn_ref(P, act, find_act(act, B.n_act, l), l);
+    // entry e of the active atoms, and the last one that starts at or before l
+    auto entry = [&](int e) -> int4 {
+        if (staged) return sact[e];
+        const DevAct A = act[e];
+        return make_int4(A.fn_loc, A.atom, P.atom_loc[A.atom], (int)P.atom_fn0[A.atom]);
+    };
+    auto find = [&](int l) -> int {
         int lo = 0, hi = B.n_act - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (sact[mid].x <= l) lo = mid; else hi = mid - 1;
+            if ((staged ? sact[mid].x : act[mid].fn_loc) <= l) lo = mid; else hi = mid - 1;
         }
-        const int4 a = sact[lo];
-        FnRef r;
-        r.atom = a.y;
-        r.li = l - a.x;
-        r.gi = (long long)a.w + r.li;
-        r.rp = __ldg(P.rowptr + r.gi);
-        r.loc = a.z;
-        r.pad = 0;
-        return r;
+        return lo;
     };
     if (threadIdx.x < 128) {
         const int j = J * 128 + threadIdx.x;
+        GatherRow g{0, -1, 0, 0, 0};
         float sc = 0.f, un = 0.f;
         if (j < B.nfn) {
-            const FnRef rj = ref_of(j);
-            rref[threadIdx.x] = rj;
-            if (fixed) fixed_scale_adaptive(__uint_as_float(gmax[rj.gi]), gsum[rj.gi], T.nkc * 64, sc, un);
+            const int4 a = entry(find(j));
+            g.li = j - a.x;
+            g.atom = a.y;
+            g.loc = a.z;
+            const long long gi = (long long)a.w + g.li;
+            g.base = P.rowptr[gi] - g.li;
+            if (NSPLIT == 3) fixed_scale_adaptive(__uint_as_float(gmax[gi]), gsum[gi], T.nkc * 64, sc, un);
         }
-        rsc[0][threadIdx.x] = sc;
-        rsc[1][threadIdx.x] = un;
+        row[threadIdx.x] = g;
+        rsc[threadIdx.x] = make_float2(sc, un);
     }
-    uint8_t *img = ws + T.img_aux;
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t g16 = (uint32_t)(lane >> 2) << 4, cb = (uint32_t)(lane & 3) * 4u;
+    uint8_t *img = ws + T.img_aux + (long long)J * T.nkc * kChunkStride;
     // D is symmetric: block row J holds only the chunks i >= 128 J, the
     // diagonal block halved (n = 2 sum_J phi_J . E_J, exact in binary); in
     // full (the adjoint's G Phi) every chunk, nothing halved
     for (int kc = full ? 0 : 2 * J; kc < T.nkc; kc++) {
         const float blk = (!full && kc < 2 * J + 2) ? 0.5f : 1.f;
-        __syncthreads();
-        if (threadIdx.x < 64) {
-            const int i = kc * 64 + threadIdx.x;
-            if (i < B.nfn) cref[threadIdx.x] = ref_of(i);
-        }
-        __syncthreads();
-        for (int u = threadIdx.x; u < 1024; u += blockDim.x) {
-            const int r = u >> 3, g = u & 7;
-            const int j = J * 128 + r;
-            const FnRef rj = rref[r];
-            // stored value of (j, i): for i >= j, base + gi (row j's run of atom(i));
-            // for i < j, rp_i - li + off (row i's run of atom(j)); cached per column atom
-            int cur_atom = -1;
-            long long off = 0;
-            bool stored = false;
-            df x[8];
+        const int i0 = kc * 64 + 2 * lane;
+        int catom[2], cloc[2], cli[2];
+        long long cbase[2] = {0, 0};                 // row i's base, for values below the diagonal
+        bool cin[2];
+        int e = find(min(i0, B.nfn - 1));
 #pragma unroll
-            for (int q = 0; q < 8; q++) {
-                const int il = g * 8 + q;
-                const int i = kc * 64 + il;
-                x[q] = df{0.f, 0.f};
-                if (j >= B.nfn || i >= B.nfn) continue;
-                const FnRef &ci = cref[il];
-                if (ci.atom != cur_atom) {
-                    cur_atom = ci.atom;
-                    if (ci.atom == rj.atom) {
-                        stored = true;
-                        off = 0;
-                    } else if (ci.atom > rj.atom) {
-                        const int pp = __ldg(pp_sys + (long long)rj.loc * nat + ci.loc);
-                        stored = pp >= 0;
-                        off = rj.rp + pp - rj.li - (ci.gi - ci.li);       // + gi
-                    } else {
-                        const int pp = __ldg(pp_sys + (long long)ci.loc * nat + rj.loc);
-                        stored = pp >= 0;
-                        off = pp + rj.li;                                   // + rp_i - li
+        for (int c = 0; c < 2; c++) {
+            const int i = i0 + c;
+            cin[c] = i < B.nfn;
+            if (c == 1 && cin[1] && e + 1 < B.n_act && (staged ? sact[e + 1].x : act[e + 1].fn_loc) <= i) e++;
+            const int4 a = entry(e);
+            catom[c] = a.y;
+            cloc[c] = a.z;
+            cli[c] = i - a.x;
+            if (cin[c] && kc < 2 * J + 2) cbase[c] = P.rowptr[(long long)a.w + cli[c]] - cli[c];
+        }
+        int cur = -2;                                // the row atom of up/low/ok
+        long long up[2] = {0, 0}, low[2] = {0, 0};
+        bool ok[2] = {false, false};
+        for (int rb = warp * 16; rb < warp * 16 + 16; rb += 4) {
+            float2 v[4][2];
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const GatherRow g = row[rb + q];
+                const int j = J * 128 + rb + q;
+                if (g.atom != cur) {                 // the same for the whole warp
+                    cur = g.atom;
+#pragma unroll
+                    for (int c = 0; c < 2; c++) {
+                        int pp = 0;
+                        if (cur >= 0 && cin[c] && catom[c] != cur)
+                            pp = catom[c] > cur ? __ldg(pp_sys + g.loc * nat + cloc[c])
+                                                : __ldg(pp_sys + cloc[c] * nat + g.loc);
+                        ok[c] = cur >= 0 && cin[c] && pp >= 0;
+                        up[c] = pp + cli[c];
+                        low[c] = cbase[c] + pp;
                     }
                 }
-                if (!stored) continue;
-                long long k;
-                if (ci.atom == rj.atom)
-                    k = i >= j ? rj.rp + (ci.gi - rj.gi) : ci.rp + (rj.gi - ci.gi);
-                else
-                    k = ci.atom > rj.atom ? off + ci.gi : ci.rp - ci.li + off;
-                const float2 v = __ldg(ddv + k);
-                const float sc = (i == j ? 1.f : offdiag_scale) * blk;
-                x[q] = df{v.x * sc, v.y * sc};
+#pragma unroll
+                for (int c = 0; c < 2; c++) {
+                    v[q][c] = make_float2(0.f, 0.f);
+                    const long long k = i0 + c >= j ? g.base + up[c] : low[c] + g.li;
+                    if (ok[c]) v[q][c] = __ldg(ddv + k);
+                }
             }
-            uint8_t *dst = img + unit_offset(J, T.nkc, kc, r, g);
-            if (fixed)
-                store_fixed8(dst, x, rsc[0][r], rsc[1][r]);
-            else
-                store_split8_df(dst, x, n_split);
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const int r = rb + q, j = J * 128 + r;
+                const float2 su = rsc[r];
+                uint32_t w0, w1 = 0, w2 = 0;
+                if (NSPLIT == 3) {
+                    float x0[2], d[2], lo[2];
+#pragma unroll
+                    for (int c = 0; c < 2; c++) {
+                        const float s = (i0 + c == j ? 1.f : offdiag_scale) * blk;
+                        const float hi = v[q][c].x * s;
+                        lo[c] = v[q][c].y * s;
+                        x0[c] = rintf(hi * su.x) * su.y;
+                        d[c] = hi - x0[c];
+                    }
+                    w0 = pack2_bf16(x0[0], x0[1]);
+                    w1 = pack2_bf16(d[0], d[1]);
+                    w2 = pack2_bf16((d[0] - __uint_as_float(w1 << 16)) + lo[0],
+                                    (d[1] - __uint_as_float(w1 & 0xFFFF0000u)) + lo[1]);
+                } else {
+                    w0 = pack2_bf16(v[q][0].x * ((i0 == j ? 1.f : offdiag_scale) * blk),
+                                    v[q][1].x * ((i0 + 1 == j ? 1.f : offdiag_scale) * blk));
+                }
+                uint8_t *dst = img + (long long)kc * kChunkStride + row_offset((uint32_t)r, g16) + cb;
+                *reinterpret_cast<uint32_t *>(dst) = w0;
+                if (NSPLIT == 3) {
+                    *reinterpret_cast<uint32_t *>(dst + kChunkBytes) = w1;
+                    *reinterpret_cast<uint32_t *>(dst + 2 * kChunkBytes) = w2;
+                }
+            }
         }
     }
 }
@@ -2447,10 +2438,11 @@ cudaError_t tc_launch_gather_d(const TcPlan &t, const DevPlan &P, const TcWave &
 {
     if (w.ng <= 0) return cudaSuccess;
     const char *base = (const char *)ws;
-    k_tc_gather_d<<<(unsigned)w.ng, 256, 0, s>>>(P, t.d_batches, t.d_items + w.g0, (uint8_t *)ws + t.img_base,
-                                                 (const float2 *)base, (const unsigned int *)(base + t.bound_off),
-                                                 (const float *)(base + t.bound_off + 4 * t.n_fn),
-                                                 (float)offdiag_scale, n_split, full ? 1 : 0);
+    auto kernel = n_split == 3 ? k_tc_gather_d<3> : k_tc_gather_d<1>;
+    kernel<<<(unsigned)w.ng, 256, 0, s>>>(P, t.d_batches, t.d_items + w.g0, (uint8_t *)ws + t.img_base,
+                                          (const float2 *)base, (const unsigned int *)(base + t.bound_off),
+                                          (const float *)(base + t.bound_off + 4 * t.n_fn), (float)offdiag_scale,
+                                          full ? 1 : 0);
     return cudaGetLastError();
 }
 
