@@ -335,8 +335,10 @@ int build_tc_plans(fgi_ctx *c, TcPlanInput tin, std::string *err)
     tin.bound_grids = bounded ? ts.bound_grids : 0;
     tin.sb_points = ts.h_sb_points;
     tin.sb_growth = ts.h_sb_growth;
+    tin.for_h = true;
     int rc = tc_build(c->tc, tin, err);
     if (rc != FGI_OK) return rc;
+    tin.for_h = false;
     tin.sb_points = ts.sb_points;
     tin.sb_growth = ts.sb_growth;
     rc = tc_build(c->tcd, tin, err);

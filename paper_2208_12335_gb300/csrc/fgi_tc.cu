@@ -16,6 +16,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <climits>
 #include <cstdint>
 #include <cstdio>
 #include <cstdlib>
@@ -110,6 +111,28 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
         : "memory");
 }
 
+// start moving [src, src + bytes) into L2 (both multiples of 16)
+__device__ __forceinline__ void bulk_prefetch(const void *src, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+
+// add to a global 64-bit word where pred holds, without a branch
+__device__ __forceinline__ void red_add_if(bool pred, unsigned long long addr, long long x)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t"
+                 "@p red.relaxed.gpu.global.add.u64 [%0], %1;\n\t}" ::"l"(addr), "l"(x), "r"((int)pred)
+                 : "memory");
+}
+
+// the largest of m, |a|, |b|; NaN when one of them is
+__device__ __forceinline__ float max_abs_nan(float m, float a, float b)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(m), "f"(fabsf(a)), "f"(fabsf(b)));
+    return r;
+}
+
 __device__ __forceinline__ void tmem_alloc(uint32_t *slot, uint32_t ncols)
 {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
@@ -148,6 +171,14 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t adesc, uint64_t
         : "memory");
 }
 
+// one lane of a converged warp
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // 32 lanes x 32 consecutive 32-bit columns: thread (lane) gets its row's 32 values
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v)
 {
@@ -164,6 +195,19 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v)
         : "r"(taddr));
 #pragma unroll
     for (int i = 0; i < 32; i++) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v)
+{
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+#pragma unroll
+    for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
 }
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
@@ -800,9 +844,38 @@ __device__ __forceinline__ void row_bounds_quad(const DevPlan &P, const DevBatch
     }
 }
 
+// The descriptor of one row block for the H scatter (threads 0 .. 127, a row
+// each; e0 the first of the block's ne active atoms)
+__device__ __forceinline__ void write_hblock(const DevPlan &P, const DevBatch &B, const DevAct *act, int r0, int e0, int ne,
+                                             HBlock *out)
+{
+    const int r = threadIdx.x;
+    if (r >= 128) return;
+    const int f = r0 + r;
+    long long base = 0;
+    int li = 0, slot = 0;
+    if (f < B.nfn) {
+        slot = find_act(act + e0, ne, f);
+        const DevAct A = act[e0 + slot];
+        li = f - A.fn_loc;
+        base = P.rowptr[P.atom_fn0[A.atom] + li] - li;
+    }
+    out->base[r] = base;
+    out->li[r] = (unsigned short)li;
+    out->slot[r] = (unsigned char)slot;
+    if (r < ne) out->loc[r] = P.atom_loc[act[e0 + r].atom];
+    if (r == 0) {
+        out->pair_off = P.sys_pair_off[B.sys];
+        out->nat = P.sys_nat[B.sys];
+        out->nslot = ne;
+        out->n = min(128, B.nfn - r0);
+
+    }
+}
+
 __global__ void __launch_bounds__(kPhiThreads, 4) k_tc_phi(DevPlan P, const TcBatch *tb, const WorkItem *items,
                                                 uint8_t *ws, const double *v, int n_split, int fixed,
-                                                int *bsign, int bound)
+                                                int *bsign, int bound, unsigned int *counter)
 {
     extern __shared__ float4 phi_smem[];            // knots of the bound pass, or offsets of the pass over the points
     __shared__ float2 wvs[kMaxBatchPoints];         // per-point image scale (double-float)
@@ -838,6 +911,8 @@ __global__ void __launch_bounds__(kPhiThreads, 4) k_tc_phi(DevPlan P, const TcBa
     neg = __syncthreads_or(neg) != 0;
     const int sgn = (pos && neg) ? 0 : (neg ? -1 : 1);
     if (I == 0 && threadIdx.x == 0) bsign[it.batch] = sgn;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0u;       // of the contraction that follows
+    write_hblock(P, B, act, r0, e0, ne, reinterpret_cast<HBlock *>(ws + T.hblock) + I);
     if (fixed && bound) {
         // row bounds from the tables: per (atom, shell) and point one lookup
         // of the suffix bound of |u(r)/r| at the point's distance (knot index
@@ -1114,8 +1189,9 @@ __device__ __forceinline__ void density_image_lanes(const DevPlan &P, const DevB
 // term is per point (column): first the largest |phi_i(p)| over all of the
 // batch's functions (FP32), then every 128-row block in double-float.
 __global__ void __launch_bounds__(kPhiThreads, 5) k_tc_phi_cols(DevPlan P, const TcBatch *tb, const WorkItem *items,
-                                                     uint8_t *ws, int n_split, int bound)
+                                                     uint8_t *ws, int n_split, int bound, unsigned int *counter)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0u;       // of the contraction that follows
     __shared__ float colmax[kPhiThreads / 64][64], colsum[kPhiThreads / 64][64];
     __shared__ float2 csc[64];                       // per point: scale, unit
     __shared__ float2 ylim[kMaxL + 1];               // per l: max over m of max |Y_lm|, bound of the sum over m
@@ -1259,55 +1335,77 @@ __global__ void k_fix_to_h(const long long *acc, double *h, long long n, int acc
 }
 
 // ----------------------------------------------- H contraction on tcgen05 (K2)
-// Persistent: one CTA per SM walks the tile list (batch, I, J), I <= J, with
-// stride gridDim.x; each tile is 128 x 128 outputs with K = the batch's
-// points in chunks of 64, computed transposed (A = phi of block J, B = w v phi
-// of block I).  Warp 8 (one lane) streams operand chunks into a two-stage
-// shared-memory ring with bulk copies; warp 9 (one lane) issues the MMAs
-// into one of two tensor-memory accumulator sets (acc0 + acc1, 256 columns
-// each); warps 0-7 drain the other set and scatter the upper triangle into
-// the fixed-point H accumulator, so the scatter of one tile overlaps the
-// MMAs of the next.  A warp's lanes hold 32 consecutive functions j, so the
-// atomics for one column i land on consecutive values of row i.
-constexpr int kThreadsTc = 320;                  // warps 0-7 epilogue, 8 producer, 9 MMA
-constexpr int kWarpProducer = 8, kWarpMma = 9;
-constexpr int kEpiThreads = 256;
-constexpr int kStages = 2;
-constexpr int kStageBytes = 6 * kChunkBytes;     // A and B operands, 3 planes each
+// Persistent: one CTA per SM takes tiles (batch, I, J), I <= J, from a shared
+// counter; each tile is 128 x 128 outputs with K = the batch's points in
+// chunks of 64, computed transposed (A = phi of block J, B = w v phi of block
+// I).  One warp (one lane) fetches tiles ahead, publishes them in a small tile
+// ring and streams operand chunks into a shared-memory ring with bulk copies;
+// one (one lane) issues the MMAs into one of two tensor-memory accumulator
+// sets (acc0 + acc1, 256 columns each); two groups of eight warps, one for each
+// set, drain and scatter the upper triangle into the fixed-point H
+// accumulator, so the scatter of one tile overlaps the MMAs of the next.  A
+// warp's lanes hold 32 consecutive functions j, so the atomics for one column
+// i land on consecutive values of row i.
+//
+// The counter keeps the tiles in flight next to each other in the list: with a
+// fixed stride the CTAs drift apart over ~90 super-batches, whose operands
+// outgrow L2 (17 GB read from DRAM for 4.7 GB of images in the 64-atom Si
+// cluster's density).
+// Two groups of eight epilogue warps, one for each accumulator set: a group's
+// table look-ups and drain of one tile overlap the other group's and the MMAs.
+constexpr int kGroupWarps = 8, kGroupThreads = 32 * kGroupWarps;
+constexpr int kWarpProducer = 2 * kGroupWarps, kWarpMma = kWarpProducer + 1;
+constexpr int kThreadsTc = 32 * (kWarpMma + 1);
+constexpr int kStages = 2;                       // ring of operand chunks, A and B of 64 contraction steps each
+constexpr int kOperandBytes = kChunkStride;      // three planes
+constexpr int kStageBytes = 2 * kOperandBytes;
 // split products kept in the density: combined order <= 3 except x2*y2 (8 of
 // 9), as in H; the order-3 pair x1*y2, x2*y1 is about 2^-27 of the leading
 // product, which over ~10^3 functions is no longer far below the 1e-7
 // relative bound on n
 constexpr int kDensityOrder = 3;
 
-struct ColRef {                                  // column i of an H tile (a row of the stored triangle)
-    long long rpl;                               // first stored value of row i minus i's index in its atom
-    int atom;                                    // global atom
-    int loc;                                     // atom index inside its system
-    int slot;                                    // i's atom among the tile's column atoms (0 = first)
-    int pad;
+// One tile, resolved by the producer so that the other roles have no chain of
+// dependent global loads.
+struct TileInfo {
+    int ti, tj;                                  // H: blocks I, J; density: point tile m, block J.  ti < 0: no more tiles
+    int np, nfn;                                 // points and functions of the batch
+    int nc, nkc, nc_alloc;                       // see TcBatch
+    int sign;                                    // H: of w v over the batch
+    long long img_phi, img_e, part_row;          // density
+    long long pad;
+};
+constexpr int kTiles = 4;                        // tile ring
+constexpr int kPairSlots = 32;                   // atoms of a block in the pair table
+
+// An H tile's rows and columns as the epilogue needs them: the descriptors of
+// blocks I and J (HBlock, written with the operand images).
+struct HTile {
+    HBlock i, j;
 };
 
-// Pair offsets of an H tile: for each of the (at most kColAtoms) atoms of
-// the tile's columns and each row j, the start of that atom's run in row i
-// relative to (rp_i - li), i.e. 0 for j's own atom, pairpos otherwise (-1:
-// not stored).  Filled once per tile so that the scatter loop has no
-// dependent global loads.
-constexpr int kColAtoms = 32;
-struct HPairTab {
-    int pp[kColAtoms][128];
-    int2 atom[2][kColAtoms];                     // (global atom, index in system) per slot
-    int nslot[2];
-    int pad[2];
+// Scatter tables of one group: for column i the address of the first stored
+// value of row i less i's index in its atom; for a pair of atoms (of I, of J)
+// the byte offset from there to atom(j)'s run, 0 for the same atom, negative
+// where the pair is not stored.
+struct HColumn {
+    unsigned long long base;
+    int pair_row;                                // first entry of the column's atom in pair
+    int pad;
+};
+struct HTables {
+    HColumn col[128];
+    int pair[kPairSlots * kPairSlots];
 };
 
 struct TcRing {
     uint64_t full[kStages], empty[kStages];
-    uint64_t tfull[2], tempty[2];
+    uint64_t tfull[2], tempty[2];                // accumulator sets
+    uint64_t nfull[kTiles], nempty[kTiles];      // tile ring
+    TileInfo tile[kTiles];
     uint32_t tmem;
     int abort;
-    int pad[2];
-    ColRef ref[2][128];
+    int go[2];                                   // per group: the tile's entry holds a tile
 };
 
 __device__ __forceinline__ uint8_t *align1024(uint8_t *p)
@@ -1315,8 +1413,11 @@ __device__ __forceinline__ uint8_t *align1024(uint8_t *p)
     return reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(p) + 1023) & ~(uintptr_t)1023);
 }
 
-// named barrier of the eight epilogue warps
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// named barrier of one group of epilogue warps
+__device__ __forceinline__ void group_sync(int group)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(kGroupThreads) : "memory");
+}
 
 __device__ __forceinline__ void ring_init(TcRing *S)
 {
@@ -1326,52 +1427,168 @@ __device__ __forceinline__ void ring_init(TcRing *S)
     }
     for (int b = 0; b < 2; b++) {
         mbar_init(&S->tfull[b], 1);
-        mbar_init(&S->tempty[b], kEpiThreads);
+        mbar_init(&S->tempty[b], kGroupThreads);
+    }
+    for (int e = 0; e < kTiles; e++) {
+        mbar_init(&S->nfull[e], 1);
+        mbar_init(&S->nempty[e], 2);             // the MMA warp and the tile's epilogue group
     }
     S->abort = 0;
     fence_mbar_init();
 }
 
-// Issue the split products of one 64-deep chunk (4 k-steps of 16): every
-// product of combined order <= ORDER except x2*y2; x0*y0 alone in
-// accumulator 0.  Fully unrolled with the descriptors of the stage computed
-// once: the plane and k-step offsets are added to the descriptors' address
-// field (addr >> 4, no carry out of it inside shared memory), so one lane
-// issues an MMA every few instructions and keeps the tensor pipe fed.
+// The operand ring: stage n % kStages holds the n-th chunk, in the order the
+// producer and the MMA warp both walk.  Producer: room for chunk n (false:
+// timed out).
+__device__ __forceinline__ bool stage_wait_empty(TcRing *S, uint32_t n, int *status)
+{
+    return n < kStages || mbar_wait_a(&S->empty[n % kStages], (n / kStages - 1) & 1, status, &S->abort);
+}
+
+__device__ __forceinline__ bool stage_wait_full(TcRing *S, uint32_t n, int *status)
+{
+    return mbar_wait_a(&S->full[n % kStages], (n / kStages) & 1, status, &S->abort);
+}
+
+// Producer, at the end: do not leave while a copy may still be landing
+__device__ __forceinline__ void ring_drain(TcRing *S, uint32_t n, int *status)
+{
+    for (uint32_t q = (n > kStages ? n - kStages : 0); q < n; q++)
+        mbar_wait_a(&S->empty[q % kStages], (q / kStages) & 1, status, &S->abort);
+}
+
+// ---- tile ring: entry lt % kTiles holds this CTA's lt-th tile, drained by
+// group lt % 2
+//
+// Producer side: the next tiles of the shared list, their tables loading while
+// the tile before them streams.
+struct TileFetch {
+    const WorkItem *items;
+    const TcBatch *tb;
+    const DevBatch *batches;
+    const int *bsign;                            // H only
+    unsigned int *counter;
+    unsigned int n_items;
+    WorkItem it;                                 // current tile and its tables
+    TcBatch T;
+    int np, nfn, sign;
+    bool have;
+    WorkItem it1;                                // the next tile
+    bool have1;
+    unsigned int idx2;                           // index of the one after it
+};
+
+__device__ __forceinline__ void fetch_tables(TileFetch &F)
+{
+    if (!F.have) return;
+    F.T = F.tb[F.it.batch];
+    F.np = F.batches[F.it.batch].np;
+    F.nfn = F.batches[F.it.batch].nfn;
+    F.sign = F.bsign ? F.bsign[F.it.batch] : 0;
+}
+
+__device__ __forceinline__ WorkItem fetch_item(const TileFetch &F, unsigned int k, bool &have)
+{
+    have = k < F.n_items;
+    return have ? F.items[k] : WorkItem{0, 0, 0};
+}
+
+__device__ __forceinline__ void fetch_start(TileFetch &F)
+{
+    const unsigned int k0 = atomicAdd(F.counter, 1u), k1 = atomicAdd(F.counter, 1u);
+    F.idx2 = atomicAdd(F.counter, 1u);
+    F.it = fetch_item(F, k0, F.have);
+    F.it1 = fetch_item(F, k1, F.have1);
+    fetch_tables(F);
+}
+
+// the following tile becomes the current one
+__device__ __forceinline__ void fetch_next(TileFetch &F)
+{
+    F.it = F.it1;
+    F.have = F.have1;
+    F.it1 = fetch_item(F, F.idx2, F.have1);
+    F.idx2 = atomicAdd(F.counter, 1u);
+    fetch_tables(F);
+}
+
+__device__ __forceinline__ bool tile_wait_empty(TcRing *S, uint32_t lt, int *status)
+{
+    return lt < kTiles || mbar_wait_a(&S->nempty[lt % kTiles], (lt / kTiles - 1) & 1, status, &S->abort);
+}
+
+__device__ __forceinline__ bool tile_wait_full(TcRing *S, uint32_t lt, int *status)
+{
+    return mbar_wait_a(&S->nfull[lt % kTiles], (lt / kTiles) & 1, status, &S->abort);
+}
+
+// Producer, after its last tile (lt of them): an end mark for each group
+__device__ __forceinline__ void tiles_end(TcRing *S, uint32_t lt, int *status)
+{
+    for (uint32_t e = lt; e < lt + 2; e++) {
+        if (!tile_wait_empty(S, e, status)) return;
+        S->tile[e % kTiles].ti = -1;
+        mbar_arrive(&S->nfull[e % kTiles]);
+    }
+}
+
+// Epilogue group: its next tile; false at the end (or after a time-out) for
+// all of the group's threads alike, so that none skips a named barrier
+__device__ __forceinline__ bool group_next_tile(TcRing *S, uint32_t lt, int group, int tid, int *status)
+{
+    if (tid == 0) S->go[group] = tile_wait_full(S, lt, status) && S->tile[lt % kTiles].ti >= 0;
+    group_sync(group);
+    // every thread looks at the barrier itself: it orders the tile's copies before its reads
+    return S->go[group] != 0 && tile_wait_full(S, lt, status);
+}
+
+// Issue the split products of the first nks 16-deep steps of a 64-deep chunk:
+// every product of combined order <= ORDER except x2*y2; x0*y0 alone in
+// accumulator 0.  The plane and k-step offsets are added to the descriptors'
+// address field (addr >> 4, no carry out of it inside shared memory).
+// The tensor pipe holds few MMAs in its queue, so what its warp does between
+// them shows: the whole warp walks the loops and one lane issues, which leaves
+// the descriptors in uniform registers (40 instead of 50 cycles an MMA, 64 the
+// pipe needs), and a stage has one barrier each way.  Without epilogues a
+// 64-deep chunk takes 2252 cycles this way, 2048 of them the pipe's, and took
+// 2880 with one lane in divergent code and a barrier an operand.
 // first: the chunk opens the item (the first product into each accumulator
 // overwrites it).
 template <int NSPLIT, int ORDER, bool B_MN>
 __device__ __forceinline__ void mma_chunk(uint32_t acc_base, const uint8_t *a_sm, const uint8_t *b_sm, uint32_t idesc,
-                                          bool first)
+                                          bool first, int nks)
 {
-    const uint64_t ad0 = desc_sw128(smem_u32(a_sm), 16, 1024);
-    const uint64_t bd0 = B_MN ? desc_sw128(smem_u32(b_sm), 8192, 1024) : desc_sw128(smem_u32(b_sm), 16, 1024);
+    uint64_t ad0 = desc_sw128(smem_u32(a_sm), 16, 1024);
+    uint64_t bd0 = B_MN ? desc_sw128(smem_u32(b_sm), 8192, 1024) : desc_sw128(smem_u32(b_sm), 16, 1024);
+#pragma unroll 1
+    for (int ks = 0; ks < nks; ks++) {
+        if (elect_one()) {
 #pragma unroll
-    for (int ks = 0; ks < 4; ks++) {
+            for (int pa = 0; pa < NSPLIT; pa++) {
 #pragma unroll
-        for (int pa = 0; pa < NSPLIT; pa++) {
-#pragma unroll
-            for (int pb = 0; pb < NSPLIT; pb++) {
-                if (pa + pb > ORDER || (pa == 2 && pb == 2)) continue;
-                const int acc = (pa + pb == 0) ? 0 : 1;
-                const uint64_t ad = ad0 + (uint64_t)((pa * kChunkBytes + ks * 32) >> 4);
-                const uint64_t bd = bd0 + (uint64_t)((pb * kChunkBytes + ks * (B_MN ? 2048 : 32)) >> 4);
-                const bool opens = ks == 0 && (acc == 0 || (pa == 0 && pb == 1));
-                tc_mma(acc_base + acc * 128, ad, bd, idesc, (first && opens) ? 0u : 1u);
+                for (int pb = 0; pb < NSPLIT; pb++) {
+                    if (pa + pb > ORDER || (pa == 2 && pb == 2)) continue;
+                    const int acc = (pa + pb == 0) ? 0 : 1;
+                    const bool opens = acc == 0 || (pa == 0 && pb == 1);
+                    tc_mma(acc_base + acc * 128, ad0 + (uint64_t)((pa * kChunkBytes) >> 4),
+                           bd0 + (uint64_t)((pb * kChunkBytes) >> 4), idesc, (opens && first && ks == 0) ? 0u : 1u);
+                }
             }
         }
+        ad0 += 32 >> 4;
+        bd0 += (B_MN ? 2048 : 32) >> 4;
     }
 }
 
 __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_h(DevPlan P, const TcBatch *tb, const WorkItem *items,
                                                         int n_items, const uint8_t *ws, unsigned long long *hfix,
-                                                        int n_split, const int *bsign)
+                                                        int n_split, const int *bsign, unsigned int *counter)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *sm = align1024(smem_raw);
-    TcRing *S = reinterpret_cast<TcRing *>(sm + kStages * kStageBytes);
-    HPairTab *PT = reinterpret_cast<HPairTab *>(
-        (reinterpret_cast<uintptr_t>(S + 1) + 15) & ~(uintptr_t)15);
+    HTile *htile = reinterpret_cast<HTile *>(sm + kStages * kStageBytes);       // [kTiles]
+    HTables *tables = reinterpret_cast<HTables *>(htile + kTiles);            // [2]
+    TcRing *S = reinterpret_cast<TcRing *>(tables + 2);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) ring_init(S);
     if (warp == kWarpMma) {
@@ -1384,176 +1601,184 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_h(DevPlan P, const TcBatch
     const uint32_t tmem = S->tmem;
     const uint32_t chunk = (uint32_t)n_split * kChunkBytes;
 
+    // A = phi rows of block J (TMEM lanes), B = w v phi rows of block I (TMEM
+    // columns): the transposed tile, so that the scatter of one column i by the
+    // 32 lanes of a warp hits consecutive values of row i.  Batches where w v has
+    // one sign hold psi = phi sqrt|w v| in the phi image, which then serves as
+    // both operands; their diagonal tiles need one chunk for the two.
     if (warp == kWarpProducer) {
         if (lane == 0) {
-            long long n = 0;
+            uint32_t n = 0, lt = 0;
             bool ok = true;
-            for (int t = blockIdx.x; t < n_items && ok; t += gridDim.x) {
-                const WorkItem it = items[t];
-                const TcBatch T = tb[it.batch];
-                // A = phi rows of block J (TMEM lanes), B = w v phi rows of block I
-                // (TMEM columns): the transposed tile, so that the scatter of one
-                // column i by the 32 lanes of a warp hits consecutive values of row i.
-                // Batches where w v has one sign hold psi = phi sqrt|w v| in the
-                // phi image, which then serves as both operands.
-                const uint8_t *a_img = ws + T.img_phi;
-                const uint8_t *b_img = ws + (bsign[it.batch] != 0 ? T.img_phi : T.img_aux);
-                for (int c = 0; c < T.nc; c++, n++) {
-                    const int st = (int)(n % kStages);
-                    const long long use = n / kStages;
-                    if (use > 0 && !mbar_wait_a(&S->empty[st], (uint32_t)((use - 1) & 1), P.status, &S->abort)) {
-                        ok = false;
-                        break;
+            TileFetch F{};
+            F.items = items;
+            F.tb = tb;
+            F.batches = P.batches;
+            F.bsign = bsign;
+            F.counter = counter;
+            F.n_items = (unsigned int)n_items;
+            for (fetch_start(F); F.have && ok; lt++) {
+                const WorkItem it = F.it;
+                const TcBatch T = F.T;
+                const bool same = F.sign != 0 && it.ti == it.tj;
+                if (!(ok = tile_wait_empty(S, lt, P.status))) break;
+                const int e = (int)(lt % kTiles);
+                TileInfo &I = S->tile[e];
+                I.ti = it.ti;
+                I.tj = it.tj;
+                I.np = F.np;
+                I.nfn = F.nfn;
+                I.nc = T.nc;
+                I.sign = F.sign;
+                mbar_expect_tx(&S->nfull[e], 2 * (uint32_t)sizeof(HBlock));
+                const HBlock *hb = reinterpret_cast<const HBlock *>(ws + T.hblock);
+                bulk_g2s(&htile[e].i, hb + it.ti, sizeof(HBlock), &S->nfull[e]);
+                bulk_g2s(&htile[e].j, hb + it.tj, sizeof(HBlock), &S->nfull[e]);
+                const uint8_t *a_img = ws + T.img_phi + (long long)it.tj * T.nc_alloc * kChunkStride;
+                const uint8_t *b_img = ws + (F.sign != 0 ? T.img_phi : T.img_aux) + (long long)it.ti * T.nc_alloc * kChunkStride;
+                fetch_next(F);
+                for (int c = 0; c < T.nc; c++) {
+                    // the next tile's operands, if it is the first to read them (the
+                    // list goes through J at I = 0 first): their trip from DRAM to L2
+                    // passes behind this tile
+                    if (c == min(1, T.nc - 1) && F.have && F.it.ti == 0) {
+                        const uint32_t bytes = (uint32_t)(F.T.nc * kChunkStride);
+                        const long long blk = (long long)F.it.tj * F.T.nc_alloc * kChunkStride;
+                        bulk_prefetch(ws + F.T.img_phi + blk, bytes);
+                        if (F.sign == 0) bulk_prefetch(ws + F.T.img_aux + blk, bytes);
                     }
-                    uint8_t *a_sm = sm + st * kStageBytes, *b_sm = a_sm + 3 * kChunkBytes;
-                    mbar_expect_tx(&S->full[st], 2 * chunk);
-                    bulk_g2s(a_sm, a_img + (long long)(it.tj * T.nc_alloc + c) * kChunkStride, chunk, &S->full[st]);
-                    bulk_g2s(b_sm, b_img + (long long)(it.ti * T.nc_alloc + c) * kChunkStride, chunk, &S->full[st]);
+                    if (!(ok = stage_wait_empty(S, n, P.status))) break;
+                    const uint32_t q = n++ % kStages;
+                    uint8_t *dst = sm + q * kStageBytes;
+                    mbar_expect_tx(&S->full[q], same ? chunk : 2 * chunk);
+                    bulk_g2s(dst, a_img + (long long)c * kChunkStride, chunk, &S->full[q]);
+                    if (!same) bulk_g2s(dst + kOperandBytes, b_img + (long long)c * kChunkStride, chunk, &S->full[q]);
                 }
             }
-            // do not leave while a copy may still be landing
-            for (long long q = (n > kStages ? n - kStages : 0); q < n; q++)
-                mbar_wait_a(&S->empty[q % kStages], (uint32_t)((q / kStages) & 1), P.status, &S->abort);
+            if (ok) tiles_end(S, lt, P.status);
+            ring_drain(S, n, P.status);
+            // nor while a tile's descriptors may (the entries of older tiles have
+            // been read: the end marks took the next two places)
+            for (uint32_t q = lt + 2 > kTiles ? lt + 2 - kTiles : 0; q < lt; q++) tile_wait_full(S, q, P.status);
         }
         __syncwarp();
     } else if (warp == kWarpMma) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16(128, 128, false, false);
-            long long n = 0;
-            int lt = 0;
-            bool ok = true;
-            for (int t = blockIdx.x; t < n_items && ok; t += gridDim.x, lt++) {
-                const TcBatch T = tb[items[t].batch];
-                const int buf = lt & 1, use = lt >> 1;
-                if (use > 0 && !mbar_wait_a(&S->tempty[buf], (uint32_t)((use - 1) & 1), P.status, &S->abort)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                for (int c = 0; c < T.nc; c++, n++) {
-                    const int st = (int)(n % kStages);
-                    if (!mbar_wait_a(&S->full[st], (uint32_t)((n / kStages) & 1), P.status, &S->abort)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint8_t *a_sm = sm + st * kStageBytes;
-                    if (n_split == 3)
-                        mma_chunk<3, 3, false>(tmem + buf * 256, a_sm, a_sm + 3 * kChunkBytes, idesc, c == 0);
-                    else
-                        mma_chunk<1, 0, false>(tmem + buf * 256, a_sm, a_sm + 3 * kChunkBytes, idesc, c == 0);
-                    tc_commit(&S->empty[st]);
-                }
-                tc_commit(&S->tfull[buf]);
+        uint32_t n = 0;
+        bool ok = true;
+        for (uint32_t lt = 0; ok && __all_sync(0xffffffffu, tile_wait_full(S, lt, P.status)); lt++) {
+            const int e = (int)(lt % kTiles);
+            const int ti = S->tile[e].ti, tj = S->tile[e].tj, np = S->tile[e].np, nfn = S->tile[e].nfn, nc = S->tile[e].nc;
+            const bool same = S->tile[e].sign != 0 && ti == tj;
+            if (ti < 0) break;
+            __syncwarp();
+            if (elect_one()) mbar_arrive(&S->nempty[e]);
+            // the columns of the last block end at n_b
+            const uint32_t idesc = idesc_bf16(128, min(128, (nfn - ti * 128 + 15) & ~15), false, false);
+            const uint32_t buf = lt & 1, use = lt >> 1;
+            ok = use == 0 || mbar_wait_a(&S->tempty[buf], (use - 1) & 1, P.status, &S->abort);
+            tc_fence_after();
+            for (int c = 0; c < nc; c++, n++) {
+                ok = __all_sync(0xffffffffu, ok && stage_wait_full(S, n, P.status));
+                if (!ok) break;
+                // steps past the batch's points would add zeros
+                const int nks = min(4, (np - c * 64 + 15) >> 4);
+                const uint8_t *a_sm = sm + (n % kStages) * kStageBytes, *b_sm = same ? a_sm : a_sm + kOperandBytes;
+                if (n_split == 3)
+                    mma_chunk<3, 3, false>(tmem + buf * 256, a_sm, b_sm, idesc, c == 0, nks);
+                else
+                    mma_chunk<1, 0, false>(tmem + buf * 256, a_sm, b_sm, idesc, c == 0, nks);
+                if (elect_one()) tc_commit(&S->empty[n % kStages]);
             }
+            if (elect_one()) tc_commit(&S->tfull[buf]);
         }
         __syncwarp();
     } else {
-        // epilogue warp w: TMEM lanes 32 (w % 4) .. + 31 (functions j of block J),
-        // columns 64 (w / 4) .. + 63 (functions i of block I)
-        int lt = 0;
+        // Warp w of a group: TMEM lanes 32 (w % 4) .. + 31 (functions j of block
+        // J), columns 64 (w / 4) .. + 63 (functions i of block I).  Bound by the
+        // instructions of the conversion to fixed point (about 20 a value).
+        const int group = warp >> 3, quad = warp & 3, half = (warp >> 2) & 1;
+        const int tid = threadIdx.x & (kGroupThreads - 1), r = quad * 32 + lane;
+        HTables &H = tables[group];
+        const uint32_t acc_base = tmem + group * 256 + ((uint32_t)(quad * 32) << 16);
         bool bad = false;
-        const int quad = warp & 3, half = warp >> 2;
-        const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
-        for (int t = blockIdx.x; t < n_items; t += gridDim.x, lt++) {
-            const WorkItem it = items[t];
-            const DevBatch B = P.batches[it.batch];
-            const DevAct *act = P.act + B.act0;
-            const int buf = lt & 1, use = lt >> 1;
-            const int i0 = it.ti * 128, j0 = it.tj * 128;
-            const int *pp_sys = P.pairpos + P.sys_pair_off[B.sys];
-            const int nat = P.sys_nat[B.sys];
-            if (threadIdx.x < 128) {
-                const int i = i0 + threadIdx.x;
-                const int ilast = min(i0 + 127, B.nfn - 1);
-                if (i <= ilast) {
-                    const int e_first = find_act(act, B.n_act, i0);
-                    const int e = find_act(act, B.n_act, i);
-                    const FnRef c = fn_ref(P, act, e, i);
-                    const int slot = e - e_first;
-                    S->ref[buf][threadIdx.x] = ColRef{c.rp - c.li, c.atom, c.loc, slot, 0};
-                    if (slot < kColAtoms && (i == i0 || act[e].fn_loc == i))
-                        PT->atom[buf][slot] = make_int2(c.atom, c.loc);
-                    if (i == ilast) PT->nslot[buf] = slot + 1;
-                } else {
-                    S->ref[buf][threadIdx.x] = ColRef{0, -1, 0, 0, 0};   // past the batch: a valid slot, never stored
+        for (uint32_t lt = group; group_next_tile(S, lt, group, tid, P.status); lt += 2) {
+            const int e = (int)(lt % kTiles);
+            const int ti = S->tile[e].ti, tj = S->tile[e].tj;
+            const HBlock &bi = htile[e].i, &bj = htile[e].j;
+            const int ncol = bi.n, ni = bi.nslot, nj = bj.nslot;
+            const float scale = S->tile[e].sign < 0 ? -256.f : 256.f;    // H = -psi^T psi
+            const int *pp_sys = P.pairpos + bi.pair_off;
+            const long long nat = bi.nat;
+            const bool tab = ni <= kPairSlots && nj <= kPairSlots;
+            if (tid < 128)
+                H.col[tid] = HColumn{(unsigned long long)__cvta_generic_to_global(hfix + bi.base[tid]),
+                                     bi.slot[tid] * kPairSlots, 0};
+            if (tab) {
+                for (int q = tid; q < ni * kPairSlots; q += kGroupThreads) {
+                    const int a = q / kPairSlots, b = q % kPairSlots;
+                    if (b >= nj) continue;
+                    const int pp = bi.loc[a] == bj.loc[b] ? 0 : __ldg(pp_sys + bi.loc[a] * nat + bj.loc[b]);
+                    H.pair[q] = pp < 0 ? INT_MIN : 8 * pp;
                 }
             }
-            const int r = quad * 32 + lane;
-            const int j = j0 + r;                  // this lane's function (block J)
-            FnRef jref{};
-            if (j < B.nfn) jref = fn_ref(P, act, find_act(act, B.n_act, j), j);
-            const bool negate = bsign[it.batch] < 0;            // H = -psi^T psi
-            epi_sync();
-            // pair offsets of this tile (the previous tile's scatter is over)
-            const int nslot = PT->nslot[buf];
-            const bool tab = nslot <= kColAtoms;
-            if (tab && j < B.nfn) {
-                for (int sl = half; sl < nslot; sl += 2) {
-                    const int2 a = PT->atom[buf][sl];
-                    PT->pp[sl][r] = a.x == jref.atom ? 0 : __ldg(pp_sys + (long long)a.y * nat + jref.loc);
-                }
-            }
-            epi_sync();
-            const bool ok = mbar_wait_a(&S->tfull[buf], (uint32_t)(use & 1), P.status, &S->abort);
+            // this lane's function j
+            const int sj = bj.slot[r], lj = 8 * bj.li[r], locj = bj.loc[sj];
+            const bool inj = r < bj.n;
+            group_sync(group);
+            const bool ok = mbar_wait_a(&S->tfull[group], (lt >> 1) & 1, P.status, &S->abort);
             tc_fence_after();
-            const uint32_t acc_base = tmem + buf * 256 + lane_base;
+            // (i, j) is stored for i <= j: only diagonal tiles cross that line
+            const int rlim = !inj ? -1 : ti == tj ? r : 127;
             for (int cq = 0; cq < 2; cq++) {
-                const int cc = 2 * half + cq;
-                if (i0 + cc * 32 >= B.nfn) break;
+                const int c0 = 64 * half + 32 * cq;
+                if (c0 >= ncol) break;
                 float a0[32], a1[32];
-                tmem_ld32(acc_base + cc * 32, a0);
-                if (n_split > 1) tmem_ld32(acc_base + 128 + cc * 32, a1);
+                tmem_ld32(acc_base + c0, a0);
+                if (n_split > 1) tmem_ld32(acc_base + 128 + c0, a1);
+                else
+#pragma unroll
+                    for (int q = 0; q < 32; q++) a1[q] = 0.f;
                 tmem_wait_ld();
-                if (!ok || j >= B.nfn) continue;
-                // stored value of (i, j), i <= j: row i, (rp_i - li) + [pair offset of
-                // atom(j) in row i, 0 for the same atom] + lj
-                unsigned long long *hj = hfix + jref.li;
-                if (tab) {
-                    // branch-free per column (predicated atomics), so the conversions
-                    // of neighbouring columns overlap
+                if (!ok) continue;
+                float size = 0.f;
+#pragma unroll
+                for (int q = 0; q < 32; q++) size = max_abs_nan(size, a0[q], a1[q]);
+                if (tab && !__any_sync(0xffffffffu, !(size < 16384.f))) {
+                    // v 2^8 = h + f with h its rounding (by an addition, the FRND unit
+                    // is slow), f exact: h 2^32 + f 2^32 in units of 2^-40, the sign of
+                    // the batch in the factor
 #pragma unroll
                     for (int q = 0; q < 32; q++) {
-                        const int il = cc * 32 + q;
-                        const int i = i0 + il;
-                        const long long rpl = S->ref[buf][il].rpl;
-                        const int ppv = PT->pp[S->ref[buf][il].slot][r];
-                        long long fx = f32_to_fix(a0[q], bad);
-                        if (n_split > 1) fx += f32_to_fix(a1[q], bad);
-                        if (negate) fx = -fx;
-                        if (i < B.nfn && i <= j && ppv >= 0 && fx != 0)
-                            atomicAdd(hj + rpl + ppv, (unsigned long long)fx);
+                        const int il = c0 + q;
+                        const HColumn col = H.col[il];
+                        const int off = H.pair[col.pair_row + sj];
+                        const float h0 = fmaf(a0[q], scale, kRoundMagic), h1 = fmaf(a1[q], scale, kRoundMagic);
+                        const float f0 = fmaf(a0[q], scale, -(h0 - kRoundMagic)), f1 = fmaf(a1[q], scale, -(h1 - kRoundMagic));
+                        // the words of kRoundMagic + h less those of kRoundMagic
+                        const int hi = (int)(__float_as_uint(h0) + __float_as_uint(h1) - 2u * 0x4B400000u);
+                        const long long fx = (((long long)hi << 32) + __float2int_rz(f0 * 4294967296.f)) +
+                                             __float2int_rz(f1 * 4294967296.f);
+                        red_add_if(off >= 0 && il <= rlim && fx != 0, col.base + (unsigned int)(off + lj), fx);
                     }
                     continue;
                 }
-                int cur_atom = -1;                 // more column atoms than table slots
-                int ppv = 0;
-                bool stored = false;
+                // values of 2^14 Ha and more (or not finite), or more atoms than the
+                // pair table holds
+                const float sgn = scale * 0.00390625f;
 #pragma unroll
                 for (int q = 0; q < 32; q++) {
-                    const int il = cc * 32 + q;
-                    const int i = i0 + il;
-                    if (i >= B.nfn || i > j) continue;
-                    const ColRef ci = S->ref[buf][il];
-                    if (ci.atom != cur_atom) {
-                        cur_atom = ci.atom;
-                        if (ci.atom == jref.atom) {
-                            ppv = 0;
-                            stored = true;
-                        } else {
-                            ppv = __ldg(pp_sys + (long long)ci.loc * nat + jref.loc);
-                            stored = ppv >= 0;
-                        }
-                    }
-                    if (!stored) continue;
-                    long long fx = f32_to_fix(a0[q], bad);
-                    if (n_split > 1) fx += f32_to_fix(a1[q], bad);
-                    if (negate) fx = -fx;
-                    if (fx != 0) atomicAdd(hj + ci.rpl + ppv, (unsigned long long)fx);
+                    const int il = c0 + q;
+                    if (il > rlim || il >= ncol) continue;
+                    const int loci = bi.loc[bi.slot[il]];
+                    const int pp = loci == locj ? 0 : __ldg(pp_sys + loci * nat + locj);
+                    const long long fx = f32_to_fix(a0[q] * sgn, bad) + f32_to_fix(a1[q] * sgn, bad);
+                    red_add_if(pp >= 0 && fx != 0, H.col[il].base + 8ll * pp + lj, fx);
                 }
             }
             tc_fence_before();
-            mbar_arrive(&S->tempty[buf]);
+            mbar_arrive(&S->tempty[group]);
+            group_sync(group);                     // the tables may be filled again
+            if (tid == 0) mbar_arrive(&S->nempty[e]);
         }
         if (bad) atomicOr(P.status, kStatusNonFinite);
     }
@@ -1776,12 +2001,13 @@ __global__ void __launch_bounds__(256) k_tc_gather_d(DevPlan P, const TcBatch *t
 }
 
 // ------------------------------------------------- density on tcgen05 (K3b)
-// Persistent: one CTA per SM walks the items (batch, 128-point tile m,
-// 128-function block J), J ascending so the longest contractions come first:
+// Persistent, with the roles, the rings and the tile counter of the H
+// contraction, over the items (batch, 128-point tile m, 128-function block J),
+// J ascending so the longest contractions come first:
 // E^T[j][p] = sum_{i >= 128 J} D'[j][i] phi_i(p) over the upper block
 // triangle of the symmetric D (D' = D with its diagonal block halved;
 // A = D image, K-major; B = phi image read as MN-major) accumulates in one of
-// two tensor-memory sets while warps 0-7 finish the previous item: the
+// two tensor-memory sets while a group of warps finishes an earlier item: the
 // partial density sum_{j in J} E^T[j][p] phi_j(p) in double-float (lane j
 // multiplies by its own phi row, the warp reduces over j), one row of 128
 // doubles per item.  Many items per batch keep the CTAs on few batches at a
@@ -1794,12 +2020,12 @@ __global__ void __launch_bounds__(256) k_tc_gather_d(DevPlan P, const TcBatch *t
 template <bool ADJ>
 __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_density(DevPlan P, const TcBatch *tb, const WorkItem *items,
                                                               int n_items, const uint8_t *ws, double *part,
-                                                              int n_split, uint8_t *ws_e)
+                                                              int n_split, uint8_t *ws_e, unsigned int *counter)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *sm = align1024(smem_raw);
     TcRing *S = reinterpret_cast<TcRing *>(sm + kStages * kStageBytes);
-    __shared__ double red[4][128];
+    __shared__ double red[2][4][128];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) ring_init(S);
     if (warp == kWarpMma) {
@@ -1814,186 +2040,194 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_density(DevPlan P, const T
 
     if (warp == kWarpProducer) {
         if (lane == 0) {
-            long long n = 0;
+            uint32_t n = 0, lt = 0;
             bool ok = true;
-            for (int t = blockIdx.x; t < n_items && ok; t += gridDim.x) {
-                const WorkItem it = items[t];
-                const TcBatch T = tb[it.batch];
-                const int m = it.ti, J = it.tj;
-                const uint8_t *d_img = ws + T.img_aux, *phi_img = ws + T.img_phi;
-                for (int kc = ADJ ? 0 : 2 * J; kc < T.nkc; kc++, n++) {
-                    const int st = (int)(n % kStages);
-                    const long long use = n / kStages;
-                    if (use > 0 && !mbar_wait_a(&S->empty[st], (uint32_t)((use - 1) & 1), P.status, &S->abort)) {
-                        ok = false;
-                        break;
+            TileFetch F{};
+            F.items = items;
+            F.tb = tb;
+            F.batches = P.batches;
+            F.counter = counter;
+            F.n_items = (unsigned int)n_items;
+            for (fetch_start(F); F.have && ok; lt++) {
+                const TcBatch T = F.T;
+                const int m = F.it.ti, J = F.it.tj;
+                if (!(ok = tile_wait_empty(S, lt, P.status))) break;
+                TileInfo &I = S->tile[lt % kTiles];
+                I.ti = m;
+                I.tj = J;
+                I.np = F.np;
+                I.nfn = F.nfn;
+                I.nkc = T.nkc;
+                I.nc_alloc = T.nc_alloc;
+                I.img_phi = T.img_phi;
+                I.img_e = T.img_e;
+                I.part_row = T.part0 + (long long)J * (T.nc_alloc / 2) + m;
+                mbar_arrive(&S->nfull[lt % kTiles]);
+                fetch_next(F);
+                const uint8_t *d_img = ws + T.img_aux + (long long)J * T.nkc * kChunkStride, *phi_img = ws + T.img_phi;
+                // a last tile of at most 64 points has one column chunk
+                const int halves = 2 * m + 1 < T.nc ? 2 : 1;
+                const int kc0 = ADJ ? 0 : 2 * J;
+                for (int kc = kc0; kc < T.nkc; kc++) {
+                    // the next tile's operands, if it is the first to read them (its
+                    // point tile at J = 0, its block of D at m = 0): their trip from
+                    // DRAM to L2 passes behind this tile
+                    if (kc == min(kc0 + 1, T.nkc - 1) && F.have) {
+                        if (F.it.tj == 0)
+                            for (int I = 0; I < F.T.nrb; I++)
+                                bulk_prefetch(ws + F.T.img_phi + (long long)(I * F.T.nc_alloc + 2 * F.it.ti) * kChunkStride,
+                                              2 * kChunkStride);
+                        if (F.it.ti == 0) {
+                            const int k0 = ADJ ? 0 : 2 * F.it.tj;
+                            bulk_prefetch(ws + F.T.img_aux + ((long long)F.it.tj * F.T.nkc + k0) * kChunkStride,
+                                          (uint32_t)(F.T.nkc - k0) * kChunkStride);
+                        }
                     }
-                    uint8_t *a_sm = sm + st * kStageBytes, *b_sm = a_sm + 3 * kChunkBytes;
-                    mbar_expect_tx(&S->full[st], 2 * chunk);
-                    const int I = kc >> 1, half = kc & 1;
-                    bulk_g2s(a_sm, d_img + (long long)(J * T.nkc + kc) * kChunkStride, chunk, &S->full[st]);
-                    for (int s = 0; s < n_split; s++)
-                        for (int c2 = 0; c2 < 2; c2++)
-                            bulk_g2s(b_sm + s * kChunkBytes + c2 * 8192,
-                                     phi_img + (long long)(I * T.nc_alloc + 2 * m + c2) * kChunkStride +
-                                         s * kChunkBytes + half * 8192,
-                                     8192, &S->full[st]);
+                    if (!(ok = stage_wait_empty(S, n, P.status))) break;
+                    const uint32_t q = n++ % kStages;
+                    uint8_t *dst = sm + q * kStageBytes;
+                    mbar_expect_tx(&S->full[q], chunk + (uint32_t)(n_split * halves * 8192));
+                    bulk_g2s(dst, d_img + (long long)kc * kChunkStride, chunk, &S->full[q]);
+                    for (int c2 = 0; c2 < halves; c2++)
+                        for (int s = 0; s < n_split; s++)
+                            bulk_g2s(dst + kOperandBytes + s * kChunkBytes + c2 * 8192,
+                                     phi_img + (long long)((kc >> 1) * T.nc_alloc + 2 * m + c2) * kChunkStride +
+                                         s * kChunkBytes + (kc & 1) * 8192,
+                                     8192, &S->full[q]);
                 }
             }
-            for (long long q = (n > kStages ? n - kStages : 0); q < n; q++)
-                mbar_wait_a(&S->empty[q % kStages], (uint32_t)((q / kStages) & 1), P.status, &S->abort);
+            if (ok) tiles_end(S, lt, P.status);
+            ring_drain(S, n, P.status);
         }
         __syncwarp();
     } else if (warp == kWarpMma) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16(128, 128, false, true);
-            long long n = 0;
-            int u = 0;
-            bool ok = true;
-            for (int t = blockIdx.x; t < n_items && ok; t += gridDim.x, u++) {
-                const WorkItem it = items[t];
-                const TcBatch T = tb[it.batch];
-                const int J = it.tj;
-                const int buf = u & 1, use = u >> 1;
-                if (use > 0 && !mbar_wait_a(&S->tempty[buf], (uint32_t)((use - 1) & 1), P.status, &S->abort)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                const int kc0 = ADJ ? 0 : 2 * J;
-                for (int kc = kc0; kc < T.nkc; kc++, n++) {
-                    const int st = (int)(n % kStages);
-                    if (!mbar_wait_a(&S->full[st], (uint32_t)((n / kStages) & 1), P.status, &S->abort)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint8_t *a_sm = sm + st * kStageBytes;
-                    if (n_split == 3)
-                        mma_chunk<3, kDensityOrder, true>(tmem + buf * 256, a_sm, a_sm + 3 * kChunkBytes, idesc,
-                                                          kc == kc0);
-                    else
-                        mma_chunk<1, 0, true>(tmem + buf * 256, a_sm, a_sm + 3 * kChunkBytes, idesc, kc == kc0);
-                    tc_commit(&S->empty[st]);
-                }
-                tc_commit(&S->tfull[buf]);
+        uint32_t n = 0;
+        bool ok = true;
+        for (uint32_t lt = 0; ok && __all_sync(0xffffffffu, tile_wait_full(S, lt, P.status)); lt++) {
+            const int e = (int)(lt % kTiles);
+            const int m = S->tile[e].ti, J = S->tile[e].tj, np = S->tile[e].np, nfn = S->tile[e].nfn, nkc = S->tile[e].nkc;
+            if (m < 0) break;
+            __syncwarp();
+            if (elect_one()) mbar_arrive(&S->nempty[e]);
+            // the last tile's columns end at the batch's points
+            const uint32_t idesc = idesc_bf16(128, min(128, (np - m * 128 + 15) & ~15), false, true);
+            const uint32_t buf = lt & 1, use = lt >> 1;
+            ok = use == 0 || mbar_wait_a(&S->tempty[buf], (use - 1) & 1, P.status, &S->abort);
+            tc_fence_after();
+            const int kc0 = ADJ ? 0 : 2 * J;
+            for (int kc = kc0; kc < nkc; kc++, n++) {
+                ok = __all_sync(0xffffffffu, ok && stage_wait_full(S, n, P.status));
+                if (!ok) break;
+                // steps past the batch's functions would add zeros
+                const int nks = min(4, (nfn - kc * 64 + 15) >> 4);
+                const uint8_t *a_sm = sm + (n % kStages) * kStageBytes, *b_sm = a_sm + kOperandBytes;
+                if (n_split == 3)
+                    mma_chunk<3, kDensityOrder, true>(tmem + buf * 256, a_sm, b_sm, idesc, kc == kc0, nks);
+                else
+                    mma_chunk<1, 0, true>(tmem + buf * 256, a_sm, b_sm, idesc, kc == kc0, nks);
+                if (elect_one()) tc_commit(&S->empty[n % kStages]);
             }
+            if (elect_one()) tc_commit(&S->tfull[buf]);
         }
         __syncwarp();
     } else {
-        // epilogue warp w: TMEM lanes 32 (w % 4) .. + 31 (functions j of the
-        // block), point columns 64 (w / 4) .. + 63
-        const int quad = warp & 3, half = warp >> 2;
-        const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
-        int u = 0;
-        bool ok = true;
-        for (int t = blockIdx.x; t < n_items; t += gridDim.x, u++) {
-            const WorkItem it = items[t];
-            const DevBatch B = P.batches[it.batch];
-            const TcBatch T = tb[it.batch];
-            const int m = it.ti, J = it.tj;
-            const uint8_t *phi_img = ws + T.img_phi;
-            const int buf = u & 1, use = u >> 1;
-            const int r = quad * 32 + lane;
+        // Warp w of a group: TMEM lanes 32 (w % 4) .. + 31 (functions j of the
+        // block), point columns 64 (w / 4) .. + 63, sixteen at a time.  Bound by
+        // its FP32 instructions (about 30 a value of E).
+        const int group = warp >> 3, quad = warp & 3, half = (warp >> 2) & 1;
+        const int tid = threadIdx.x & (kGroupThreads - 1), r = quad * 32 + lane;
+        const uint32_t acc_base = tmem + group * 256 + ((uint32_t)(quad * 32) << 16);
+        for (uint32_t lt = group; group_next_tile(S, lt, group, tid, P.status); lt += 2) {
+            const TileInfo T = S->tile[lt % kTiles];
+            const int m = T.ti, J = T.tj;
             const int j = J * 128 + r;
-            // this warp's phi rows for the first of its two column chunks: issued
-            // before the wait so the loads overlap the MMAs
-            uint4 pre[3][4];
-            {
-                const int cc = 2 * half, c = 2 * m + (cc >> 1);
+            const bool live = j < T.nfn;
+            // this lane's phi row at the warp's 64 points (one chunk): two 16-byte
+            // units a plane for 16 points, loaded ahead of their use
+            const uint8_t *row = ws + T.img_phi + (long long)(J * T.nc_alloc + 2 * m + half) * kChunkStride;
+            uint4 w[2][3];
+            auto load_units = [&](int piece) {
 #pragma unroll
-                for (int gg = 0; gg < 4; gg++) {
-                    const long long off = unit_offset(J, T.nc_alloc, c, r, (cc & 1) * 4 + gg);
-#pragma unroll
-                    for (int sp = 0; sp < 3; sp++)
-                        pre[sp][gg] = sp < n_split ? *reinterpret_cast<const uint4 *>(phi_img + off + sp * kChunkBytes)
-                                                   : make_uint4(0u, 0u, 0u, 0u);
-                }
-            }
-            ok = mbar_wait_a(&S->tfull[buf], (uint32_t)(use & 1), P.status, &S->abort);
-            tc_fence_after();
-            const uint32_t acc_base = tmem + buf * 256 + lane_base;
-            for (int cq = 0; cq < 2; cq++) {
-                const int cc = 2 * half + cq;
-                float a0[32], a1[32];
-                tmem_ld32(acc_base + cc * 32, a0);
-                if (n_split > 1)
-                    tmem_ld32(acc_base + 128 + cc * 32, a1);
-                else
-#pragma unroll
-                    for (int q = 0; q < 32; q++) a1[q] = 0.f;
-                tmem_wait_ld();
-                if (cq == 1) {
-                    tc_fence_before();
-                    mbar_arrive(&S->tempty[buf]);     // accumulator set may be reused
-                }
-                // E^T[j][p] phi_j(p) for the 32 points of this column chunk in
-                // double-float (FP32 pipe): e = acc0 + acc1, phi = sum of its planes
-                const int c = 2 * m + (cc >> 1);
-                const bool live = ok && j < B.nfn;
-                if (ADJ && live) {
-                    // this lane's row of E at the chunk's 32 points, for the gradient
-                    float4 *dst = reinterpret_cast<float4 *>(ws_e + T.img_e) +
-                                  ((long long)j * T.nc_alloc * 64 + m * 128 + cc * 32) / 4;
-#pragma unroll
-                    for (int q4 = 0; q4 < 8; q4++)
-                        dst[q4] = make_float4(a0[4 * q4] + a1[4 * q4], a0[4 * q4 + 1] + a1[4 * q4 + 1],
-                                              a0[4 * q4 + 2] + a1[4 * q4 + 2], a0[4 * q4 + 3] + a1[4 * q4 + 3]);
-                }
-#pragma unroll
-                for (int gg = 0; gg < 4; gg++) {
-                    const int g = (cc & 1) * 4 + gg;
-                    const long long off = unit_offset(J, T.nc_alloc, c, r, g);
-                    uint32_t w[3][4] = {};
+                for (int g = 0; g < 2; g++)
 #pragma unroll
                     for (int sp = 0; sp < 3; sp++) {
-                        uint4 uu;
-                        if (cq == 0)
-                            uu = pre[sp][gg];
-                        else
-                            uu = sp < n_split ? *reinterpret_cast<const uint4 *>(phi_img + off + sp * kChunkBytes)
-                                              : make_uint4(0u, 0u, 0u, 0u);
-                        w[sp][0] = uu.x; w[sp][1] = uu.y; w[sp][2] = uu.z; w[sp][3] = uu.w;
+                        w[g][sp] = make_uint4(0u, 0u, 0u, 0u);
+                        if (live && sp < n_split)
+                            w[g][sp] = *reinterpret_cast<const uint4 *>(
+                                row + row_offset((uint32_t)r, (uint32_t)(2 * piece + g) << 4) + sp * kChunkBytes);
                     }
+            };
+            load_units(0);
+            const bool ok = mbar_wait_a(&S->tfull[group], (lt >> 1) & 1, P.status, &S->abort);
+            tc_fence_after();
+#pragma unroll 1
+            for (int piece = 0; piece < 4; piece++) {
+                const int c0 = 64 * half + 16 * piece;
+                float hi[16], lo[16];
+                tmem_ld16(acc_base + c0, hi);
+                if (n_split > 1) tmem_ld16(acc_base + 128 + c0, lo);
+                else
+#pragma unroll
+                    for (int q = 0; q < 16; q++) lo[q] = 0.f;
+                tmem_wait_ld();
+                if (piece == 3) {
+                    tc_fence_before();
+                    mbar_arrive(&S->tempty[group]);   // accumulator set may be reused
+                }
+                if (ADJ && live && ok) {
+                    // this lane's row of E at the 16 points, for the gradient
+                    float4 *dst = reinterpret_cast<float4 *>(ws_e + T.img_e) +
+                                  ((long long)j * T.nc_alloc * 64 + m * 128 + c0) / 4;
+#pragma unroll
+                    for (int q = 0; q < 4; q++)
+                        dst[q] = make_float4(hi[4 * q] + lo[4 * q], hi[4 * q + 1] + lo[4 * q + 1],
+                                             hi[4 * q + 2] + lo[4 * q + 2], hi[4 * q + 3] + lo[4 * q + 3]);
+                }
+                // E^T[j][p] phi_j(p) in double-float: e = acc0 + acc1, phi = f0 + (f1 +
+                // f2), whose inner sum is exact and never larger than a non-zero f0
+#pragma unroll
+                for (int g = 0; g < 2; g++)
 #pragma unroll
                     for (int q = 0; q < 8; q++) {
-                        const int col = gg * 8 + q;
-                        const float f0 = __uint_as_float((q & 1) ? (w[0][q >> 1] & 0xFFFF0000u) : (w[0][q >> 1] << 16));
-                        const float f1 = __uint_as_float((q & 1) ? (w[1][q >> 1] & 0xFFFF0000u) : (w[1][q >> 1] << 16));
-                        const float f2 = __uint_as_float((q & 1) ? (w[2][q >> 1] & 0xFFFF0000u) : (w[2][q >> 1] << 16));
-                        df ph = df_two_sum(f0, f1);
-                        ph = df_fast_two_sum(ph.hi, ph.lo + f2);
-                        const df e = df_two_sum(a0[col], n_split > 1 ? a1[col] : 0.f);
-                        const df pr = df_mul(e, ph);
-                        a0[col] = live ? pr.hi : 0.f;
-                        a1[col] = live ? pr.lo : 0.f;
+                        const int k = 8 * g + q;
+                        auto term = [&](const uint4 &u) {
+                            const uint32_t x = (q >> 1) == 0 ? u.x : (q >> 1) == 1 ? u.y : (q >> 1) == 2 ? u.z : u.w;
+                            return __uint_as_float((q & 1) ? (x & 0xFFFF0000u) : (x << 16));
+                        };
+                        const df ph = df_fast_two_sum(term(w[g][0]), term(w[g][1]) + term(w[g][2]));
+                        const df e = df_two_sum(hi[k], lo[k]);
+                        const float p = e.hi * ph.hi;
+                        lo[k] = fmaf(e.lo, ph.hi, fmaf(e.hi, ph.lo, fmaf(e.hi, ph.hi, -p)));
+                        hi[k] = p;
                     }
-                }
-                // reduce over the 32 lanes (rows j): lane q ends with column q
+                if (piece < 3) load_units(piece + 1);
+                // sum over the 32 lanes (rows j), halving the columns a lane holds: the
+                // high parts with their rounding errors, the low parts plainly
 #pragma unroll
-                for (int wd = 16; wd >= 1; wd >>= 1) {
-                    const bool upper = (lane & wd) != 0;
+                for (int wd = 8; wd >= 1; wd >>= 1) {
+                    const bool upper = (lane & (2 * wd)) != 0;
 #pragma unroll
                     for (int q = 0; q < wd; q++) {
-                        const float sh = upper ? a0[q] : a0[q + wd], sl = upper ? a1[q] : a1[q + wd];
-                        const float kh = upper ? a0[q + wd] : a0[q], kl = upper ? a1[q + wd] : a1[q];
-                        const df rcv{__shfl_xor_sync(0xffffffffu, sh, wd), __shfl_xor_sync(0xffffffffu, sl, wd)};
-                        const df sum = df_add(df{kh, kl}, rcv);
-                        a0[q] = sum.hi;
-                        a1[q] = sum.lo;
+                        const float sh = upper ? hi[q] : hi[q + wd], sl = upper ? lo[q] : lo[q + wd];
+                        const float kh = upper ? hi[q + wd] : hi[q], kl = upper ? lo[q + wd] : lo[q];
+                        const df t2 = df_two_sum(kh, __shfl_xor_sync(0xffffffffu, sh, 2 * wd));
+                        hi[q] = t2.hi;
+                        lo[q] = t2.lo + (kl + __shfl_xor_sync(0xffffffffu, sl, 2 * wd));
                     }
                 }
-                red[quad][cc * 32 + lane] = (double)a0[0] + (double)a1[0];
+                const df t2 = df_two_sum(hi[0], __shfl_xor_sync(0xffffffffu, hi[0], 1));
+                const float tl = t2.lo + (lo[0] + __shfl_xor_sync(0xffffffffu, lo[0], 1));
+                if ((lane & 1) == 0) red[group][quad][c0 + (lane >> 1)] = (double)t2.hi + (double)tl;
             }
             // item complete: this block's partial density at the tile's 128 points
-            epi_sync();
-            if (threadIdx.x < 128) {
-                const long long row = T.part0 + (long long)J * (T.nc_alloc / 2) + m;
-                part[row * 128 + threadIdx.x] =
-                    ok ? (red[0][threadIdx.x] + red[1][threadIdx.x]) + (red[2][threadIdx.x] + red[3][threadIdx.x])
-                       : 0.0;
+            group_sync(group);
+            if (tid == 0) mbar_arrive(&S->nempty[lt % kTiles]);
+            if (tid < 128) {
+                part[T.part_row * 128 + tid] = ok ? (red[group][0][tid] + red[group][1][tid]) +
+                                                  (red[group][2][tid] + red[group][3][tid])
+                                            : 0.0;
             }
-            epi_sync();
+            group_sync(group);
         }
     }
     tc_fence_before();
@@ -2126,7 +2360,9 @@ size_t smem_tc(int n_split)
 // the bound pass keeps knots (bound_grids 2), the pass over the points offsets
 size_t smem_phi(bool bound) { return bound ? kKnotCache * sizeof(unsigned short) : kGeoCache * sizeof(float4); }
 
-size_t smem_tc_h() { return smem_tc(3) + sizeof(HPairTab) + 16; }
+size_t smem_tc_h() { return smem_tc(3) + kTiles * sizeof(HTile) + 2 * sizeof(HTables); }
+static_assert(1024 + kStages * kStageBytes + sizeof(TcRing) + kTiles * sizeof(HTile) + 2 * sizeof(HTables) <= 232448,
+              "the H contraction's shared memory");
 
 bool attrs_set = false;
 
@@ -2232,6 +2468,11 @@ int tc_build(TcPlan &t, const TcPlanInput &in, std::string *err)
         T.plane_phi = (long long)T.nrb * T.nc_alloc * kChunkBytes;
         T.plane_d = (long long)T.nrb * T.nkc * kChunkBytes;
         foot[b] = 3 * (size_t)T.plane_phi + 3 * (size_t)std::max(T.plane_phi, T.plane_d);
+        T.hblock = -1;
+        if (in.for_h) {
+            // phi and w v phi images, and the row blocks' descriptors
+            foot[b] = 6 * (size_t)T.plane_phi + ((size_t)T.nrb * sizeof(HBlock) + 1023) / 1024 * 1024;
+        }
         T.img_e = -1;
         if (in.with_e) foot[b] += 2 * (size_t)T.plane_phi;     // E in FP32: twice a BF16 plane
     }
@@ -2266,6 +2507,7 @@ int tc_build(TcPlan &t, const TcPlanInput &in, std::string *err)
         TcBatch &T = t.batches[b];
         T.img_phi = (long long)off;
         T.img_aux = (long long)(off + 3 * (size_t)T.plane_phi);
+        if (in.for_h) T.hblock = (long long)(off + 6 * (size_t)T.plane_phi);
         if (in.with_e) T.img_e = (long long)(off + 3 * (size_t)T.plane_phi + 3 * (size_t)std::max(T.plane_phi, T.plane_d));
         T.part0 = part;
         part += part_rows(b);
@@ -2337,7 +2579,8 @@ int tc_build(TcPlan &t, const TcPlanInput &in, std::string *err)
     t.n_fn = in.n_fn;
     t.bound_off = ((size_t)in.nnz * 8 + 255) / 256 * 256;
     t.sign_off = (t.bound_off + 8 * (size_t)in.n_fn + 255) / 256 * 256;
-    t.img_base = (t.sign_off + 4 * (size_t)n_sb + 1023) / 1024 * 1024;
+    t.counter_off = (t.sign_off + 4 * (size_t)n_sb + 255) / 256 * 256;
+    t.img_base = (t.counter_off + 256 + 1023) / 1024 * 1024;
     t.ws_bytes = t.img_base + max_ws + 1024;
     // items must not be empty for the device copy
     if (!in.host_only) {
@@ -2399,7 +2642,8 @@ cudaError_t tc_launch_phi(const TcPlan &t, const DevPlan &P, const TcWave &w, co
     k_tc_phi<<<(unsigned)w.nphi, kPhiThreads, dyn, s>>>(P, t.d_batches, t.d_items + w.phi0,
                                                        (uint8_t *)ws + t.img_base, v, n_split, fixed,
                                                        reinterpret_cast<int *>((uint8_t *)ws + t.sign_off),
-                                                       t.bound_grids >= 2 ? 1 : 0);
+                                                       t.bound_grids >= 2 ? 1 : 0,
+                                                       reinterpret_cast<unsigned int *>((uint8_t *)ws + t.counter_off));
     return cudaGetLastError();
 }
 
@@ -2409,7 +2653,8 @@ cudaError_t tc_launch_phi_cols(const TcPlan &t, const DevPlan &P, const TcWave &
     if (w.npc <= 0) return cudaSuccess;
     k_tc_phi_cols<<<(unsigned)w.npc, kPhiThreads, 0, s>>>(P, t.d_batches, t.d_items + w.pc0,
                                                            (uint8_t *)ws + t.img_base, n_split,
-                                                           t.bound_grids >= 1 ? 1 : 0);
+                                                           t.bound_grids >= 1 ? 1 : 0,
+                                                           reinterpret_cast<unsigned int *>((uint8_t *)ws + t.counter_off));
     return cudaGetLastError();
 }
 
@@ -2420,7 +2665,8 @@ cudaError_t tc_launch_h(const TcPlan &t, const DevPlan &P, const TcWave &w, cons
     const int grid = (int)std::min<long long>(w.nh, t.num_sms);
     k_tc_h<<<grid, kThreadsTc, smem_tc_h(), s>>>(P, t.d_batches, t.d_items + w.h0, (int)w.nh,
                                                 (const uint8_t *)ws + t.img_base, (unsigned long long *)ws, n_split,
-                                                reinterpret_cast<const int *>((const uint8_t *)ws + t.sign_off));
+                                                reinterpret_cast<const int *>((const uint8_t *)ws + t.sign_off),
+                                                (unsigned int *)((const uint8_t *)ws + t.counter_off));
     return cudaGetLastError();
 }
 
@@ -2470,7 +2716,8 @@ cudaError_t tc_launch_density(const TcPlan &t, const DevPlan &P, const TcWave &w
     const int grid = (int)std::min<long long>(w.ne, t.num_sms);
     k_tc_density<false><<<grid, kThreadsTc, smem_tc(3), s>>>(P, t.d_batches, t.d_items + w.e0, (int)w.ne,
                                                              (const uint8_t *)ws + t.img_base, part, n_split,
-                                                             nullptr);
+                                                             nullptr,
+                                                             (unsigned int *)((const uint8_t *)ws + t.counter_off));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_density_sum<<<(unsigned)w.nd, 128, 0, s>>>(P, t.d_batches, t.d_items + w.d0, part, n, 2.0);
@@ -2486,7 +2733,8 @@ cudaError_t tc_launch_adjoint(const TcPlan &t, const DevPlan &P, const TcWave &w
     double *part = reinterpret_cast<double *>(img + w.part_off);
     const int grid = (int)std::min<long long>(w.ne, t.num_sms);
     k_tc_density<true><<<grid, kThreadsTc, smem_tc(3), s>>>(P, t.d_batches, t.d_items + w.e0, (int)w.ne, img, part,
-                                                            n_split, img);
+                                                            n_split, img,
+                                                            (unsigned int *)((const uint8_t *)ws + t.counter_off));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_density_sum<<<(unsigned)w.nd, 128, 0, s>>>(P, t.d_batches, t.d_items + w.d0, part, dv, 1.0);

@@ -20,6 +20,21 @@ constexpr int kChunkBytes = 16384;       // 128 rows x 64 columns x 2 bytes
 constexpr int kChunkStride = 3 * kChunkBytes;   // the three planes of a chunk are adjacent: one bulk copy
                                                 // moves them, and a value's planes are one address apart
 
+// One 128-row block of a super-batch as the H scatter needs it, written with
+// the operand images: per row the first stored value of its function's row of
+// H less the function's index in its atom, that index, and the place of its
+// atom among the block's; the atoms' indices in their system.
+struct HBlock {
+    long long base[128];
+    long long pair_off;    // the system's pair positions in DevPlan::pairpos
+    int loc[128];
+    unsigned short li[128];
+    unsigned char slot[128];
+    int nat, nslot;        // atoms of the system, of the block
+    int n, pad[3];         // rows that are functions
+};
+static_assert(sizeof(HBlock) % 16 == 0, "HBlock is moved by bulk copies");
+
 struct TcBatch {
     long long img_phi;     // byte offset (in the wave's workspace) of the phi image
     long long img_aux;     // byte offset of the w v phi image (H) or the D image (density)
@@ -32,6 +47,7 @@ struct TcBatch {
     long long part0;       // first partial-density row of the batch in its wave (128 doubles each)
     long long img_e;       // byte offset of E = G Phi (FP32 [row][point], rows of 64 nc_alloc points)
                            // for the adjoint, -1 when the plan keeps no room for it
+    long long hblock;      // byte offset of the row blocks' descriptors (H plans), else -1
 };
 
 struct TcWave {
@@ -60,6 +76,7 @@ struct TcPlanInput {
     bool host_only = false;              // build host tables only (no device copies)
     long long wave_mb = 0;               // operand images per wave, MiB (0: default)
     int bound_grids = 0;                 // leading-digit grids from table bounds: 1 density, 2 also H
+    bool for_h = false;                  // the H integration's plan (descriptors of the row blocks)
     bool with_e = false;                 // room for E = G Phi per batch (the adjoint's tiles)
 };
 
@@ -70,6 +87,7 @@ struct TcPlan {
     size_t img_base = 0;                 // workspace offset of the wave images (scratch below)
     size_t bound_off = 0;                // workspace offset of the per-function bounds of D
     size_t sign_off = 0;                 // workspace offset of the per-batch sign of w v (H images)
+    size_t counter_off = 0;              // workspace offset of the contractions' tile counter
     long long nnz = 0, n_fn = 0;
     int num_sms = 1;                     // persistent grids: one CTA per SM
     int bound_grids = 0;                 // see TcPlanInput
