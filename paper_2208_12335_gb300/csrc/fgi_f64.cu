@@ -13,7 +13,38 @@ namespace fgi {
 namespace {
 
 // ---------------------------------------------------------------- basis (FP64)
-// ws block of batch b: Phi[nfn][kpad], zero for padded points.
+// ws block of batch b: Phi[nfn][kpad], zero for padded points and beyond the
+// cutoff.  Bound by the FP64 pipe (1/64 of the FP32 rate): the shells are
+// walked grouped by l, so the harmonics of an l are formed once an atom and
+// point, and 1/d is a multiplication a shell.  (A division and harmonics a
+// shell: 20-atom molecule, two calls on 101 k points, 1.49 ms.)
+template <int L>
+__device__ __forceinline__ void phi_shells_f64(const DevPlan &P, const DevSpecies &S, int &sh, double d, double inv,
+                                               double nx, double ny, double nz, double *col, int kpad)
+{
+    if (S.nl[L] == 0) return;
+    double Y[2 * L + 1];
+    ylm_unit<double>(L, nx, ny, nz, Y);
+    for (const int end = sh + S.nl[L]; sh < end; sh++) {
+        const int f0 = P.shells[S.shell0 + sh].fn0;
+        double ud = 0.0;
+        const DevRadial &R = P.radials[P.shell_rad_l[S.shell0 + sh]];
+        const double *c0 = P.coef + 4 * R.coef_off;
+        if (d < 1e-12) {
+            ud = L == 0 ? c0[1] * R.inv_h : 0.0;          // the limit u'(0)
+        } else if (d < R.rcut) {
+            const double s = d * R.inv_h;
+            const int k = min((int)s, R.nk - 2);
+            const double t = s - (double)k;
+            const double2 *c = reinterpret_cast<const double2 *>(c0 + 4 * (long long)k);
+            const double2 a = __ldg(c), b = __ldg(c + 1);
+            ud = (a.x + t * (a.y + t * (b.x + t * b.y))) * inv;
+        }
+#pragma unroll
+        for (int m = 0; m < 2 * L + 1; m++) col[(long long)(f0 + m) * kpad] = ud * Y[m];
+    }
+}
+
 __global__ void k_phi_f64(DevPlan P, int b0, double *ws)
 {
     const DevBatch B = P.batches[b0 + blockIdx.x];
@@ -25,31 +56,36 @@ __global__ void k_phi_f64(DevPlan P, int b0, double *ws)
         const DevAct A = P.act[B.act0 + e];
         const DevSpecies S = P.species[P.atom_species[A.atom]];
         double *col = out + (long long)A.fn_loc * B.kpad + p;
-        if (p >= B.np) {
+        double x = 0.0, y = 0.0, z = 0.0, d2 = 1e300;
+        if (p < B.np) {
+            const long long g = B.pt0 + p;
+            x = P.px[g] - P.atom_xyz[3 * A.atom + 0];
+            y = P.py[g] - P.atom_xyz[3 * A.atom + 1];
+            z = P.pz[g] - P.atom_xyz[3 * A.atom + 2];
+            d2 = x * x + y * y + z * z;
+        }
+        // beyond the largest cutoff (with a margin for the rounding of the squares)
+        if (d2 > S.rcut * S.rcut * (1.0 + 1e-12)) {
             for (int f = 0; f < S.n_fn; f++) col[(long long)f * B.kpad] = 0.0;
             continue;
         }
-        const long long g = B.pt0 + p;
-        const double x = P.px[g] - P.atom_xyz[3 * A.atom + 0];
-        const double y = P.py[g] - P.atom_xyz[3 * A.atom + 1];
-        const double z = P.pz[g] - P.atom_xyz[3 * A.atom + 2];
-        const double d = sqrt(x * x + y * y + z * z);
+        const double d = sqrt(d2);
         const double inv = d > 1e-12 ? 1.0 / d : 0.0;
         const double nx = x * inv, ny = y * inv, nz = z * inv;
-        int f = 0;
-        for (int sh = 0; sh < S.n_shell; sh++) {
-            const DevRadial R = P.radials[P.shell_rad[S.shell0 + sh]];
-            const double ud = radial_over_d_f64(R, P.coef, d);
-            double Y[7];
-            ylm_unit<double>(R.l, nx, ny, nz, Y);
-            for (int m = 0; m < 2 * R.l + 1; m++, f++) col[(long long)f * B.kpad] = ud * Y[m];
-        }
+        int sh = 0;
+        phi_shells_f64<0>(P, S, sh, d, inv, nx, ny, nz, col, B.kpad);
+        phi_shells_f64<1>(P, S, sh, d, inv, nx, ny, nz, col, B.kpad);
+        phi_shells_f64<2>(P, S, sh, d, inv, nx, ny, nz, col, B.kpad);
+        phi_shells_f64<3>(P, S, sh, d, inv, nx, ny, nz, col, B.kpad);
     }
 }
 
 // ------------------------------------------------------- H contraction (FP64)
 // One 64x64 tile (ti <= tj) of h_b = Phi_b diag(w v) Phi_b^T, then FP64
-// atomic scatter of the upper triangle into the stored values.
+// atomic scatter of the upper triangle into the stored values.  Bound by the
+// FP64 pipe, a warp's instruction at a time: on a diagonal tile the 136 4x4
+// blocks that meet the upper triangle are dealt to consecutive threads, five
+// warps instead of eight, and warps whose rows lie past n_b do nothing.
 constexpr int TF = 64;     // tile edge
 constexpr int TK = 16;     // points per step
 
@@ -59,8 +95,18 @@ __global__ void __launch_bounds__(256) k_h_f64(DevPlan P, const WorkItem *items,
     const WorkItem it = items[blockIdx.x];
     const DevBatch B = P.batches[it.batch];
     const double *phi = ws + B.ws_off;
-    const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+    const int t = threadIdx.x;
     const int i0 = it.ti * TF, j0 = it.tj * TF;
+    int tx = t & 15, ty = t >> 4;
+    bool mine = i0 + ty * 4 < B.nfn;
+    if (it.ti == it.tj) {
+        // block number t of the triangle tx >= ty, row by row
+        mine = t < 136;
+        int rest = min(t, 135);
+        for (ty = 0; rest >= 16 - ty; ty++) rest -= 16 - ty;
+        tx = ty + rest;
+        mine = mine && i0 + ty * 4 < B.nfn;
+    }
     __shared__ double As[TK][TF + 1];
     __shared__ double Bs[TK][TF + 1];
     __shared__ double wv[TK];
@@ -93,18 +139,21 @@ __global__ void __launch_bounds__(256) k_h_f64(DevPlan P, const WorkItem *items,
             Bs[kk][r] = (j0 + r < B.nfn && kin) ? phi[(long long)(j0 + r) * B.kpad + k] : 0.0;
         }
         __syncthreads();
+        if (mine) {
 #pragma unroll
-        for (int kk = 0; kk < TK; kk++) {
-            double a[4], b[4];
+            for (int kk = 0; kk < TK; kk++) {
+                double a[4], b[4];
 #pragma unroll
-            for (int q = 0; q < 4; q++) { a[q] = As[kk][ty * 4 + q]; b[q] = Bs[kk][tx * 4 + q]; }
+                for (int q = 0; q < 4; q++) { a[q] = As[kk][ty * 4 + q]; b[q] = Bs[kk][tx * 4 + q]; }
 #pragma unroll
-            for (int r = 0; r < 4; r++)
+                for (int r = 0; r < 4; r++)
 #pragma unroll
-                for (int c = 0; c < 4; c++) acc[r][c] = fma(a[r], b[c], acc[r][c]);
+                    for (int c = 0; c < 4; c++) acc[r][c] = fma(a[r], b[c], acc[r][c]);
+            }
         }
         __syncthreads();
     }
+    if (!mine) return;
 #pragma unroll
     for (int r = 0; r < 4; r++) {
         const int il = ty * 4 + r;
@@ -123,7 +172,12 @@ __global__ void __launch_bounds__(256) k_h_f64(DevPlan P, const WorkItem *items,
 // One 64-point tile of batch b: n_p = sum_j (sum_i phi_i(p) D_ij) phi_j(p),
 // D gathered from the stored upper triangle (off-diagonal values scaled by
 // offdiag_scale: 1 for a matrix, 1/2 for a gradient with respect to stored
-// values).  Optionally writes E[j][p] = sum_i phi_i(p) D_ij (adjoint).
+// values).  FULL (the adjoint) writes E[j][p] = sum_i phi_i(p) D_ij;
+// otherwise the symmetry of D halves the FP64 work that bounds the kernel:
+// n = 2 sum_J phi_J . (sum_{K >= J} D'_JK phi_K) over 64-function blocks, D' = D
+// with its diagonal blocks halved (exact).  Warps past the batch's points skip
+// the products.
+template <bool FULL>
 __global__ void __launch_bounds__(256) k_density_f64(DevPlan P, const WorkItem *items,
                                                      const double *ws, const double *dval,
                                                      double offdiag_scale, double *n_out,
@@ -144,7 +198,8 @@ __global__ void __launch_bounds__(256) k_density_f64(DevPlan P, const WorkItem *
     double part[4] = {0, 0, 0, 0};
     for (int j0 = 0; j0 < B.nfn; j0 += TF) {
         double acc[4][4] = {};
-        for (int k0 = 0; k0 < B.nfn; k0 += TK) {
+        for (int k0 = FULL ? 0 : j0; k0 < B.nfn; k0 += TK) {
+            const double half = !FULL && k0 < j0 + TF ? 0.5 : 1.0;
 #pragma unroll
             for (int e = 0; e < 4; e++) {
                 const int idx = t + 256 * e;
@@ -158,20 +213,22 @@ __global__ void __launch_bounds__(256) k_density_f64(DevPlan P, const WorkItem *
                     const FnRef a = fn_ref(P, act, fnact[lo], lo);
                     const FnRef b = fn_ref(P, act, fnact[hi], hi);
                     const long long k = value_index(P, B.sys, a, b);
-                    if (k >= 0) dv = dval[k] * (lo == hi ? 1.0 : offdiag_scale);
+                    if (k >= 0) dv = dval[k] * (lo == hi ? half : offdiag_scale * half);
                 }
                 Bs[kk][c] = dv;
             }
             __syncthreads();
+            if (p0 + ty * 4 < B.np) {
 #pragma unroll
-            for (int kk = 0; kk < TK; kk++) {
-                double a[4], b[4];
+                for (int kk = 0; kk < TK; kk++) {
+                    double a[4], b[4];
 #pragma unroll
-                for (int q = 0; q < 4; q++) { a[q] = As[kk][ty * 4 + q]; b[q] = Bs[kk][tx * 4 + q]; }
+                    for (int q = 0; q < 4; q++) { a[q] = As[kk][ty * 4 + q]; b[q] = Bs[kk][tx * 4 + q]; }
 #pragma unroll
-                for (int r = 0; r < 4; r++)
+                    for (int r = 0; r < 4; r++)
 #pragma unroll
-                    for (int c = 0; c < 4; c++) acc[r][c] = fma(a[r], b[c], acc[r][c]);
+                        for (int c = 0; c < 4; c++) acc[r][c] = fma(a[r], b[c], acc[r][c]);
+                }
             }
             __syncthreads();
         }
@@ -184,7 +241,7 @@ __global__ void __launch_bounds__(256) k_density_f64(DevPlan P, const WorkItem *
                 const int j = j0 + tx * 4 + c;
                 if (j >= B.nfn) continue;
                 part[r] = fma(acc[r][c], phi[(long long)j * B.kpad + p], part[r]);
-                if (e_out) e_out[B.ws_off + (long long)j * B.kpad + p] = acc[r][c];
+                if (FULL) e_out[B.ws_off + (long long)j * B.kpad + p] = acc[r][c];
             }
         }
     }
@@ -198,7 +255,7 @@ __global__ void __launch_bounds__(256) k_density_f64(DevPlan P, const WorkItem *
 #pragma unroll
         for (int r = 0; r < 4; r++) {
             const int p = p0 + ty * 4 + r;
-            if (p < B.np) n_out[B.pt0 + p] = part[r];
+            if (p < B.np) n_out[B.pt0 + p] = FULL ? part[r] : 2.0 * part[r];
         }
     }
 }
@@ -361,8 +418,8 @@ cudaError_t launch_density_f64(const DevPlan &P, const WorkItem *items, int n_it
                                double *n_out, double *e_out, cudaStream_t s)
 {
     if (n_items <= 0) return cudaSuccess;
-    k_density_f64<<<n_items, 256, kMaxBatchFns * sizeof(unsigned short), s>>>(
-        P, items, ws, d, offdiag_scale, n_out, e_out);
+    auto kernel = e_out ? k_density_f64<true> : k_density_f64<false>;
+    kernel<<<n_items, 256, kMaxBatchFns * sizeof(unsigned short), s>>>(P, items, ws, d, offdiag_scale, n_out, e_out);
     return cudaGetLastError();
 }
 

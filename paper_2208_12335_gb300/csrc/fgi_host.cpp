@@ -760,6 +760,7 @@ int build_plan(fgi_ctx *c, const char *tune_path)
            i_sp = add(dsp.data(), dsp.size() * sizeof(DevSpecies)),
            i_shr = add(shell_rad.data(), shell_rad.size() * 4),
            i_dsh = add(dshell.data(), dshell.size() * sizeof(DevShell)),
+           i_srl = add(shell_by_l.data(), shell_by_l.size() * 4),
            i_rad = add(drad.data(), drad.size() * sizeof(DevRadial)),
            i_coef = add(coef.data(), coef.size() * 8), i_coefdd = add(coef_dd.data(), coef_dd.size() * 4),
            i_scoef = add(scoef.data(), scoef.size() * 4),
@@ -799,6 +800,7 @@ int build_plan(fgi_ctx *c, const char *tune_path)
     P.species = (const DevSpecies *)at(i_sp);
     P.shell_rad = (const int *)at(i_shr);
     P.shells = (const DevShell *)at(i_dsh);
+    P.shell_rad_l = (const int *)at(i_srl);
     P.n_shells = (int)shell_rad.size();
     P.radials = (const DevRadial *)at(i_rad);
     P.coef = (const double *)at(i_coef);

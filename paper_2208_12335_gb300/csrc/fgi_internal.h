@@ -89,6 +89,7 @@ struct DevPlan {
     const DevSpecies *species;
     const int *shell_rad;         // radial id per species shell
     const DevShell *shells;       // the same shells, packed for the tensor-core basis kernels
+    const int *shell_rad_l;       // their radial ids, in the order of shells
     int n_shells;                 // entries of shell_rad / shells
     const DevRadial *radials;
     const double *coef;           // [sum intervals][4] FP64

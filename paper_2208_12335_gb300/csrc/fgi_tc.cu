@@ -111,12 +111,6 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
         : "memory");
 }
 
-// start moving [src, src + bytes) into L2 (both multiples of 16)
-__device__ __forceinline__ void bulk_prefetch(const void *src, uint32_t bytes)
-{
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
-}
-
 // add to a global 64-bit word where pred holds, without a branch
 __device__ __forceinline__ void red_add_if(bool pred, unsigned long long addr, long long x)
 {
@@ -1350,7 +1344,8 @@ __global__ void k_fix_to_h(const long long *acc, double *h, long long n, int acc
 // The counter keeps the tiles in flight next to each other in the list: with a
 // fixed stride the CTAs drift apart over ~90 super-batches, whose operands
 // outgrow L2 (17 GB read from DRAM for 4.7 GB of images in the 64-atom Si
-// cluster's density).
+// cluster's density).  Prefetching the next tile's operands into L2 was
+// measured 1-3 % slower and is not done.
 // Two groups of eight epilogue warps, one for each accumulator set: a group's
 // table look-ups and drain of one tile overlap the other group's and the MMAs.
 constexpr int kGroupWarps = 8, kGroupThreads = 32 * kGroupWarps;
@@ -1638,15 +1633,6 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_h(DevPlan P, const TcBatch
                 const uint8_t *b_img = ws + (F.sign != 0 ? T.img_phi : T.img_aux) + (long long)it.ti * T.nc_alloc * kChunkStride;
                 fetch_next(F);
                 for (int c = 0; c < T.nc; c++) {
-                    // the next tile's operands, if it is the first to read them (the
-                    // list goes through J at I = 0 first): their trip from DRAM to L2
-                    // passes behind this tile
-                    if (c == min(1, T.nc - 1) && F.have && F.it.ti == 0) {
-                        const uint32_t bytes = (uint32_t)(F.T.nc * kChunkStride);
-                        const long long blk = (long long)F.it.tj * F.T.nc_alloc * kChunkStride;
-                        bulk_prefetch(ws + F.T.img_phi + blk, bytes);
-                        if (F.sign == 0) bulk_prefetch(ws + F.T.img_aux + blk, bytes);
-                    }
                     if (!(ok = stage_wait_empty(S, n, P.status))) break;
                     const uint32_t q = n++ % kStages;
                     uint8_t *dst = sm + q * kStageBytes;
@@ -2067,22 +2053,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_density(DevPlan P, const T
                 const uint8_t *d_img = ws + T.img_aux + (long long)J * T.nkc * kChunkStride, *phi_img = ws + T.img_phi;
                 // a last tile of at most 64 points has one column chunk
                 const int halves = 2 * m + 1 < T.nc ? 2 : 1;
-                const int kc0 = ADJ ? 0 : 2 * J;
-                for (int kc = kc0; kc < T.nkc; kc++) {
-                    // the next tile's operands, if it is the first to read them (its
-                    // point tile at J = 0, its block of D at m = 0): their trip from
-                    // DRAM to L2 passes behind this tile
-                    if (kc == min(kc0 + 1, T.nkc - 1) && F.have) {
-                        if (F.it.tj == 0)
-                            for (int I = 0; I < F.T.nrb; I++)
-                                bulk_prefetch(ws + F.T.img_phi + (long long)(I * F.T.nc_alloc + 2 * F.it.ti) * kChunkStride,
-                                              2 * kChunkStride);
-                        if (F.it.ti == 0) {
-                            const int k0 = ADJ ? 0 : 2 * F.it.tj;
-                            bulk_prefetch(ws + F.T.img_aux + ((long long)F.it.tj * F.T.nkc + k0) * kChunkStride,
-                                          (uint32_t)(F.T.nkc - k0) * kChunkStride);
-                        }
-                    }
+                for (int kc = ADJ ? 0 : 2 * J; kc < T.nkc; kc++) {
                     if (!(ok = stage_wait_empty(S, n, P.status))) break;
                     const uint32_t q = n++ % kStages;
                     uint8_t *dst = sm + q * kStageBytes;
