@@ -4,11 +4,15 @@
 // uses for the electrostatic potential (the paper's Fig. 4 caption notes that
 // this potential was not yet accelerated on GPUs).
 //
-//  1. k_hartree_moments (FP64): per point p on atom a's radial shell k,
-//       rho~_a,lm(r_k) += (w_p / (r_k^3 ln q)) n_p A_lm(rhat_p)
+//  1. k_hartree_moments: a warp per (atom a, radial shell k), over its points p
+//     (listed once at set-up),
+//       rho~_a,lm(r_k) = sum_p (w_p / (r_k^3 ln q)) n_p A_lm(rhat_p)
 //     (w_p / (r_k^3 ln q) is the partitioned angular weight; A_lm = Y_lm / K_lm
-//     the unnormalised harmonics), FP64 atomics.
-//  2. k_hartree_radial (FP64): per (atom, l, m) the radial Poisson equation
+//     the unnormalised harmonics).  Harmonics and sums are double-float (about
+//     2^-45 relative), w_p n_p and the final scale FP64: GB300's FP64 pipe has
+//     1/64 of the FP32 rate.
+//  2. k_hartree_radial (FP64): a warp per (atom, l), lanes along the shells, the
+//     radial Poisson equation
 //       V(r) = 4 pi/(2l+1) [r^-(l+1) int_0^r rho r'^(l+2) dr' + r^l int_r^inf rho r'^(1-l) dr']
 //     with the partial integrals in x = ln r interval by interval, each by the
 //     integral of the cubic through its four nearest shells, plus
@@ -29,6 +33,8 @@
 //     carries a relative error of a few FP32 roundings of the l >= 1 part,
 //     against the FP64 pipe's 1/64 rate on GB300.  The sum over atoms is a
 //     double-float.
+#include <vector>
+
 #include "fgi_dd.cuh"
 #include "fgi_hartree.h"
 #include "fgi_ylm.cuh"
@@ -110,32 +116,6 @@ __device__ __forceinline__ df df_rsqrt(df a, float y)
     return df_fast_two_sum(y, y * (0.5f * e));
 }
 
-template <int LMAX>
-__global__ void __launch_bounds__(256) k_hartree_moments(DevPlan P, HartreeDev H, long long n_pts, const double *n,
-                                                         double *rho)
-{
-    constexpr int L = (LMAX + 1) * (LMAX + 1);
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n_pts;
-         p += (long long)gridDim.x * blockDim.x) {
-        const int a = H.owner[p];
-        if (a < 0) continue;
-        const int k = H.shell[p];
-        const HartreeRad g = H.rad[a];
-        const double dx = P.px[p] - P.atom_xyz[3 * a], dy = P.py[p] - P.atom_xyz[3 * a + 1],
-                     dz = P.pz[p] - P.atom_xyz[3 * a + 2];
-        const double r = sqrt(dx * dx + dy * dy + dz * dz);
-        if (!(r > 0.0)) continue;
-        const double rk = g.r0 * exp(g.lnq * (double)k);
-        const double val = P.pw[p] / (rk * rk * rk * g.lnq) * n[p];
-        const double ir = 1.0 / r;
-        double A[L];
-        ylm_unnormalised<LMAX, double>(dx * ir, dy * ir, dz * ir, A);
-        double *dst = rho + (H.rad_off[a] + k) * kL;
-#pragma unroll
-        for (int q = 0; q < L; q++) atomicAdd(dst + q, val * A[q]);
-    }
-}
-
 __device__ __forceinline__ double ipow(double r, int n)      // r^n, 0 <= n <= 9
 {
     double p = 1.0;
@@ -143,71 +123,244 @@ __device__ __forceinline__ double ipow(double r, int n)      // r^n, 0 <= n <= 9
     return p;
 }
 
-// one thread per (atom, lm); the thread with lm = 0 also packs the atom's
-// record for the evaluation
-__global__ void __launch_bounds__(32) k_hartree_radial(DevPlan P, HartreeDev H, int l_max, HartreeTabs T)
+// acc += a b (double-floats; acc's low part a plain FP32 sum)
+__device__ __forceinline__ void df_fma_acc(df &acc, df a, df b)
 {
-    const int L = (l_max + 1) * (l_max + 1);
-    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (t >= (long long)H.n_atoms * L) return;
-    const int a = (int)(t / L), lm = (int)(t % L);
-    int l = 0;
-    while ((l + 1) * (l + 1) <= lm) l++;
+    df p = df_two_prod(a.hi, b.hi);
+    p.lo = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, p.lo));
+    const df t = df_two_sum(acc.hi, p.hi);
+    acc.hi = t.hi;
+    acc.lo += t.lo + p.lo;
+}
+
+// Sum of v[0 .. n) over the 32 lanes: each step halves the values a lane
+// holds; lane's values end up as v[0 .. ceil(n/32)) = sums off .. of the n,
+// those below lim.
+template <int N, int MASK>
+__device__ __forceinline__ void warp_sum_split(df *v, int &off, int &lim)
+{
+    if constexpr (MASK > 0) {
+        constexpr int H = (N + 1) / 2;
+        const bool upper = (threadIdx.x & MASK) != 0;
+#pragma unroll
+        for (int q = 0; q < H; q++) {
+            const df b = q + H < N ? v[q + H < N ? q + H : 0] : df{0.f, 0.f};
+            const float sh = upper ? v[q].hi : b.hi, sl = upper ? v[q].lo : b.lo;
+            const float kh = upper ? b.hi : v[q].hi, kl = upper ? b.lo : v[q].lo;
+            const df t = df_two_sum(kh, __shfl_xor_sync(0xffffffffu, sh, MASK));
+            v[q].hi = t.hi;
+            v[q].lo = t.lo + (kl + __shfl_xor_sync(0xffffffffu, sl, MASK));
+        }
+        if (upper) off += H;
+        else lim = min(lim, off + H);
+        warp_sum_split<H, MASK / 2>(v, off, lim);
+    }
+}
+
+// One warp per (atom, shell).  (A thread per point with FP64 harmonics and
+// (l_max + 1)^2 FP64 atomics was bound by the FP64 pipe: 250-atom cluster, 7.3 M
+// points, l_max 6, 3.30 ms; now 0.51 ms.)
+template <int LMAX>
+__global__ void __launch_bounds__(128) k_hartree_moments(DevPlan P, HartreeDev H, const double *n, double *rho)
+{
+    constexpr int L = (LMAX + 1) * (LMAX + 1);
+    const long long bin = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (bin >= H.n_shells) return;
+    const long long i0 = H.bin_off[bin], i1 = H.bin_off[bin + 1];
+    df acc[L];
+#pragma unroll
+    for (int q = 0; q < L; q++) acc[q] = df{0.f, 0.f};
+    int a = 0;
+    if (i0 < i1) a = H.owner[H.order[i0]];
+    const float *aa = P.atom_dd + 6 * a;
+    for (long long i = i0 + lane; i < i1; i += 32) {
+        const long long p = H.order[i];
+        const float2 *pp = reinterpret_cast<const float2 *>(P.pts_dd + 6 * p);
+        const float2 px = pp[0], py = pp[1], pz = pp[2];
+        df x = dfa(df{px.x, px.y}, df{-aa[0], -aa[1]}), y = dfa(df{py.x, py.y}, df{-aa[2], -aa[3]}),
+           z = dfa(df{pz.x, pz.y}, df{-aa[4], -aa[5]});
+        const df d2 = dfa(dfa(df_sqr(x), df_sqr(y)), df_sqr(z));
+        if (!(d2.hi > 0.f)) continue;
+        const df ir = df_rsqrt(d2, rsqrtf(d2.hi));
+        x = df_mul(x, ir);
+        y = df_mul(y, ir);
+        z = df_mul(z, ir);
+        df cm = df_from_double(P.pw[p] * n[p]), sm{0.f, 0.f};      // w n Re, Im (x + i y)^m
+        float pmm = 1.f;
+#pragma unroll
+        for (int m = 0; m <= LMAX; m++) {
+            if (m > 0) {
+                const df c = dfa(df_mul(cm, x), df_mul(df{-sm.hi, -sm.lo}, y));
+                sm = dfa(df_mul(cm, y), df_mul(sm, x));
+                cm = c;
+                pmm *= (float)(2 * m - 1);                          // Pbar_m^m, exact
+            }
+            df p2{0.f, 0.f}, p1{pmm, 0.f};
+#pragma unroll
+            for (int l = m; l <= LMAX; l++) {
+                df pl = p1;
+                if (l == m + 1) {
+                    pl = df_mul_f(z, (float)(2 * m + 1) * pmm);
+                } else if (l > m + 1) {
+                    // 1/(l-m) as a double-float
+                    constexpr double one = 1.0;
+                    const double iv = one / (double)(l - m);
+                    const df inv{(float)iv, (float)(iv - (double)(float)iv)};
+                    const df u = df_mul(df_mul_f(z, (float)(2 * l - 1)), p1);
+                    pl = df_mul(dfa(u, df_mul_f(p2, -(float)(l + m - 1))), inv);
+                }
+                if (l > m) {
+                    p2 = p1;
+                    p1 = pl;
+                }
+                df_fma_acc(acc[l * l + l + m], pl, cm);
+                if (m > 0) df_fma_acc(acc[l * l + l - m], pl, sm);
+            }
+        }
+    }
+    int off = 0, lim = L;
+    warp_sum_split<L, 16>(acc, off, lim);
+    double scale = 0.0;
+    if (i0 < i1) {
+        const HartreeRad g = H.rad[a];
+        const double rk = g.r0 * exp(g.lnq * (double)(bin - H.rad_off[a]));
+        scale = 1.0 / (rk * rk * rk * g.lnq);
+    }
+#pragma unroll
+    for (int q = 0; q < (L + 31) / 32; q++)
+        if (off + q < lim) rho[bin * kL + off + q] = ((double)acc[q].hi + (double)acc[q].lo) * scale;
+}
+
+__device__ __forceinline__ double warp_scan_up(double v, int lane)       // inclusive, towards higher lanes
+{
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+    }
+    return v;
+}
+
+__device__ __forceinline__ double warp_scan_down(double v, int lane)     // inclusive, towards lower lanes
+{
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double u = __shfl_down_sync(0xffffffffu, v, o);
+        if (lane + o < 32) v += u;
+    }
+    return v;
+}
+
+// The radial equation of atom a for one l by one warp, lanes along the shells:
+// the partial integrals as warp scans, the 2l+1 functions side by side.
+template <int l>
+__device__ void radial_l(const DevPlan &P, const HartreeRad &g, int a, long long o, const HartreeTabs &T)
+{
+    constexpr int NM = 2 * l + 1;
+    const int lane = threadIdx.x & 31, n = g.nrad;
+    const double h = g.lnq, h24 = h / 24.0;
+    auto rk = [&](int k) { return g.r0 * exp(h * (double)k); };
+    // the integrands per dx = dr / r: f = rho r^(l+3) (inner), g = rho r^(2-l) (outer, over rho)
+    double *rho = T.rho + o * kL + l * l, *F = T.F + o * kL + l * l, *Vd = T.Vd + o * kL + l * l;
+    for (int k = lane; k < n; k += 32) {
+        const double r = rk(k), rf = ipow(r, l + 3), rg = l <= 2 ? ipow(r, 2 - l) : 1.0 / ipow(r, l - 2);
+#pragma unroll
+        for (int m = 0; m < NM; m++) {
+            const double rr = rho[k * kL + m];
+            F[k * kL + m] = rr * rf;
+            rho[k * kL + m] = rr * rg;
+        }
+    }
+    __syncwarp();
+    // integral over interval [k, k+1] of the cubic through the nearest four samples (n >= 4)
+    auto seg = [&](const double *fn, int k) {
+        auto v = [&](int j) { return fn[j * kL]; };
+        if (k == 0) return h24 * (9.0 * v(0) + 19.0 * v(1) - 5.0 * v(2) + v(3));
+        if (k == n - 2) return h24 * (v(n - 4) - 5.0 * v(n - 3) + 19.0 * v(n - 2) + 9.0 * v(n - 1));
+        return h24 * (13.0 * (v(k) + v(k + 1)) - (v(k - 1) + v(k + 2)));
+    };
+    // 4 pi/(2l+1), times K_lm^2 for the two unnormalised harmonics (moment, evaluation)
+    double pref[NM], carry[NM];
+#pragma unroll
+    for (int m = 0; m < NM; m++) {
+        pref[m] = 4.0 * 3.14159265358979323846 / (2.0 * l + 1.0) * ylm_norm2(l, m - l);
+        carry[m] = F[m] / (double)(l + 3);
+    }
+    // inner integrals, forward: the inner part of V in FP64 scratch
+    for (int k0 = 0; k0 < n; k0 += 32) {
+        const int k = k0 + lane;
+        const double ir = 1.0 / ipow(rk(min(k, n - 1)), l + 1);
+#pragma unroll
+        for (int m = 0; m < NM; m++) {
+            const double iin = carry[m] + warp_scan_up(k > 0 && k < n ? seg(F + m, k - 1) : 0.0, lane);
+            if (k < n) Vd[k * kL + m] = pref[m] * iin * ir;
+            carry[m] = __shfl_sync(0xffffffffu, iin, 31);
+        }
+    }
+    if (lane == 0) {
+        if (l == 0) {
+            const float *aa = P.atom_dd + 6 * a;
+            const df q = df_from_double(pref[0] * carry[0]);
+            T.rec[3 * a] = make_float4(aa[0], aa[1], aa[2], aa[3]);
+            T.rec[3 * a + 1] = make_float4(aa[4], aa[5], g.rmax2_hi, g.rmax2_lo);
+            T.rec[3 * a + 2] = make_float4(q.hi, q.lo, 0.f, 0.f);
+        } else {
+#pragma unroll
+            for (int m = 0; m < NM; m++) T.Qf[(long long)a * kLf + l * l + m - 1] = (float)(pref[m] * carry[m]);
+        }
+    }
+    // outer integrals, backward; V = inner + outer part, stored once
+#pragma unroll
+    for (int m = 0; m < NM; m++) carry[m] = 0.0;
+    for (int k0 = (n - 1) / 32 * 32; k0 >= 0; k0 -= 32) {
+        const int k = k0 + lane;
+        const double rl = ipow(rk(min(k, n - 1)), l);
+#pragma unroll
+        for (int m = 0; m < NM; m++) {
+            const double iout = carry[m] + warp_scan_down(k < n - 1 ? seg(rho + m, k) : 0.0, lane);
+            if (k < n) {
+                const double v = Vd[k * kL + m] + pref[m] * iout * rl;
+                if (l == 0) T.V0[o + k] = v;
+                else T.Vf[(o + k) * kLf + l * l + m - 1] = (float)v;
+            }
+            carry[m] = __shfl_sync(0xffffffffu, iout, 0);
+        }
+    }
+}
+
+// One warp per (atom, l); the warp with l = 0 also packs the atom's records for
+// the evaluation.  (One thread per (atom, l, m) along the shells was a serial
+// chain: 0.44 ms on 64 atoms of 60 shells; now 0.08 ms.)
+__global__ void __launch_bounds__(128) k_hartree_radial(DevPlan P, HartreeDev H, int l_max, HartreeTabs T)
+{
+    const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (w >= (long long)H.n_atoms * (l_max + 1)) return;
+    const int a = (int)(w / (l_max + 1)), l = (int)(w % (l_max + 1));
     const HartreeRad g = H.rad[a];
     const int n = g.nrad;
     const long long o = H.rad_off[a];
-    const double h = g.lnq;
-    double *rho = T.rho + o * kL + lm, *F = T.F + o * kL + lm, *Vin = T.Vd + o * kL + lm;
-    auto rk = [&](int k) { return g.r0 * exp(h * (double)k); };
-    // the integrands per dx = dr / r: f = rho r^(l+3) (inner), g = rho r^(2-l) (outer, over rho)
-    for (int k = 0; k < n; k++) {
-        const double r = rk(k), rr = rho[(long long)k * kL];
-        F[(long long)k * kL] = rr * ipow(r, l + 3);
-        rho[(long long)k * kL] = l <= 2 ? rr * ipow(r, 2 - l) : rr / ipow(r, l - 2);
+    switch (l) {
+    case 0: radial_l<0>(P, g, a, o, T); break;
+    case 1: radial_l<1>(P, g, a, o, T); return;
+    case 2: radial_l<2>(P, g, a, o, T); return;
+    case 3: radial_l<3>(P, g, a, o, T); return;
+    case 4: radial_l<4>(P, g, a, o, T); return;
+    case 5: radial_l<5>(P, g, a, o, T); return;
+    default: radial_l<6>(P, g, a, o, T); return;
     }
-    // integral over interval [k, k+1] of the cubic through the nearest four samples (n >= 4)
-    auto seg = [&](const double *fn, int k) {
-        auto v = [&](int j) { return fn[(long long)j * kL]; };
-        if (k == 0) return h * (9.0 * v(0) + 19.0 * v(1) - 5.0 * v(2) + v(3)) / 24.0;
-        if (k == n - 2) return h * (v(n - 4) - 5.0 * v(n - 3) + 19.0 * v(n - 2) + 9.0 * v(n - 1)) / 24.0;
-        return h * (-v(k - 1) + 13.0 * v(k) + 13.0 * v(k + 1) - v(k + 2)) / 24.0;
-    };
-    // 4 pi/(2l+1), times K_lm^2 for the two unnormalised harmonics (moment, evaluation)
-    const double pref = 4.0 * 3.14159265358979323846 / (2.0 * l + 1.0) * ylm_norm2(l, lm - l * l - l);
-    // inner integrals, forward: the inner part of V in FP64 scratch
-    double iin = F[0] / (double)(l + 3);
-    for (int k = 0; k < n; k++) {
-        if (k > 0) iin += seg(F, k - 1);
-        Vin[(long long)k * kL] = pref * iin / ipow(rk(k), l + 1);
-    }
-    if (lm == 0) {
-        const float *aa = P.atom_dd + 6 * a;
-        const df q = df_from_double(pref * iin);
-        T.rec[3 * a] = make_float4(aa[0], aa[1], aa[2], aa[3]);
-        T.rec[3 * a + 1] = make_float4(aa[4], aa[5], g.rmax2_hi, g.rmax2_lo);
-        T.rec[3 * a + 2] = make_float4(q.hi, q.lo, 0.f, 0.f);
-    } else {
-        T.Qf[(long long)a * kLf + lm - 1] = (float)(pref * iin);
-    }
-    // outer integrals, backward; V = inner + outer part, stored once
-    double iout = 0.0;
-    for (int k = n - 1; k >= 0; k--) {
-        if (k < n - 1) iout += seg(rho, k);
-        const double v = Vin[(long long)k * kL] + pref * iout * ipow(rk(k), l);
-        if (lm == 0) T.V0[o + k] = v;
-        else T.Vf[(o + k) * kLf + lm - 1] = (float)v;
-    }
-    if (lm != 0) return;
+    __syncwarp();
     // the shells' radii, and V_00 on each interval k as the cubic through
     // shells i0 .. i0+3 (i0 = k - 1 clamped to [0, n-4]) in f = x - k,
     // x = ln(r / r_0) / ln q: a_m = p^(m)(o) / m! with o = k - i0 and
     // p(t) = V_i0 + t D1 + t(t-1)/2 D2 + t(t-1)(t-2)/6 D3 (forward differences)
-    for (int k = 0; k < n; k++) {
-        const double r = rk(k);
+    for (int k = lane; k < n; k += 32) {
+        const double r = g.r0 * exp(g.lnq * (double)k);
         const df rh = df_from_double(r), ri = df_from_double(1.0 / r);
         T.rk[o + k] = make_float4(rh.hi, rh.lo, ri.hi, ri.lo);
     }
-    for (int k = 0; k + 1 < n; k++) {
+    for (int k = lane; k + 1 < n; k += 32) {
         const int i0 = k - 1 < 0 ? 0 : (k - 1 > n - 4 ? n - 4 : k - 1);
         const double t = (double)(k - i0);
         const double *v = T.V0 + o + i0;
@@ -221,9 +374,56 @@ __global__ void __launch_bounds__(32) k_hartree_radial(DevPlan P, HartreeDev H, 
     }
 }
 
-// CTA per batch, thread per point; the atoms of the batch's system
+// ---- pairs of FP32 numbers, one instruction for both (the FMA pipe takes two
+// cycles for it, the issue slots are halved); each half is rounded as the
+// scalar operation would be
+struct pk {
+    unsigned long long v;
+};
+__device__ __forceinline__ pk pk_make(float a, float b)
+{
+    pk r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 pk_get(pk a)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+    return r;
+}
+__device__ __forceinline__ pk operator*(pk a, pk b)
+{
+    pk r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ pk fma2(pk a, pk b, pk c)
+{
+    pk r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+// A row of 48 FP32 coefficients, or the first of it, in 32-byte loads: a load
+// costs the L1 a look-up for each lane whose row differs, whatever its width.
+template <int N>
+__device__ __forceinline__ void load_row(const float *p, float *v)
+{
+#pragma unroll
+    for (int j = 0; j < (N + 7) / 8; j++)
+        asm("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+            : "=f"(v[8 * j]), "=f"(v[8 * j + 1]), "=f"(v[8 * j + 2]), "=f"(v[8 * j + 3]), "=f"(v[8 * j + 4]),
+              "=f"(v[8 * j + 5]), "=f"(v[8 * j + 6]), "=f"(v[8 * j + 7])
+            : "l"(p + 8 * j));
+}
+
+// CTA per batch, thread per point; the atoms of the batch's system.  Bound by
+// the FP32 pipe (about 330 operations a pair of a point and a far atom at l_max
+// 6).  Two far atoms at a time in packed FP32 pairs issued a fifth fewer
+// instructions and took as long; six CTAs an SM instead of four: 250-atom
+// cluster, l_max 6, 28.9 -> 27.2 ms.
 template <int LMAX>
-__global__ void __launch_bounds__(128) k_hartree_eval(DevPlan P, HartreeDev H, HartreeTabs T, double *vh)
+__global__ void __launch_bounds__(128, 6) k_hartree_eval(DevPlan P, HartreeDev H, HartreeTabs T, double *vh)
 {
     constexpr int L = (LMAX + 1) * (LMAX + 1);
     const DevBatch B = P.batches[blockIdx.x];
@@ -361,11 +561,27 @@ __global__ void __launch_bounds__(128) k_hartree_eval(DevPlan P, HartreeDev H, H
                         const float f2 = -t * (t - 1.f) * (t - 3.f) * 0.5f;
                         const float f3 = t * (t - 1.f) * (t - 2.f) * (1.f / 6.f);
                         const float *vf = T.Vf + (o + i0) * kLf;
+                        // eight coefficients of the four rows at a time, in pairs
+                        const pk w0 = pk_make(f0, f0), w1 = pk_make(f1, f1), w2 = pk_make(f2, f2), w3 = pk_make(f3, f3);
 #pragma unroll
-                        for (int q = 1; q < L; q++)
-                            part = fmaf(f0 * vf[q - 1] + f1 * vf[kLf + q - 1] + f2 * vf[2 * kLf + q - 1] +
-                                            f3 * vf[3 * kLf + q - 1],
-                                        A[q], part);
+                        for (int q8 = 0; q8 < L - 1; q8 += 8) {
+                            float v0[8], v1[8], v2[8], v3[8];
+                            load_row<8>(vf + q8, v0);
+                            load_row<8>(vf + kLf + q8, v1);
+                            load_row<8>(vf + 2 * kLf + q8, v2);
+                            load_row<8>(vf + 3 * kLf + q8, v3);
+#pragma unroll
+                            for (int q = 0; q < 8; q += 2) {
+                                if (q8 + q >= L - 1) break;
+                                const pk v = fma2(w3, pk_make(v3[q], v3[q + 1]),
+                                                  fma2(w2, pk_make(v2[q], v2[q + 1]),
+                                                       fma2(w0, pk_make(v0[q], v0[q + 1]),
+                                                            w1 * pk_make(v1[q], v1[q + 1]))));
+                                const float2 u = pk_get(v);
+                                part = fmaf(u.x, A[q8 + q + 1], part);
+                                if (q8 + q + 1 < L - 1) part = fmaf(u.y, A[q8 + q + 2 < L ? q8 + q + 2 : 0], part);
+                            }
+                        }
                     }
                 }
             }
@@ -376,6 +592,41 @@ __global__ void __launch_bounds__(128) k_hartree_eval(DevPlan P, HartreeDev H, H
 }
 
 }  // namespace
+
+// points per (owner, shell), then their places
+__global__ void k_bin_count(HartreeDev H, long long n_pts, unsigned int *count)
+{
+    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n_pts; p += (long long)gridDim.x * blockDim.x)
+        if (H.owner[p] >= 0) atomicAdd(count + H.rad_off[H.owner[p]] + H.shell[p], 1u);
+}
+
+__global__ void k_bin_fill(HartreeDev H, long long n_pts, unsigned int *count, unsigned int *order)
+{
+    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n_pts; p += (long long)gridDim.x * blockDim.x)
+        if (H.owner[p] >= 0) {
+            const long long bin = H.rad_off[H.owner[p]] + H.shell[p];
+            order[H.bin_off[bin] + atomicSub(count + bin, 1u) - 1] = (unsigned int)p;
+        }
+}
+
+cudaError_t hartree_bin_points(const HartreeDev &H, long long n_pts, unsigned int *count, unsigned int *order,
+                               long long *bin_off)
+{
+    cudaError_t e = cudaMemset(count, 0, sizeof(unsigned int) * (size_t)H.n_shells);
+    if (e != cudaSuccess) return e;
+    if (n_pts > 0) k_bin_count<<<1216, 256>>>(H, n_pts, count);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    std::vector<unsigned int> host((size_t)H.n_shells);
+    e = cudaMemcpy(host.data(), count, sizeof(unsigned int) * host.size(), cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return e;
+    std::vector<long long> off(host.size() + 1, 0);
+    for (size_t k = 0; k < host.size(); k++) off[k + 1] = off[k] + host[k];
+    e = cudaMemcpy(bin_off, off.data(), sizeof(long long) * off.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return e;
+    if (n_pts > 0) k_bin_fill<<<1216, 256>>>(H, n_pts, count, order);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return cudaStreamSynchronize(0);
+}
 
 HartreeRad hartree_rad(double r_min, double ln_q, int n_rad)
 {
@@ -414,24 +665,23 @@ cudaError_t launch_hartree(const DevPlan &P, const HartreeDev &H, int n_batch, l
                            const double *n, double *vh, double *ws, cudaStream_t s)
 {
     const HartreeTabs T = carve(H, ws);
-    cudaError_t e = cudaMemsetAsync(T.rho, 0, sizeof(double) * kL * (size_t)H.n_shells, s);
-    if (e != cudaSuccess) return e;
-    if (n_pts > 0) {
-        const unsigned grid = (unsigned)std::min<long long>((n_pts + 255) / 256, 4864);
+    cudaError_t e = cudaSuccess;
+    if (H.n_shells > 0) {
+        const unsigned grid = (unsigned)((H.n_shells + 3) / 4);
         switch (l_max) {
-        case 0: k_hartree_moments<0><<<grid, 256, 0, s>>>(P, H, n_pts, n, T.rho); break;
-        case 1: k_hartree_moments<1><<<grid, 256, 0, s>>>(P, H, n_pts, n, T.rho); break;
-        case 2: k_hartree_moments<2><<<grid, 256, 0, s>>>(P, H, n_pts, n, T.rho); break;
-        case 3: k_hartree_moments<3><<<grid, 256, 0, s>>>(P, H, n_pts, n, T.rho); break;
-        case 4: k_hartree_moments<4><<<grid, 256, 0, s>>>(P, H, n_pts, n, T.rho); break;
-        case 5: k_hartree_moments<5><<<grid, 256, 0, s>>>(P, H, n_pts, n, T.rho); break;
-        default: k_hartree_moments<6><<<grid, 256, 0, s>>>(P, H, n_pts, n, T.rho); break;
+        case 0: k_hartree_moments<0><<<grid, 128, 0, s>>>(P, H, n, T.rho); break;
+        case 1: k_hartree_moments<1><<<grid, 128, 0, s>>>(P, H, n, T.rho); break;
+        case 2: k_hartree_moments<2><<<grid, 128, 0, s>>>(P, H, n, T.rho); break;
+        case 3: k_hartree_moments<3><<<grid, 128, 0, s>>>(P, H, n, T.rho); break;
+        case 4: k_hartree_moments<4><<<grid, 128, 0, s>>>(P, H, n, T.rho); break;
+        case 5: k_hartree_moments<5><<<grid, 128, 0, s>>>(P, H, n, T.rho); break;
+        default: k_hartree_moments<6><<<grid, 128, 0, s>>>(P, H, n, T.rho); break;
         }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    const long long nt = (long long)H.n_atoms * (l_max + 1) * (l_max + 1);
-    if (nt > 0) {
-        k_hartree_radial<<<(unsigned)((nt + 31) / 32), 32, 0, s>>>(P, H, l_max, T);
+    const long long nw = (long long)H.n_atoms * (l_max + 1);
+    if (nw > 0) {
+        k_hartree_radial<<<(unsigned)((nw + 3) / 4), 128, 0, s>>>(P, H, l_max, T);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (n_batch > 0) {

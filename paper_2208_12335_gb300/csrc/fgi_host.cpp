@@ -1456,7 +1456,10 @@ int fgi_set_atom_grids(fgi_ctx *c, const int32_t *owner, const int32_t *shell, c
         const size_t s_own = align_up(4 * (size_t)c->n_pts + 4, 256), s_off = align_up(8 * (size_t)(n_at + 1), 256),
                      s_rg = align_up(sizeof(HartreeRad) * (size_t)(n_at + 1), 256),
                      s_sys = align_up(8 * sys_atom0.size(), 256);
-        const size_t tot = 2 * s_own + s_off + s_rg + s_sys;
+        const size_t n_sh = (size_t)c->hd.n_shells;
+        const size_t s_bin = align_up(8 * (n_sh + 1), 256), s_cnt = align_up(4 * n_sh + 4, 256);
+        const size_t at_ord = 2 * s_own + s_off + s_rg + s_sys, at_bin = at_ord + s_own, at_cnt = at_bin + s_bin;
+        const size_t tot = at_cnt + s_cnt;
         CUDA_TRY(c, cudaMalloc((void **)&c->d_hartree, tot));
         char *b = c->d_hartree;
         CUDA_TRY(c, cudaMemcpy(b, owner, 4 * (size_t)c->n_pts, cudaMemcpyHostToDevice));
@@ -1471,6 +1474,10 @@ int fgi_set_atom_grids(fgi_ctx *c, const int32_t *owner, const int32_t *shell, c
         c->hd.rad_off = (const long long *)(b + 2 * s_own);
         c->hd.rad = (const HartreeRad *)(b + 2 * s_own + s_off);
         c->hd.sys_atom0 = (const long long *)(b + 2 * s_own + s_off + s_rg);
+        c->hd.order = (const unsigned int *)(b + at_ord);
+        c->hd.bin_off = (const long long *)(b + at_bin);
+        CUDA_TRY(c, hartree_bin_points(c->hd, c->n_pts, (unsigned int *)(b + at_cnt), (unsigned int *)(b + at_ord),
+                                       (long long *)(b + at_bin)));
     }
     c->have_atom_grids = true;
     return FGI_OK;
