@@ -129,4 +129,81 @@ __host__ __device__ __forceinline__ df df_from_double(double x)
     return {hi, (float)(x - (double)hi)};
 }
 
+#if defined(__CUDACC__)
+// ---- pairs of FP32 numbers, one instruction for both: the FMA pipe takes two
+// cycles for it, the issue slots are halved.  Each half is rounded as the
+// scalar operation would be.
+struct pk {
+    unsigned long long v;
+};
+__device__ __forceinline__ pk pk_make(float a, float b)
+{
+    pk r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ pk pk_dup(float a) { return pk_make(a, a); }
+__device__ __forceinline__ float2 pk_get(pk a)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+    return r;
+}
+__device__ __forceinline__ pk operator+(pk a, pk b)
+{
+    pk r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ pk operator*(pk a, pk b)
+{
+    pk r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ pk fma2(pk a, pk b, pk c)
+{
+    pk r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ pk operator-(pk a) { return pk{a.v ^ 0x8000000080000000ull}; }
+__device__ __forceinline__ pk operator-(pk a, pk b) { return fma2(b, pk_dup(-1.f), a); }   // one rounding, as a - b
+
+// two double-floats, and the operations above on them, step by step
+struct df2 {
+    pk hi, lo;
+};
+__device__ __forceinline__ df2 df2_two_sum(pk a, pk b)
+{
+    const pk s = a + b, bb = s - a;
+    return {s, (a - (s - bb)) + (b - bb)};
+}
+__device__ __forceinline__ df2 df2_fast_two_sum(pk a, pk b)
+{
+    const pk s = a + b;
+    return {s, b - (s - a)};
+}
+__device__ __forceinline__ df2 df2_add_sloppy(df2 a, df2 b)
+{
+    const df2 s = df2_two_sum(a.hi, b.hi);
+    return df2_fast_two_sum(s.hi, s.lo + (a.lo + b.lo));
+}
+__device__ __forceinline__ df2 df2_mul(df2 a, df2 b)
+{
+    const pk p = a.hi * b.hi;
+    return df2_fast_two_sum(p, fma2(a.hi, b.lo, fma2(a.lo, b.hi, fma2(a.hi, b.hi, -p))));
+}
+__device__ __forceinline__ df2 df2_rsqrt(df2 a)                   // df_rsqrt_refine
+{
+    const float2 ah = pk_get(a.hi);
+    const pk y = pk_make(rsqrtf(ah.x), rsqrtf(ah.y)), y2h = y * y, y2l = fma2(y, y, -y2h);
+    const pk ph = a.hi * y2h, pl = fma2(a.hi, y2h, -ph);
+    const pk rho = ((pk_dup(1.f) - ph) - pl) - fma2(a.hi, y2l, a.lo * y2h);
+    const pk c = y * (rho * fma2(pk_dup(0.375f), rho, pk_dup(0.5f)));
+    const pk s = y + c;
+    return {s, c - (s - y)};
+}
+#endif
+
 }  // namespace fgi

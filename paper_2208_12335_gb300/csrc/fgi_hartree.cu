@@ -374,36 +374,6 @@ __global__ void __launch_bounds__(128) k_hartree_radial(DevPlan P, HartreeDev H,
     }
 }
 
-// ---- pairs of FP32 numbers, one instruction for both (the FMA pipe takes two
-// cycles for it, the issue slots are halved); each half is rounded as the
-// scalar operation would be
-struct pk {
-    unsigned long long v;
-};
-__device__ __forceinline__ pk pk_make(float a, float b)
-{
-    pk r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 pk_get(pk a)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
-    return r;
-}
-__device__ __forceinline__ pk operator*(pk a, pk b)
-{
-    pk r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ pk fma2(pk a, pk b, pk c)
-{
-    pk r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-    return r;
-}
 // A row of 48 FP32 coefficients, or the first of it, in 32-byte loads: a load
 // costs the L1 a look-up for each lane whose row differs, whatever its width.
 template <int N>
@@ -562,7 +532,7 @@ __global__ void __launch_bounds__(128, 6) k_hartree_eval(DevPlan P, HartreeDev H
                         const float f3 = t * (t - 1.f) * (t - 2.f) * (1.f / 6.f);
                         const float *vf = T.Vf + (o + i0) * kLf;
                         // eight coefficients of the four rows at a time, in pairs
-                        const pk w0 = pk_make(f0, f0), w1 = pk_make(f1, f1), w2 = pk_make(f2, f2), w3 = pk_make(f3, f3);
+                        const pk w0 = pk_dup(f0), w1 = pk_dup(f1), w2 = pk_dup(f2), w3 = pk_dup(f3);
 #pragma unroll
                         for (int q8 = 0; q8 < L - 1; q8 += 8) {
                             float v0[8], v1[8], v2[8], v3[8];

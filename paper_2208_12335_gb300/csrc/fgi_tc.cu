@@ -191,17 +191,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v)
     for (int i = 0; i < 32; i++) v[i] = __uint_as_float(r[i]);
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v)
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float *v)
 {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
 #pragma unroll
-    for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 8; i++) v[i] = __uint_as_float(r[i]);
 }
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
@@ -1549,29 +1546,33 @@ __device__ __forceinline__ bool group_next_tile(TcRing *S, uint32_t lt, int grou
 // 2880 with one lane in divergent code and a barrier an operand.
 // first: the chunk opens the item (the first product into each accumulator
 // overwrites it).
-template <int NSPLIT, int ORDER, bool B_MN>
-__device__ __forceinline__ void mma_chunk(uint32_t acc_base, const uint8_t *a_sm, const uint8_t *b_sm, uint32_t idesc,
+// The planes of the first operand go slowest.  It is A (K-major) for H; for the
+// density (PHI_A) it is B and the second operand, read as MN-major, is A, so
+// that the points lie along the lanes of the accumulators.
+template <int NSPLIT, int ORDER, bool PHI_A>
+__device__ __forceinline__ void mma_chunk(uint32_t acc_base, const uint8_t *sm1, const uint8_t *sm2, uint32_t idesc,
                                           bool first, int nks)
 {
-    uint64_t ad0 = desc_sw128(smem_u32(a_sm), 16, 1024);
-    uint64_t bd0 = B_MN ? desc_sw128(smem_u32(b_sm), 8192, 1024) : desc_sw128(smem_u32(b_sm), 16, 1024);
+    uint64_t d1 = desc_sw128(smem_u32(sm1), 16, 1024);
+    uint64_t d2 = PHI_A ? desc_sw128(smem_u32(sm2), 8192, 1024) : desc_sw128(smem_u32(sm2), 16, 1024);
 #pragma unroll 1
     for (int ks = 0; ks < nks; ks++) {
         if (elect_one()) {
 #pragma unroll
-            for (int pa = 0; pa < NSPLIT; pa++) {
+            for (int p1 = 0; p1 < NSPLIT; p1++) {
 #pragma unroll
-                for (int pb = 0; pb < NSPLIT; pb++) {
-                    if (pa + pb > ORDER || (pa == 2 && pb == 2)) continue;
-                    const int acc = (pa + pb == 0) ? 0 : 1;
-                    const bool opens = acc == 0 || (pa == 0 && pb == 1);
-                    tc_mma(acc_base + acc * 128, ad0 + (uint64_t)((pa * kChunkBytes) >> 4),
-                           bd0 + (uint64_t)((pb * kChunkBytes) >> 4), idesc, (opens && first && ks == 0) ? 0u : 1u);
+                for (int p2 = 0; p2 < NSPLIT; p2++) {
+                    if (p1 + p2 > ORDER || (p1 == 2 && p2 == 2)) continue;
+                    const int acc = (p1 + p2 == 0) ? 0 : 1;
+                    const bool opens = acc == 0 || (p1 == 0 && p2 == 1);
+                    const uint64_t e1 = d1 + (uint64_t)((p1 * kChunkBytes) >> 4), e2 = d2 + (uint64_t)((p2 * kChunkBytes) >> 4);
+                    tc_mma(acc_base + acc * 128, PHI_A ? e2 : e1, PHI_A ? e1 : e2, idesc,
+                           (opens && first && ks == 0) ? 0u : 1u);
                 }
             }
         }
-        ad0 += 32 >> 4;
-        bd0 += (B_MN ? 2048 : 32) >> 4;
+        d1 += 32 >> 4;
+        d2 += (PHI_A ? 2048 : 32) >> 4;
     }
 }
 
@@ -1990,19 +1991,19 @@ __global__ void __launch_bounds__(256) k_tc_gather_d(DevPlan P, const TcBatch *t
 // Persistent, with the roles, the rings and the tile counter of the H
 // contraction, over the items (batch, 128-point tile m, 128-function block J),
 // J ascending so the longest contractions come first:
-// E^T[j][p] = sum_{i >= 128 J} D'[j][i] phi_i(p) over the upper block
+// E[p][j] = sum_{i >= 128 J} phi_i(p) D'[j][i] over the upper block
 // triangle of the symmetric D (D' = D with its diagonal block halved;
-// A = D image, K-major; B = phi image read as MN-major) accumulates in one of
+// A = phi image read as MN-major, B = D image, K-major) accumulates in one of
 // two tensor-memory sets while a group of warps finishes an earlier item: the
-// partial density sum_{j in J} E^T[j][p] phi_j(p) in double-float (lane j
-// multiplies by its own phi row, the warp reduces over j), one row of 128
-// doubles per item.  Many items per batch keep the CTAs on few batches at a
+// partial density sum_{j in J} E[p][j] phi_j(p) in double-float, a thread its
+// own point p (tensor-memory lane) and half of the j, one row of 128 doubles
+// per item.  Many items per batch keep the CTAs on few batches at a
 // time, so the D and phi images are read from L2.  k_density_sum then forms
 // n_p = 2 sum_J partial_J(p).
 //
 // ADJ (the adjoint's E = G Phi): every function chunk of the full G image,
-// and each lane also stores its row of E (acc0 + acc1 in FP32) for the
-// position gradient.
+// and each thread also stores its point's E (acc0 + acc1 in FP32; rows of
+// points) for the position gradient.
 template <bool ADJ>
 __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_density(DevPlan P, const TcBatch *tb, const WorkItem *items,
                                                               int n_items, const uint8_t *ws, double *part,
@@ -2011,7 +2012,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_density(DevPlan P, const T
     extern __shared__ uint8_t smem_raw[];
     uint8_t *sm = align1024(smem_raw);
     TcRing *S = reinterpret_cast<TcRing *>(sm + kStages * kStageBytes);
-    __shared__ double red[2][4][128];
+    __shared__ double red[2][2][128];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) ring_init(S);
     if (warp == kWarpMma) {
@@ -2076,12 +2077,12 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_density(DevPlan P, const T
         bool ok = true;
         for (uint32_t lt = 0; ok && __all_sync(0xffffffffu, tile_wait_full(S, lt, P.status)); lt++) {
             const int e = (int)(lt % kTiles);
-            const int m = S->tile[e].ti, J = S->tile[e].tj, np = S->tile[e].np, nfn = S->tile[e].nfn, nkc = S->tile[e].nkc;
+            const int m = S->tile[e].ti, J = S->tile[e].tj, nfn = S->tile[e].nfn, nkc = S->tile[e].nkc;
             if (m < 0) break;
             __syncwarp();
             if (elect_one()) mbar_arrive(&S->nempty[e]);
-            // the last tile's columns end at the batch's points
-            const uint32_t idesc = idesc_bf16(128, min(128, (np - m * 128 + 15) & ~15), false, true);
+            // the columns of the last block end at n_b
+            const uint32_t idesc = idesc_bf16(128, min(128, (nfn - J * 128 + 15) & ~15), true, false);
             const uint32_t buf = lt & 1, use = lt >> 1;
             ok = use == 0 || mbar_wait_a(&S->tempty[buf], (use - 1) & 1, P.status, &S->abort);
             tc_fence_after();
@@ -2102,102 +2103,88 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_density(DevPlan P, const T
         }
         __syncwarp();
     } else {
-        // Warp w of a group: TMEM lanes 32 (w % 4) .. + 31 (functions j of the
-        // block), point columns 64 (w / 4) .. + 63, sixteen at a time.  Bound by
-        // its FP32 instructions (about 30 a value of E).
+        // Warp w of a group: TMEM lanes 32 (w % 4) .. + 31 (points of the tile),
+        // columns 64 (w / 4) .. + 63 (functions j of the block), eight at a time.
+        // Bound by its instructions, about 17 a value of E in packed pairs of j.
+        // (With the functions along the lanes, the sum over them took a butterfly
+        // of selects and shuffles and 37 instructions a value: the epilogue alone
+        // needed 6.4 of the 7.4 ms of 64 molecules' density.)
         const int group = warp >> 3, quad = warp & 3, half = (warp >> 2) & 1;
-        const int tid = threadIdx.x & (kGroupThreads - 1), r = quad * 32 + lane;
-        const uint32_t acc_base = tmem + group * 256 + ((uint32_t)(quad * 32) << 16);
+        const int tid = threadIdx.x & (kGroupThreads - 1), pl = quad * 32 + lane;
+        const uint32_t acc_base = tmem + group * 256 + ((uint32_t)(quad * 32) << 16) + 64 * half;
+        const uint32_t g16 = (uint32_t)((pl >> 3) & 7) << 4, pb = (uint32_t)(pl & 7) * 2u;
         for (uint32_t lt = group; group_next_tile(S, lt, group, tid, P.status); lt += 2) {
             const TileInfo T = S->tile[lt % kTiles];
             const int m = T.ti, J = T.tj;
-            const int j = J * 128 + r;
-            const bool live = j < T.nfn;
-            // this lane's phi row at the warp's 64 points (one chunk): two 16-byte
-            // units a plane for 16 points, loaded ahead of their use
-            const uint8_t *row = ws + T.img_phi + (long long)(J * T.nc_alloc + 2 * m + half) * kChunkStride;
-            uint4 w[2][3];
-            auto load_units = [&](int piece) {
+            const int nj = min(64, T.nfn - J * 128 - 64 * half);     // this warp's functions
+            // phi of rows 64 half + .. at this thread's point, in row order: row r at
+            // r 128 + its swizzled unit, the planes a chunk's bytes apart
+            const uint8_t *row = ws + T.img_phi + (long long)(J * T.nc_alloc + 2 * m + (pl >> 6)) * kChunkStride +
+                                 64 * half * 128 + pb;
+            unsigned short w[2][8][3];
+            auto load_phi = [&](int piece, unsigned short (*v)[3]) {
 #pragma unroll
-                for (int g = 0; g < 2; g++)
+                for (int q = 0; q < 8; q++) {
+                    const uint8_t *src = row + piece * 1024 + row_offset(q, g16);
 #pragma unroll
-                    for (int sp = 0; sp < 3; sp++) {
-                        w[g][sp] = make_uint4(0u, 0u, 0u, 0u);
-                        if (live && sp < n_split)
-                            w[g][sp] = *reinterpret_cast<const uint4 *>(
-                                row + row_offset((uint32_t)r, (uint32_t)(2 * piece + g) << 4) + sp * kChunkBytes);
-                    }
+                    for (int sp = 0; sp < 3; sp++)
+                        v[q][sp] = sp < n_split ? *reinterpret_cast<const unsigned short *>(src + sp * kChunkBytes) : 0;
+                }
             };
-            load_units(0);
+            if (nj > 0) load_phi(0, w[0]);
+            if (nj > 8) load_phi(1, w[1]);
             const bool ok = mbar_wait_a(&S->tfull[group], (lt >> 1) & 1, P.status, &S->abort);
             tc_fence_after();
-#pragma unroll 1
-            for (int piece = 0; piece < 4; piece++) {
-                const int c0 = 64 * half + 16 * piece;
-                float hi[16], lo[16];
-                tmem_ld16(acc_base + c0, hi);
-                if (n_split > 1) tmem_ld16(acc_base + 128 + c0, lo);
+            pk s2 = pk_dup(0.f), c2 = pk_dup(0.f);       // sums over even and odd j
+            auto piece_sum = [&](int piece, unsigned short (*v)[3]) {
+                float hi[8], lo[8];
+                tmem_ld8(acc_base + 8 * piece, hi);
+                if (n_split > 1) tmem_ld8(acc_base + 128 + 8 * piece, lo);
                 else
 #pragma unroll
-                    for (int q = 0; q < 16; q++) lo[q] = 0.f;
+                    for (int q = 0; q < 8; q++) lo[q] = 0.f;
                 tmem_wait_ld();
-                if (piece == 3) {
-                    tc_fence_before();
-                    mbar_arrive(&S->tempty[group]);   // accumulator set may be reused
+                if (ADJ && ok) {
+                    float *dst = reinterpret_cast<float *>(ws_e + T.img_e) +
+                                 (long long)(J * 128 + 64 * half + 8 * piece) * T.nc_alloc * 64 + m * 128 + pl;
+#pragma unroll
+                    for (int q = 0; q < 8; q++)
+                        if (8 * piece + q < nj) dst[(long long)q * T.nc_alloc * 64] = hi[q] + lo[q];
                 }
-                if (ADJ && live && ok) {
-                    // this lane's row of E at the 16 points, for the gradient
-                    float4 *dst = reinterpret_cast<float4 *>(ws_e + T.img_e) +
-                                  ((long long)j * T.nc_alloc * 64 + m * 128 + c0) / 4;
+                // E phi in double-float: e = acc0 + acc1, phi = f0 + (f1 + f2), whose
+                // inner sum is exact and never larger than a non-zero f0.  Rows past
+                // n_b up to the next 16 are zero in both images.
 #pragma unroll
-                    for (int q = 0; q < 4; q++)
-                        dst[q] = make_float4(hi[4 * q] + lo[4 * q], hi[4 * q + 1] + lo[4 * q + 1],
-                                             hi[4 * q + 2] + lo[4 * q + 2], hi[4 * q + 3] + lo[4 * q + 3]);
+                for (int q = 0; q < 8; q += 2) {
+                    auto term = [&](int sp) {
+                        return pk_make(__uint_as_float((uint32_t)v[q][sp] << 16), __uint_as_float((uint32_t)v[q + 1][sp] << 16));
+                    };
+                    const df2 ph = df2_fast_two_sum(term(0), term(1) + term(2));
+                    const df2 e = df2_two_sum(pk_make(hi[q], hi[q + 1]), pk_make(lo[q], lo[q + 1]));
+                    const pk pr = e.hi * ph.hi;
+                    const pk pl2 = fma2(e.lo, ph.hi, fma2(e.hi, ph.lo, fma2(e.hi, ph.hi, -pr)));
+                    const df2 t = df2_two_sum(s2, pr);
+                    s2 = t.hi;
+                    c2 = c2 + (t.lo + pl2);
                 }
-                // E^T[j][p] phi_j(p) in double-float: e = acc0 + acc1, phi = f0 + (f1 +
-                // f2), whose inner sum is exact and never larger than a non-zero f0
-#pragma unroll
-                for (int g = 0; g < 2; g++)
-#pragma unroll
-                    for (int q = 0; q < 8; q++) {
-                        const int k = 8 * g + q;
-                        auto term = [&](const uint4 &u) {
-                            const uint32_t x = (q >> 1) == 0 ? u.x : (q >> 1) == 1 ? u.y : (q >> 1) == 2 ? u.z : u.w;
-                            return __uint_as_float((q & 1) ? (x & 0xFFFF0000u) : (x << 16));
-                        };
-                        const df ph = df_fast_two_sum(term(w[g][0]), term(w[g][1]) + term(w[g][2]));
-                        const df e = df_two_sum(hi[k], lo[k]);
-                        const float p = e.hi * ph.hi;
-                        lo[k] = fmaf(e.lo, ph.hi, fmaf(e.hi, ph.lo, fmaf(e.hi, ph.hi, -p)));
-                        hi[k] = p;
-                    }
-                if (piece < 3) load_units(piece + 1);
-                // sum over the 32 lanes (rows j), halving the columns a lane holds: the
-                // high parts with their rounding errors, the low parts plainly
-#pragma unroll
-                for (int wd = 8; wd >= 1; wd >>= 1) {
-                    const bool upper = (lane & (2 * wd)) != 0;
-#pragma unroll
-                    for (int q = 0; q < wd; q++) {
-                        const float sh = upper ? hi[q] : hi[q + wd], sl = upper ? lo[q] : lo[q + wd];
-                        const float kh = upper ? hi[q + wd] : hi[q], kl = upper ? lo[q + wd] : lo[q];
-                        const df t2 = df_two_sum(kh, __shfl_xor_sync(0xffffffffu, sh, 2 * wd));
-                        hi[q] = t2.hi;
-                        lo[q] = t2.lo + (kl + __shfl_xor_sync(0xffffffffu, sl, 2 * wd));
-                    }
+            };
+#pragma unroll 1
+            for (int piece = 0; 8 * piece < nj; piece += 2) {
+                piece_sum(piece, w[0]);
+                if (8 * (piece + 2) < nj) load_phi(piece + 2, w[0]);
+                if (8 * (piece + 1) < nj) {
+                    piece_sum(piece + 1, w[1]);
+                    if (8 * (piece + 3) < nj) load_phi(piece + 3, w[1]);
                 }
-                const df t2 = df_two_sum(hi[0], __shfl_xor_sync(0xffffffffu, hi[0], 1));
-                const float tl = t2.lo + (lo[0] + __shfl_xor_sync(0xffffffffu, lo[0], 1));
-                if ((lane & 1) == 0) red[group][quad][c0 + (lane >> 1)] = (double)t2.hi + (double)tl;
             }
+            tc_fence_before();
+            mbar_arrive(&S->tempty[group]);              // accumulator set may be reused
+            const float2 sf = pk_get(s2), cf = pk_get(c2);
+            red[group][half][pl] = ((double)sf.x + (double)sf.y) + ((double)cf.x + (double)cf.y);
             // item complete: this block's partial density at the tile's 128 points
             group_sync(group);
             if (tid == 0) mbar_arrive(&S->nempty[lt % kTiles]);
-            if (tid < 128) {
-                part[T.part_row * 128 + tid] = ok ? (red[group][0][tid] + red[group][1][tid]) +
-                                                  (red[group][2][tid] + red[group][3][tid])
-                                            : 0.0;
-            }
+            if (tid < 128) part[T.part_row * 128 + tid] = ok ? red[group][0][tid] + red[group][1][tid] : 0.0;
             group_sync(group);
         }
     }
