@@ -643,6 +643,9 @@ int build_plan(fgi_ctx *c, const char *tune_path)
         for (int sh : s.shells)
             shared = shared && c->radials[sh].h == c->radials[s.shells[0]].h &&
                      c->radials[sh].nk == c->radials[s.shells[0]].nk;
+        // (its points beyond the cutoff multiply interval 0 by zero: finite in FP32)
+        for (int sh : s.shells)
+            for (int q = 0; q < 4; q++) shared = shared && std::isfinite(coef_ddn[8 * (size_t)drad[sh].coef_off + q]);
         d.shared_grid = shared ? 1 : 0;
         // the shells grouped by l (stable), with each one's first function
         std::vector<int> first(s.shells.size()), lord;
@@ -675,7 +678,7 @@ int build_plan(fgi_ctx *c, const char *tune_path)
                     const size_t src = 8 * ((size_t)drad[s.shells[i]].coef_off + k);
                     scoefn.insert(scoefn.end(), coef_ddn.begin() + src, coef_ddn.begin() + src + 8);
                 }
-            if (r0.nk < 65536) {
+            {
                 const size_t ns = s.shells.size();
                 d.sbound_stride = (int)((ns + 3) / 4 * 4);
                 d.sbound_off = (long long)sbound.size();
@@ -985,7 +988,7 @@ int internal_integrate_h(fgi_ctx *c, const double *v, double *h, int accumulate,
     CUDA_TRY(c, cudaMemsetAsync(ws, 0, (size_t)c->nnz * 8, s));       // fixed-point accumulator
     for (const TcWave &w : c->tc.waves) {
         {
-            ProfScope ps(c, s, 0, w.phi_flops, w.phi_bytes);
+            ProfScope ps(c, s, 0, w.phi_flops, w.phi_bytes, 2);
             CUDA_TRY(c, tc_launch_phi(c->tc, P, w, v, ws, n_split, s));
         }
         ProfScope ps(c, s, 1, w.h_flops, w.h_bytes);

@@ -118,7 +118,7 @@ struct DevPlan {
     // [16] max |Y_lm| (index l*l + l + m), then per radial, per knot
     // interval k, a bound of |u(r)/r| over r >= k h
     const float *rbound;
-    // the same bounds for species on one knot grid of fewer than 65536 knots,
+    // the same bounds for species on one knot grid,
     // interleaved by interval in the order of DevPlan::shells and padded with
     // zeros to four shells, so that one 16-byte load serves four shells
     const float *sbound;

@@ -351,17 +351,15 @@ __device__ __forceinline__ const float4 *spline_tab(const DevPlan &P, const DevS
     return P.coef_dd + 2 * R.coef_off;
 }
 
-// ----------------------------------------- lane-per-point basis evaluation
-// One lane evaluates every function of one atom at its own point and hands
-// each value straight to an emitter (split + 16-bit stores into the operand
-// image): values never pass through shared memory, and the 32 lanes of a
-// warp (32 consecutive points, one atom) store 64 contiguous bytes of one
-// image row per plane.  The geometry (offset, distance, 1/d^(l+1)) is
-// double-float once per (point, atom); the radial factor once per shell,
-// times the per-point scale of each image; the angular polynomial FP32.
-// (Two points per lane with 32-bit stores of BF16 pairs was measured
-// slower: the doubled per-lane state costs occupancy or spills, and these
-// kernels wait mostly on their loads.)
+// ----------------------------------------- basis evaluation, two points a lane
+// A warp evaluates every function of one atom at the 64 points of a chunk, two
+// neighbouring points a lane in packed FP32 pairs (half the issue slots, which
+// bound the kernels), and hands each pair of values straight to an emitter
+// (split + one 32-bit store a plane into the operand image): values never pass
+// through shared memory, and a warp stores whole 128-byte image rows.  The
+// geometry (offset, distance, 1/d^(l+1)) is double-float once per (point,
+// atom); the radial factor once per shell, times the per-point scale of each
+// image; the angular polynomial FP32.
 
 // One value split on its row's or point's grid (as above; NSPLIT 1:
 // plain BF16) and stored as one 16-bit BF16 per plane
@@ -382,6 +380,27 @@ __device__ __forceinline__ void store_value(uint8_t *dst, df x, float scale, flo
         *reinterpret_cast<unsigned short *>(dst + 2 * kChunkBytes) = __bfloat16_as_ushort(c);
     } else {
         *reinterpret_cast<unsigned short *>(dst) = __bfloat16_as_ushort(__float2bfloat16_rn(x.hi));
+    }
+}
+
+// The same for the values hi - nlo of two neighbouring points (scale and unit a
+// pair too): one 32-bit store a plane
+template <int NSPLIT>
+__device__ __forceinline__ void store_pair(uint8_t *dst, pk hi, pk nlo, pk scale, pk unit)
+{
+    if (NSPLIT == 3) {
+        const pk x0 = (fma2(hi, scale, pk_dup(kRoundMagic)) + pk_dup(-kRoundMagic)) * unit;
+        const pk d = hi - x0;
+        const float2 xf = pk_get(x0), df_ = pk_get(d);
+        const uint32_t b = pack2_bf16(df_.x, df_.y);
+        const pk e = (d - pk_make(__uint_as_float(b << 16), __uint_as_float(b & 0xFFFF0000u))) - nlo;
+        const float2 ef = pk_get(e);
+        *reinterpret_cast<uint32_t *>(dst) = __byte_perm(__float_as_uint(xf.x), __float_as_uint(xf.y), 0x7632);
+        *reinterpret_cast<uint32_t *>(dst + kChunkBytes) = b;
+        *reinterpret_cast<uint32_t *>(dst + 2 * kChunkBytes) = pack2_bf16(ef.x, ef.y);
+    } else {
+        const float2 hf = pk_get(hi);
+        *reinterpret_cast<uint32_t *>(dst) = pack2_bf16(hf.x, hf.y);
     }
 }
 
@@ -416,14 +435,18 @@ __device__ __forceinline__ void ylm_poly_unit(float x, float y, float z, float *
         Q[0] = y; Q[1] = z; Q[2] = x;
         g[0] = g[1] = g[2] = 0;
     } else if (L == 2) {
-        Q[0] = x * y; Q[1] = y * z; Q[2] = 2.f * z * z - x * x - y * y; Q[3] = x * z;
-        Q[4] = 0.5f * (x * x - y * y);
+        Q[0] = x * y; Q[1] = y * z; Q[2] = fmaf(-y, y, fmaf(2.f * z, z, -(x * x))); Q[3] = x * z;
+        Q[4] = 0.5f * fmaf(x, x, -(y * y));
         g[0] = 0; g[1] = 0; g[2] = 1; g[3] = 0; g[4] = 0;
     } else {
-        const float q = 4.f * z * z - x * x - y * y;
-        Q[0] = y * (3.f * x * x - y * y); Q[1] = 2.f * (x * y * z); Q[2] = y * q;
-        Q[3] = z * (2.f * z * z - 3.f * x * x - 3.f * y * y); Q[4] = x * q; Q[5] = z * (x * x - y * y);
-        Q[6] = x * (x * x - 3.f * y * y);
+        const float xx = x * x, q = fmaf(-y, y, fmaf(4.f * z, z, -xx));
+        Q[0] = y * fmaf(-y, y, (3.f * x) * x);
+        Q[1] = 2.f * ((x * y) * z);
+        Q[2] = y * q;
+        Q[3] = z * fmaf(-(3.f * y), y, fmaf(2.f * z, z, -((3.f * x) * x)));
+        Q[4] = x * q;
+        Q[5] = z * fmaf(-y, y, xx);
+        Q[6] = x * fmaf(-(3.f * y), y, xx);
         g[0] = 0; g[1] = 1; g[2] = 2; g[3] = 3; g[4] = 2; g[5] = 1; g[6] = 0;
     }
 }
@@ -462,6 +485,35 @@ __device__ __forceinline__ void emit_shell_lane(const df *rk, float x, float y, 
 #pragma unroll
         for (int k = 0; k < NIMG; k++) val[k] = df_mul_f_raw(rc[k][gi[m]], Q[m]);
         emit(fm, val);
+    }
+}
+
+// the same polynomials for two points, rounding for rounding
+template <int L>
+__device__ __forceinline__ void ylm_poly_unit2(pk x, pk y, pk z, pk *Q, int *g)
+{
+    if (L == 1) {
+        Q[0] = y; Q[1] = z; Q[2] = x;
+        g[0] = g[1] = g[2] = 0;
+    } else if (L == 2) {
+        const pk two = pk_dup(2.f), half = pk_dup(0.5f);
+        Q[0] = x * y; Q[1] = y * z;
+        Q[2] = fma2(-y, y, fma2(two * z, z, -(x * x)));
+        Q[3] = x * z;
+        Q[4] = half * fma2(x, x, -(y * y));
+        g[0] = 0; g[1] = 0; g[2] = 1; g[3] = 0; g[4] = 0;
+    } else {
+        const pk two = pk_dup(2.f), three = pk_dup(3.f), four = pk_dup(4.f);
+        const pk xx = x * x;
+        const pk q = fma2(-y, y, fma2(four * z, z, -xx));
+        Q[0] = y * fma2(-y, y, (three * x) * x);
+        Q[1] = two * ((x * y) * z);
+        Q[2] = y * q;
+        Q[3] = z * fma2(-(three * y), y, fma2(two * z, z, -((three * x) * x)));
+        Q[4] = x * q;
+        Q[5] = z * fma2(-y, y, xx);
+        Q[6] = x * fma2(-(three * y), y, xx);
+        g[0] = 0; g[1] = 1; g[2] = 2; g[3] = 3; g[4] = 2; g[5] = 1; g[6] = 0;
     }
 }
 
@@ -588,70 +640,150 @@ __device__ __forceinline__ void eval_atom_general(const DevPlan &P, const DevSpe
     if (S.lmax >= 3) shells_of_l(std::integral_constant<int, 3>{});
 }
 
-// The same for the 32 lanes of a warp together (one atom, a point each).
-// Warps whose lanes are all beyond the species' cutoff call zero_all() and
-// clear their part of the image with 16-byte stores.  Where the species'
-// shells share one knot grid (and no lane sits on the nucleus) the lanes run
-// one path without divergence: a lane beyond the cutoff or without a point
-// multiplies by zero instead of branching, the interval and its fraction are
-// found once, and the next shell's coefficients load while the present ones
-// are used.  The order of operations of a value is that of the general path.
-template <int NIMG, bool SCALED, class Emit, class Emit0, class Zero>
-__device__ __forceinline__ void eval_atom_warp(const DevPlan &P, const DevSpecies &S, const DevShell *sh_tab,
-                                               const Dd3 &aa, const Dd3 &pp, bool has, int f_lo, int f_hi,
-                                               const df *scale, Emit &emit, Emit0 &emit0, Zero &zero_all)
+// two points' coordinates as pairs of double-floats
+struct Dd3x2 {
+    df2 x, y, z;
+};
+__device__ __forceinline__ Dd3x2 pair_dd3(const Dd3 &a, const Dd3 &b)
 {
-    const df zero{0.f, 0.f};
+    return Dd3x2{{pk_make(a.x.x, b.x.x), pk_make(a.x.y, b.x.y)},
+                 {pk_make(a.y.x, b.y.x), pk_make(a.y.y, b.y.y)},
+                 {pk_make(a.z.x, b.z.x), pk_make(a.z.y, b.z.y)}};
+}
+
+// The same for a warp together (one atom, two points a lane: p0, p1 their
+// coordinates, has0, has1 whether there are such points).  Warps whose points
+// are all beyond the species' cutoff call zero_all() and clear their part of
+// the image with 16-byte stores.  Where the species' shells share one knot grid
+// (and no point sits on the nucleus) the lanes run one path without
+// divergence: a point beyond the cutoff multiplies by zero instead of
+// branching, and the interval and its fraction are found once.  emit2(f, hi, nlo)
+// receives the pair of values hi[k] - nlo[k] of image k: the low parts are kept
+// negated from the radial factor on, which saves the packed negations and
+// changes no rounding.  The operations of a value are those of the general
+// path, in its order.
+//
+// What bounds it is instruction issue, then the L1's look-ups: two points a lane
+// halve the FP32 instructions a point (f32x2) and fill four bytes a store where
+// one filled two.  The 64-atom Si cluster's density images 1.84 -> 1.66 ms, 64
+// molecules' (2.3 M points) phi images 15.7 -> 13.9 ms with the preparation below.
+// Loading the next shell's coefficients ahead costs registers that a third CTA
+// an SM is worth more of: 2.14 -> 2.06 ms of H images without it.
+template <int NIMG, bool SCALED, class Emit2, class General, class Zero>
+__device__ __forceinline__ void eval_atom_warp(const DevPlan &P, const DevSpecies &S, const DevShell *sh_tab,
+                                               const Dd3 &aa, const Dd3x2 &pp, bool has0, bool has1, int f_lo,
+                                               int f_hi, const df2 *scale, Emit2 &emit2, General &general,
+                                               Zero &zero_all)
+{
     // beyond the species' largest cutoff every value is zero (FP32 distance,
     // relative error ~1e-7, against the cutoff with a 1e-5 margin)
-    const float3 o = offset_f32(pp, aa);
+    const df2 ax{pk_dup(-aa.x.x), pk_dup(-aa.x.y)}, ay{pk_dup(-aa.y.x), pk_dup(-aa.y.y)}, az{pk_dup(-aa.z.x), pk_dup(-aa.z.y)};
+    const pk ox = (pp.x.hi + ax.hi) + (pp.x.lo + ax.lo), oy = (pp.y.hi + ay.hi) + (pp.y.lo + ay.lo),
+             oz = (pp.z.hi + az.hi) + (pp.z.lo + az.lo);
+    const float2 o2 = pk_get(fma2(oz, oz, fma2(oy, oy, ox * ox)));
     const float rcs = (float)S.rcut * 1.00001f;
-    bool none = !has || o.x * o.x + o.y * o.y + o.z * o.z > rcs * rcs;
-    if (__all_sync(0xffffffffu, none)) {
+    const bool in0 = has0 && o2.x <= rcs * rcs, in1 = has1 && o2.y <= rcs * rcs;
+    if (__all_sync(0xffffffffu, !in0 && !in1)) {
         zero_all();
         return;
     }
     // offset from the atom (the rounding of the low parts differs from point
     // to point), d^2 (terms of one sign), 1/d from a refined rsqrtf, d = d^2/d
-    const df x = df_sub_sloppy(df{pp.x.x, pp.x.y}, df{aa.x.x, aa.x.y});
-    const df y = df_sub_sloppy(df{pp.y.x, pp.y.y}, df{aa.y.x, aa.y.y});
-    const df z = df_sub_sloppy(df{pp.z.x, pp.z.y}, df{aa.z.x, aa.z.y});
-    const df d2 = df_add_sloppy(df_add_sloppy(df_mul(x, x), df_mul(y, y)), df_mul(z, z));
-    if (!S.shared_grid || __any_sync(0xffffffffu, !none && d2.hi < 1e-24f)) {
-        eval_atom_general<NIMG, SCALED>(P, S, sh_tab, aa, pp, has, f_lo, f_hi, scale, emit, emit0);
+    const df2 x = df2_add_sloppy(pp.x, ax), y = df2_add_sloppy(pp.y, ay), z = df2_add_sloppy(pp.z, az);
+    const df2 d2 = df2_add_sloppy(df2_add_sloppy(df2_mul(x, x), df2_mul(y, y)), df2_mul(z, z));
+    const float2 d2h = pk_get(d2.hi);
+    if (!S.shared_grid || __any_sync(0xffffffffu, (in0 && d2h.x < 1e-24f) || (in1 && d2h.y < 1e-24f))) {
+        general(0);
+        general(1);
         return;
     }
-    const df i0 = df_rsqrt(d2);
-    const df d = df_mul(d2, i0);
-    const bool live = !none && d.hi < sh_tab[S.shell0].rcut_f;
-    const df sd = df_mul(d, df{S.inv_h_hi, S.inv_h_lo});
-    const int kk = live ? max(0, min((int)floorf(sd.hi), S.nk - 2)) : 0;
-    const float t = sd.hi - (float)kk, tl = sd.lo;
-    const float4 *ce = P.scoefn + S.scoef_off + 2 * ((long long)kk * S.n_shell);
-    SplineEntry next = load_entry(ce);
+    const df2 i0 = df2_rsqrt(d2);
+    const df2 d = df2_mul(d2, i0);
+    const float rcut = sh_tab[S.shell0].rcut_f;
+    const float2 dh = pk_get(d.hi);
+    const bool live0 = in0 && dh.x < rcut, live1 = in1 && dh.y < rcut;
+    const df2 sd = df2_mul(d, {pk_dup(S.inv_h_hi), pk_dup(S.inv_h_lo)});
+    const float2 sh2 = pk_get(sd.hi);
+    const int k0 = live0 ? max(0, min((int)floorf(sh2.x), S.nk - 2)) : 0;
+    const int k1 = live1 ? max(0, min((int)floorf(sh2.y), S.nk - 2)) : 0;
+    const float2 tl2 = pk_get(sd.lo);
+    // a point that is not live: t = 0 on interval 0, times ip = 0
+    const pk t = pk_make(live0 ? sh2.x - (float)k0 : 0.f, live1 ? sh2.y - (float)k1 : 0.f);
+    const pk nt = -t, ntl = pk_make(live0 ? -tl2.x : 0.f, live1 ? -tl2.y : 0.f), tt = t * t;
+    const float4 *tab = P.scoefn + S.scoef_off;
+    const float4 *c0 = tab + 2 * ((long long)k0 * S.n_shell), *c1 = tab + 2 * ((long long)k1 * S.n_shell);
     int sh = 0;
-    df pw = i0;                                         // 1/d^(l+1)
+    df2 pw = i0;                                        // 1/d^(l+1)
     auto shells_of_l = [&](auto lc) {
         constexpr int L = decltype(lc)::value;
         constexpr int NM = 2 * L + 1;
+        constexpr int NG = L < 2 ? 1 : (L == 2 ? 2 : 4);
+        constexpr int G0 = L == 2 ? 0 : 1;              // first kYlmRatio entry of groups 1..
         const int end = sh + S.nl[L];
-        if (L > 0) pw = df_mul(pw, i0);
-        df ip[NIMG];                                    // times each image's scale
+        if (L > 0) pw = df2_mul(pw, i0);
+        if (sh == end) return;
+        df2 ip[NIMG], nip[NIMG];                        // times each image's scale; and negated
 #pragma unroll
-        for (int k = 0; k < NIMG; k++) ip[k] = (SCALED || k > 0) ? df_mul(pw, scale[k]) : pw;
+        for (int k = 0; k < NIMG; k++) {
+            const df2 v = (SCALED || k > 0) ? df2_mul(pw, scale[k]) : pw;
+            const float2 vh = pk_get(v.hi), vl = pk_get(v.lo);
+            ip[k] = df2{pk_make(live0 ? vh.x : 0.f, live1 ? vh.y : 0.f), pk_make(live0 ? vl.x : 0.f, live1 ? vl.y : 0.f)};
+            nip[k] = df2{-ip[k].hi, -ip[k].lo};
+        }
+        pk Q[NM];
+        int gi[7];
+        if constexpr (L > 0) ylm_poly_unit2<L>(x.hi, y.hi, z.hi, Q, gi);
         for (; sh < end; sh++) {
-            const SplineEntry e = next;
-            if (sh + 1 < S.n_shell) next = load_entry(ce + 2 * (sh + 1));
+            const SplineEntry a = load_entry(c0 + 2 * sh), b = load_entry(c1 + 2 * sh);
             const int f = sh_tab[S.shell0 + sh].fn0;
             if (f + NM <= f_lo || f >= f_hi) continue;
-            const df u = spline_value(e, t, tl);
-            df rk[NIMG];
+            // u = c0 + t c1 + t^2 (c2 + t c3), c0 + t c1 in double-float (spline_value)
+            const pk h1 = pk_make(a.h.y, b.h.y), lin = t * h1;
+            const pk nlin_lo = fma2(nt, pk_make(a.l.y, b.l.y), fma2(ntl, h1, fma2(nt, h1, lin)));
+            const pk quad = tt * fma2(t, pk_make(a.h.w, b.h.w), pk_make(a.h.z, b.h.z));
+            const df2 u1 = df2_two_sum(pk_make(a.h.x, b.h.x), lin);
+            const df2 u = df2_two_sum(u1.hi, u1.lo + ((pk_make(a.l.x, b.l.x) - nlin_lo) + quad));
+            pk rh[NIMG][NG], nrh[NIMG][NG], nrl[NIMG][NG];   // radial factors: high, -high, -low
 #pragma unroll
             for (int k = 0; k < NIMG; k++) {
-                rk[k] = df_mul(u, ip[k]);
-                if (!live) rk[k] = zero;
+                const pk p = u.hi * ip[k].hi;
+                const pk nlo = fma2(u.hi, nip[k].lo, fma2(u.lo, nip[k].hi, fma2(u.hi, nip[k].hi, p)));
+                rh[k][0] = p - nlo;
+                nrl[k][0] = nlo + (rh[k][0] - p);
+#pragma unroll
+                for (int c = 1; c < NG; c++) {
+                    const float2 K = kYlmRatio[G0 + c - 1];
+                    const pk kh = pk_dup(K.x), kl = pk_dup(K.y), pc = rh[k][0] * kh;
+                    // -(rh kl + (rl kh + (rh kh - pc)))
+                    const pk nl = fma2(-rh[k][0], kl, fma2(nrl[k][0], kh, fma2(-rh[k][0], kh, pc)));
+                    rh[k][c] = pc - nl;
+                    nrl[k][c] = nl + (rh[k][c] - pc);
+                }
+#pragma unroll
+                for (int c = 0; c < NG; c++) nrh[k][c] = -rh[k][c];
             }
-            emit_shell_lane<L, NIMG>(rk, x.hi, y.hi, z.hi, f, f_lo, f_hi, emit);
+            if constexpr (L == 0) {                     // the angular factor is 1
+                pk hi[NIMG], nlo[NIMG];
+#pragma unroll
+                for (int k = 0; k < NIMG; k++) {
+                    hi[k] = rh[k][0];
+                    nlo[k] = nrl[k][0];
+                }
+                emit2(f, hi, nlo);
+            } else {
+                const bool whole = f >= f_lo && f + NM <= f_hi;
+#pragma unroll
+                for (int m = 0; m < NM; m++) {
+                    if (!whole && (f + m < f_lo || f + m >= f_hi)) continue;
+                    pk hi[NIMG], nlo[NIMG];
+#pragma unroll
+                    for (int k = 0; k < NIMG; k++) {    // df_mul_f_raw
+                        hi[k] = rh[k][gi[m]] * Q[m];
+                        nlo[k] = fma2(nrl[k][gi[m]], Q[m], fma2(nrh[k][gi[m]], Q[m], hi[k]));
+                    }
+                    emit2(f + m, hi, nlo);
+                }
+            }
         }
     };
     shells_of_l(std::integral_constant<int, 0>{});
@@ -672,55 +804,71 @@ __device__ __forceinline__ const DevShell *stage_shells(const DevPlan &P, DevShe
 // swizzled place of point column group g16 = g << 4 in row r of a chunk
 __device__ __forceinline__ uint32_t row_offset(uint32_t r, uint32_t g16) { return r * 128u + (((r << 4) ^ g16) & 0x70u); }
 
-// H images of one 128-row block: warp tasks (atom of the block, 32-point
-// group), lane = point.  NIMG 1: psi = phi sqrt|w v| on the second grid set;
-// NIMG 2: phi (first set) and w v phi (second set) into two images.
+// H images of one 128-row block: warp tasks (atom of the block, 64-point
+// chunk).  NIMG 1: psi = phi sqrt|w v| on the second grid set; NIMG 2: phi
+// (first set) and w v phi (second set) into two images.
 template <int NIMG, int NSPLIT>
 __device__ __forceinline__ void h_image_lanes(const DevPlan &P, const DevBatch &B, const TcBatch &T,
                                               const DevAct *act, const DevShell *sh_tab, int I, int e0, int ne,
                                               uint8_t *img0, uint8_t *img1, const float2 *wvs,
-                                              const float2 (*fsc)[128])
+                                              const float4 (*fsc)[128])
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
     const int r0 = I * 128;
-    const int ng = 2 * T.nc;                       // 32-point groups covering the image's chunks
-    for (int task = warp; task < ne * ng; task += nwarp) {
-        const int eq = task / ng, q = task - eq * ng;
+    const uint32_t g16 = (uint32_t)(lane >> 2) << 4, pb = (uint32_t)(lane & 3) * 4u;
+    for (int task = warp; task < ne * T.nc; task += nwarp) {
+        const int eq = task / T.nc, c = task - eq * T.nc;
         const DevAct A = act[e0 + eq];
         const DevSpecies S = P.species[P.atom_species[A.atom]];
         const int f_lo = max(0, r0 - A.fn_loc), f_hi = min(S.n_fn, r0 + 128 - A.fn_loc);
-        const int p = q * 32 + lane;
-        const bool has = p < B.np;
-        const Dd3 pp = load_dd3(P.pts_dd + 6 * (B.pt0 + (has ? p : 0)));
+        const int p = c * 64 + 2 * lane;
+        const bool has0 = p < B.np, has1 = p + 1 < B.np;
+        const Dd3 q0 = load_dd3(P.pts_dd + 6 * (B.pt0 + (has0 ? p : 0)));
+        const Dd3 q1 = load_dd3(P.pts_dd + 6 * (B.pt0 + (has1 ? p + 1 : 0)));
         const Dd3 aa = load_dd3(P.atom_dd + 6 * A.atom);
-        df scale[NIMG];
-        const float2 s2 = has ? wvs[p] : make_float2(0.f, 0.f);
+        const float2 s0 = has0 ? wvs[p] : make_float2(0.f, 0.f), s1 = has1 ? wvs[p + 1] : make_float2(0.f, 0.f);
+        df2 scale[NIMG];
 #pragma unroll
-        for (int k = 0; k < NIMG; k++) scale[k] = df{s2.x, s2.y};
+        for (int k = 0; k < NIMG; k++) scale[k] = df2{pk_make(s0.x, s1.x), pk_make(s0.y, s1.y)};
         const int rb = A.fn_loc - r0;
-        uint8_t *const c0 = img0 + (long long)(I * T.nc_alloc + (q >> 1)) * kChunkStride;
-        uint8_t *const c1 = img1 + (long long)(I * T.nc_alloc + (q >> 1)) * kChunkStride;
-        const uint32_t g16 = (uint32_t)((p >> 3) & 7) << 4, pb = (uint32_t)(p & 7) * 2u;
-        auto emit = [&](int f, const df *val) {
+        uint8_t *const c0 = img0 + (long long)(I * T.nc_alloc + c) * kChunkStride;
+        uint8_t *const c1 = img1 + (long long)(I * T.nc_alloc + c) * kChunkStride;
+        auto emit2 = [&](int f, const pk *hi, const pk *nlo) {
             const int r = rb + f;
             const uint32_t off = row_offset((uint32_t)r, g16) + pb;
 #pragma unroll
             for (int k = 0; k < NIMG; k++) {
-                const float2 su = fsc[NIMG == 1 ? 1 : k][r];
-                store_value<NSPLIT>((k == 0 ? c0 : c1) + off, val[k], su.x, su.y);
+                const float4 su = fsc[NIMG == 1 ? 1 : k][r];
+                store_pair<NSPLIT>((k == 0 ? c0 : c1) + off, hi[k], nlo[k], pk_make(su.x, su.y), pk_make(su.z, su.w));
             }
         };
-        auto emit0 = [&](int f) {
-            const uint32_t off = row_offset((uint32_t)(rb + f), g16) + pb;
+        auto general = [&](int half) {
+            df sc[NIMG];
+            const float2 s2 = half ? s1 : s0;
 #pragma unroll
-            for (int k = 0; k < NIMG; k++) store_zero<NSPLIT>((k == 0 ? c0 : c1) + off);
+            for (int k = 0; k < NIMG; k++) sc[k] = df{s2.x, s2.y};
+            const uint32_t hb = pb + 2u * half;
+            auto emit = [&](int f, const df *val) {
+                const int r = rb + f;
+                const uint32_t off = row_offset((uint32_t)r, g16) + hb;
+#pragma unroll
+                for (int k = 0; k < NIMG; k++) {
+                    const float4 su = fsc[NIMG == 1 ? 1 : k][r];
+                    store_value<NSPLIT>((k == 0 ? c0 : c1) + off, val[k], su.x, su.z);
+                }
+            };
+            auto emit0 = [&](int f) {
+                const uint32_t off = row_offset((uint32_t)(rb + f), g16) + hb;
+#pragma unroll
+                for (int k = 0; k < NIMG; k++) store_zero<NSPLIT>((k == 0 ? c0 : c1) + off);
+            };
+            eval_atom_general<NIMG, NIMG == 1>(P, S, sh_tab, aa, half ? q1 : q0, half ? has1 : has0, f_lo, f_hi, sc,
+                                               emit, emit0);
         };
-        // the warp's 32 columns of rows rb + [f_lo, f_hi): four 16-byte units
-        // per row and plane
+        // the chunk's columns of rows rb + [f_lo, f_hi): eight 16-byte units a row and plane
         auto zero_all = [&]() {
-            for (int u = lane; u < (f_hi - f_lo) * 4; u += 32) {
-                const uint32_t off = row_offset((uint32_t)(rb + f_lo + (u >> 2)),
-                                                (uint32_t)((q & 1) * 4 + (u & 3)) << 4);
+            for (int u = lane; u < (f_hi - f_lo) * 8; u += 32) {
+                const uint32_t off = row_offset((uint32_t)(rb + f_lo + (u >> 3)), (uint32_t)(u & 7) << 4);
 #pragma unroll
                 for (int k = 0; k < NIMG; k++)
 #pragma unroll
@@ -729,55 +877,28 @@ __device__ __forceinline__ void h_image_lanes(const DevPlan &P, const DevBatch &
                             make_uint4(0u, 0u, 0u, 0u);
             }
         };
-        eval_atom_warp<NIMG, NIMG == 1>(P, S, sh_tab, aa, pp, has, f_lo, f_hi, scale, emit, emit0, zero_all);
+        eval_atom_warp<NIMG, NIMG == 1>(P, S, sh_tab, aa, pair_dd3(q0, q1), has0, has1, f_lo, f_hi, scale, emit2,
+                                        general, zero_all);
     }
 }
 
-// -------------------------------------------- basis -> operand images (K1)
-// CTA per (batch, 128-row block).  A first pass takes bounds of the rows'
-// maxima and sums for the fixed-point grids; then every function is evaluated
-// lane per point and the split planes of psi = phi sqrt|w v| (batches where
-// w v has one sign) or of phi and w v phi (mixed signs) are written.
-//
-// The radial factor N_lm u(d)/d^(l+1) -- shared by all angular points of a
-// radial shell, so its rounding would be systematic -- is evaluated in
-// double-float from a double-float spline table and double-float
-// coordinates; only the angular polynomial Q_lm(x, y, z) is FP32 (its
-// rounding varies from point to point).
-
+// ------------------------------------- preparation of the H images (K0)
+// CTA per super-batch: the sign of w v, the images' scale of every point, the
+// digit grid (scale, unit) of every function in both images, and the
+// descriptors of the row blocks.  A kernel of its own: these passes want many
+// small warps in flight, the evaluation few with many registers, and a
+// super-batch's atoms and points are looked at once instead of once a row
+// block.  H images with it and two points a lane: 64-atom Si cluster, 1.11 M
+// points, 2.73 -> 2.06 ms (0.46 of it here), 75-atom cluster with f shells,
+// two images a batch, 3.80 -> 3.08 ms (0.73 here).
 constexpr int kPhiThreads = 256;
-constexpr int kKnotCache = 8448;                      // (atom, point) knots of the bound pass kept in shared memory
-constexpr int kGeoCache = 128 * 33 / 2;               // float4 slots of the pass over the points
-
-// FP32 distance from atom `atom` to point `pt` (from the double-float
-// coordinates), for the bounds of the digit grids
-__device__ __forceinline__ float point_atom_dist_f32(const DevPlan &P, int atom, long long pt)
-{
-    const float3 o = offset_f32(load_dd3(P.pts_dd + 6 * pt), load_dd3(P.atom_dd + 6 * atom));
-    return sqrtf(o.x * o.x + o.y * o.y + o.z * o.z);
-}
 
 // Knot interval of distance d from below (against FP32 rounding of d) for the
-// suffix bounds of |u(r)/r|, or kNoKnot beyond the cutoff
-constexpr int kNoKnot = 0xFFFF;
+// suffix bounds of |u(r)/r|, or -1 beyond the cutoff
 __device__ __forceinline__ int knot_below(float d, float rcut_f, float inv_h, int nk)
 {
-    if (!(d < rcut_f * 1.00001f)) return kNoKnot;
+    if (!(d < rcut_f * 1.00001f)) return -1;
     return min(max((int)(d * 0.999999f * inv_h), 0), nk - 2);
-}
-
-// lane m folds function m of a shell (first function f1 of its atom, 2l+1 of
-// them) into its row: the bound of the radial factor times max |Y_lm|
-__device__ __forceinline__ void fold_row(const DevPlan &P, const DevShell &R, int fn_loc, int r0, int f_lo, int f_hi,
-                                         int lane, float m, float s, unsigned int *rowmax, float *rowsum)
-{
-    const int fr = R.fn0 + lane;
-    if (lane < 2 * R.l + 1 && m > 0.f && fr >= f_lo && fr < f_hi) {
-        const int row = fn_loc + fr - r0;
-        const float yl = __ldg(P.rbound + R.l * R.l + lane);
-        rowmax[row] = __float_as_uint(fminf(m * yl, 1.0e30f));
-        rowsum[row] = fminf(s * 1.0001f * yl, 1.0e30f);       // 1.0001: FP32 sums
-    }
 }
 
 __device__ __forceinline__ float warp_sum(float s)
@@ -787,61 +908,174 @@ __device__ __forceinline__ float warp_sum(float s)
     return s;
 }
 
-// Row bounds of one atom's functions from the interleaved table of its
-// species: four shells per task, one 16-byte look-up per point for all four.
-// MIXED: also the bounds of |phi| itself (set 0), which only batches with
-// both signs use.
+__device__ __forceinline__ float warp_max(float m)                   // m >= 0
+{
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
+}
+
+// digit grid of function f (row of its block) in image `set`
+__device__ __forceinline__ void put_grid(HGrid *grids, int set, int f, float mx, float sum, int depth)
+{
+    float sc, un;
+    fixed_scale_adaptive(mx, sum, depth, sc, un);
+    grids[f >> 7].s[set][f & 127] = make_float2(sc, un);
+}
+
+// lane m: the grid of function m of a shell (first function f0 in the batch) from
+// the bound of its radial factor and of the factor's sum, times max |Y_lm|
+__device__ __forceinline__ void put_shell_grid(const DevPlan &P, HGrid *grids, int set, int l, int f0, float m, float s,
+                                               int depth, int lane)
+{
+    if (lane > 2 * l) return;
+    const float yl = __ldg(P.rbound + l * l + lane);
+    put_grid(grids, set, f0 + lane, m > 0.f ? fminf(m * yl, 1.0e30f) : 0.f, fminf(s * 1.0001f * yl, 1.0e30f), depth);
+}
+
+// Grids of one atom's functions by a warp from the interleaved table bounds: per
+// point one look-up of the suffix bounds of |u(r)/r| serves four shells, times
+// sqrt|w v| (psi) or |w v| (w v phi) of the point; the maximum over the points
+// times max |Y_lm| bounds each row, and the same products summed over the
+// points bound the row sums, so that rows whose sum allows it keep an 8-bit
+// digit.  MIXED: also |phi| itself (set 0), which only batches with both signs
+// use.
 template <bool MIXED>
-__device__ __forceinline__ void row_bounds_quad(const DevPlan &P, const DevBatch &B, const DevAct &A,
-                                                const DevSpecies &S, const DevShell *sh_tab, int quad, int r0, int f_lo,
-                                                int f_hi, const unsigned short *kc, const float *wvf,
-                                                unsigned int (*rowmax)[128], float (*rowsum)[128])
+__device__ __forceinline__ void atom_grids(const DevPlan &P, const DevBatch &B, const DevAct &A, const DevSpecies &S,
+                                           const DevShell *sh_tab, const Dd3 *pts, const float *wvf, HGrid *grids,
+                                           int depth)
 {
     const int lane = threadIdx.x & 31;
-    const float *bt = P.sbound + S.sbound_off + 4 * quad;
-    float m0[4] = {}, m1[4] = {}, s0[4] = {}, s1[4] = {};
-    for (int p = lane; p < B.np; p += 32) {
-        const int ki = kc ? (int)kc[p]
-                          : knot_below(point_atom_dist_f32(P, A.atom, B.pt0 + p), sh_tab[S.shell0].rcut_f, S.inv_h_hi, S.nk);
-        if (ki != kNoKnot) {
-            const float4 t4 = __ldg(reinterpret_cast<const float4 *>(bt + (long long)ki * S.sbound_stride));
-            const float t[4] = {t4.x, t4.y, t4.z, t4.w};
+    const Dd3 aa = load_dd3(P.atom_dd + 6 * A.atom);
+    const float rcut = sh_tab[S.shell0].rcut_f;
+    for (int q0 = 0; 4 * q0 < S.n_shell; q0 += 3) {                // twelve shells a pass
+        const int nq = min(3, (S.n_shell + 3) / 4 - q0);
+        const float *bt = P.sbound + S.sbound_off + 4 * q0;
+        float m0[12], m1[12], s0[12], s1[12];
+#pragma unroll
+        for (int j = 0; j < 12; j++) m0[j] = m1[j] = s0[j] = s1[j] = 0.f;
+        for (int p = lane; p < B.np; p += 32) {
+            const float3 o = offset_f32(pts[p], aa);
+            const int ki = knot_below(sqrtf(o.x * o.x + o.y * o.y + o.z * o.z), rcut, S.inv_h_hi, S.nk);
+            if (ki < 0) continue;
+            const float4 *row = reinterpret_cast<const float4 *>(bt + (long long)ki * S.sbound_stride);
             const float w = wvf[p];
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const float tw = t[j] * w;
-                m1[j] = fmaxf(m1[j], tw);
-                s1[j] += tw;
-                if (MIXED) {
-                    m0[j] = fmaxf(m0[j], t[j]);
-                    s0[j] += t[j];
+            for (int q = 0; q < 3; q++) {
+                if (q >= nq) break;
+                const float4 t4 = __ldg(row + q);
+                const float t[4] = {t4.x, t4.y, t4.z, t4.w};
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    const float tw = t[j] * w;
+                    m1[4 * q + j] = fmaxf(m1[4 * q + j], tw);
+                    s1[4 * q + j] += tw;
+                    if (MIXED) {
+                        m0[4 * q + j] = fmaxf(m0[4 * q + j], t[j]);
+                        s0[4 * q + j] += t[j];
+                    }
                 }
             }
         }
-    }
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
-        const int sh = 4 * quad + j;
-        if (sh >= S.n_shell) break;
-        const DevShell R = sh_tab[S.shell0 + sh];
-        if (R.fn0 + 2 * R.l + 1 <= f_lo || R.fn0 >= f_hi) continue;
-        const float a1 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m1[j]))), b1 = warp_sum(s1[j]);
-        fold_row(P, R, A.fn_loc, r0, f_lo, f_hi, lane, a1, b1, rowmax[1], rowsum[1]);
-        if (MIXED) {
-            const float a0 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m0[j])));
-            const float b0 = warp_sum(s0[j]);
-            fold_row(P, R, A.fn_loc, r0, f_lo, f_hi, lane, a0, b0, rowmax[0], rowsum[0]);
+        for (int j = 0; j < 12; j++) {
+            const int sh = 4 * q0 + j;
+            if (sh >= S.n_shell) break;
+            const int l = sh_tab[S.shell0 + sh].l, f0 = A.fn_loc + sh_tab[S.shell0 + sh].fn0;
+            const float a1 = warp_max(m1[j]), b1 = warp_sum(s1[j]);
+            put_shell_grid(P, grids, 1, l, f0, a1, b1, depth, lane);
+            if (MIXED) {
+                const float a0 = warp_max(m0[j]), b0 = warp_sum(s0[j]);
+                put_shell_grid(P, grids, 0, l, f0, a0, b0, depth, lane);
+            }
         }
+    }
+}
+
+// The same for any species, a shell at a time from its own table
+__device__ __forceinline__ void atom_grids_general(const DevPlan &P, const DevBatch &B, const DevAct &A,
+                                                   const DevSpecies &S, const DevShell *sh_tab, const Dd3 *pts,
+                                                   const float *wvf, HGrid *grids, int depth)
+{
+    const int lane = threadIdx.x & 31;
+    const Dd3 aa = load_dd3(P.atom_dd + 6 * A.atom);
+    for (int sh = 0; sh < S.n_shell; sh++) {
+        const DevShell R = sh_tab[S.shell0 + sh];
+        const float *bt = P.rbound + R.bound_off;
+        float m0 = 0.f, m1 = 0.f, s0 = 0.f, s1 = 0.f;
+        for (int p = lane; p < B.np; p += 32) {
+            const float3 o = offset_f32(pts[p], aa);
+            const int ki = knot_below(sqrtf(o.x * o.x + o.y * o.y + o.z * o.z), R.rcut_f, R.inv_h_hi, R.nk);
+            if (ki < 0) continue;
+            const float t = __ldg(bt + ki), tw = t * wvf[p];
+            m0 = fmaxf(m0, t);
+            m1 = fmaxf(m1, tw);
+            s0 += t;
+            s1 += tw;
+        }
+        m0 = warp_max(m0);
+        m1 = warp_max(m1);
+        s0 = warp_sum(s0);
+        s1 = warp_sum(s1);
+        put_shell_grid(P, grids, 0, R.l, A.fn_loc + R.fn0, m0, s0, depth, lane);
+        put_shell_grid(P, grids, 1, R.l, A.fn_loc + R.fn0, m1, s1, depth, lane);
+    }
+}
+
+// The exact maxima and sums of |phi| and |w v phi| (or |psi|) over the points,
+// in FP32 (bound_grids 0 and 1)
+__device__ __forceinline__ void atom_grids_exact(const DevPlan &P, const DevBatch &B, const DevAct &A, const DevSpecies &S,
+                                                 const Dd3 *pts, const float *wvf, HGrid *grids, int depth)
+{
+    const int lane = threadIdx.x & 31;
+    const float *aa = P.atom_dd + 6 * A.atom;
+    const float ax = aa[0] + aa[1], ay = aa[2] + aa[3], az = aa[4] + aa[5];
+    int f = A.fn_loc;
+    for (int sh = 0; sh < S.n_shell; sh++) {
+        const DevRadial R = P.radials[P.shell_rad[S.shell0 + sh]];
+        const int nm = 2 * R.l + 1;
+        int tstep;
+        const float4 *tab = spline_tab(P, S, R, sh, tstep);
+        float mx[7], sm[7], mxw[7], smw[7];
+#pragma unroll
+        for (int m = 0; m < 7; m++) mx[m] = sm[m] = mxw[m] = smw[m] = 0.f;
+        for (int p = lane; p < B.np; p += 32) {
+            const Dd3 pp = pts[p];
+            const float x = (pp.x.x + pp.x.y) - ax, y = (pp.y.x + pp.y.y) - ay, z = (pp.z.x + pp.z.y) - az;
+            const float d = sqrtf(x * x + y * y + z * z);
+            const float rad = radial_over_d_f32(R, tab, tstep, d, __frcp_rn(d));
+            if (rad == 0.f) continue;
+            float Q[7];
+            int ci[7];
+            ylm_poly_f32(R.l, x, y, z, Q, ci);
+            const float wvp = wvf[p];
+#pragma unroll
+            for (int m = 0; m < 7; m++) {
+                if (m >= nm) break;
+                const float a = fminf(fabsf(rad * kYlmC[ci[m]].x * Q[m]), 1.0e30f);
+                const float aw = fminf(a * wvp, 1.0e30f);
+                mx[m] = fmaxf(mx[m], a);
+                sm[m] += a;
+                mxw[m] = fmaxf(mxw[m], aw);
+                smw[m] += aw;
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < 7; m++) {
+            if (m >= nm) break;
+            const float a = warp_max(mx[m]), aw = warp_max(mxw[m]), s1 = warp_sum(sm[m]), s2 = warp_sum(smw[m]);
+            if (lane == 0) {
+                put_grid(grids, 0, f + m, a, s1, depth);
+                put_grid(grids, 1, f + m, aw, s2, depth);
+            }
+        }
+        f += nm;
     }
 }
 
 // The descriptor of one row block for the H scatter (threads 0 .. 127, a row
 // each; e0 the first of the block's ne active atoms)
-__device__ __forceinline__ void write_hblock(const DevPlan &P, const DevBatch &B, const DevAct *act, int r0, int e0, int ne,
-                                             HBlock *out)
+__device__ __forceinline__ void write_hblock(const DevPlan &P, const DevBatch &B, const DevAct *act, int r0, int r, int e0,
+                                             int ne, HBlock *out)
 {
-    const int r = threadIdx.x;
-    if (r >= 128) return;
     const int f = r0 + r;
     long long base = 0;
     int li = 0, slot = 0;
@@ -860,21 +1094,88 @@ __device__ __forceinline__ void write_hblock(const DevPlan &P, const DevBatch &B
         out->nat = P.sys_nat[B.sys];
         out->nslot = ne;
         out->n = min(128, B.nfn - r0);
-
     }
 }
 
-__global__ void __launch_bounds__(kPhiThreads, 4) k_tc_phi(DevPlan P, const TcBatch *tb, const WorkItem *items,
-                                                uint8_t *ws, const double *v, int n_split, int fixed,
-                                                int *bsign, int bound, unsigned int *counter)
+__global__ void __launch_bounds__(kPhiThreads, 4) k_h_prep(DevPlan P, const TcBatch *tb, int b0, uint8_t *ws, const double *v,
+                                                        int fixed, int bound, int *bsign, unsigned int *counter)
 {
-    extern __shared__ float4 phi_smem[];            // knots of the bound pass, or offsets of the pass over the points
+    __shared__ Dd3 pts[kMaxBatchPoints];
+    __shared__ float wvf[kMaxBatchPoints];           // |w v| or its root per point (FP32)
+    __shared__ DevShell shs[kMaxShellsSmem];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0u;       // of the contraction that follows
+    const int b = b0 + blockIdx.x;
+    const DevBatch B = P.batches[b];
+    if (B.np <= 0 || B.nfn <= 0) return;
+    const TcBatch T = tb[b];
+    const DevAct *act = P.act + B.act0;
+    const DevShell *sh_tab = stage_shells(P, shs);
+    // sign of w v over the batch: one sign s (or zero) everywhere lets H use a
+    // single image psi = phi sqrt|w v| for both operands, H = s psi^T psi;
+    // mixed signs keep the phi and w v phi images
+    bool pos = false, neg = false, bad = false;
+    for (int p = threadIdx.x; p < B.np; p += blockDim.x) {
+        const double vv = v[B.pt0 + p], wv = P.pw[B.pt0 + p] * vv;
+        pos |= wv > 0.0;
+        neg |= wv < 0.0;
+        bad |= !isfinite(vv);
+        pts[p] = load_dd3(P.pts_dd + 6 * (B.pt0 + p));
+    }
+    if (bad) atomicOr(P.status, kStatusNonFinite);
+    pos = __syncthreads_or(pos) != 0;
+    neg = __syncthreads_or(neg) != 0;
+    const int sgn = (pos && neg) ? 0 : (neg ? -1 : 1);
+    if (threadIdx.x == 0) bsign[b] = sgn;
+    // the per-point scale of the images, sqrt|w v| (psi) or w v (mixed signs),
+    // and its size for the grids
+    HGrid *grids = reinterpret_cast<HGrid *>(ws + T.hgrid);
+    float2 *wvs = reinterpret_cast<float2 *>(ws + T.hscale);
+    const float up = bound ? 1.f + 1.f / 1048576.f : 1.f;
+    for (int p = threadIdx.x; p < B.np; p += blockDim.x) {
+        const double s = P.pw[B.pt0 + p] * v[B.pt0 + p];
+        df sd = df_from_double(sgn != 0 ? fabs(s) : s);
+        if (sgn != 0) sd = df_sqrt(sd);
+        wvs[p] = make_float2(sd.hi, sd.lo);
+        const float a = fabsf((float)s) * up;
+        wvf[p] = fminf(sgn != 0 ? sqrtf(a) * up : a, 1.0e30f);
+    }
+    for (int q = threadIdx.x; q < T.nrb * 128; q += blockDim.x) {
+        const int r0 = q & ~127, rend = min(r0 + 128, B.nfn);
+        const int e0 = find_act(act, B.n_act, r0), e1 = find_act(act, B.n_act, rend - 1);
+        write_hblock(P, B, act, r0, q & 127, e0, e1 - e0 + 1, reinterpret_cast<HBlock *>(ws + T.hblock) + (q >> 7));
+    }
+    if (!fixed) return;
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5, depth = T.nc * 64;
+    for (int e = warp; e < B.n_act; e += nwarp) {
+        const DevAct A = act[e];
+        const DevSpecies S = P.species[P.atom_species[A.atom]];
+        if (!bound) atom_grids_exact(P, B, A, S, pts, wvf, grids, depth);
+        else if (S.sbound_stride == 0) atom_grids_general(P, B, A, S, sh_tab, pts, wvf, grids, depth);
+        else if (sgn != 0) atom_grids<false>(P, B, A, S, sh_tab, pts, wvf, grids, depth);
+        else atom_grids<true>(P, B, A, S, sh_tab, pts, wvf, grids, depth);
+    }
+}
+
+// -------------------------------------------- basis -> operand images (K1)
+// CTA per (batch, 128-row block): every function of the block is evaluated, two
+// points a lane, and the split planes of psi = phi sqrt|w v| (batches where w v
+// has one sign) or of phi and w v phi (mixed signs) are written on the grids of
+// the preparation.
+//
+// The radial factor N_lm u(d)/d^(l+1) -- shared by all angular points of a
+// radial shell, so its rounding would be systematic -- is evaluated in
+// double-float from a double-float spline table and double-float
+// coordinates; only the angular polynomial Q_lm(x, y, z) is FP32 (its
+// rounding varies from point to point).
+//
+// Three CTAs an SM: two take 2.28 ms where three take 2.06 (four 2.08: spills).
+__global__ void __launch_bounds__(kPhiThreads, 3) k_tc_phi(DevPlan P, const TcBatch *tb, const WorkItem *items,
+                                                uint8_t *ws, int fixed, const int *bsign)
+{
     __shared__ float2 wvs[kMaxBatchPoints];         // per-point image scale (double-float)
     __shared__ DevShell shs[kMaxShellsSmem];
-    __shared__ unsigned int rowmax[2][128];          // |phi|, |w v phi| maxima (float bits)
-    __shared__ float rowsum[2][128];                 // sums of |phi|, |w v phi| over the points
-    __shared__ float2 fsc[2][128];                   // per row: scale, unit
-    __shared__ float wvf[kMaxBatchPoints];           // |w v| per point (FP32), first pass
+    __shared__ float4 fsc[2][128];                   // per row: scale twice, unit twice
     const WorkItem it = items[blockIdx.x];
     const DevBatch B = P.batches[it.batch];
     const TcBatch T = tb[it.batch];
@@ -887,232 +1188,15 @@ __global__ void __launch_bounds__(kPhiThreads, 4) k_tc_phi(DevPlan P, const TcBa
     const int ne = e1 - e0 + 1;
     uint8_t *phi_img = ws + T.img_phi;
     uint8_t *a_img = ws + T.img_aux;
-    // the species' shells (visible after the barrier below)
     const DevShell *sh_tab = stage_shells(P, shs);
-    // sign of w v over the batch: one sign s (or zero) everywhere lets H use a
-    // single image psi = phi sqrt|w v| for both operands, H = s psi^T psi;
-    // mixed signs keep the phi and w v phi images
-    bool pos = false, neg = false;
-    for (int p = threadIdx.x; p < B.np; p += blockDim.x) {
-        const double wv = P.pw[B.pt0 + p] * v[B.pt0 + p];
-        pos |= wv > 0.0;
-        neg |= wv < 0.0;
-    }
-    pos = __syncthreads_or(pos) != 0;
-    neg = __syncthreads_or(neg) != 0;
-    const int sgn = (pos && neg) ? 0 : (neg ? -1 : 1);
-    if (I == 0 && threadIdx.x == 0) bsign[it.batch] = sgn;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0u;       // of the contraction that follows
-    write_hblock(P, B, act, r0, e0, ne, reinterpret_cast<HBlock *>(ws + T.hblock) + I);
-    if (fixed && bound) {
-        // row bounds from the tables: per (atom, shell) and point one lookup
-        // of the suffix bound of |u(r)/r| at the point's distance (knot index
-        // taken from below), times sqrt|w v| (psi) or |w v| (w v phi) of the
-        // point; the maximum over the points times max |Y_lm| bounds each
-        // row, and the same products summed over the points bound the row
-        // sums, so that rows whose sum allows it keep an 8-bit digit.
+    const int sgn = bsign[it.batch];
+    for (int p = threadIdx.x; p < B.np; p += blockDim.x) wvs[p] = reinterpret_cast<const float2 *>(ws + T.hscale)[p];
+    if (fixed) {
+        const HGrid *g = reinterpret_cast<const HGrid *>(ws + T.hgrid) + I;
         for (int q = threadIdx.x; q < 256; q += blockDim.x) {
-            (&rowmax[0][0])[q] = 0u;          // rows past n_b stay zero
-            (&rowsum[0][0])[q] = 0.f;
+            const float2 su = g->s[q >> 7][q & 127];
+            fsc[q >> 7][q & 127] = make_float4(su.x, su.x, su.y, su.y);
         }
-        for (int p = threadIdx.x; p < B.np; p += blockDim.x) {
-            const float a = fabsf((float)(P.pw[B.pt0 + p] * v[B.pt0 + p])) * (1.f + 1.f / 1048576.f);
-            wvf[p] = fminf(sgn != 0 ? sqrtf(a) * (1.f + 1.f / 1048576.f) : a, 1.0e30f);
-        }
-        // knots of the points on the block's atoms' grids, once, when they fit
-        unsigned short *kcache = reinterpret_cast<unsigned short *>(phi_smem);
-        const bool cached = ne * B.np <= kKnotCache;
-        if (cached) {
-            for (int q = threadIdx.x; q < ne * B.np; q += blockDim.x) {
-                const int eq = q / B.np, p = q - eq * B.np;
-                const int atom = act[e0 + eq].atom;
-                const DevSpecies &S = P.species[P.atom_species[atom]];
-                if (S.sbound_stride > 0)
-                    kcache[q] = (unsigned short)knot_below(point_atom_dist_f32(P, atom, B.pt0 + p),
-                                                           sh_tab[S.shell0].rcut_f, S.inv_h_hi, S.nk);
-            }
-        }
-        __syncthreads();
-        // warp tasks (atom of the block, four of its shells): the lanes stride
-        // over the batch's points and keep the maxima and sums in registers;
-        // one warp reduction per shell, whose rows the warp alone writes
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-        int job0 = 0;
-        for (int e = e0; e <= e1; e++) {
-            const DevAct A = act[e];
-            const DevSpecies S = P.species[P.atom_species[A.atom]];
-            const int f_lo = max(0, r0 - A.fn_loc), f_hi = min(S.n_fn, r0 + 128 - A.fn_loc);
-            const int first = ((warp - job0) % nwarp + nwarp) % nwarp;
-            if (S.sbound_stride > 0) {
-                const int nq = (S.n_shell + 3) >> 2;
-                job0 += nq;
-                const unsigned short *kc = cached ? kcache + (e - e0) * B.np : nullptr;
-                for (int qd = first; qd < nq; qd += nwarp) {
-                    if (sgn != 0)
-                        row_bounds_quad<false>(P, B, A, S, sh_tab, qd, r0, f_lo, f_hi, kc, wvf, rowmax, rowsum);
-                    else
-                        row_bounds_quad<true>(P, B, A, S, sh_tab, qd, r0, f_lo, f_hi, kc, wvf, rowmax, rowsum);
-                }
-                continue;
-            }
-            // shells on knot grids of their own (or too long for the cache's index)
-            job0 += S.n_shell;
-            for (int sh = first; sh < S.n_shell; sh += nwarp) {
-                const DevShell R = sh_tab[S.shell0 + sh];
-                if (R.fn0 + 2 * R.l + 1 <= f_lo || R.fn0 >= f_hi) continue;
-                const float rcl = R.rcut_f * 1.00001f;
-                const float *bt = P.rbound + R.bound_off;
-                float m0 = 0.f, m1 = 0.f, s0 = 0.f, s1 = 0.f;
-                for (int p = lane; p < B.np; p += 32) {
-                    const float d = point_atom_dist_f32(P, A.atom, B.pt0 + p);
-                    if (d < rcl) {
-                        const int ki = min(max((int)(d * 0.999999f * R.inv_h_hi), 0), R.nk - 2);
-                        const float t = __ldg(bt + ki);
-                        const float tw = t * wvf[p];
-                        m0 = fmaxf(m0, t);
-                        m1 = fmaxf(m1, tw);
-                        s0 += t;
-                        s1 += tw;
-                    }
-                }
-                m0 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m0)));
-                m1 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m1)));
-                s0 = warp_sum(s0);
-                s1 = warp_sum(s1);
-                fold_row(P, R, A.fn_loc, r0, f_lo, f_hi, lane, m0, s0, rowmax[0], rowsum[0]);
-                fold_row(P, R, A.fn_loc, r0, f_lo, f_hi, lane, m1, s1, rowmax[1], rowsum[1]);
-            }
-        }
-        __syncthreads();
-        for (int q = threadIdx.x; q < 256; q += blockDim.x) {
-            const int which = q >> 7, r = q & 127;
-            float sc, un;
-            fixed_scale_adaptive(__uint_as_float(rowmax[which][r]), rowsum[which][r], T.nc * 64, sc, un);
-            fsc[which][r] = make_float2(sc, un);
-        }
-        __syncthreads();
-    } else if (fixed) {
-        // pass 1: row maxima and sums of |phi| and |w v phi| (or of |psi|,
-        // kept in the second set) over the batch's points (FP32).  One warp
-        // per (atom, shell) of the block; lanes stride over the points and
-        // keep per-function partials in registers.
-        for (int q = threadIdx.x; q < 256; q += blockDim.x) {
-            (&rowmax[0][0])[q] = 0u;          // rows past n_b stay zero
-            (&rowsum[0][0])[q] = 0.f;
-        }
-        for (int p = threadIdx.x; p < B.np; p += blockDim.x) {
-            const float a = fabsf((float)(P.pw[B.pt0 + p] * v[B.pt0 + p]));
-            wvf[p] = fminf(sgn != 0 ? sqrtf(a) : a, 1.0e30f);
-        }
-        // FP32 offsets and distances of the block's atoms to the batch's points,
-        // once, in the (not yet used) value buffer when they fit: every shell
-        // job of an atom reads them instead of recomputing them
-        float4 *geo = phi_smem;
-        const bool geo_cached = ne * B.np <= kGeoCache;
-        if (geo_cached) {
-            for (int q = threadIdx.x; q < ne * B.np; q += blockDim.x) {
-                const int eq = q / B.np, p = q - eq * B.np;
-                const float *aa = P.atom_dd + 6 * act[e0 + eq].atom;
-                const float *pp = P.pts_dd + 6 * (B.pt0 + p);
-                const float x = (pp[0] + pp[1]) - (aa[0] + aa[1]);
-                const float y = (pp[2] + pp[3]) - (aa[2] + aa[3]);
-                const float z = (pp[4] + pp[5]) - (aa[4] + aa[5]);
-                geo[q] = make_float4(x, y, z, sqrtf(x * x + y * y + z * z));
-            }
-        }
-        __syncthreads();
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-        int job = 0;
-        for (int e = e0; e <= e1; e++) {
-            const DevAct A = act[e];
-            const DevSpecies S = P.species[P.atom_species[A.atom]];
-            const int f_lo = max(0, r0 - A.fn_loc), f_hi = min(S.n_fn, r0 + 128 - A.fn_loc);
-            const float *aa = P.atom_dd + 6 * A.atom;
-            const float ax = aa[0] + aa[1], ay = aa[2] + aa[3], az = aa[4] + aa[5];
-            int f = 0;
-            for (int sh = 0; sh < S.n_shell; sh++) {
-                const DevRadial R = P.radials[P.shell_rad[S.shell0 + sh]];
-                const int nm = 2 * R.l + 1;
-                const int f1 = f;
-                f += nm;
-                if (f <= f_lo || f1 >= f_hi) continue;
-                if ((job++ % nwarp) != warp) continue;
-                int tstep;
-                const float4 *tab = spline_tab(P, S, R, sh, tstep);
-                float mx[7], sm[7], mxw[7], smw[7];
-#pragma unroll
-                for (int m = 0; m < 7; m++) mx[m] = sm[m] = mxw[m] = smw[m] = 0.f;
-                for (int p = lane; p < B.np; p += 32) {
-                    float x, y, z, d;
-                    if (geo_cached) {
-                        const float4 gq = geo[(e - e0) * B.np + p];
-                        x = gq.x;
-                        y = gq.y;
-                        z = gq.z;
-                        d = gq.w;
-                    } else {
-                        const float *pp = P.pts_dd + 6 * (B.pt0 + p);
-                        x = (pp[0] + pp[1]) - ax;
-                        y = (pp[2] + pp[3]) - ay;
-                        z = (pp[4] + pp[5]) - az;
-                        d = sqrtf(x * x + y * y + z * z);
-                    }
-                    const float rad = radial_over_d_f32(R, tab, tstep, d, __frcp_rn(d));
-                    if (rad == 0.f) continue;
-                    float Q[7];
-                    int ci[7];
-                    ylm_poly_f32(R.l, x, y, z, Q, ci);
-                    const float wvp = wvf[p];
-#pragma unroll
-                    for (int m = 0; m < 7; m++) {
-                        if (m >= nm) break;
-                        const float a = fminf(fabsf(rad * kYlmC[ci[m]].x * Q[m]), 1.0e30f);
-                        const float aw = fminf(a * wvp, 1.0e30f);
-                        mx[m] = fmaxf(mx[m], a);
-                        sm[m] += a;
-                        mxw[m] = fmaxf(mxw[m], aw);
-                        smw[m] += aw;
-                    }
-                }
-#pragma unroll
-                for (int m = 0; m < 7; m++) {
-                    if (m >= nm) break;
-                    unsigned int a = __reduce_max_sync(0xffffffffu, __float_as_uint(mx[m]));
-                    unsigned int aw = __reduce_max_sync(0xffffffffu, __float_as_uint(mxw[m]));
-                    float s1 = sm[m], s2 = smw[m];
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-                        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-                    }
-                    const int fr = f1 + m;
-                    if (lane == 0 && fr >= f_lo && fr < f_hi) {
-                        const int row = A.fn_loc + fr - r0;
-                        rowmax[0][row] = a;
-                        rowmax[1][row] = aw;
-                        rowsum[0][row] = s1;
-                        rowsum[1][row] = s2;
-                    }
-                }
-            }
-        }
-        __syncthreads();
-        for (int q = threadIdx.x; q < 256; q += blockDim.x) {
-            const int which = q >> 7, r = q & 127;
-            float sc, un;
-            fixed_scale_adaptive(__uint_as_float(rowmax[which][r]), rowsum[which][r], T.nc * 64, sc, un);
-            fsc[which][r] = make_float2(sc, un);
-        }
-        __syncthreads();
-    }
-    // the per-point scale of the images: sqrt|w v| (psi) or w v (mixed signs)
-    for (int p = threadIdx.x; p < B.np; p += blockDim.x) {
-        const double vv = v ? v[B.pt0 + p] : 0.0;
-        if (!isfinite(vv)) atomicOr(P.status, kStatusNonFinite);
-        const double s = P.pw[B.pt0 + p] * vv;
-        df sd = df_from_double(sgn != 0 ? fabs(s) : s);
-        if (sgn != 0) sd = df_sqrt(sd);
-        wvs[p] = make_float2(sd.hi, sd.lo);
     }
     __syncthreads();
     uint8_t *img1 = sgn == 0 ? a_img : phi_img;
@@ -1123,36 +1207,31 @@ __global__ void __launch_bounds__(kPhiThreads, 4) k_tc_phi(DevPlan P, const TcBa
         if (fixed) h_image_lanes<2, 3>(P, B, T, act, sh_tab, I, e0, ne, phi_img, img1, wvs, fsc);
         else h_image_lanes<2, 1>(P, B, T, act, sh_tab, I, e0, ne, phi_img, img1, wvs, fsc);
     }
-    // rows past n_b in the last block: zeros (whole 16-byte units)
-    const int nlive = rend - r0;
-    const int nplanes = fixed ? 3 : 1;
-    for (int u = threadIdx.x; u < (128 - nlive) * T.nc * 8; u += blockDim.x) {
-        const int r = nlive + u / (T.nc * 8), cg = u % (T.nc * 8);
-        const long long off = unit_offset(I, T.nc_alloc, cg >> 3, r, cg & 7);
-        for (int pl = 0; pl < nplanes; pl++) {
-            *reinterpret_cast<uint4 *>(phi_img + off + pl * kChunkBytes) = make_uint4(0u, 0u, 0u, 0u);
-            if (sgn == 0) *reinterpret_cast<uint4 *>(a_img + off + pl * kChunkBytes) = make_uint4(0u, 0u, 0u, 0u);
-        }
-    }
+    // rows past n_b in the last block stay as they are: a row or column of a
+    // product depends on its own operand row alone, and the scatter leaves
+    // those out (the padding of the points is zero)
 }
 
-// The density's image of one 64-point chunk: warp tasks (active atom, 32-point
-// half of the chunk), lane = point (the same point for all of a warp's
-// tasks), every function of the atom, split on the point's grid.
+// The density's image of one 64-point chunk: a warp an active atom, two
+// neighbouring points a lane (the same for all of the warp's atoms), every
+// function of the atom, split on the points' grids.
 template <int NSPLIT>
 __device__ __forceinline__ void density_image_lanes(const DevPlan &P, const DevBatch &B, const TcBatch &T,
                                                     const DevAct *act, const DevShell *sh_tab, int c, uint8_t *phi_img,
                                                     const float2 *csc)
 {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;   // nwarp even
-    const int half = warp & 1, k = half * 32 + lane, p = c * 64 + k;
-    const bool has = p < B.np;
-    const Dd3 pp = load_dd3(P.pts_dd + 6 * (B.pt0 + (has ? p : 0)));
-    const float2 su = NSPLIT == 3 ? csc[k] : make_float2(0.f, 0.f);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+    const int k = 2 * lane, p = c * 64 + k;
+    const bool has0 = p < B.np, has1 = p + 1 < B.np;
+    const Dd3 q0 = load_dd3(P.pts_dd + 6 * (B.pt0 + (has0 ? p : 0)));
+    const Dd3 q1 = load_dd3(P.pts_dd + 6 * (B.pt0 + (has1 ? p + 1 : 0)));
+    const Dd3x2 pp = pair_dd3(q0, q1);
+    const float2 s0 = NSPLIT == 3 ? csc[k] : make_float2(0.f, 0.f), s1 = NSPLIT == 3 ? csc[k + 1] : make_float2(0.f, 0.f);
+    const pk sc = pk_make(s0.x, s1.x), un = pk_make(s0.y, s1.y);
     uint8_t *const img = phi_img + (long long)c * kChunkStride;
-    const uint32_t g16 = (uint32_t)(k >> 3) << 4, pb = (uint32_t)(k & 7) * 2u;
+    const uint32_t g16 = (uint32_t)(lane >> 2) << 4, pb = (uint32_t)(lane & 3) * 4u;
     const uint32_t blk = (uint32_t)T.nc_alloc * kChunkStride - 128u * 128u;   // a row block, less its rows' offsets
-    for (int e = warp >> 1; e < B.n_act; e += nwarp >> 1) {
+    for (int e = warp; e < B.n_act; e += nwarp) {
         const DevAct A = act[e];
         const DevSpecies S = P.species[P.atom_species[A.atom]];
         const Dd3 aa = load_dd3(P.atom_dd + 6 * A.atom);
@@ -1160,18 +1239,28 @@ __device__ __forceinline__ void density_image_lanes(const DevPlan &P, const DevB
             const uint32_t rg = (uint32_t)(A.fn_loc + f);
             return (rg >> 7) * blk + row_offset(rg, g);
         };
-        auto emit = [&](int f, const df *val) { store_value<NSPLIT>(img + place(f, g16) + pb, val[0], su.x, su.y); };
-        auto emit0 = [&](int f) { store_zero<NSPLIT>(img + place(f, g16) + pb); };
-        // the warp's 32 columns of the atom's rows: four 16-byte units per row and plane
+        auto emit2 = [&](int f, const pk *hi, const pk *nlo) {
+            store_pair<NSPLIT>(img + place(f, g16) + pb, hi[0], nlo[0], sc, un);
+        };
+        auto general = [&](int half) {
+            const uint32_t hb = pb + 2u * half;
+            const float2 su = half ? s1 : s0;
+            auto emit = [&](int f, const df *val) { store_value<NSPLIT>(img + place(f, g16) + hb, val[0], su.x, su.y); };
+            auto emit0 = [&](int f) { store_zero<NSPLIT>(img + place(f, g16) + hb); };
+            eval_atom_general<1, false>(P, S, sh_tab, aa, half ? q1 : q0, half ? has1 : has0, 0, S.n_fn, nullptr, emit,
+                                        emit0);
+        };
+        // the chunk's columns of the atom's rows: eight 16-byte units a row and plane
         auto zero_all = [&]() {
-            for (int u = lane; u < S.n_fn * 4; u += 32) {
-                const uint32_t off = place(u >> 2, (uint32_t)(half * 4 + (u & 3)) << 4);
+            for (int u = lane; u < S.n_fn * 8; u += 32) {
+                const uint32_t off = place(u >> 3, (uint32_t)(u & 7) << 4);
 #pragma unroll
                 for (int pl = 0; pl < NSPLIT; pl++)
                     *reinterpret_cast<uint4 *>(img + off + pl * kChunkBytes) = make_uint4(0u, 0u, 0u, 0u);
             }
         };
-        eval_atom_warp<1, false>(P, S, sh_tab, aa, pp, has, 0, S.n_fn, nullptr, emit, emit0, zero_all);
+        eval_atom_warp<1, false>(P, S, sh_tab, aa, pp, has0, has1, 0, S.n_fn, (const df2 *)nullptr, emit2, general,
+                                 zero_all);
     }
 }
 
@@ -1179,7 +1268,7 @@ __device__ __forceinline__ void density_image_lanes(const DevPlan &P, const DevB
 // density contracts over functions, so the fixed-point grid of the leading
 // term is per point (column): first the largest |phi_i(p)| over all of the
 // batch's functions (FP32), then every 128-row block in double-float.
-__global__ void __launch_bounds__(kPhiThreads, 5) k_tc_phi_cols(DevPlan P, const TcBatch *tb, const WorkItem *items,
+__global__ void __launch_bounds__(kPhiThreads, 3) k_tc_phi_cols(DevPlan P, const TcBatch *tb, const WorkItem *items,
                                                      uint8_t *ws, int n_split, int bound, unsigned int *counter)
 {
     if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0u;       // of the contraction that follows
@@ -1223,7 +1312,7 @@ __global__ void __launch_bounds__(kPhiThreads, 5) k_tc_phi_cols(DevPlan P, const
                 if (bound && S.sbound_stride > 0) {
                     // table bounds, four shells a look-up
                     const int ki = knot_below(d, sh_tab[S.shell0].rcut_f, S.inv_h_hi, S.nk);
-                    if (ki == kNoKnot) continue;
+                    if (ki < 0) continue;
                     const float4 *bt = reinterpret_cast<const float4 *>(P.sbound + S.sbound_off +
                                                                         (long long)ki * S.sbound_stride);
                     for (int q = 0; 4 * q < S.n_shell; q++) {
@@ -1288,9 +1377,9 @@ __global__ void __launch_bounds__(kPhiThreads, 5) k_tc_phi_cols(DevPlan P, const
     }
     if (fixed) density_image_lanes<3>(P, B, T, act, sh_tab, c, phi_img, csc);
     else density_image_lanes<1>(P, B, T, act, sh_tab, c, phi_img, csc);
-    // rows [n_b, 64 nkc) of the contraction's last function chunk: zeros
+    // rows from n_b to the end of the contraction's last 16-deep step: zeros
     const int nplanes = fixed ? 3 : 1;
-    for (int u = threadIdx.x; u < (T.nkc * 64 - B.nfn) * 8; u += blockDim.x) {
+    for (int u = threadIdx.x; u < (-B.nfn & 15) * 8; u += blockDim.x) {
         const int rg = B.nfn + (u >> 3), g = u & 7;
         const long long off = unit_offset(rg >> 7, T.nc_alloc, c, rg & 127, g);
         for (int pl = 0; pl < nplanes; pl++)
@@ -1730,6 +1819,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_h(DevPlan P, const TcBatch
                 float size = 0.f;
 #pragma unroll
                 for (int q = 0; q < 32; q++) size = max_abs_nan(size, a0[q], a1[q]);
+                if (!inj) size = 0.f;              // a row past n_b
                 if (tab && !__any_sync(0xffffffffu, !(size < 16384.f))) {
                     // v 2^8 = h + f with h its rounding (by an addition, the FRND unit
                     // is slow), f exact: h 2^32 + f 2^32 in units of 2^-40, the sign of
@@ -2315,9 +2405,6 @@ size_t smem_tc(int n_split)
     return 1024 + (size_t)kStages * kStageBytes + sizeof(TcRing);
 }
 
-// the bound pass keeps knots (bound_grids 2), the pass over the points offsets
-size_t smem_phi(bool bound) { return bound ? kKnotCache * sizeof(unsigned short) : kGeoCache * sizeof(float4); }
-
 size_t smem_tc_h() { return smem_tc(3) + kTiles * sizeof(HTile) + 2 * sizeof(HTables); }
 static_assert(1024 + kStages * kStageBytes + sizeof(TcRing) + kTiles * sizeof(HTile) + 2 * sizeof(HTables) <= 232448,
               "the H contraction's shared memory");
@@ -2332,8 +2419,6 @@ cudaError_t set_attrs()
     e = cudaFuncSetAttribute(k_tc_density<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_tc(3));
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_tc_density<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_tc(3));
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_tc_phi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_phi(false));
     if (e != cudaSuccess) return e;
     attrs_set = true;
     return cudaSuccess;
@@ -2426,10 +2511,12 @@ int tc_build(TcPlan &t, const TcPlanInput &in, std::string *err)
         T.plane_phi = (long long)T.nrb * T.nc_alloc * kChunkBytes;
         T.plane_d = (long long)T.nrb * T.nkc * kChunkBytes;
         foot[b] = 3 * (size_t)T.plane_phi + 3 * (size_t)std::max(T.plane_phi, T.plane_d);
-        T.hblock = -1;
+        T.hblock = T.hgrid = T.hscale = -1;
         if (in.for_h) {
-            // phi and w v phi images, and the row blocks' descriptors
-            foot[b] = 6 * (size_t)T.plane_phi + ((size_t)T.nrb * sizeof(HBlock) + 1023) / 1024 * 1024;
+            // phi and w v phi images; the row blocks' descriptors and grids, the
+            // points' scales
+            foot[b] = 6 * (size_t)T.plane_phi +
+                      ((size_t)T.nrb * (sizeof(HBlock) + sizeof(HGrid)) + (size_t)T.nc * 512 + 1023) / 1024 * 1024;
         }
         T.img_e = -1;
         if (in.with_e) foot[b] += 2 * (size_t)T.plane_phi;     // E in FP32: twice a BF16 plane
@@ -2465,7 +2552,11 @@ int tc_build(TcPlan &t, const TcPlanInput &in, std::string *err)
         TcBatch &T = t.batches[b];
         T.img_phi = (long long)off;
         T.img_aux = (long long)(off + 3 * (size_t)T.plane_phi);
-        if (in.for_h) T.hblock = (long long)(off + 6 * (size_t)T.plane_phi);
+        if (in.for_h) {
+            T.hblock = (long long)(off + 6 * (size_t)T.plane_phi);
+            T.hgrid = T.hblock + (long long)T.nrb * (long long)sizeof(HBlock);
+            T.hscale = T.hgrid + (long long)T.nrb * (long long)sizeof(HGrid);
+        }
         if (in.with_e) T.img_e = (long long)(off + 3 * (size_t)T.plane_phi + 3 * (size_t)std::max(T.plane_phi, T.plane_d));
         T.part0 = part;
         part += part_rows(b);
@@ -2506,7 +2597,7 @@ int tc_build(TcPlan &t, const TcPlanInput &in, std::string *err)
         wv.ng = (long long)t.items.size() - wv.g0;
         wv.pc0 = (long long)t.items.size();
         for (int b : ord)
-            for (int c = 0; c < t.batches[b].nc_alloc; c++) t.items.push_back(WorkItem{b, (short)c, 0});
+            for (int c = 0; c < t.batches[b].nc; c++) t.items.push_back(WorkItem{b, (short)c, 0});
         wv.npc = (long long)t.items.size() - wv.pc0;
         wv.d0 = (long long)t.items.size();
         for (int b : ord)
@@ -2594,14 +2685,14 @@ cudaError_t tc_launch_phi(const TcPlan &t, const DevPlan &P, const TcWave &w, co
                           int n_split, cudaStream_t s)
 {
     if (w.nphi <= 0) return cudaSuccess;
-    // the H images (v given) of the split mode use the fixed-point leading term
-    const int fixed = (v != nullptr && n_split == 3) ? 1 : 0;
-    const size_t dyn = smem_phi(t.bound_grids >= 2);
-    k_tc_phi<<<(unsigned)w.nphi, kPhiThreads, dyn, s>>>(P, t.d_batches, t.d_items + w.phi0,
-                                                       (uint8_t *)ws + t.img_base, v, n_split, fixed,
-                                                       reinterpret_cast<int *>((uint8_t *)ws + t.sign_off),
-                                                       t.bound_grids >= 2 ? 1 : 0,
-                                                       reinterpret_cast<unsigned int *>((uint8_t *)ws + t.counter_off));
+    const int fixed = n_split == 3 ? 1 : 0;             // the split mode's fixed-point leading term
+    uint8_t *img = (uint8_t *)ws + t.img_base;
+    int *bsign = reinterpret_cast<int *>((uint8_t *)ws + t.sign_off);
+    k_h_prep<<<(unsigned)w.nb, kPhiThreads, 0, s>>>(P, t.d_batches, w.b0, img, v, fixed, t.bound_grids >= 2 ? 1 : 0,
+                                                    bsign, reinterpret_cast<unsigned int *>((uint8_t *)ws + t.counter_off));
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_tc_phi<<<(unsigned)w.nphi, kPhiThreads, 0, s>>>(P, t.d_batches, t.d_items + w.phi0, img, fixed, bsign);
     return cudaGetLastError();
 }
 

@@ -35,6 +35,12 @@ struct HBlock {
 };
 static_assert(sizeof(HBlock) % 16 == 0, "HBlock is moved by bulk copies");
 
+// Digit grids of one row block: (scale, unit) per row of the phi image (set 0)
+// and of the psi or w v phi image (set 1)
+struct HGrid {
+    float2 s[2][128];
+};
+
 struct TcBatch {
     long long img_phi;     // byte offset (in the wave's workspace) of the phi image
     long long img_aux;     // byte offset of the w v phi image (H) or the D image (density)
@@ -48,6 +54,8 @@ struct TcBatch {
     long long img_e;       // byte offset of E = G Phi (FP32 [row][point], rows of 64 nc_alloc points)
                            // for the adjoint, -1 when the plan keeps no room for it
     long long hblock;      // byte offset of the row blocks' descriptors (H plans), else -1
+    long long hgrid;       // of their digit grids
+    long long hscale;      // of the points' image scales (a double-float each)
 };
 
 struct TcWave {
