@@ -149,4 +149,14 @@ inline void radial_over_r_bounds(const double *coef, int n_int, double h, float 
     }
 }
 
+// Sum over m of |Y_lm| <= (2l+1)/sqrt(4 pi): Cauchy-Schwarz with
+// sum_m Y_lm^2 = (2l+1)/(4 pi) (Unsold's theorem)
+#if defined(__CUDACC__)
+__host__ __device__
+#endif
+inline float ylm_sum_bound(int l)
+{
+    return (float)(2 * l + 1) * (0.28209479f * 1.000001f);
+}
+
 }  // namespace fgi

@@ -631,10 +631,11 @@ int build_plan(fgi_ctx *c, const char *tune_path)
     // species whose shells share one knot grid also get their coefficients
     // interleaved by interval, so that one point's shells read neighbouring
     // cache lines
-    std::vector<float> scoef, scoefn, sbound;
+    std::vector<float> scoef, scoefn, sbound, cbound;
     std::vector<int> shell_fn0, shell_by_l;     // per species slot: first function, radial (grouped by l)
     for (const SpeciesH &s : c->species) {
         DevSpecies d{};
+        d.cbound_off = -1;
         d.shell0 = (int)shell_rad.size();
         d.n_shell = (int)s.shells.size();
         d.n_fn = s.n_fn;
@@ -687,6 +688,21 @@ int build_plan(fgi_ctx *c, const char *tune_path)
                 for (int k = 0; k < r0.nk - 1; k++)
                     for (size_t i = 0; i < ns; i++)
                         dst[(size_t)k * d.sbound_stride + i] = rbound[drad[s.shells[lord[i]]].bound_off + k];
+                // the same over all shells, in FP32 and the shells' order
+                d.cbound_off = (long long)(cbound.size() / 2);
+                for (int k = 0; k < r0.nk - 1; k++) {
+                    float mx = 0.f, sm = 0.f;
+                    for (int i : lord) {
+                        const int l = c->radials[s.shells[i]].l;
+                        float y = 0.f;
+                        for (int m = 0; m <= 2 * l; m++) y = std::max(y, rbound[l * l + m]);
+                        const float tb = rbound[drad[s.shells[i]].bound_off + k];
+                        mx = std::max(mx, std::min(tb * y, 1.0e30f));
+                        sm += std::min(tb * ylm_sum_bound(l), 1.0e30f);
+                    }
+                    cbound.push_back(mx);
+                    cbound.push_back(sm);
+                }
             }
         }
         shell_rad.insert(shell_rad.end(), s.shells.begin(), s.shells.end());
@@ -715,6 +731,7 @@ int build_plan(fgi_ctx *c, const char *tune_path)
     if (scoef.empty()) scoef.assign(8, 0.f);
     if (scoefn.empty()) scoefn.assign(8, 0.f);
     if (sbound.empty()) sbound.assign(4, 0.f);
+    if (cbound.empty()) cbound.assign(2, 0.f);
     BigVec<double> px(c->n_pts), py(c->n_pts), pz(c->n_pts);
 #pragma omp parallel for schedule(static)
     for (int64_t p = 0; p < c->n_pts; p++) {
@@ -779,7 +796,8 @@ int build_plan(fgi_ctx *c, const char *tune_path)
            i_sv0 = add(sys_val0.data(), sys_val0.size() * 8), i_sf0 = add(sys_fn0.data(), sys_fn0.size() * 8),
            i_fsys = add(c->fn_sys.data(), c->fn_sys.size() * 4), i_status = add(nullptr, 64),
            i_snnz = add(sys_nnz.data(), sys_nnz.size() * 8), i_colg = add(col_glob.data(), col_glob.size() * 4),
-           i_rbnd = add(rbound.data(), rbound.size() * 4), i_sbnd = add(sbound.data(), sbound.size() * 4);
+           i_rbnd = add(rbound.data(), rbound.size() * 4), i_sbnd = add(sbound.data(), sbound.size() * 4),
+           i_cbnd = add(cbound.data(), cbound.size() * 4);
     cudaError_t e = cudaMalloc((void **)&c->d_arena, total);
     if (e != cudaSuccess) {
         c->d_arena = nullptr;
@@ -829,6 +847,7 @@ int build_plan(fgi_ctx *c, const char *tune_path)
     P.col_glob = (const int *)at(i_colg);
     P.rbound = (const float *)at(i_rbnd);
     P.sbound = (const float *)at(i_sbnd);
+    P.cbound = (const float2 *)at(i_cbnd);
     c->d_status = (int *)at(i_status);
 
     // tensor-core path plan (operand images, tiles, waves)

@@ -38,6 +38,7 @@ struct DevSpecies {
     int lmax;             // largest angular momentum of its shells
     int sbound_stride;    // floats per interval of its interleaved bounds (0: none, see DevPlan::sbound)
     long long sbound_off; // first of them in DevPlan::sbound
+    long long cbound_off; // first of its column bounds in DevPlan::cbound, -1: none
     int nl[4];            // shells of each l (DevPlan::shells holds them grouped by l)
 };
 
@@ -122,6 +123,10 @@ struct DevPlan {
     // interleaved by interval in the order of DevPlan::shells and padded with
     // zeros to four shells, so that one 16-byte load serves four shells
     const float *sbound;
+    // per species on one knot grid, per interval: the maximum over its shells
+    // and m of the bound of |phi|, and the bound of their sum (the column
+    // bounds of the density's digit grids)
+    const float2 *cbound;
 };
 
 // ---- launchers (return the launch status) ----

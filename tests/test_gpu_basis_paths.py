@@ -65,3 +65,28 @@ def test_shared_knots_equal_general_path(molecule, both_signs, points, precision
     assert np.array_equal(a, b)                                   # the same active functions
     assert np.abs(h0).max() > 0 and np.array_equal(h0, h1)
     assert np.abs(n0).max() > 0 and np.array_equal(n0, n1)
+
+
+def test_column_bounds_of_many_atoms(tmp_path):
+    """More active atoms at a point than the column bounds stage at a time
+    (128), the last group partly filled; the same two paths, equal bit by bit."""
+    import paper_2208_12335_gb300 as fgi
+    rc = 4.0 * W.BOHR_PER_ANG
+    radials = [W.make_radial(W.RadialSpec(l, (0.5 + 0.2 * l, 1.7), (1.0, -0.2), rc, rc - W.BOHR_PER_ANG, 900))
+               for l in (0, 1)]
+    species = [W.Species("A", 1.0, [0, 1])]
+    xyz = np.stack(np.meshgrid(*[1.2 * np.arange(n) for n in (6, 5, 5)], indexing="ij"), -1).reshape(-1, 3)
+    prob = W.build_problem("many", radials, species, [(np.zeros(150, dtype=np.int32), xyz)], lambda k: (4, 14), 9,
+                           (200, 50, None))
+    r = radials[1]
+    padded = [radials[0], W.Radial(r.l, r.h, np.concatenate([r.coef, np.zeros((1, 4))]), r.spec, r.norm)]
+    out = []
+    for rads in (radials, padded):
+        ctx = fgi.Context(0).load(dataclasses.replace(prob, radials=rads), "split_bf16")
+        d = torch.from_numpy(np.random.default_rng(5).standard_normal(ctx.sizes()[1])).cuda()
+        n = ctx.density(d)[0]
+        ctx.sync()
+        out.append((ctx.batch_work()[1], n.cpu().numpy()))
+    (a, n0), (b, n1) = out
+    assert np.array_equal(a, b) and a.max() > 4 * 128
+    assert np.abs(n0).max() > 0 and np.array_equal(n0, n1)
