@@ -2305,100 +2305,263 @@ __global__ void __launch_bounds__(128) k_density_sum(DevPlan P, const TcBatch *t
     n_out[B.pt0 + p] = factor * s;
 }
 
-// sum over the shell's 2l+1 functions of E_i grad phi_i (FP32), unrolled per l
-template <int L>
-__device__ __forceinline__ void adj_shell(float g, float gp, float x, float y, float z, float nx, float ny, float nz,
-                                          const float *Erow, long long Pa, float &gx, float &gy, float &gz)
+// What the position gradient needs of a shell (in the species' own order) and
+// of an active atom
+struct AdjShell {
+    int l, nk, coef_off;
+    float rcut_f, inv_h;
+};
+struct AdjAtom {
+    Dd3 pos;
+    float rlim, rcut_f;                              // the species' cutoff with its margin; of the shared knots
+    float inv_h;
+    int nk, shared, shell0, n_shell, fn_loc, atom;
+    const float4 *tab;                               // shared knots: interval 0 of the species' splines
+};
+constexpr int kAdjAtoms = 64;                        // staged at a time
+
+__device__ __forceinline__ AdjShell adj_shell_entry(const DevPlan &P, int i)
 {
-    float Y[2 * L + 1], G[2 * L + 1][3];
-    ylm_unit<float>(L, x, y, z, Y);                      // P(r) = r^l Y_lm
-    ylm_poly_grad<float>(L, x, y, z, G);
-#pragma unroll
-    for (int m = 0; m < 2 * L + 1; m++) {
-        const float e = __ldg(Erow + m * Pa);
-        const float a = gp * Y[m];
-        gx = fmaf(e, fmaf(a, nx, g * G[m][0]), gx);
-        gy = fmaf(e, fmaf(a, ny, g * G[m][1]), gy);
-        gz = fmaf(e, fmaf(a, nz, g * G[m][2]), gz);
+    const DevRadial &R = P.radials[P.shell_rad[i]];
+    return AdjShell{R.l, R.nk, (int)R.coef_off, R.rcut_f, R.inv_h_hi};
+}
+
+// Two points' P = r^l Y_lm and its gradient: add(m, Y_m, G_m, mask) for every m, mask the
+// components of the gradient that are not zero
+template <int L, class Add>
+__device__ __forceinline__ void adj_angular(pk x, pk y, pk z, Add &&add)
+{
+    const pk no = pk_dup(0.f);
+    auto g3 = [&](int m, pk Y, pk gx, pk gy, pk gz, int mask) {
+        const pk G[3] = {gx, gy, gz};
+        add(m, Y, G, mask);
+    };
+    if constexpr (L == 0) {
+        g3(0, pk_dup(0.28209479177387814f), no, no, no, 0);
+    } else if constexpr (L == 1) {
+        const pk c = pk_dup(0.4886025119029199f);
+        g3(0, c * y, no, c, no, 2);
+        g3(1, c * z, no, no, c, 4);
+        g3(2, c * x, c, no, no, 1);
+    } else if constexpr (L == 2) {
+        constexpr float fb = 0.31539156525252005f, fc = 0.5462742152960396f;
+        const pk a = pk_dup(1.0925484305920792f), b = pk_dup(fb), c = pk_dup(fc);
+        const pk ax = a * x, ay = a * y, az = a * z, xx = x * x, yy = y * y;
+        g3(0, ax * y, ay, ax, no, 3);
+        g3(1, ay * z, no, az, ay, 6);
+        g3(2, b * (fma2(pk_dup(2.f) * z, z, -xx) - yy), pk_dup(-2.f * fb) * x, pk_dup(-2.f * fb) * y, pk_dup(4.f * fb) * z,
+           7);
+        g3(3, ax * z, az, no, ax, 5);
+        g3(4, c * (xx - yy), pk_dup(2.f * fc) * x, pk_dup(-2.f * fc) * y, no, 3);
+    } else {
+        constexpr float f3 = 0.5900435899266435f, f2 = 2.890611442640554f, f1 = 0.4570457994644658f,
+                        f0 = 0.3731763325901154f, f2b = 1.445305721320277f;
+        const pk c3 = pk_dup(f3), c2 = pk_dup(f2), c1 = pk_dup(f1), c0 = pk_dup(f0), c2b = pk_dup(f2b);
+        const pk xx = x * x, yy = y * y, y3 = pk_dup(3.f) * y, txx = (pk_dup(3.f) * x) * x;
+        const pk fz = pk_dup(4.f) * z, zx = fma2(fz, z, -xx), q = zx - yy, dxy = xx - yy;
+        const pk c2x = c2 * x;
+        g3(0, (c3 * y) * (txx - yy), (pk_dup(6.f * f3) * x) * y, pk_dup(3.f * f3) * dxy, no, 3);
+        g3(1, (c2x * y) * z, (c2 * y) * z, c2x * z, c2x * y, 7);
+        g3(2, (c1 * y) * q, (pk_dup(-2.f * f1) * x) * y, c1 * fma2(-y3, y, zx), (pk_dup(8.f * f1) * y) * z, 7);
+        g3(3, (c0 * z) * fma2(-y3, y, fma2(pk_dup(2.f) * z, z, -txx)), (pk_dup(-6.f * f0) * x) * z,
+           (pk_dup(-6.f * f0) * y) * z, c0 * fma2(-y3, y, fma2(pk_dup(6.f) * z, z, -txx)), 7);
+        g3(4, (c1 * x) * q, c1 * (fma2(fz, z, -txx) - yy), (pk_dup(-2.f * f1) * x) * y, (pk_dup(8.f * f1) * x) * z, 7);
+        g3(5, (c2b * z) * dxy, (pk_dup(2.f * f2b) * x) * z, (pk_dup(-2.f * f2b) * y) * z, c2b * dxy, 7);
+        g3(6, (c3 * x) * fma2(-y3, y, xx), pk_dup(3.f * f3) * dxy, (pk_dup(-6.f * f3) * x) * y, no, 3);
     }
 }
 
+// Two points' place in an atom's shells
+struct AdjPair {
+    float d[2];
+    bool live[2];
+    pk x, y, z, n[3], inv;
+    pk t;                                            // on the species' knots: fraction of the interval
+    const float4 *c[2];                              // and the interval's splines
+};
+
+// the run of shells of one l that starts at sh (SHARED: all on the species' knots
+// and with its cutoff): sums over their functions of E_i grad phi_i
+template <int L, bool SHARED>
+__device__ __forceinline__ void adj_run(const AdjAtom &A, const AdjShell *sh_tab, const DevPlan &P, const AdjPair &q,
+                                        int &sh, const float *&Erow, long long Pa, pk *gr)
+{
+    constexpr int NM = 2 * L + 1;
+    pk ipl = q.inv;                                     // 1/d^(l+1)
+#pragma unroll
+    for (int i = 0; i < L; i++) ipl = ipl * q.inv;
+    AdjShell R;
+    if (!SHARED) R = sh_tab ? sh_tab[A.shell0 + sh] : adj_shell_entry(P, A.shell0 + sh);
+    do {
+        pk t = q.t, ih = pk_dup(A.inv_h);
+        const float4 *c0 = q.c[0] + 2 * sh, *c1 = q.c[1] + 2 * sh;
+        bool in0 = true, in1 = true;
+        if (!SHARED) {
+            in0 = q.live[0] && q.d[0] < R.rcut_f;
+            in1 = q.live[1] && q.d[1] < R.rcut_f;
+            const float a0 = q.d[0] * R.inv_h, a1 = q.d[1] * R.inv_h;
+            const int k0 = in0 ? min((int)a0, R.nk - 2) : 0, k1 = in1 ? min((int)a1, R.nk - 2) : 0;
+            t = pk_make(__fsub_rn(a0, (float)k0), __fsub_rn(a1, (float)k1));
+            ih = pk_dup(R.inv_h);
+            c0 = P.coef_dd + 2 * ((long long)R.coef_off + k0);
+            c1 = P.coef_dd + 2 * ((long long)R.coef_off + k1);
+        }
+        const float4 a = __ldg(c0), b = __ldg(c1);
+        pk e[NM];
+#pragma unroll
+        for (int m = 0; m < NM; m++) {
+            const float2 v = __ldg(reinterpret_cast<const float2 *>(Erow + m * Pa));
+            e[m] = pk_make(v.x, v.y);
+        }
+        Erow += NM * Pa;
+        const pk w = pk_make(a.w, b.w), zc = pk_make(a.z, b.z), yc = pk_make(a.y, b.y);
+        const pk u = fma2(t, fma2(t, fma2(t, w, zc), yc), pk_make(a.x, b.x));
+        const pk dq = fma2(t, fma2(pk_dup(2.f), zc, (pk_dup(3.f) * t) * w), yc);
+        pk g = u * ipl, gp = fma2(pk_dup(-(float)(L + 1)) * u, q.inv, dq * ih) * ipl;
+        if (!SHARED) {
+            const float2 gv = pk_get(g), pv = pk_get(gp);
+            g = pk_make(in0 ? gv.x : 0.f, in1 ? gv.y : 0.f);
+            gp = pk_make(in0 ? pv.x : 0.f, in1 ? pv.y : 0.f);
+        }
+        adj_angular<L>(q.x, q.y, q.z, [&](int m, pk Ym, const pk *Gm, int mask) {
+            const pk am = gp * Ym;
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                const pk v = (mask >> c & 1) ? fma2(am, q.n[c], g * Gm[c]) : am * q.n[c];
+                gr[c] = fma2(e[m], v, gr[c]);
+            }
+        });
+        sh++;
+        if (sh == A.n_shell) break;
+        R = sh_tab ? sh_tab[A.shell0 + sh] : adj_shell_entry(P, A.shell0 + sh);
+    } while (R.l == L);
+}
+
+template <bool SHARED>
+__device__ __forceinline__ void adj_atom(const AdjAtom &A, const AdjShell *sh_tab, const DevPlan &P, const AdjPair &q,
+                                         const float *Erow, long long Pa, pk *gr)
+{
+    for (int sh = 0; sh < A.n_shell;) {
+        switch ((sh_tab ? sh_tab[A.shell0 + sh] : adj_shell_entry(P, A.shell0 + sh)).l) {
+        case 0: adj_run<0, SHARED>(A, sh_tab, P, q, sh, Erow, Pa, gr); break;
+        case 1: adj_run<1, SHARED>(A, sh_tab, P, q, sh, Erow, Pa, gr); break;
+        case 2: adj_run<2, SHARED>(A, sh_tab, P, q, sh, Erow, Pa, gr); break;
+        default: adj_run<3, SHARED>(A, sh_tab, P, q, sh, Erow, Pa, gr); break;
+        }
+    }
+}
+
+// distance (x^2 and y^2 are shared with the polynomials and rounded before the sum)
+__device__ __forceinline__ float adj_dist(const float3 &o)
+{
+    return sqrtf(fmaf(o.z, o.z, __fadd_rn(__fmul_rn(o.x, o.x), __fmul_rn(o.y, o.y))));
+}
+
 // Position gradient of the adjoint on CUDA cores (FP32): CTA per (batch,
-// 64-point chunk); warp tasks (active atom, 32-point half), lane = point.
-// The lane forms sum_{i on the atom} grad phi_i(p) . E_i(p) from the E rows
-// the contraction stored, times -2 w_p v_p; the warp sums its 32 points and
-// adds the atom's three components to dR (FP64 atomics).
+// 64-point chunk), a warp an active atom, two neighbouring points a lane in
+// packed pairs.  The lane forms sum_{i on the atom} grad phi_i(p) . E_i(p) from
+// the E rows the contraction stored, times -2 w_p v_p; the warp sums each half
+// of its 64 points and adds the atom's three components to dR (FP64 atomics).
 //   grad phi = g'(d) (r/d) P(r) + g(d) grad P(r),  g = u/d^(l+1),
 //   g' = u'/d^(l+1) - (l+1) u/d^(l+2),  P = r^l Y_lm (a polynomial in x, y, z)
-__global__ void __launch_bounds__(256) k_tc_adj_grad(DevPlan P, const TcBatch *tb, const WorkItem *items,
+// The rows of E are read once, in 256-byte pieces.  What bounds it is the
+// latency of those loads: a point a lane, with the species' and shells' tables
+// found through a chain of dependent look-ups a shell, took 3.1 ms where the
+// atoms and shells staged in shared memory and two points a lane take 1.26
+// (64-atom Si cluster, 1.11 M points; 3.1 GB of E, 0.45 ms at the measured
+// copy rate); 0.38 -> 0.17 ms for a molecule of 30 atoms.  Four CTAs an SM: two
+// and three are slower (1.9, 1.6 ms), six spill.
+__global__ void __launch_bounds__(256, 4) k_tc_adj_grad(DevPlan P, const TcBatch *tb, const WorkItem *items,
                                                      const uint8_t *ws, const double *v, double *dR)
 {
+    __shared__ AdjAtom at[kAdjAtoms];
+    __shared__ AdjShell shs[kMaxShellsSmem];
     const WorkItem it = items[blockIdx.x];
     const DevBatch B = P.batches[it.batch];
     const TcBatch T = tb[it.batch];
-    const int c = it.ti;
     const DevAct *act = P.act + B.act0;
     const float *E = reinterpret_cast<const float *>(ws + T.img_e);
     const long long Pa = (long long)T.nc_alloc * 64;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-    for (int task = warp; task < B.n_act * 2; task += nwarp) {
-        const DevAct A = act[task >> 1];
-        const int p = c * 64 + (task & 1) * 32 + lane;
-        float gx = 0.f, gy = 0.f, gz = 0.f;
-        if (p < B.np) {
-            const DevSpecies S = P.species[P.atom_species[A.atom]];
-            const float *pp = P.pts_dd + 6 * (B.pt0 + p);
-            const float *aa = P.atom_dd + 6 * A.atom;
-            const float x = (pp[0] - aa[0]) + (pp[1] - aa[1]);
-            const float y = (pp[2] - aa[2]) + (pp[3] - aa[3]);
-            const float z = (pp[4] - aa[4]) + (pp[5] - aa[5]);
-            const float d = sqrtf(x * x + y * y + z * z);
-            if (d > 1e-12f && d < (float)S.rcut * 1.00001f) {
-                const float inv = 1.f / d;
-                const float nx = x * inv, ny = y * inv, nz = z * inv;
-                int f = 0;
-                for (int sh = 0; sh < S.n_shell; sh++) {
-                    const DevRadial R = P.radials[P.shell_rad[S.shell0 + sh]];
-                    const int nm = 2 * R.l + 1;
-                    if (d >= R.rcut_f) {
-                        f += nm;
-                        continue;
-                    }
-                    const float s = d * R.inv_h_hi;
-                    const int k = min((int)s, R.nk - 2);
-                    const float t = s - (float)k;
-                    const float4 ch = __ldg(P.coef_dd + 2 * (R.coef_off + k));
-                    const float u = ch.x + t * (ch.y + t * (ch.z + t * ch.w));
-                    const float du = (ch.y + t * (2.f * ch.z + 3.f * t * ch.w)) * R.inv_h_hi;
-                    float ipl = inv;
-                    for (int q = 0; q < R.l; q++) ipl *= inv;          // 1/d^(l+1)
-                    const float g = u * ipl;
-                    const float gp = (du - (float)(R.l + 1) * u * inv) * ipl;
-                    const float *Erow = E + (long long)(A.fn_loc + f) * Pa + p;
-                    switch (R.l) {
-                    case 0: adj_shell<0>(g, gp, x, y, z, nx, ny, nz, Erow, Pa, gx, gy, gz); break;
-                    case 1: adj_shell<1>(g, gp, x, y, z, nx, ny, nz, Erow, Pa, gx, gy, gz); break;
-                    case 2: adj_shell<2>(g, gp, x, y, z, nx, ny, nz, Erow, Pa, gx, gy, gz); break;
-                    default: adj_shell<3>(g, gp, x, y, z, nx, ny, nz, Erow, Pa, gx, gy, gz); break;
-                    }
-                    f += nm;
-                }
-                const float pref = (float)(-2.0 * P.pw[B.pt0 + p] * v[B.pt0 + p]);
-                gx *= pref;
-                gy *= pref;
-                gz *= pref;
+    const AdjShell *sh_tab = P.n_shells <= kMaxShellsSmem ? shs : nullptr;
+    if (sh_tab)
+        for (int i = threadIdx.x; i < P.n_shells; i += blockDim.x) shs[i] = adj_shell_entry(P, i);
+    const int p = it.ti * 64 + 2 * lane;
+    const bool has0 = p < B.np, has1 = p + 1 < B.np;
+    const Dd3 q0 = load_dd3(P.pts_dd + 6 * (B.pt0 + (has0 ? p : 0)));
+    const Dd3 q1 = load_dd3(P.pts_dd + 6 * (B.pt0 + (has1 ? p + 1 : 0)));
+    const float w0 = has0 ? (float)(-2.0 * P.pw[B.pt0 + p] * v[B.pt0 + p]) : 0.f;
+    const float w1 = has1 ? (float)(-2.0 * P.pw[B.pt0 + p + 1] * v[B.pt0 + p + 1]) : 0.f;
+    for (int e0 = 0; e0 < B.n_act; e0 += kAdjAtoms) {
+        const int ne = min(kAdjAtoms, B.n_act - e0);
+        __syncthreads();
+        if (threadIdx.x < ne) {
+            const DevAct D = act[e0 + threadIdx.x];
+            const DevSpecies &S = P.species[P.atom_species[D.atom]];
+            at[threadIdx.x] = AdjAtom{load_dd3(P.atom_dd + 6 * D.atom), (float)S.rcut * 1.00001f, (float)S.rcut, S.inv_h_hi,
+                                      S.nk, S.shared_grid, S.shell0, S.n_shell, D.fn_loc, D.atom,
+                                      P.scoef + S.scoef_off};
+        }
+        __syncthreads();
+        for (int e = warp; e < ne; e += nwarp) {
+            const AdjAtom &A = at[e];
+            const float3 o0 = offset_f32(q0, A.pos), o1 = offset_f32(q1, A.pos);
+            AdjPair q;
+            q.d[0] = adj_dist(o0);
+            q.d[1] = adj_dist(o1);
+            q.live[0] = has0 && q.d[0] > 1e-12f && q.d[0] < A.rlim;
+            q.live[1] = has1 && q.d[1] > 1e-12f && q.d[1] < A.rlim;
+            if (!__any_sync(0xffffffffu, q.live[0] || q.live[1])) continue;
+            const float i0 = 1.f / q.d[0], i1 = 1.f / q.d[1];
+            q.x = pk_make(o0.x, o1.x);
+            q.y = pk_make(o0.y, o1.y);
+            q.z = pk_make(o0.z, o1.z);
+            q.inv = pk_make(i0, i1);
+            q.n[0] = q.x * q.inv;
+            q.n[1] = q.y * q.inv;
+            q.n[2] = q.z * q.inv;
+            const float *Erow = E + (long long)A.fn_loc * Pa + p;
+            pk gr[3] = {pk_dup(0.f), pk_dup(0.f), pk_dup(0.f)};
+            if (A.shared) {
+                q.live[0] = q.live[0] && q.d[0] < A.rcut_f;
+                q.live[1] = q.live[1] && q.d[1] < A.rcut_f;
+                const float a0 = q.d[0] * A.inv_h, a1 = q.d[1] * A.inv_h;
+                const int k0 = q.live[0] ? min((int)a0, A.nk - 2) : 0, k1 = q.live[1] ? min((int)a1, A.nk - 2) : 0;
+                q.t = pk_make(__fsub_rn(a0, (float)k0), __fsub_rn(a1, (float)k1));
+                q.c[0] = A.tab + 2ll * k0 * A.n_shell;
+                q.c[1] = A.tab + 2ll * k1 * A.n_shell;
+                adj_atom<true>(A, sh_tab, P, q, Erow, Pa, gr);
+            } else {
+                q.t = pk_dup(0.f);
+                q.c[0] = q.c[1] = P.coef_dd;
+                adj_atom<false>(A, sh_tab, P, q, Erow, Pa, gr);
             }
-        }
+            float s0[3], s1[3];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            gx += __shfl_xor_sync(0xffffffffu, gx, o);
-            gy += __shfl_xor_sync(0xffffffffu, gy, o);
-            gz += __shfl_xor_sync(0xffffffffu, gz, o);
-        }
-        if (lane == 0 && (gx != 0.f || gy != 0.f || gz != 0.f)) {
-            atomicAdd(dR + 3 * A.atom + 0, (double)gx);
-            atomicAdd(dR + 3 * A.atom + 1, (double)gy);
-            atomicAdd(dR + 3 * A.atom + 2, (double)gz);
+            for (int c = 0; c < 3; c++) {
+                const float2 r = pk_get(gr[c]);
+                s0[c] = q.live[0] ? r.x * w0 : 0.f;
+                s1[c] = q.live[1] ? r.y * w1 : 0.f;
+            }
+            // sums over 32 points each: lanes 0 .. 15 hold the first half's,
+            // 16 .. 31 the second's; the lanes' pairs are taken apart at the
+            // first step (bit 3: the first or the second of a pair)
+            const bool up = lane & 8;
+            float r[3];
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                const float mine = up ? s1[c] : s0[c];
+                r[c] = mine + __shfl_xor_sync(0xffffffffu, up ? s0[c] : s1[c], 8);
+            }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+                for (int c = 0; c < 3; c++) r[c] += __shfl_xor_sync(0xffffffffu, r[c], o);
+#pragma unroll
+            for (int c = 0; c < 3; c++) r[c] += __shfl_xor_sync(0xffffffffu, r[c], 8);
+            const int c = lane & 15;
+            if (c < 3 && (r[0] != 0.f || r[1] != 0.f || r[2] != 0.f))
+                atomicAdd(dR + 3 * A.atom + c, (double)(c == 0 ? r[0] : c == 1 ? r[1] : r[2]));
         }
     }
 }

@@ -90,3 +90,27 @@ def test_column_bounds_of_many_atoms(tmp_path):
     (a, n0), (b, n1) = out
     assert np.array_equal(a, b) and a.max() > 4 * 128
     assert np.abs(n0).max() > 0 and np.array_equal(n0, n1)
+
+
+@pytest.mark.parametrize("points", [0, 512])
+def test_position_gradient_paths(molecule, points, tmp_path):
+    """The adjoint's position gradient on shared knots and shell by shell: the
+    same FP32 operations, summed into dR by FP64 atomics in no fixed order
+    (below 10^5 terms of 2^-53 each, against the largest component)."""
+    import paper_2208_12335_gb300 as fgi
+    tune = tmp_path / "tune.txt"
+    tune.write_text("h_sb_points %d\ndensity_sb_points %d\n" % (points, points))
+    padded = list(molecule.radials)
+    for i in (8, 12):
+        r = padded[i]
+        padded[i] = W.Radial(r.l, r.h, np.concatenate([r.coef, np.zeros((1, 4))]), r.spec, r.norm)
+    out = []
+    for radials in (molecule.radials, padded):
+        ctx = fgi.Context(0).load(dataclasses.replace(molecule, radials=radials), "split_bf16", tune_path=str(tune))
+        g = torch.from_numpy(np.random.default_rng(7).standard_normal(ctx.sizes()[1])).cuda()
+        dv, dR = ctx.adjoint(g, torch.from_numpy(molecule.v).cuda())
+        ctx.sync()
+        out.append((dv.cpu().numpy(), dR.cpu().numpy()))
+    (v0, r0), (v1, r1) = out
+    assert np.abs(v0).max() > 0 and np.array_equal(v0, v1)
+    assert np.abs(r0).max() > 0 and np.abs(r0 - r1).max() <= 1e5 * 2.0 ** -53 * np.abs(r0).max()
