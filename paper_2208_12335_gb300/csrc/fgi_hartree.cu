@@ -252,103 +252,113 @@ __device__ __forceinline__ double warp_scan_down(double v, int lane)     // incl
     return v;
 }
 
-// The radial equation of atom a for one l by one warp, lanes along the shells:
-// the partial integrals as warp scans, the 2l+1 functions side by side.
-template <int l>
-__device__ void radial_l(const DevPlan &P, const HartreeRad &g, int a, long long o, const HartreeTabs &T)
+constexpr int kRadShells = 256;         // shells the radial equation keeps in shared memory
+constexpr int kRadWarps = 4;            // warps a CTA
+
+// The radial equation of atom a for one (l, m) by one warp, lanes along the
+// shells: the partial integrals as warp scans.  F and V: n doubles each of
+// the warp's own, `st` apart (shared memory, or the global scratch of an atom
+// with more shells than that).
+template <int l, class Radius>
+__device__ void radial_lm(const DevPlan &P, const HartreeRad &g, int a, int mi, long long o, const HartreeTabs &T,
+                          const Radius &rk, double *F, double *V, int st)
 {
-    constexpr int NM = 2 * l + 1;
     const int lane = threadIdx.x & 31, n = g.nrad;
-    const double h = g.lnq, h24 = h / 24.0;
-    auto rk = [&](int k) { return g.r0 * exp(h * (double)k); };
-    // the integrands per dx = dr / r: f = rho r^(l+3) (inner), g = rho r^(2-l) (outer, over rho)
-    double *rho = T.rho + o * kL + l * l, *F = T.F + o * kL + l * l, *Vd = T.Vd + o * kL + l * l;
-    for (int k = lane; k < n; k += 32) {
-        const double r = rk(k), rf = ipow(r, l + 3), rg = l <= 2 ? ipow(r, 2 - l) : 1.0 / ipow(r, l - 2);
-#pragma unroll
-        for (int m = 0; m < NM; m++) {
-            const double rr = rho[k * kL + m];
-            F[k * kL + m] = rr * rf;
-            rho[k * kL + m] = rr * rg;
-        }
-    }
+    const double h24 = g.lnq / 24.0;
+    const double *rho = T.rho + o * kL + l * l + mi;
+    // the integrands per dx = dr / r: f = rho r^(l+3) (inner), g = rho r^(2-l) (outer, over f)
+    for (int k = lane; k < n; k += 32) F[k * st] = rho[k * kL] * ipow(rk(k), l + 3);
     __syncwarp();
     // integral over interval [k, k+1] of the cubic through the nearest four samples (n >= 4)
-    auto seg = [&](const double *fn, int k) {
-        auto v = [&](int j) { return fn[j * kL]; };
+    auto seg = [&](int k) {
+        auto v = [&](int j) { return F[j * st]; };
         if (k == 0) return h24 * (9.0 * v(0) + 19.0 * v(1) - 5.0 * v(2) + v(3));
         if (k == n - 2) return h24 * (v(n - 4) - 5.0 * v(n - 3) + 19.0 * v(n - 2) + 9.0 * v(n - 1));
         return h24 * (13.0 * (v(k) + v(k + 1)) - (v(k - 1) + v(k + 2)));
     };
     // 4 pi/(2l+1), times K_lm^2 for the two unnormalised harmonics (moment, evaluation)
-    double pref[NM], carry[NM];
+    double pref = 0.0;
 #pragma unroll
-    for (int m = 0; m < NM; m++) {
-        pref[m] = 4.0 * 3.14159265358979323846 / (2.0 * l + 1.0) * ylm_norm2(l, m - l);
-        carry[m] = F[m] / (double)(l + 3);
-    }
-    // inner integrals, forward: the inner part of V in FP64 scratch
+    for (int m = 0; m < 2 * l + 1; m++)
+        if (m == mi) pref = 4.0 * 3.14159265358979323846 / (2.0 * l + 1.0) * ylm_norm2(l, m - l);
+    double carry = F[0] / (double)(l + 3);
+    // inner integrals, forward: the inner part of V
     for (int k0 = 0; k0 < n; k0 += 32) {
         const int k = k0 + lane;
         const double ir = 1.0 / ipow(rk(min(k, n - 1)), l + 1);
-#pragma unroll
-        for (int m = 0; m < NM; m++) {
-            const double iin = carry[m] + warp_scan_up(k > 0 && k < n ? seg(F + m, k - 1) : 0.0, lane);
-            if (k < n) Vd[k * kL + m] = pref[m] * iin * ir;
-            carry[m] = __shfl_sync(0xffffffffu, iin, 31);
-        }
+        const double iin = carry + warp_scan_up(k > 0 && k < n ? seg(k - 1) : 0.0, lane);
+        if (k < n) V[k * st] = pref * iin * ir;
+        carry = __shfl_sync(0xffffffffu, iin, 31);
     }
     if (lane == 0) {
         if (l == 0) {
             const float *aa = P.atom_dd + 6 * a;
-            const df q = df_from_double(pref[0] * carry[0]);
+            const df q = df_from_double(pref * carry);
             T.rec[3 * a] = make_float4(aa[0], aa[1], aa[2], aa[3]);
             T.rec[3 * a + 1] = make_float4(aa[4], aa[5], g.rmax2_hi, g.rmax2_lo);
             T.rec[3 * a + 2] = make_float4(q.hi, q.lo, 0.f, 0.f);
         } else {
-#pragma unroll
-            for (int m = 0; m < NM; m++) T.Qf[(long long)a * kLf + l * l + m - 1] = (float)(pref[m] * carry[m]);
+            T.Qf[(long long)a * kLf + l * l + mi - 1] = (float)(pref * carry);
         }
     }
+    __syncwarp();
+    for (int k = lane; k < n; k += 32) {
+        const double r = rk(k), rg = l <= 2 ? ipow(r, 2 - l) : 1.0 / ipow(r, l - 2);
+        F[k * st] = rho[k * kL] * rg;
+    }
+    __syncwarp();
     // outer integrals, backward; V = inner + outer part, stored once
-#pragma unroll
-    for (int m = 0; m < NM; m++) carry[m] = 0.0;
+    carry = 0.0;
     for (int k0 = (n - 1) / 32 * 32; k0 >= 0; k0 -= 32) {
         const int k = k0 + lane;
         const double rl = ipow(rk(min(k, n - 1)), l);
-#pragma unroll
-        for (int m = 0; m < NM; m++) {
-            const double iout = carry[m] + warp_scan_down(k < n - 1 ? seg(rho + m, k) : 0.0, lane);
-            if (k < n) {
-                const double v = Vd[k * kL + m] + pref[m] * iout * rl;
-                if (l == 0) T.V0[o + k] = v;
-                else T.Vf[(o + k) * kLf + l * l + m - 1] = (float)v;
-            }
-            carry[m] = __shfl_sync(0xffffffffu, iout, 0);
+        const double iout = carry + warp_scan_down(k < n - 1 ? seg(k) : 0.0, lane);
+        if (k < n) {
+            const double v = V[k * st] + pref * iout * rl;
+            if (l == 0) T.V0[o + k] = v;
+            else T.Vf[(o + k) * kLf + l * l + mi - 1] = (float)v;
         }
+        carry = __shfl_sync(0xffffffffu, iout, 0);
     }
 }
 
-// One warp per (atom, l); the warp with l = 0 also packs the atom's records for
-// the evaluation.  (One thread per (atom, l, m) along the shells was a serial
-// chain: 0.44 ms on 64 atoms of 60 shells; now 0.08 ms.)
-__global__ void __launch_bounds__(128) k_hartree_radial(DevPlan P, HartreeDev H, int l_max, HartreeTabs T)
+// One warp per (atom, l, m), the warps of a CTA on one atom; the warp with
+// l = 0 also packs the atom's records for the evaluation.
+//
+// Bound by latency and by the FP64 unit (two lanes a clock and SM): an
+// exponential a shell, once a CTA, and chains of FP64 sums.  A warp per
+// (atom, l) with its 2l+1 functions side by side in global scratch kept a few
+// SMs busy and the others idle: 67 -> 19 us for 3 atoms, l_max 4; 79 -> 24
+// for 64 atoms; 300 -> 184 for 250 atoms, l_max 6.  One warp a CTA gives the
+// same for the small systems and 244 us for 250 atoms.
+__global__ void __launch_bounds__(32 * kRadWarps) k_hartree_radial(DevPlan P, HartreeDev H, int l_max, HartreeTabs T)
 {
-    const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+    __shared__ double rs[kRadShells], sF[kRadWarps][kRadShells], sV[kRadWarps][kRadShells];
+    const int nlm = (l_max + 1) * (l_max + 1), per = (nlm + kRadWarps - 1) / kRadWarps;
+    const int a = blockIdx.x / per, warp = threadIdx.x >> 5, lm = (blockIdx.x - a * per) * kRadWarps + warp;
     const int lane = threadIdx.x & 31;
-    if (w >= (long long)H.n_atoms * (l_max + 1)) return;
-    const int a = (int)(w / (l_max + 1)), l = (int)(w % (l_max + 1));
     const HartreeRad g = H.rad[a];
     const int n = g.nrad;
     const long long o = H.rad_off[a];
+    const bool smem = n <= kRadShells;
+    if (smem)
+        for (int k = threadIdx.x; k < n; k += blockDim.x) rs[k] = g.r0 * exp(g.lnq * (double)k);
+    __syncthreads();
+    if (lm >= nlm) return;
+    int l = 0;
+    while ((l + 1) * (l + 1) <= lm) l++;
+    const int m = lm - l * l;
+    auto rk = [&](int k) { return smem ? rs[k] : g.r0 * exp(g.lnq * (double)k); };
+    double *F = smem ? sF[warp] : T.F + o * kL + lm, *V = smem ? sV[warp] : T.Vd + o * kL + lm;
+    const int st = smem ? 1 : kL;
     switch (l) {
-    case 0: radial_l<0>(P, g, a, o, T); break;
-    case 1: radial_l<1>(P, g, a, o, T); return;
-    case 2: radial_l<2>(P, g, a, o, T); return;
-    case 3: radial_l<3>(P, g, a, o, T); return;
-    case 4: radial_l<4>(P, g, a, o, T); return;
-    case 5: radial_l<5>(P, g, a, o, T); return;
-    default: radial_l<6>(P, g, a, o, T); return;
+    case 0: radial_lm<0>(P, g, a, m, o, T, rk, F, V, st); break;
+    case 1: radial_lm<1>(P, g, a, m, o, T, rk, F, V, st); return;
+    case 2: radial_lm<2>(P, g, a, m, o, T, rk, F, V, st); return;
+    case 3: radial_lm<3>(P, g, a, m, o, T, rk, F, V, st); return;
+    case 4: radial_lm<4>(P, g, a, m, o, T, rk, F, V, st); return;
+    case 5: radial_lm<5>(P, g, a, m, o, T, rk, F, V, st); return;
+    default: radial_lm<6>(P, g, a, m, o, T, rk, F, V, st); return;
     }
     __syncwarp();
     // the shells' radii, and V_00 on each interval k as the cubic through
@@ -356,7 +366,7 @@ __global__ void __launch_bounds__(128) k_hartree_radial(DevPlan P, HartreeDev H,
     // x = ln(r / r_0) / ln q: a_m = p^(m)(o) / m! with o = k - i0 and
     // p(t) = V_i0 + t D1 + t(t-1)/2 D2 + t(t-1)(t-2)/6 D3 (forward differences)
     for (int k = lane; k < n; k += 32) {
-        const double r = g.r0 * exp(g.lnq * (double)k);
+        const double r = rk(k);
         const df rh = df_from_double(r), ri = df_from_double(1.0 / r);
         T.rk[o + k] = make_float4(rh.hi, rh.lo, ri.hi, ri.lo);
     }
@@ -649,9 +659,9 @@ cudaError_t launch_hartree(const DevPlan &P, const HartreeDev &H, int n_batch, l
         }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    const long long nw = (long long)H.n_atoms * (l_max + 1);
-    if (nw > 0) {
-        k_hartree_radial<<<(unsigned)((nw + 3) / 4), 128, 0, s>>>(P, H, l_max, T);
+    if (H.n_atoms > 0) {
+        const int nlm = (l_max + 1) * (l_max + 1), per = (nlm + kRadWarps - 1) / kRadWarps;
+        k_hartree_radial<<<(unsigned)(H.n_atoms * per), 32 * kRadWarps, 0, s>>>(P, H, l_max, T);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (n_batch > 0) {

@@ -25,3 +25,15 @@ def test_hartree_shells(n_rad, n_ang, l_max):
     vh = ctx.hartree(torch.from_numpy(n).cuda(), l_max=l_max).cpu().numpy()
     ctx.sync()
     assert np.all(np.abs(vh - ref) <= 1e-10 * np.abs(ref).max() + 2.0 ** -18 * bound)
+
+
+def test_more_shells_than_shared_memory_holds():
+    """Beyond 256 shells the radial equation works in global scratch."""
+    import paper_2208_12335_gb300 as fgi
+    prob = W.tiny_water(n_rad=300, n_ang=6)
+    n = np.random.default_rng(2).standard_normal(prob.n_pts) * np.exp(-0.3 * np.linalg.norm(prob.pts, axis=1))
+    ref, bound = OH.hartree(prob, n, l_max=3, l1_bound=True)
+    ctx = fgi.Context(0).load(prob, "fp64")
+    vh = ctx.hartree(torch.from_numpy(n).cuda(), l_max=3).cpu().numpy()
+    ctx.sync()
+    assert np.all(np.abs(vh - ref) <= 1e-10 * np.abs(ref).max() + 2.0 ** -18 * bound)
