@@ -890,8 +890,8 @@ __device__ __forceinline__ void h_image_lanes(const DevPlan &P, const DevBatch &
 // small warps in flight, the evaluation few with many registers, and a
 // super-batch's atoms and points are looked at once instead of once a row
 // block.  H images with it and two points a lane: 64-atom Si cluster, 1.11 M
-// points, 2.73 -> 2.06 ms (0.46 of it here), 75-atom cluster with f shells,
-// two images a batch, 3.80 -> 3.08 ms (0.73 here).
+// points, 2.73 -> 1.85 ms (0.25 of it here), 75-atom cluster with f shells,
+// two images a batch, 3.80 -> 2.9 ms (0.49 here).
 constexpr int kPhiThreads = 256;
 
 // Knot interval of distance d from below (against FP32 rounding of d) for the
@@ -932,13 +932,51 @@ __device__ __forceinline__ void put_shell_grid(const DevPlan &P, HGrid *grids, i
     put_grid(grids, set, f0 + lane, m > 0.f ? fminf(m * yl, 1.0e30f) : 0.f, fminf(s * 1.0001f * yl, 1.0e30f), depth);
 }
 
+// Sum over the warp of twelve values at once: lane L receives the sum of value
+// L / 2 (zero beyond).  Each step adds across one lane bit and hands half of the
+// values to the other lane: 16 shuffles where twelve sums take 60, every sum in
+// the order of warp_sum.
+__device__ __forceinline__ float warp_sums12(const float *v, int lane)
+{
+    float a[8], b[4], c[2];
+    const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4, h1 = lane & 2;
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+        const float lo = v[j], hi = j < 4 ? v[8 + j] : 0.f;
+        a[j] = (h4 ? hi : lo) + __shfl_xor_sync(0xffffffffu, h4 ? lo : hi, 16);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; j++)
+        b[j] = (h3 ? a[4 + j] : a[j]) + __shfl_xor_sync(0xffffffffu, h3 ? a[j] : a[4 + j], 8);
+#pragma unroll
+    for (int j = 0; j < 2; j++)
+        c[j] = (h2 ? b[2 + j] : b[j]) + __shfl_xor_sync(0xffffffffu, h2 ? b[j] : b[2 + j], 4);
+    float d = (h1 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, h1 ? c[0] : c[1], 2);
+    return d + __shfl_xor_sync(0xffffffffu, d, 1);
+}
+
+// The maxima of twelve values (>= 0) in the same places
+__device__ __forceinline__ float warp_maxs12(const float *v, int lane)
+{
+    float r = 0.f;
+#pragma unroll
+    for (int j = 0; j < 12; j++) {
+        const float m = warp_max(v[j]);
+        if (lane >> 1 == j) r = m;
+    }
+    return r;
+}
+
 // Grids of one atom's functions by a warp from the interleaved table bounds: per
 // point one look-up of the suffix bounds of |u(r)/r| serves four shells, times
 // sqrt|w v| (psi) or |w v| (w v phi) of the point; the maximum over the points
 // times max |Y_lm| bounds each row, and the same products summed over the
 // points bound the row sums, so that rows whose sum allows it keep an 8-bit
 // digit.  MIXED: also |phi| itself (set 0), which only batches with both signs
-// use.
+// use.  The grids themselves are found a function a lane: a shell at a time
+// (2l+1 lanes of 32, after its own reductions) that part took as long as the
+// points: the preparation 0.46 -> 0.25 ms for the 64-atom Si cluster, 0.67 ->
+// 0.49 for the 75-atom cluster, 1.34 -> 1.17 for 64 molecules.
 template <bool MIXED>
 __device__ __forceinline__ void atom_grids(const DevPlan &P, const DevBatch &B, const DevAct &A, const DevSpecies &S,
                                            const DevShell *sh_tab, const Dd3 *pts, const float *wvf, HGrid *grids,
@@ -976,16 +1014,39 @@ __device__ __forceinline__ void atom_grids(const DevPlan &P, const DevBatch &B, 
                 }
             }
         }
-#pragma unroll
-        for (int j = 0; j < 12; j++) {
-            const int sh = 4 * q0 + j;
-            if (sh >= S.n_shell) break;
-            const int l = sh_tab[S.shell0 + sh].l, f0 = A.fn_loc + sh_tab[S.shell0 + sh].fn0;
-            const float a1 = warp_max(m1[j]), b1 = warp_sum(s1[j]);
-            put_shell_grid(P, grids, 1, l, f0, a1, b1, depth, lane);
+        __syncwarp();
+        // lane 2 j: shell j of the pass
+        const float a1 = warp_maxs12(m1, lane), b1 = warp_sums12(s1, lane);
+        float a0 = 0.f, b0 = 0.f;
+        if (MIXED) {
+            a0 = warp_maxs12(m0, lane);
+            b0 = warp_sums12(s0, lane);
+        }
+        // function i in the order of the shell table (by l): its shell and m
+        for (int i0 = 0; i0 < S.n_fn; i0 += 32) {
+            int i = i0 + lane, sh = 0, l = 0;
+            for (; l < kMaxL; l++) {
+                const int nf = S.nl[l] * (2 * l + 1);
+                if (i < nf) break;
+                i -= nf;
+                sh += S.nl[l];
+            }
+            const int q = i / (2 * l + 1), m = i - q * (2 * l + 1), j = sh + q - 4 * q0;
+            const bool mine = i0 + lane < S.n_fn && j >= 0 && j < 12;
+            const int src = 2 * max(0, min(j, 11));
+            const float mx1 = __shfl_sync(0xffffffffu, a1, src), sm1 = __shfl_sync(0xffffffffu, b1, src);
+            float mx0 = 0.f, sm0 = 0.f;
             if (MIXED) {
-                const float a0 = warp_max(m0[j]), b0 = warp_sum(s0[j]);
-                put_shell_grid(P, grids, 0, l, f0, a0, b0, depth, lane);
+                mx0 = __shfl_sync(0xffffffffu, a0, src);
+                sm0 = __shfl_sync(0xffffffffu, b0, src);
+            }
+            if (mine) {
+                const int f = A.fn_loc + sh_tab[S.shell0 + sh + q].fn0 + m;
+                const float yl = __ldg(P.rbound + l * l + m);
+                put_grid(grids, 1, f, mx1 > 0.f ? fminf(mx1 * yl, 1.0e30f) : 0.f, fminf(sm1 * 1.0001f * yl, 1.0e30f), depth);
+                if (MIXED)
+                    put_grid(grids, 0, f, mx0 > 0.f ? fminf(mx0 * yl, 1.0e30f) : 0.f, fminf(sm0 * 1.0001f * yl, 1.0e30f),
+                             depth);
             }
         }
     }
