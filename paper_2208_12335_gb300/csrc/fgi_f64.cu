@@ -17,7 +17,7 @@ namespace {
 // cutoff.  Bound by the FP64 pipe (1/64 of the FP32 rate): the shells are
 // walked grouped by l, so the harmonics of an l are formed once an atom and
 // point, and 1/d is a multiplication a shell.  (A division and harmonics a
-// shell: 20-atom molecule, two calls on 101 k points, 1.49 ms.)
+// shell: 20-atom molecule, two calls on 101 k points, 1.49 ms; 0.87 so.)
 template <int L>
 __device__ __forceinline__ void phi_shells_f64(const DevPlan &P, const DevSpecies &S, int &sh, double d, double inv,
                                                double nx, double ny, double nz, double *col, int kpad)
@@ -45,12 +45,14 @@ __device__ __forceinline__ void phi_shells_f64(const DevPlan &P, const DevSpecie
     }
 }
 
+// gridDim.y CTAs a batch: one a batch left the SMs unevenly loaded (two calls,
+// 512 batches: 0.87 ms; 0.70 with eight)
 __global__ void k_phi_f64(DevPlan P, int b0, double *ws)
 {
     const DevBatch B = P.batches[b0 + blockIdx.x];
     double *out = ws + B.ws_off;
     const int total = B.n_act * B.kpad;
-    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+    for (int idx = blockIdx.y * blockDim.x + threadIdx.x; idx < total; idx += gridDim.y * blockDim.x) {
         const int e = idx / B.kpad;
         const int p = idx - e * B.kpad;
         const DevAct A = P.act[B.act0 + e];
@@ -83,9 +85,12 @@ __global__ void k_phi_f64(DevPlan P, int b0, double *ws)
 // ------------------------------------------------------- H contraction (FP64)
 // One 64x64 tile (ti <= tj) of h_b = Phi_b diag(w v) Phi_b^T, then FP64
 // atomic scatter of the upper triangle into the stored values.  Bound by the
-// FP64 pipe, a warp's instruction at a time: on a diagonal tile the 136 4x4
-// blocks that meet the upper triangle are dealt to consecutive threads, five
-// warps instead of eight, and warps whose rows lie past n_b do nothing.
+// FP64 pipe (94 % busy), a warp's instruction at a time: the 4x4 blocks that the
+// tile has (up to n_b, and on a diagonal tile those that meet the upper
+// triangle) are dealt to consecutive threads, so that no more warps work
+// than they fill, and the points end at the batch's.
+// 20-atom molecule, 101 k points: 4.35 ms with 64x64 tiles whose rows alone were
+// trimmed, 3.25 now.
 constexpr int TF = 64;     // tile edge
 constexpr int TK = 16;     // points per step
 
@@ -97,15 +102,19 @@ __global__ void __launch_bounds__(256) k_h_f64(DevPlan P, const WorkItem *items,
     const double *phi = ws + B.ws_off;
     const int t = threadIdx.x;
     const int i0 = it.ti * TF, j0 = it.tj * TF;
-    int tx = t & 15, ty = t >> 4;
-    bool mine = i0 + ty * 4 < B.nfn;
+    const int rows = (min(TF, B.nfn - i0) + 3) >> 2, cols = (min(TF, B.nfn - j0) + 3) >> 2;
+    int tx, ty;
+    bool mine;
     if (it.ti == it.tj) {
         // block number t of the triangle tx >= ty, row by row
-        mine = t < 136;
-        int rest = min(t, 135);
-        for (ty = 0; rest >= 16 - ty; ty++) rest -= 16 - ty;
+        mine = t < rows * (rows + 1) / 2;
+        int rest = mine ? t : 0;
+        for (ty = 0; rest >= rows - ty; ty++) rest -= rows - ty;
         tx = ty + rest;
-        mine = mine && i0 + ty * 4 < B.nfn;
+    } else {
+        mine = t < rows * cols;
+        ty = mine ? t / cols : 0;
+        tx = mine ? t - ty * cols : 0;
     }
     __shared__ double As[TK][TF + 1];
     __shared__ double Bs[TK][TF + 1];
@@ -140,8 +149,10 @@ __global__ void __launch_bounds__(256) k_h_f64(DevPlan P, const WorkItem *items,
         }
         __syncthreads();
         if (mine) {
+            const int kn = B.np - k0;
 #pragma unroll
             for (int kk = 0; kk < TK; kk++) {
+                if (kk >= kn) break;
                 double a[4], b[4];
 #pragma unroll
                 for (int q = 0; q < 4; q++) { a[q] = As[kk][ty * 4 + q]; b[q] = Bs[kk][tx * 4 + q]; }
@@ -174,11 +185,15 @@ __global__ void __launch_bounds__(256) k_h_f64(DevPlan P, const WorkItem *items,
 // offdiag_scale: 1 for a matrix, 1/2 for a gradient with respect to stored
 // values).  FULL (the adjoint) writes E[j][p] = sum_i phi_i(p) D_ij;
 // otherwise the symmetry of D halves the FP64 work that bounds the kernel:
-// n = 2 sum_J phi_J . (sum_{K >= J} D'_JK phi_K) over 64-function blocks, D' = D
-// with its diagonal blocks halved (exact).  Warps past the batch's points skip
-// the products.
+// n = 2 sum_j phi_j (sum_{i >= j} D'_ij phi_i), D' = D with its diagonal halved
+// (exact).  The functions j come in blocks of equal width, at most 64; the 4x4
+// blocks of points and functions are dealt to consecutive threads, the points
+// fastest, so that warps skip the steps of the triangle that they do not need
+// and no more warps work than the batch's points and functions fill.
+// 20-atom molecule, 101 k points: 4.7 ms with whole 64x64 blocks and whole
+// diagonal blocks, 3.5 now (four CTAs an SM; two 3.7).
 template <bool FULL>
-__global__ void __launch_bounds__(256) k_density_f64(DevPlan P, const WorkItem *items,
+__global__ void __launch_bounds__(256, 4) k_density_f64(DevPlan P, const WorkItem *items,
                                                      const double *ws, const double *dval,
                                                      double offdiag_scale, double *n_out,
                                                      double *e_out)
@@ -186,20 +201,26 @@ __global__ void __launch_bounds__(256) k_density_f64(DevPlan P, const WorkItem *
     const WorkItem it = items[blockIdx.x];
     const DevBatch B = P.batches[it.batch];
     const double *phi = ws + B.ws_off;
-    const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+    const int t = threadIdx.x;
     const int p0 = it.ti * TF;
     extern __shared__ unsigned short fnact[];          // local function -> active entry
-    __shared__ double As[TK][TF + 1];                  // phi[i][p]
-    __shared__ double Bs[TK][TF + 1];                  // D[i][j]
+    __shared__ double stage[2][TK][TF + 1];
+    auto &As = stage[0], &Bs = stage[1];               // phi[i][p], D[i][j]
+    double (*red)[17] = reinterpret_cast<double (*)[17]>(&stage[0][0][0]);   // in their place at the end
+    static_assert(sizeof(stage) >= TF * 17 * sizeof(double), "the sums over functions");
     const DevAct *act = P.act + B.act0;
     for (int l = t; l < B.nfn; l += 256) fnact[l] = (unsigned short)find_act(act, B.n_act, l);
     __syncthreads();
 
+    const int nblk = (B.nfn + 3) >> 2, nj = (nblk + 15) >> 4;
+    const int cols = (nblk + nj - 1) / nj, width = 4 * cols;      // functions of a block
+    const int rows = (min(TF, B.np - p0) + 3) >> 2;
+    const bool mine = t < rows * cols;
+    const int tx = mine ? t / rows : 0, ty = mine ? t - tx * rows : 0;
     double part[4] = {0, 0, 0, 0};
-    for (int j0 = 0; j0 < B.nfn; j0 += TF) {
+    for (int j0 = 0; j0 < B.nfn; j0 += width) {
         double acc[4][4] = {};
         for (int k0 = FULL ? 0 : j0; k0 < B.nfn; k0 += TK) {
-            const double half = !FULL && k0 < j0 + TF ? 0.5 : 1.0;
 #pragma unroll
             for (int e = 0; e < 4; e++) {
                 const int idx = t + 256 * e;
@@ -208,19 +229,21 @@ __global__ void __launch_bounds__(256) k_density_f64(DevPlan P, const WorkItem *
                 As[kk][c] = (i < B.nfn && p0 + c < B.kpad) ? phi[(long long)i * B.kpad + p0 + c] : 0.0;
                 const int j = j0 + c;
                 double dv = 0.0;
-                if (i < B.nfn && j < B.nfn) {
+                if (c < width && i < B.nfn && j < B.nfn && (FULL || i >= j)) {
                     const int lo = i < j ? i : j, hi = i < j ? j : i;
                     const FnRef a = fn_ref(P, act, fnact[lo], lo);
                     const FnRef b = fn_ref(P, act, fnact[hi], hi);
                     const long long k = value_index(P, B.sys, a, b);
-                    if (k >= 0) dv = dval[k] * (lo == hi ? half : offdiag_scale * half);
+                    if (k >= 0) dv = dval[k] * (lo != hi ? offdiag_scale : FULL ? 1.0 : 0.5);
                 }
                 Bs[kk][c] = dv;
             }
             __syncthreads();
-            if (p0 + ty * 4 < B.np) {
+            if (mine && (FULL || k0 + TK > j0 + 4 * tx)) {
+                const int kn = B.nfn - k0;
 #pragma unroll
                 for (int kk = 0; kk < TK; kk++) {
+                    if (kk >= kn) break;
                     double a[4], b[4];
 #pragma unroll
                     for (int q = 0; q < 4; q++) { a[q] = As[kk][ty * 4 + q]; b[q] = Bs[kk][tx * 4 + q]; }
@@ -232,6 +255,7 @@ __global__ void __launch_bounds__(256) k_density_f64(DevPlan P, const WorkItem *
             }
             __syncthreads();
         }
+        if (!mine) continue;
 #pragma unroll
         for (int r = 0; r < 4; r++) {
             const int p = p0 + ty * 4 + r;
@@ -245,18 +269,15 @@ __global__ void __launch_bounds__(256) k_density_f64(DevPlan P, const WorkItem *
             }
         }
     }
+    if (mine) {
 #pragma unroll
-    for (int r = 0; r < 4; r++) {
-        double s = part[r];
-        for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        part[r] = s;
+        for (int r = 0; r < 4; r++) red[ty * 4 + r][tx] = part[r];
     }
-    if (tx == 0) {
-#pragma unroll
-        for (int r = 0; r < 4; r++) {
-            const int p = p0 + ty * 4 + r;
-            if (p < B.np) n_out[B.pt0 + p] = FULL ? part[r] : 2.0 * part[r];
-        }
+    __syncthreads();
+    if (t < TF && p0 + t < B.np) {
+        double s = 0.0;
+        for (int c = 0; c < cols; c++) s += red[t][c];
+        n_out[B.pt0 + p0 + t] = FULL ? s : 2.0 * s;
     }
 }
 
@@ -401,7 +422,7 @@ __global__ void k_check_finite(DevPlan P, const double *x, long long n)
 cudaError_t launch_phi_f64(const DevPlan &P, int b0, int nb, double *ws, cudaStream_t s)
 {
     if (nb <= 0) return cudaSuccess;
-    k_phi_f64<<<nb, 256, 0, s>>>(P, b0, ws);
+    k_phi_f64<<<dim3((unsigned)nb, 8), 256, 0, s>>>(P, b0, ws);
     return cudaGetLastError();
 }
 
