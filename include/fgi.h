@@ -222,8 +222,10 @@ int fgi_integrate_h(fgi_ctx *ctx, const double *v_dev, double *h_dev, int accumu
      onto the device and reserves the array there: the first call can then
      fail for lack of device memory (reported as FGI_ERR_CUDA), and only
      devices on which the call has run hold the array.
-   - A plan whose fgi_workspace_size() exceeds FGI_STATIC_SCRATCH_BYTES is
-     rejected with FGI_ERR_WORKSPACE and a message giving both sizes.
+   - A plan whose workspace exceeds FGI_STATIC_SCRATCH_BYTES is rejected with
+     FGI_ERR_WORKSPACE and a message giving both sizes (not counting the
+     descriptors of H's row blocks, at most 2.6 % of the workspace, for which
+     the array has room beyond that size).
    - All calls on a device share the one array, which keeps the last call's
      contents (what must start at zero is cleared on the device by each
      call); calls whose GPU work overlaps (other streams, other host
@@ -295,12 +297,14 @@ int fgi_hartree_workspace_size(fgi_ctx *ctx, size_t *bytes);
         interpolation in the fractional shell index, 4 pi/(2l+1) Q_lm /
         d^(l+1) beyond the last shell, V(r_0) (d/r_0)^l inside the first.
    n_dev, vh_dev: device [n_pts] FP64 in the caller's point order;
-   0 <= l_max <= 6 (FGI_ERR_UNSUPPORTED otherwise).  Moments and the radial
-   solve in FP64; the evaluation (every (point, atom) pair of a system) takes
+   0 <= l_max <= 6 (FGI_ERR_UNSUPPORTED otherwise).  The moments are
+   FP64 sums for l = 0 and double-float sums for l >= 1 (about 2^-45 of their
+   terms), the radial solve is FP64; the evaluation (every (point, atom) pair of a system) takes
    the l = 0 terms as double-floats (~1e-12 relative; FP64 interpolation for
    radial grids with ln q > 0.6) and the l >= 1 terms in FP32 (a few FP32
-   roundings of the l >= 1 part).  The moments are summed with FP64 atomics:
-   not bitwise reproducible.  Needs a plan and fgi_set_atom_grids;
+   roundings of the l >= 1 part).  The moments are summed in an order
+   fixed when the grids are set: calls of one context repeat bit by
+   bit, another context's may differ in the last bits.  Needs a plan and fgi_set_atom_grids;
    ws: device, 256-byte aligned, at least fgi_hartree_workspace_size bytes
    (FGI_ERR_WORKSPACE otherwise).  Enqueued on stream, no allocation, no host
    synchronisation (graph-capturable). */

@@ -8,10 +8,10 @@
 //     (listed once at set-up),
 //       rho~_a,lm(r_k) = sum_p (w_p / (r_k^3 ln q)) n_p A_lm(rhat_p)
 //     (w_p / (r_k^3 ln q) is the partitioned angular weight; A_lm = Y_lm / K_lm
-//     the unnormalised harmonics).  Harmonics and sums are double-float (about
-//     2^-45 relative), w_p n_p and the final scale FP64: GB300's FP64 pipe has
-//     1/64 of the FP32 rate.
-//  2. k_hartree_radial (FP64): a warp per (atom, l), lanes along the shells, the
+//     the unnormalised harmonics).  Harmonics and sums of l >= 1 are double-float
+//     (about 2^-45 relative), w_p n_p, the sum for l = 0 and the final scale FP64:
+//     GB300's FP64 pipe has 1/64 of the FP32 rate.
+//  2. k_hartree_radial (FP64): a warp per (atom, l, m), lanes along the shells, the
 //     radial Poisson equation
 //       V(r) = 4 pi/(2l+1) [r^-(l+1) int_0^r rho r'^(l+2) dr' + r^l int_r^inf rho r'^(1-l) dr']
 //     with the partial integrals in x = ln r interval by interval, each by the
@@ -159,7 +159,8 @@ __device__ __forceinline__ void warp_sum_split(df *v, int &off, int &lim)
 
 // One warp per (atom, shell).  (A thread per point with FP64 harmonics and
 // (l_max + 1)^2 FP64 atomics was bound by the FP64 pipe: 250-atom cluster, 7.3 M
-// points, l_max 6, 3.30 ms; now 0.51 ms.)
+// points, l_max 6, 3.30 ms; now 0.51 ms.)  The monopole's sum stays FP64: the
+// l = 0 terms are all there is at l_max 0, and the others end in FP32.
 template <int LMAX>
 __global__ void __launch_bounds__(128) k_hartree_moments(DevPlan P, HartreeDev H, const double *n, double *rho)
 {
@@ -171,6 +172,7 @@ __global__ void __launch_bounds__(128) k_hartree_moments(DevPlan P, HartreeDev H
     df acc[L];
 #pragma unroll
     for (int q = 0; q < L; q++) acc[q] = df{0.f, 0.f};
+    double mono = 0.0;
     int a = 0;
     if (i0 < i1) a = H.owner[H.order[i0]];
     const float *aa = P.atom_dd + 6 * a;
@@ -186,7 +188,9 @@ __global__ void __launch_bounds__(128) k_hartree_moments(DevPlan P, HartreeDev H
         x = df_mul(x, ir);
         y = df_mul(y, ir);
         z = df_mul(z, ir);
-        df cm = df_from_double(P.pw[p] * n[p]), sm{0.f, 0.f};      // w n Re, Im (x + i y)^m
+        const double wn = P.pw[p] * n[p];
+        mono += wn;
+        df cm = df_from_double(wn), sm{0.f, 0.f};                  // w n Re, Im (x + i y)^m
         float pmm = 1.f;
 #pragma unroll
         for (int m = 0; m <= LMAX; m++) {
@@ -214,13 +218,15 @@ __global__ void __launch_bounds__(128) k_hartree_moments(DevPlan P, HartreeDev H
                     p2 = p1;
                     p1 = pl;
                 }
-                df_fma_acc(acc[l * l + l + m], pl, cm);
+                if (l > 0) df_fma_acc(acc[l * l + l + m], pl, cm);
                 if (m > 0) df_fma_acc(acc[l * l + l - m], pl, sm);
             }
         }
     }
     int off = 0, lim = L;
     warp_sum_split<L, 16>(acc, off, lim);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mono += __shfl_xor_sync(0xffffffffu, mono, o);
     double scale = 0.0;
     if (i0 < i1) {
         const HartreeRad g = H.rad[a];
@@ -229,7 +235,8 @@ __global__ void __launch_bounds__(128) k_hartree_moments(DevPlan P, HartreeDev H
     }
 #pragma unroll
     for (int q = 0; q < (L + 31) / 32; q++)
-        if (off + q < lim) rho[bin * kL + off + q] = ((double)acc[q].hi + (double)acc[q].lo) * scale;
+        if (off + q < lim)
+            rho[bin * kL + off + q] = (off + q == 0 ? mono : (double)acc[q].hi + (double)acc[q].lo) * scale;
 }
 
 __device__ __forceinline__ double warp_scan_up(double v, int lane)       // inclusive, towards higher lanes
