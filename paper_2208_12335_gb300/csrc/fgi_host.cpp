@@ -957,6 +957,14 @@ void wave_work(fgi_ctx *c)
 // ========================================================= internal entry points
 namespace fgi {
 
+// what the static scratch is held against: the workspace without the H
+// descriptors, for which it keeps room of its own
+size_t internal_static_need(fgi_ctx *c)
+{
+    return std::max(std::max(c->ws_f64_bytes, tc_workspace_bytes(c->tca)),
+                    std::max(c->tc.ws_images, tc_workspace_bytes(c->tcd)));
+}
+
 int internal_device(const fgi_ctx *c) { return c ? c->device : -1; }
 
 int internal_error(fgi_ctx *c, int code, const char *msg)

@@ -155,6 +155,7 @@ struct fgi_ctx;
 namespace fgi {
 // host-side helpers shared between the runtime's translation units
 int internal_device(const fgi_ctx *c);
+size_t internal_static_need(fgi_ctx *c);
 int internal_error(fgi_ctx *c, int code, const char *msg);
 int internal_integrate_h(fgi_ctx *c, const double *v, double *h, int accumulate, void *ws, size_t ws_bytes,
                          void *stream, bool allow_profile);

@@ -18,7 +18,10 @@ namespace {
 
 // The scratch: every GPU that loads the library holds it until the process
 // exits.  All calls on a device share it and it keeps the last call's data.
-__device__ __align__(256) unsigned char g_static_scratch[FGI_STATIC_SCRATCH_BYTES];
+// Beside the documented size it has room for the H descriptors (at most 2.6 % of
+// the images), which plans near that size may need on top.
+constexpr size_t kScratchBytes = (size_t)FGI_STATIC_SCRATCH_BYTES + ((size_t)FGI_STATIC_SCRATCH_BYTES >> 5);
+__device__ __align__(256) unsigned char g_static_scratch[kScratchBytes];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_setup_mutex;
@@ -56,6 +59,7 @@ extern "C" int fgi_integrate_h_static(fgi_ctx *ctx, const double *v_dev, double 
     size_t need = 0;
     int rc = fgi_workspace_size(ctx, &need);
     if (rc) return rc;
+    need = fgi::internal_static_need(ctx);
     if (need > FGI_STATIC_SCRATCH_BYTES) {
         char msg[256];
         snprintf(msg, sizeof msg,
@@ -72,6 +76,6 @@ extern "C" int fgi_integrate_h_static(fgi_ctx *ctx, const double *v_dev, double 
         return fgi::internal_error(ctx, FGI_ERR_CUDA, msg);
     }
     // profiling off: the event pool may grow, and this call must not allocate
-    return fgi::internal_integrate_h(ctx, v_dev, h_dev, accumulate, scratch, FGI_STATIC_SCRATCH_BYTES, stream,
+    return fgi::internal_integrate_h(ctx, v_dev, h_dev, accumulate, scratch, kScratchBytes, stream,
                                      false);
 }

@@ -667,7 +667,7 @@ __device__ __forceinline__ Dd3x2 pair_dd3(const Dd3 &a, const Dd3 &b)
 // What bounds it is instruction issue, then the L1's look-ups: two points a lane
 // halve the FP32 instructions a point (f32x2) and fill four bytes a store where
 // one filled two.  The 64-atom Si cluster's density images 1.84 -> 1.66 ms, 64
-// molecules' (2.3 M points) phi images 15.7 -> 13.9 ms with the preparation below.
+// molecules' (9.0 M points) images 15.7 -> 13.9 ms with the preparation below.
 // Loading the next shell's coefficients ahead costs registers that a third CTA
 // an SM is worth more of: 2.14 -> 2.06 ms of H images without it.
 template <int NIMG, bool SCALED, class Emit2, class General, class Zero>
@@ -1343,7 +1343,7 @@ constexpr int kColAtoms = 128;                       // staged at a time
 // The bounds of a column take one 8-byte look-up an atom (the species' maximum
 // and sum over its shells and m at the knot), the atoms' tables are staged in
 // shared memory.  With look-ups of four shells and a chain of table loads an
-// atom the bounds took a quarter of the kernel: 64 molecules of 20 to 40 atoms,
+// atom the bounds took a quarter of the kernel: 64 molecules (9.0 M points),
 // images 13.9 -> 12.7 ms (H's included); the 64-atom Si cluster 1.66 -> 1.43 ms.
 __global__ void __launch_bounds__(kPhiThreads, 3) k_tc_phi_cols(DevPlan P, const TcBatch *tb, const WorkItem *items,
                                                      uint8_t *ws, int n_split, int bound, unsigned int *counter)
@@ -1504,7 +1504,11 @@ __global__ void k_fix_to_h(const long long *acc, double *h, long long n, int acc
 constexpr int kGroupWarps = 8, kGroupThreads = 32 * kGroupWarps;
 constexpr int kWarpProducer = 2 * kGroupWarps, kWarpMma = kWarpProducer + 1;
 constexpr int kThreadsTc = 32 * (kWarpMma + 1);
-constexpr int kStages = 2;                       // ring of operand chunks, A and B of 64 contraction steps each
+// Ring of operand chunks, A and B of 64 contraction steps each.  Four stages of
+// 32 (64-byte rows) are slower, 64-atom Si cluster: H 3.15 -> 3.44 ms, density
+// 3.57 -> 3.84: a stage boundary costs the MMA warp about 220 clocks that the
+// queue behind it does not hide.
+constexpr int kStages = 2;
 constexpr int kOperandBytes = kChunkStride;      // three planes
 constexpr int kStageBytes = 2 * kOperandBytes;
 // split products kept in the density: combined order <= 3 except x2*y2 (8 of
@@ -2742,17 +2746,11 @@ int tc_build(TcPlan &t, const TcPlanInput &in, std::string *err)
         T.plane_d = (long long)T.nrb * T.nkc * kChunkBytes;
         foot[b] = 3 * (size_t)T.plane_phi + 3 * (size_t)std::max(T.plane_phi, T.plane_d);
         T.hblock = T.hgrid = T.hscale = -1;
-        if (in.for_h) {
-            // phi and w v phi images; the row blocks' descriptors and grids, the
-            // points' scales
-            foot[b] = 6 * (size_t)T.plane_phi +
-                      ((size_t)T.nrb * (sizeof(HBlock) + sizeof(HGrid)) + (size_t)T.nc * 512 + 1023) / 1024 * 1024;
-        }
         T.img_e = -1;
         if (in.with_e) foot[b] += 2 * (size_t)T.plane_phi;     // E in FP32: twice a BF16 plane
     }
     t.bound_grids = in.bound_grids;
-    size_t max_ws = 0;
+    size_t max_ws = 0, max_all = 0;
     TcWave w;
     size_t off = 0;
     auto close_wave = [&](int b_end) {
@@ -2765,10 +2763,29 @@ int tc_build(TcPlan &t, const TcPlanInput &in, std::string *err)
     // of 128 doubles per (point tile, function block))
     long long part = 0;
     auto part_rows = [&](int b) { return (long long)(t.batches[b].nc_alloc / 2) * t.batches[b].nrb; };
+    // H: the row blocks' descriptors and grids and the points' scales of a batch
+    // go behind its two images where the room for D is larger, else to the end
+    // of the wave (at most 2.6 % of the images), outside the wave's budget
+    std::vector<int> at_end;
+    auto desc_bytes = [&](const TcBatch &T) {
+        return ((size_t)T.nrb * (sizeof(HBlock) + sizeof(HGrid)) + (size_t)T.nc * 512 + 1023) / 1024 * 1024;
+    };
+    auto place_desc = [&](TcBatch &T, size_t at) {
+        T.hblock = (long long)at;
+        T.hgrid = T.hblock + (long long)T.nrb * (long long)sizeof(HBlock);
+        T.hscale = T.hgrid + (long long)T.nrb * (long long)sizeof(HGrid);
+    };
     auto finish_wave = [&](int b_end) {
         w.part_off = (off + 1023) / 1024 * 1024;
         off = w.part_off + (size_t)part * 128 * sizeof(double);
         close_wave(b_end);
+        size_t at = (off + 1023) / 1024 * 1024;
+        for (int b : at_end) {
+            place_desc(t.batches[b], at);
+            at += desc_bytes(t.batches[b]);
+        }
+        max_all = std::max(max_all, at_end.empty() ? off : at);
+        at_end.clear();
     };
     for (int b = 0; b < n_sb; b++) {
         const size_t pb = (size_t)part_rows(b) * 128 * sizeof(double);
@@ -2783,9 +2800,8 @@ int tc_build(TcPlan &t, const TcPlanInput &in, std::string *err)
         T.img_phi = (long long)off;
         T.img_aux = (long long)(off + 3 * (size_t)T.plane_phi);
         if (in.for_h) {
-            T.hblock = (long long)(off + 6 * (size_t)T.plane_phi);
-            T.hgrid = T.hblock + (long long)T.nrb * (long long)sizeof(HBlock);
-            T.hscale = T.hgrid + (long long)T.nrb * (long long)sizeof(HGrid);
+            if (6 * (size_t)T.plane_phi + desc_bytes(T) <= foot[b]) place_desc(T, off + 6 * (size_t)T.plane_phi);
+            else at_end.push_back(b);
         }
         if (in.with_e) T.img_e = (long long)(off + 3 * (size_t)T.plane_phi + 3 * (size_t)std::max(T.plane_phi, T.plane_d));
         T.part0 = part;
@@ -2805,7 +2821,7 @@ int tc_build(TcPlan &t, const TcPlanInput &in, std::string *err)
     for (TcWave &wv : t.waves) {
         // longest first: the wave's batches by contraction cost P n^2, each
         // batch's items kept together (they share image tiles in L2); the
-        // persistent kernels stride over this list, so the small items land last
+        // persistent kernels take them in this order, so the small items land last
         std::vector<int> ord;
         for (int b = wv.b0; b < wv.b0 + wv.nb; b++)
             if (t.sb[b].np > 0 && t.sb[b].nfn > 0) ord.push_back(b);
@@ -2858,9 +2874,12 @@ int tc_build(TcPlan &t, const TcPlanInput &in, std::string *err)
     t.n_fn = in.n_fn;
     t.bound_off = ((size_t)in.nnz * 8 + 255) / 256 * 256;
     t.sign_off = (t.bound_off + 8 * (size_t)in.n_fn + 255) / 256 * 256;
-    t.counter_off = (t.sign_off + 4 * (size_t)n_sb + 255) / 256 * 256;
-    t.img_base = (t.counter_off + 256 + 1023) / 1024 * 1024;
-    t.ws_bytes = t.img_base + max_ws + 1024;
+    // the contraction's tile counter in scratch of the other call: H has no bounds
+    // of D, the density no signs of w v
+    t.counter_off = in.for_h ? t.bound_off : t.sign_off;
+    t.img_base = (t.sign_off + 4 * (size_t)n_sb + 1023) / 1024 * 1024;
+    t.ws_images = t.img_base + max_ws + 1024;
+    t.ws_bytes = t.img_base + std::max(max_ws, max_all) + 1024;
     // items must not be empty for the device copy
     if (!in.host_only) {
         const size_t nb_bytes = t.batches.size() * sizeof(TcBatch);

@@ -91,11 +91,13 @@ struct TcPlanInput {
 struct TcPlan {
     bool built = false;
     size_t ws_bytes = 0;
+    size_t ws_images = 0;                // of it without the descriptors behind the waves' images
     size_t wave_cap = 0;
     size_t img_base = 0;                 // workspace offset of the wave images (scratch below)
     size_t bound_off = 0;                // workspace offset of the per-function bounds of D
     size_t sign_off = 0;                 // workspace offset of the per-batch sign of w v (H images)
     size_t counter_off = 0;              // workspace offset of the contractions' tile counter
+                                         // (in scratch that the plan's other call uses)
     long long nnz = 0, n_fn = 0;
     int num_sms = 1;                     // persistent grids: one CTA per SM
     int bound_grids = 0;                 // see TcPlanInput
