@@ -446,7 +446,9 @@ int build_plan(fgi_ctx *c, const char *tune_path)
             double dc = 0.0;
             for (int k = 0; k < 3; k++) dc += (xa[k] - cen[k]) * (xa[k] - cen[k]);
             dc = std::sqrt(dc);
-            if (dc >= rad + rc) continue;
+            // far beyond the rounding of dc and rad (and of squares that overflow): a
+            // batch may hold a point so far away that rc is lost beside its radius
+            if (std::isfinite(dc) && dc >= (rad + rc) * (1.0 + 1e-12)) continue;
             bool on = dc + rad < rc;
             for (int64_t p = p0; p < p1 && !on; p++) {
                 double d2 = 0.0;
