@@ -711,6 +711,11 @@ __device__ __forceinline__ void eval_atom_warp(const DevPlan &P, const DevSpecie
     // a point that is not live: t = 0 on interval 0, times ip = 0
     const pk t = pk_make(live0 ? sh2.x - (float)k0 : 0.f, live1 ? sh2.y - (float)k1 : 0.f);
     const pk nt = -t, ntl = pk_make(live0 ? -tl2.x : 0.f, live1 ? -tl2.y : 0.f), tt = t * t;
+    // and the polynomials of offset 0: those of a far point overflow FP32 (f shells
+    // from 7e12 Bohr on), and zero times infinity is not zero
+    const float2 xh = pk_get(x.hi), yh = pk_get(y.hi), zh = pk_get(z.hi);
+    const pk qx = pk_make(live0 ? xh.x : 0.f, live1 ? xh.y : 0.f), qy = pk_make(live0 ? yh.x : 0.f, live1 ? yh.y : 0.f),
+             qz = pk_make(live0 ? zh.x : 0.f, live1 ? zh.y : 0.f);
     const float4 *tab = P.scoefn + S.scoef_off;
     const float4 *c0 = tab + 2 * ((long long)k0 * S.n_shell), *c1 = tab + 2 * ((long long)k1 * S.n_shell);
     int sh = 0;
@@ -733,7 +738,7 @@ __device__ __forceinline__ void eval_atom_warp(const DevPlan &P, const DevSpecie
         }
         pk Q[NM];
         int gi[7];
-        if constexpr (L > 0) ylm_poly_unit2<L>(x.hi, y.hi, z.hi, Q, gi);
+        if constexpr (L > 0) ylm_poly_unit2<L>(qx, qy, qz, Q, gi);
         for (; sh < end; sh++) {
             const SplineEntry a = load_entry(c0 + 2 * sh), b = load_entry(c1 + 2 * sh);
             const int f = sh_tab[S.shell0 + sh].fn0;
