@@ -157,14 +157,41 @@ __device__ __forceinline__ void warp_sum_split(df *v, int &off, int &lim)
     }
 }
 
+// Exponent field of a double, and a float 2^e (zero below FP32's range)
+__device__ __forceinline__ int exp_field(double x) { return (int)((unsigned)__double2hiint(x) >> 20) & 0x7FF; }
+__device__ __forceinline__ float pow2f(int e) { return e < -126 ? 0.f : __int_as_float((e + 127) << 23); }
+
+// x 2^(1023 - e) as a double-float, for a field e not below x's own (or by at most
+// 40), in integers: the leading 24 bits of x are the high part, the other 29
+// the low part.  Zero where |x| is 2^126 times smaller than 2^(e - 1023).  Infinity and
+// NaN give NaN.  (A conversion each way and a subtraction in FP64 would take
+// the pipe that has 1/64 of the FP32 rate.)
+__device__ __forceinline__ df df_scaled(double x, int e)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const int f = (int)(hi >> 20) & 0x7FF, q = f - e;
+    if (f == 0x7FF) return {__int_as_float(0x7FFFFFFF), 0.f};
+    if (f == 0 || q < -126) return {0.f, 0.f};
+    const unsigned sign = hi & 0x80000000u;
+    const float h = __uint_as_float(sign | (unsigned)(q + 127) << 23 | (__funnelshift_l(lo, hi, 3) & 0x7FFFFFu));
+    const float l = __uint2float_rn(lo & 0x1FFFFFFFu) * pow2f(q - 52);
+    return df_fast_two_sum(h, sign ? -l : l);
+}
+
 // One warp per (atom, shell).  (A thread per point with FP64 harmonics and
 // (l_max + 1)^2 FP64 atomics was bound by the FP64 pipe: 250-atom cluster, 7.3 M
 // points, l_max 6, 3.30 ms; now 0.51 ms.)  The monopole's sum stays FP64: the
 // l = 0 terms are all there is at l_max 0, and the others end in FP32.
+//
+// The offsets are differences in FP64 and w n a product in FP64; both become
+// double-floats relative to a power of two (the largest component's; that of the
+// warp's largest |w n| so far), so that neither an atom far from the origin nor
+// the range of FP32 costs any of the 48 bits.
 template <int LMAX>
 __global__ void __launch_bounds__(128) k_hartree_moments(DevPlan P, HartreeDev H, const double *n, double *rho)
 {
     constexpr int L = (LMAX + 1) * (LMAX + 1);
+    constexpr int kHeadroom = 40;                                      // binades w n may grow before the sums are scaled
     const long long bin = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (bin >= H.n_shells) return;
@@ -173,24 +200,35 @@ __global__ void __launch_bounds__(128) k_hartree_moments(DevPlan P, HartreeDev H
 #pragma unroll
     for (int q = 0; q < L; q++) acc[q] = df{0.f, 0.f};
     double mono = 0.0;
-    int a = 0;
+    int a = 0, ew = 0;                                                 // the sums hold w n 2^(1023 - ew)
     if (i0 < i1) a = H.owner[H.order[i0]];
-    const float *aa = P.atom_dd + 6 * a;
-    for (long long i = i0 + lane; i < i1; i += 32) {
-        const long long p = H.order[i];
-        const float2 *pp = reinterpret_cast<const float2 *>(P.pts_dd + 6 * p);
-        const float2 px = pp[0], py = pp[1], pz = pp[2];
-        df x = dfa(df{px.x, px.y}, df{-aa[0], -aa[1]}), y = dfa(df{py.x, py.y}, df{-aa[2], -aa[3]}),
-           z = dfa(df{pz.x, pz.y}, df{-aa[4], -aa[5]});
+    const double ax = P.atom_xyz[3 * a], ay = P.atom_xyz[3 * a + 1], az = P.atom_xyz[3 * a + 2];
+    for (long long ib = i0; ib < i1; ib += 32) {
+        const bool has = ib + lane < i1;
+        const long long p = H.order[has ? ib + lane : i0];
+        const double dx = P.px[p] - ax, dy = P.py[p] - ay, dz = P.pz[p] - az;
+        const int ed = max(exp_field(dx), max(exp_field(dy), exp_field(dz)));
+        // a point on the nucleus has no direction
+        const bool live = has && ed > 0;
+        const double wn = live ? P.pw[p] * n[p] : 0.0;
+        mono += wn;
+        if (LMAX == 0) continue;
+        const int fw = exp_field(wn);
+        const int top = (int)__reduce_max_sync(0xffffffffu, fw == 0x7FF ? 0u : (unsigned)fw);
+        if (top > ew + kHeadroom || ew == 0) {                         // the same for the whole warp
+            const float down = ew == 0 ? 0.f : pow2f(ew - top);
+#pragma unroll
+            for (int q = 1; q < L; q++) acc[q] = df{acc[q].hi * down, acc[q].lo * down};
+            ew = top;
+        }
+        if (!live) continue;
+        df x = df_scaled(dx, ed), y = df_scaled(dy, ed), z = df_scaled(dz, ed);
         const df d2 = dfa(dfa(df_sqr(x), df_sqr(y)), df_sqr(z));
-        if (!(d2.hi > 0.f)) continue;
         const df ir = df_rsqrt(d2, rsqrtf(d2.hi));
         x = df_mul(x, ir);
         y = df_mul(y, ir);
         z = df_mul(z, ir);
-        const double wn = P.pw[p] * n[p];
-        mono += wn;
-        df cm = df_from_double(wn), sm{0.f, 0.f};                  // w n Re, Im (x + i y)^m
+        df cm = df_scaled(wn, ew), sm{0.f, 0.f};                   // w n Re, Im (x + i y)^m
         float pmm = 1.f;
 #pragma unroll
         for (int m = 0; m <= LMAX; m++) {
@@ -233,10 +271,11 @@ __global__ void __launch_bounds__(128) k_hartree_moments(DevPlan P, HartreeDev H
         const double rk = g.r0 * exp(g.lnq * (double)(bin - H.rad_off[a]));
         scale = 1.0 / (rk * rk * rk * g.lnq);
     }
+    const double unit = __hiloint2double(ew << 20, 0);                 // 2^(ew - 1023)
 #pragma unroll
     for (int q = 0; q < (L + 31) / 32; q++)
         if (off + q < lim)
-            rho[bin * kL + off + q] = (off + q == 0 ? mono : (double)acc[q].hi + (double)acc[q].lo) * scale;
+            rho[bin * kL + off + q] = (off + q == 0 ? mono : ((double)acc[q].hi + (double)acc[q].lo) * unit) * scale;
 }
 
 __device__ __forceinline__ double warp_scan_up(double v, int lane)       // inclusive, towards higher lanes
