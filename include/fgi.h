@@ -271,9 +271,10 @@ int fgi_adjoint(fgi_ctx *ctx, const double *g_dev, const double *v_dev, double *
    grid r_k = r_min[a] exp(k ln_q[a]), k = 0 .. n_rad[a]-1 (n_rad >= 4).  The point weights
    given to fgi_set_grid are then read as (partition weight) x r_k^3 ln q x
    (angular weight).  Call after fgi_set_grid; fgi_set_systems or
-   fgi_set_grid discard it.  Copies the tables to the device (a setup call:
-   it allocates).  FGI_ERR_ARG for an owner outside the point's system or a
-   shell beyond its grid. */
+   fgi_set_grid discard it.  Lists the points by (owner, shell), in their own
+   order within a shell, and copies the list (4 bytes a point) and the
+   tables to the device (a setup call: it allocates).  FGI_ERR_ARG for an
+   owner outside the point's system or a shell beyond its grid. */
 int fgi_set_atom_grids(fgi_ctx *ctx, const int32_t *owner, const int32_t *shell, const double *r_min,
                        const double *ln_q, const int32_t *n_rad);
 
@@ -302,9 +303,9 @@ int fgi_hartree_workspace_size(fgi_ctx *ctx, size_t *bytes);
    terms), the radial solve is FP64; the evaluation (every (point, atom) pair of a system) takes
    the l = 0 terms as double-floats (~1e-12 relative; FP64 interpolation for
    radial grids with ln q > 0.6) and the l >= 1 terms in FP32 (a few FP32
-   roundings of the l >= 1 part).  The moments are summed in an order
-   fixed when the grids are set: calls of one context repeat bit by
-   bit, another context's may differ in the last bits.  Needs a plan and fgi_set_atom_grids;
+   roundings of the l >= 1 part).  The moments are summed in the order
+   of the points: calls repeat bit by bit, also those of another context
+   set up alike.  Needs a plan and fgi_set_atom_grids;
    ws: device, 256-byte aligned, at least fgi_hartree_workspace_size bytes
    (FGI_ERR_WORKSPACE otherwise).  Enqueued on stream, no allocation, no host
    synchronisation (graph-capturable). */

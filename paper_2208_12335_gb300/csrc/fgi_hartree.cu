@@ -33,8 +33,6 @@
 //     carries a relative error of a few FP32 roundings of the l >= 1 part,
 //     against the FP64 pipe's 1/64 rate on GB300.  The sum over atoms is a
 //     double-float.
-#include <vector>
-
 #include "fgi_dd.cuh"
 #include "fgi_hartree.h"
 #include "fgi_ylm.cuh"
@@ -200,8 +198,8 @@ __global__ void __launch_bounds__(128) k_hartree_moments(DevPlan P, HartreeDev H
 #pragma unroll
     for (int q = 0; q < L; q++) acc[q] = df{0.f, 0.f};
     double mono = 0.0;
-    int a = 0, ew = 0;                                                 // the sums hold w n 2^(1023 - ew)
-    if (i0 < i1) a = H.owner[H.order[i0]];
+    int ew = 0;                                                        // the sums hold w n 2^(1023 - ew)
+    const int a = H.bin_atom[bin];
     const double ax = P.atom_xyz[3 * a], ay = P.atom_xyz[3 * a + 1], az = P.atom_xyz[3 * a + 2];
     for (long long ib = i0; ib < i1; ib += 32) {
         const bool has = ib + lane < i1;
@@ -618,41 +616,6 @@ __global__ void __launch_bounds__(128, 6) k_hartree_eval(DevPlan P, HartreeDev H
 }
 
 }  // namespace
-
-// points per (owner, shell), then their places
-__global__ void k_bin_count(HartreeDev H, long long n_pts, unsigned int *count)
-{
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n_pts; p += (long long)gridDim.x * blockDim.x)
-        if (H.owner[p] >= 0) atomicAdd(count + H.rad_off[H.owner[p]] + H.shell[p], 1u);
-}
-
-__global__ void k_bin_fill(HartreeDev H, long long n_pts, unsigned int *count, unsigned int *order)
-{
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n_pts; p += (long long)gridDim.x * blockDim.x)
-        if (H.owner[p] >= 0) {
-            const long long bin = H.rad_off[H.owner[p]] + H.shell[p];
-            order[H.bin_off[bin] + atomicSub(count + bin, 1u) - 1] = (unsigned int)p;
-        }
-}
-
-cudaError_t hartree_bin_points(const HartreeDev &H, long long n_pts, unsigned int *count, unsigned int *order,
-                               long long *bin_off)
-{
-    cudaError_t e = cudaMemset(count, 0, sizeof(unsigned int) * (size_t)H.n_shells);
-    if (e != cudaSuccess) return e;
-    if (n_pts > 0) k_bin_count<<<1216, 256>>>(H, n_pts, count);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    std::vector<unsigned int> host((size_t)H.n_shells);
-    e = cudaMemcpy(host.data(), count, sizeof(unsigned int) * host.size(), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return e;
-    std::vector<long long> off(host.size() + 1, 0);
-    for (size_t k = 0; k < host.size(); k++) off[k + 1] = off[k] + host[k];
-    e = cudaMemcpy(bin_off, off.data(), sizeof(long long) * off.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return e;
-    if (n_pts > 0) k_bin_fill<<<1216, 256>>>(H, n_pts, count, order);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    return cudaStreamSynchronize(0);
-}
 
 HartreeRad hartree_rad(double r_min, double ln_q, int n_rad)
 {

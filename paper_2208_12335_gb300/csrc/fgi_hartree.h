@@ -24,25 +24,18 @@ struct HartreeRad {
 
 // the grid's atom-centred structure on the device
 struct HartreeDev {
-    const int *owner = nullptr;          // [n_pts] owner atom (global index, -1: none)
-    const int *shell = nullptr;          // [n_pts] radial shell on the owner's grid
     const long long *rad_off = nullptr;  // [n_atoms + 1] first shell of each atom in the shell tables
     const HartreeRad *rad = nullptr;     // [n_atoms]
     const long long *sys_atom0 = nullptr;  // [n_sys + 1] first atom of each system
     const unsigned int *order = nullptr;   // the points that have an owner, grouped by (owner, shell)
     const long long *bin_off = nullptr;    // [n_shells + 1] first of each group in order
+    const int *bin_atom = nullptr;         // [n_shells] owner of each group
     int n_atoms = 0;
     long long n_shells = 0;
 };
 
 // radial grid record of one atom (host)
 HartreeRad hartree_rad(double r_min, double ln_q, int n_rad);
-
-// group the points by (owner, shell): fills order and bin_off (device) from
-// H.owner, H.shell and H.rad_off; count: device scratch of n_shells words.
-// A set-up call: waits for the default stream.
-cudaError_t hartree_bin_points(const HartreeDev &H, long long n_pts, unsigned int *count, unsigned int *order,
-                               long long *bin_off);
 
 // scratch of one call: multipoles and potentials on the shells, exterior moments
 size_t hartree_ws_bytes(const HartreeDev &H);

@@ -144,8 +144,6 @@ struct fgi_ctx {
     TcPlan tca;                               // the density's super-batches with room for E (the adjoint)
     // atom-centred structure of the grid (the Hartree potential)
     bool have_atom_grids = false;
-    std::vector<int> hg_owner, hg_shell, hg_nrad;
-    std::vector<double> hg_rmin, hg_lnq;
     char *d_hartree = nullptr;
     HartreeDev hd{};
     // per-kernel CUDA-event profile
@@ -875,6 +873,40 @@ int check_ready(fgi_ctx *c)
     return FGI_OK;
 }
 
+constexpr int64_t kSerialPoints = 65536;   // loops over fewer points stay on one thread (starting more takes longer)
+
+// The points that have an owner, grouped by (owner, shell) and in their own order
+// within a group (group k, of owner a's shell k - rad_off[a], is order[bin_off[k] .. bin_off[k + 1])):
+// a counting sort by pieces of consecutive points, so that it does not depend on
+// the threads.  order: room for n; returns how many of them it took.
+size_t group_points(int64_t n, const int32_t *owner, const int32_t *shell, const std::vector<long long> &rad_off,
+                    unsigned int *order, long long *bin_off)
+{
+    const size_t n_bin = (size_t)rad_off.back();
+    const int pieces = (int)std::max<int64_t>(1, std::min<int64_t>(16, n / kSerialPoints));
+    std::vector<unsigned int> at((size_t)pieces * n_bin, 0);        // per piece: points of a group, then its next place
+    auto each = [&](int q, auto &&visit) {
+        for (int64_t p = n * q / pieces; p < n * (q + 1) / pieces; p++)
+            if (owner[p] >= 0) visit(p, at[(size_t)q * n_bin + (size_t)(rad_off[owner[p]] + shell[p])]);
+    };
+#pragma omp parallel for schedule(static, 1) if (pieces > 1)
+    for (int q = 0; q < pieces; q++) each(q, [](int64_t, unsigned int &k) { k++; });
+    unsigned int place = 0;
+    for (size_t k = 0; k < n_bin; k++) {
+        bin_off[k] = place;
+        for (int q = 0; q < pieces; q++) {
+            unsigned int &slot = at[(size_t)q * n_bin + k];
+            const unsigned int points = slot;
+            slot = place;
+            place += points;
+        }
+    }
+    bin_off[n_bin] = place;
+#pragma omp parallel for schedule(static, 1) if (pieces > 1)
+    for (int q = 0; q < pieces; q++) each(q, [&](int64_t p, unsigned int &k) { order[k++] = (unsigned int)p; });
+    return place;
+}
+
 int check_compute(fgi_ctx *c)
 {
     int rc = check_ready(c);
@@ -1444,7 +1476,7 @@ int fgi_adjoint(fgi_ctx *c, const double *gv, const double *v, double *dv, doubl
 
 int fgi_set_atom_grids(fgi_ctx *c, const int32_t *owner, const int32_t *shell, const double *r_min,
                        const double *ln_q, const int32_t *n_rad)
-{
+try {
     if (!c) return FGI_ERR_ARG;
     if (!c->have_systems || !c->have_grid) return set_err(c, FGI_ERR_STATE, "set systems and grid first");
     const int n_at = (int)c->atom_species.size();
@@ -1454,65 +1486,65 @@ int fgi_set_atom_grids(fgi_ctx *c, const int32_t *owner, const int32_t *shell, c
         if (!(r_min[a] > 0.0) || !(ln_q[a] > 0.0) || !std::isfinite(r_min[a]) || !std::isfinite(ln_q[a]) || n_rad[a] < 4)
             return set_err(c, FGI_ERR_ARG, "atom grids: atom %d needs r_min > 0, ln q > 0, n_rad >= 4", a);
     // every point's owner lies in the point's own system, its shell on the owner's grid
-    std::vector<int> pt_sys((size_t)c->n_pts);
-    for (size_t b = 0; b + 1 < c->batch_off.size(); b++)
-        for (int64_t p = c->batch_off[b]; p < c->batch_off[b + 1]; p++) pt_sys[(size_t)p] = c->batch_sys[b];
-    for (int64_t p = 0; p < c->n_pts; p++) {
-        const int a = owner[p];
-        if (a == -1) continue;
-        if (a < 0 || a >= n_at || shell[p] < 0 || shell[p] >= n_rad[a])
-            return set_err(c, FGI_ERR_ARG, "atom grids: point %lld has owner %d, shell %d", (long long)p, a,
-                           (int)shell[p]);
-        if (a < c->atom_off[pt_sys[(size_t)p]] || a >= c->atom_off[pt_sys[(size_t)p] + 1])
-            return set_err(c, FGI_ERR_ARG, "atom grids: point %lld belongs to another system than its owner",
-                           (long long)p);
+    int64_t first_bad = c->n_pts;
+#pragma omp parallel for schedule(static) reduction(min : first_bad) if (c->n_pts > kSerialPoints)
+    for (int64_t b = 0; b < (int64_t)c->batch_sys.size(); b++) {
+        const int s = c->batch_sys[b];
+        const int64_t a0 = s < c->n_sys ? c->atom_off[s] : 0, a1 = s < c->n_sys ? c->atom_off[s + 1] : 0;
+        for (int64_t p = c->batch_off[b]; p < c->batch_off[b + 1]; p++) {
+            const int a = owner[p];
+            if (a != -1 && (a < a0 || a >= a1 || shell[p] < 0 || shell[p] >= n_rad[a])) first_bad = std::min(first_bad, p);
+        }
+    }
+    if (first_bad < c->n_pts) {
+        const int a = owner[first_bad], sh = shell[first_bad];
+        if (a < 0 || a >= n_at || sh < 0 || sh >= n_rad[a])
+            return set_err(c, FGI_ERR_ARG, "atom grids: point %lld has owner %d, shell %d", (long long)first_bad, a, sh);
+        return set_err(c, FGI_ERR_ARG, "atom grids: point %lld belongs to another system than its owner",
+                       (long long)first_bad);
     }
     if (c->device >= 0) {
         DeviceGuard g(c->device);
         free_atom_grids(c);
     }
-    c->hg_owner.assign(owner, owner + c->n_pts);
-    c->hg_shell.assign(shell, shell + c->n_pts);
-    c->hg_rmin.assign(r_min, r_min + n_at);
-    c->hg_lnq.assign(ln_q, ln_q + n_at);
-    c->hg_nrad.assign(n_rad, n_rad + n_at);
     std::vector<long long> rad_off(n_at + 1, 0);
     for (int a = 0; a < n_at; a++) rad_off[a + 1] = rad_off[a] + n_rad[a];
-    std::vector<HartreeRad> rgrid(n_at);
-    for (int a = 0; a < n_at; a++) rgrid[a] = hartree_rad(r_min[a], ln_q[a], n_rad[a]);
-    std::vector<long long> sys_atom0(c->atom_off.begin(), c->atom_off.end());
     c->hd.n_atoms = n_at;
     c->hd.n_shells = rad_off[n_at];
     if (c->device >= 0) {
         DeviceGuard g(c->device);
-        const size_t s_own = align_up(4 * (size_t)c->n_pts + 4, 256), s_off = align_up(8 * (size_t)(n_at + 1), 256),
-                     s_rg = align_up(sizeof(HartreeRad) * (size_t)(n_at + 1), 256),
-                     s_sys = align_up(8 * sys_atom0.size(), 256);
+        // the tables and the points that have an owner, listed by (owner, shell), in
+        // one copy
         const size_t n_sh = (size_t)c->hd.n_shells;
-        const size_t s_bin = align_up(8 * (n_sh + 1), 256), s_cnt = align_up(4 * n_sh + 4, 256);
-        const size_t at_ord = 2 * s_own + s_off + s_rg + s_sys, at_bin = at_ord + s_own, at_cnt = at_bin + s_bin;
-        const size_t tot = at_cnt + s_cnt;
-        CUDA_TRY(c, cudaMalloc((void **)&c->d_hartree, tot));
+        const size_t at_rg = align_up(8 * rad_off.size(), 256), at_sys = at_rg + align_up(sizeof(HartreeRad) * (size_t)n_at, 256),
+                     at_bin = at_sys + align_up(8 * c->atom_off.size(), 256),
+                     at_atom = at_bin + align_up(8 * (n_sh + 1), 256), at_ord = at_atom + align_up(4 * n_sh, 256);
+        BigVec<char> tab(at_ord + 4 * (size_t)c->n_pts);
+        memcpy(tab.data(), rad_off.data(), 8 * rad_off.size());
+        for (int a = 0; a < n_at; a++) {
+            const HartreeRad r = hartree_rad(r_min[a], ln_q[a], n_rad[a]);
+            memcpy(tab.data() + at_rg + sizeof r * (size_t)a, &r, sizeof r);
+        }
+        std::copy(c->atom_off.begin(), c->atom_off.end(), (long long *)(tab.data() + at_sys));
+        int *bin_atom = (int *)(tab.data() + at_atom);
+        for (int a = 0; a < n_at; a++) std::fill(bin_atom + rad_off[a], bin_atom + rad_off[a + 1], a);
+        const size_t listed = group_points(c->n_pts, owner, shell, rad_off, (unsigned int *)(tab.data() + at_ord),
+                                           (long long *)(tab.data() + at_bin));
+        const size_t bytes = at_ord + 4 * listed;
+        CUDA_TRY(c, cudaMalloc((void **)&c->d_hartree, bytes));
         char *b = c->d_hartree;
-        CUDA_TRY(c, cudaMemcpy(b, owner, 4 * (size_t)c->n_pts, cudaMemcpyHostToDevice));
-        CUDA_TRY(c, cudaMemcpy(b + s_own, shell, 4 * (size_t)c->n_pts, cudaMemcpyHostToDevice));
-        CUDA_TRY(c, cudaMemcpy(b + 2 * s_own, rad_off.data(), 8 * rad_off.size(), cudaMemcpyHostToDevice));
-        CUDA_TRY(c, cudaMemcpy(b + 2 * s_own + s_off, rgrid.data(), sizeof(HartreeRad) * (size_t)n_at,
-                               cudaMemcpyHostToDevice));
-        CUDA_TRY(c, cudaMemcpy(b + 2 * s_own + s_off + s_rg, sys_atom0.data(), 8 * sys_atom0.size(),
-                               cudaMemcpyHostToDevice));
-        c->hd.owner = (const int *)b;
-        c->hd.shell = (const int *)(b + s_own);
-        c->hd.rad_off = (const long long *)(b + 2 * s_own);
-        c->hd.rad = (const HartreeRad *)(b + 2 * s_own + s_off);
-        c->hd.sys_atom0 = (const long long *)(b + 2 * s_own + s_off + s_rg);
-        c->hd.order = (const unsigned int *)(b + at_ord);
+        CUDA_TRY(c, cudaMemcpy(b, tab.data(), bytes, cudaMemcpyHostToDevice));
+        c->hd.rad_off = (const long long *)b;
+        c->hd.rad = (const HartreeRad *)(b + at_rg);
+        c->hd.sys_atom0 = (const long long *)(b + at_sys);
         c->hd.bin_off = (const long long *)(b + at_bin);
-        CUDA_TRY(c, hartree_bin_points(c->hd, c->n_pts, (unsigned int *)(b + at_cnt), (unsigned int *)(b + at_ord),
-                                       (long long *)(b + at_bin)));
+        c->hd.bin_atom = (const int *)(b + at_atom);
+        c->hd.order = (const unsigned int *)(b + at_ord);
     }
     c->have_atom_grids = true;
     return FGI_OK;
+} catch (const std::bad_alloc &) {
+    return set_err(c, FGI_ERR_NOMEM, "atom grids: host allocation failed");
 }
 
 int fgi_hartree_workspace_size(fgi_ctx *c, size_t *bytes)
