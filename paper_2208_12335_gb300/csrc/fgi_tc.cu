@@ -1892,6 +1892,15 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_h(DevPlan P, const TcBatch
                     for (int q = 0; q < 32; q++) a1[q] = 0.f;
                 tmem_wait_ld();
                 if (!ok) continue;
+                if (ncol - c0 < 32) {
+                    // columns past n_b hold what was there before: products of stale image
+                    // rows, an earlier tile's values or none at all
+#pragma unroll
+                    for (int q = 0; q < 32; q++) {
+                        a0[q] = c0 + q < ncol ? a0[q] : 0.f;
+                        a1[q] = c0 + q < ncol ? a1[q] : 0.f;
+                    }
+                }
                 float size = 0.f;
 #pragma unroll
                 for (int q = 0; q < 32; q++) size = max_abs_nan(size, a0[q], a1[q]);
