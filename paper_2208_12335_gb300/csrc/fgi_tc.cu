@@ -1618,7 +1618,11 @@ __device__ __forceinline__ void ring_drain(TcRing *S, uint32_t n, int *status)
 // group lt % 2
 //
 // Producer side: the next tiles of the shared list, their tables loading while
-// the tile before them streams.
+// the tile before them streams.  A CTA holds three tiles of the list at a time; its
+// first three are a grid apart and the counter gives the rest, so that a list
+// shorter than that is spread evenly.  (With the first three from the counter too, the first
+// CTAs to arrive took three each and the others none: a water molecule's H, 32
+// tiles, 55.6 -> 43.3 us.)
 struct TileFetch {
     const WorkItem *items;
     const TcBatch *tb;
@@ -1652,10 +1656,9 @@ __device__ __forceinline__ WorkItem fetch_item(const TileFetch &F, unsigned int 
 
 __device__ __forceinline__ void fetch_start(TileFetch &F)
 {
-    const unsigned int k0 = atomicAdd(F.counter, 1u), k1 = atomicAdd(F.counter, 1u);
-    F.idx2 = atomicAdd(F.counter, 1u);
-    F.it = fetch_item(F, k0, F.have);
-    F.it1 = fetch_item(F, k1, F.have1);
+    F.idx2 = blockIdx.x + 2 * gridDim.x;
+    F.it = fetch_item(F, blockIdx.x, F.have);
+    F.it1 = fetch_item(F, blockIdx.x + gridDim.x, F.have1);
     fetch_tables(F);
 }
 
@@ -1665,7 +1668,7 @@ __device__ __forceinline__ void fetch_next(TileFetch &F)
     F.it = F.it1;
     F.have = F.have1;
     F.it1 = fetch_item(F, F.idx2, F.have1);
-    F.idx2 = atomicAdd(F.counter, 1u);
+    F.idx2 = 3 * gridDim.x + atomicAdd(F.counter, 1u);
     fetch_tables(F);
 }
 
