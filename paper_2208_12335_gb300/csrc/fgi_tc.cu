@@ -573,7 +573,7 @@ __device__ __forceinline__ df spline_value(const SplineEntry &e, float t, float 
 // nucleus.  emit(f, val[NIMG]) receives phi times the image's scale (SCALED
 // false: image 0 unscaled); emit0(f) a value that is zero in every image.
 template <int NIMG, bool SCALED, class Emit, class Emit0>
-__device__ __forceinline__ void eval_atom_general(const DevPlan &P, const DevSpecies &S, const DevShell *sh_tab,
+__device__ __forceinline__ void eval_atom_general(const float4 *coef, const DevSpecies &S, const DevShell *sh_tab,
                                                   const Dd3 &aa, const Dd3 &pp, bool has, int f_lo, int f_hi,
                                                   const df *scale, Emit &emit, Emit0 &emit0)
 {
@@ -613,7 +613,7 @@ __device__ __forceinline__ void eval_atom_general(const DevPlan &P, const DevSpe
             }
             df rk[NIMG];
             if (origin) {                               // the l = 0 limit C_0 c1/h
-                const SplineEntry e = load_entry(P.coef_ddn + 2 * R.coef_off);
+                const SplineEntry e = load_entry(coef + 2 * R.coef_off);
                 const df u = df_mul(df{e.h.y, e.l.y}, df{R.inv_h_hi, R.inv_h_lo});
 #pragma unroll
                 for (int k = 0; k < NIMG; k++) rk[k] = (SCALED || k > 0) ? df_mul(u, scale[k]) : u;
@@ -628,7 +628,7 @@ __device__ __forceinline__ void eval_atom_general(const DevPlan &P, const DevSpe
                     t = s2.hi - (float)kk;
                     tl = s2.lo;
                 }
-                const df u = spline_value(load_entry(P.coef_ddn + 2 * (R.coef_off + kk)), t, tl);
+                const df u = spline_value(load_entry(coef + 2 * (R.coef_off + kk)), t, tl);
 #pragma unroll
                 for (int k = 0; k < NIMG; k++) rk[k] = df_mul(u, (SCALED || k > 0) ? df_mul(pw, scale[k]) : pw);
             }
@@ -688,14 +688,19 @@ __device__ __forceinline__ void eval_atom_warp(const DevPlan &P, const DevSpecie
         zero_all();
         return;
     }
+    // (the density's kernel gains from leaving here; H's, whose general path is a call,
+    // from looking once: the 75-atom cluster's H 4.83 ms, 4.90 with the look here)
+    if (NIMG == 1 && !SCALED && !S.shared_grid) {
+        general();
+        return;
+    }
     // offset from the atom (the rounding of the low parts differs from point
     // to point), d^2 (terms of one sign), 1/d from a refined rsqrtf, d = d^2/d
     const df2 x = df2_add_sloppy(pp.x, ax), y = df2_add_sloppy(pp.y, ay), z = df2_add_sloppy(pp.z, az);
     const df2 d2 = df2_add_sloppy(df2_add_sloppy(df2_mul(x, x), df2_mul(y, y)), df2_mul(z, z));
     const float2 d2h = pk_get(d2.hi);
     if (!S.shared_grid || __any_sync(0xffffffffu, (in0 && d2h.x < 1e-24f) || (in1 && d2h.y < 1e-24f))) {
-        general(0);
-        general(1);
+        general();
         return;
     }
     const df2 i0 = df2_rsqrt(d2);
@@ -810,6 +815,47 @@ __device__ __forceinline__ const DevShell *stage_shells(const DevPlan &P, DevShe
 // swizzled place of point column group g16 = g << 4 in row r of a chunk
 __device__ __forceinline__ uint32_t row_offset(uint32_t r, uint32_t g16) { return r * 128u + (((r << 4) ^ g16) & 0x70u); }
 
+// One atom's functions [f_lo, f_hi) at the points of chunk c by the general path,
+// a point a lane: 64 consecutive bytes of a row a store.  (Every second point a
+// lane wrote half sectors: 64 atoms, shells on knots of their own, potential of both
+// signs, H 5.15 -> 4.58 ms with the rest below.)  A function of its own, for its
+// registers would cost the path on shared knots.
+template <int NIMG, int NSPLIT>
+__device__ __noinline__ void h_image_general(const float4 *coef, const DevSpecies *species, const DevShell *sh_tab,
+                                             const float *atom, const float *pts, int np, int c, int rb, int f_lo,
+                                             int f_hi, uint8_t *c0, uint8_t *c1, const float2 *wvs,
+                                             const float4 (*fsc)[128])
+{
+    const DevSpecies S = *species;
+    const Dd3 aa = load_dd3(atom);
+#pragma unroll 1
+    for (int kg = threadIdx.x & 31; kg < 64; kg += 32) {
+        const int pg = c * 64 + kg;
+        const bool has = pg < np;
+        const Dd3 q = load_dd3(pts + 6 * (has ? pg : 0));
+        const float2 s2 = has ? wvs[pg] : make_float2(0.f, 0.f);
+        df sc[NIMG];
+#pragma unroll
+        for (int k = 0; k < NIMG; k++) sc[k] = df{s2.x, s2.y};
+        const uint32_t g16 = (uint32_t)(kg >> 3) << 4, hb = (uint32_t)(kg & 7) * 2u;
+        auto emit = [&](int f, const df *val) {
+            const int r = rb + f;
+            const uint32_t off = row_offset((uint32_t)r, g16) + hb;
+#pragma unroll
+            for (int k = 0; k < NIMG; k++) {
+                const float4 su = fsc[NIMG == 1 ? 1 : k][r];
+                store_value<NSPLIT>((k == 0 ? c0 : c1) + off, val[k], su.x, su.z);
+            }
+        };
+        auto emit0 = [&](int f) {
+            const uint32_t off = row_offset((uint32_t)(rb + f), g16) + hb;
+#pragma unroll
+            for (int k = 0; k < NIMG; k++) store_zero<NSPLIT>((k == 0 ? c0 : c1) + off);
+        };
+        eval_atom_general<NIMG, NIMG == 1>(coef, S, sh_tab, aa, q, has, f_lo, f_hi, sc, emit, emit0);
+    }
+}
+
 // H images of one 128-row block: warp tasks (atom of the block, 64-point
 // chunk).  NIMG 1: psi = phi sqrt|w v| on the second grid set; NIMG 2: phi
 // (first set) and w v phi (second set) into two images.
@@ -848,28 +894,9 @@ __device__ __forceinline__ void h_image_lanes(const DevPlan &P, const DevBatch &
                 store_pair<NSPLIT>((k == 0 ? c0 : c1) + off, hi[k], nlo[k], pk_make(su.x, su.y), pk_make(su.z, su.w));
             }
         };
-        auto general = [&](int half) {
-            df sc[NIMG];
-            const float2 s2 = half ? s1 : s0;
-#pragma unroll
-            for (int k = 0; k < NIMG; k++) sc[k] = df{s2.x, s2.y};
-            const uint32_t hb = pb + 2u * half;
-            auto emit = [&](int f, const df *val) {
-                const int r = rb + f;
-                const uint32_t off = row_offset((uint32_t)r, g16) + hb;
-#pragma unroll
-                for (int k = 0; k < NIMG; k++) {
-                    const float4 su = fsc[NIMG == 1 ? 1 : k][r];
-                    store_value<NSPLIT>((k == 0 ? c0 : c1) + off, val[k], su.x, su.z);
-                }
-            };
-            auto emit0 = [&](int f) {
-                const uint32_t off = row_offset((uint32_t)(rb + f), g16) + hb;
-#pragma unroll
-                for (int k = 0; k < NIMG; k++) store_zero<NSPLIT>((k == 0 ? c0 : c1) + off);
-            };
-            eval_atom_general<NIMG, NIMG == 1>(P, S, sh_tab, aa, half ? q1 : q0, half ? has1 : has0, f_lo, f_hi, sc,
-                                               emit, emit0);
+        auto general = [&]() {
+            h_image_general<NIMG, NSPLIT>(P.coef_ddn, P.species + P.atom_species[A.atom], sh_tab, P.atom_dd + 6 * A.atom,
+                                          P.pts_dd + 6 * B.pt0, B.np, c, rb, f_lo, f_hi, c0, c1, wvs, fsc);
         };
         // the chunk's columns of rows rb + [f_lo, f_hi): eight 16-byte units a row and plane
         auto zero_all = [&]() {
@@ -1057,33 +1084,42 @@ __device__ __forceinline__ void atom_grids(const DevPlan &P, const DevBatch &B, 
     }
 }
 
-// The same for any species, a shell at a time from its own table
+// The same for any species, each shell on its own table, four shells a look at the
+// points
 __device__ __forceinline__ void atom_grids_general(const DevPlan &P, const DevBatch &B, const DevAct &A,
                                                    const DevSpecies &S, const DevShell *sh_tab, const Dd3 *pts,
                                                    const float *wvf, HGrid *grids, int depth)
 {
     const int lane = threadIdx.x & 31;
     const Dd3 aa = load_dd3(P.atom_dd + 6 * A.atom);
-    for (int sh = 0; sh < S.n_shell; sh++) {
-        const DevShell R = sh_tab[S.shell0 + sh];
-        const float *bt = P.rbound + R.bound_off;
-        float m0 = 0.f, m1 = 0.f, s0 = 0.f, s1 = 0.f;
+    for (int sh0 = 0; sh0 < S.n_shell; sh0 += 4) {
+        const DevShell *sh = sh_tab + S.shell0 + sh0;
+        const int ns = min(4, S.n_shell - sh0);
+        float m0[4], m1[4], s0[4], s1[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) m0[j] = m1[j] = s0[j] = s1[j] = 0.f;
         for (int p = lane; p < B.np; p += 32) {
             const float3 o = offset_f32(pts[p], aa);
-            const int ki = knot_below(sqrtf(o.x * o.x + o.y * o.y + o.z * o.z), R.rcut_f, R.inv_h_hi, R.nk);
-            if (ki < 0) continue;
-            const float t = __ldg(bt + ki), tw = t * wvf[p];
-            m0 = fmaxf(m0, t);
-            m1 = fmaxf(m1, tw);
-            s0 += t;
-            s1 += tw;
+            const float d = sqrtf(o.x * o.x + o.y * o.y + o.z * o.z), w = wvf[p];
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                if (j >= ns) break;
+                const int ki = knot_below(d, sh[j].rcut_f, sh[j].inv_h_hi, sh[j].nk);
+                if (ki < 0) continue;
+                const float t = __ldg(P.rbound + sh[j].bound_off + ki), tw = t * w;
+                m0[j] = fmaxf(m0[j], t);
+                m1[j] = fmaxf(m1[j], tw);
+                s0[j] += t;
+                s1[j] += tw;
+            }
         }
-        m0 = warp_max(m0);
-        m1 = warp_max(m1);
-        s0 = warp_sum(s0);
-        s1 = warp_sum(s1);
-        put_shell_grid(P, grids, 0, R.l, A.fn_loc + R.fn0, m0, s0, depth, lane);
-        put_shell_grid(P, grids, 1, R.l, A.fn_loc + R.fn0, m1, s1, depth, lane);
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            if (j >= ns) break;
+            const float a0 = warp_max(m0[j]), a1 = warp_max(m1[j]), b0 = warp_sum(s0[j]), b1 = warp_sum(s1[j]);
+            put_shell_grid(P, grids, 0, sh[j].l, A.fn_loc + sh[j].fn0, a0, b0, depth, lane);
+            put_shell_grid(P, grids, 1, sh[j].l, A.fn_loc + sh[j].fn0, a1, b1, depth, lane);
+        }
     }
 }
 
@@ -1309,13 +1345,18 @@ __device__ __forceinline__ void density_image_lanes(const DevPlan &P, const DevB
         auto emit2 = [&](int f, const pk *hi, const pk *nlo) {
             store_pair<NSPLIT>(img + place(f, g16) + pb, hi[0], nlo[0], sc, un);
         };
-        auto general = [&](int half) {
-            const uint32_t hb = pb + 2u * half;
-            const float2 su = half ? s1 : s0;
-            auto emit = [&](int f, const df *val) { store_value<NSPLIT>(img + place(f, g16) + hb, val[0], su.x, su.y); };
-            auto emit0 = [&](int f) { store_zero<NSPLIT>(img + place(f, g16) + hb); };
-            eval_atom_general<1, false>(P, S, sh_tab, aa, half ? q1 : q0, half ? has1 : has0, 0, S.n_fn, nullptr, emit,
-                                        emit0);
+        auto general = [&]() {                       // a point a lane, 64 consecutive bytes of a row a store
+#pragma unroll
+            for (int kg = lane; kg < 64; kg += 32) {
+                const int pg = c * 64 + kg;
+                const bool has = pg < B.np;
+                const Dd3 q = load_dd3(P.pts_dd + 6 * (B.pt0 + (has ? pg : 0)));
+                const float2 su = NSPLIT == 3 ? csc[kg] : make_float2(0.f, 0.f);
+                const uint32_t gg16 = (uint32_t)(kg >> 3) << 4, hb = (uint32_t)(kg & 7) * 2u;
+                auto emit = [&](int f, const df *val) { store_value<NSPLIT>(img + place(f, gg16) + hb, val[0], su.x, su.y); };
+                auto emit0 = [&](int f) { store_zero<NSPLIT>(img + place(f, gg16) + hb); };
+                eval_atom_general<1, false>(P.coef_ddn, S, sh_tab, aa, q, has, 0, S.n_fn, nullptr, emit, emit0);
+            }
         };
         // the chunk's columns of the atom's rows: eight 16-byte units a row and plane
         auto zero_all = [&]() {
