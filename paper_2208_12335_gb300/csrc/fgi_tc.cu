@@ -103,6 +103,18 @@ __device__ __forceinline__ bool mbar_wait_a(uint64_t *bar, uint32_t parity, int 
     return true;
 }
 
+// At the end of a role: wait, as long at most, for what it has itself in flight (bulk
+// copies, MMAs), whatever the abort flag says: shared and tensor memory are
+// given up when the CTA leaves, also after a time-out.
+__device__ __forceinline__ bool mbar_drain(uint64_t *bar, uint32_t parity)
+{
+    if (mbar_try_wait(bar, parity)) return true;
+    const uint64_t t0 = global_ns();
+    while (!mbar_try_wait(bar, parity))
+        if (global_ns() - t0 > kWaitLimitNs) return false;
+    return true;
+}
+
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
 {
     asm volatile(
@@ -1648,11 +1660,10 @@ __device__ __forceinline__ bool stage_wait_full(TcRing *S, uint32_t n, int *stat
     return mbar_wait_a(&S->full[n % kStages], (n / kStages) & 1, status, &S->abort);
 }
 
-// Producer, at the end: do not leave while a copy may still be landing
-__device__ __forceinline__ void ring_drain(TcRing *S, uint32_t n, int *status)
+// Producer, at the end: do not leave while one of its n copies may still be landing
+__device__ __forceinline__ void ring_drain(TcRing *S, uint32_t n)
 {
-    for (uint32_t q = (n > kStages ? n - kStages : 0); q < n; q++)
-        mbar_wait_a(&S->empty[q % kStages], (q / kStages) & 1, status, &S->abort);
+    for (uint32_t q = (n > kStages ? n - kStages : 0); q < n; q++) mbar_drain(&S->full[q % kStages], (q / kStages) & 1);
 }
 
 // ---- tile ring: entry lt % kTiles holds this CTA's lt-th tile, drained by
@@ -1723,14 +1734,16 @@ __device__ __forceinline__ bool tile_wait_full(TcRing *S, uint32_t lt, int *stat
     return mbar_wait_a(&S->nfull[lt % kTiles], (lt / kTiles) & 1, status, &S->abort);
 }
 
-// Producer, after its last tile (lt of them): an end mark for each group
-__device__ __forceinline__ void tiles_end(TcRing *S, uint32_t lt, int *status)
+// Producer, after its last tile (lt of them): an end mark for each group; returns
+// how many places of the ring they took
+__device__ __forceinline__ uint32_t tiles_end(TcRing *S, uint32_t lt, int *status)
 {
-    for (uint32_t e = lt; e < lt + 2; e++) {
-        if (!tile_wait_empty(S, e, status)) return;
-        S->tile[e % kTiles].ti = -1;
-        mbar_arrive(&S->nfull[e % kTiles]);
+    for (uint32_t k = 0; k < 2; k++) {
+        if (!tile_wait_empty(S, lt + k, status)) return k;
+        S->tile[(lt + k) % kTiles].ti = -1;
+        mbar_arrive(&S->nfull[(lt + k) % kTiles]);
     }
+    return 2;
 }
 
 // Epilogue group: its next tile; false at the end (or after a time-out) for
@@ -1851,17 +1864,19 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_h(DevPlan P, const TcBatch
                     if (!same) bulk_g2s(dst + kOperandBytes, b_img + (long long)c * kChunkStride, chunk, &S->full[q]);
                 }
             }
-            if (ok) tiles_end(S, lt, P.status);
-            ring_drain(S, n, P.status);
-            // nor while a tile's descriptors may (the entries of older tiles have
-            // been read: the end marks took the next two places)
-            for (uint32_t q = lt + 2 > kTiles ? lt + 2 - kTiles : 0; q < lt; q++) tile_wait_full(S, q, P.status);
+            const uint32_t marks = ok ? tiles_end(S, lt, P.status) : 0;
+            ring_drain(S, n);
+            // nor while a tile's descriptors may (those of older tiles and those in
+            // the places of the marks have been read)
+            for (uint32_t q = lt + marks > kTiles ? lt + marks - kTiles : 0; q < lt; q++)
+                mbar_drain(&S->nfull[q % kTiles], (q / kTiles) & 1);
         }
         __syncwarp();
     } else if (warp == kWarpMma) {
         uint32_t n = 0;
+        uint32_t lt = 0;
         bool ok = true;
-        for (uint32_t lt = 0; ok && __all_sync(0xffffffffu, tile_wait_full(S, lt, P.status)); lt++) {
+        for (; ok && __all_sync(0xffffffffu, tile_wait_full(S, lt, P.status)); lt++) {
             const int e = (int)(lt % kTiles);
             const int ti = S->tile[e].ti, tj = S->tile[e].tj, np = S->tile[e].np, nfn = S->tile[e].nfn, nc = S->tile[e].nc;
             const bool same = S->tile[e].sign != 0 && ti == tj;
@@ -1887,6 +1902,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_h(DevPlan P, const TcBatch
             }
             if (elect_one()) tc_commit(&S->tfull[buf]);
         }
+        // the last commit covers every MMA before it
+        if (lt > 0) mbar_drain(&S->tfull[(lt - 1) & 1], ((lt - 1) >> 1) & 1);
         __syncwarp();
     } else {
         // Warp w of a group: TMEM lanes 32 (w % 4) .. + 31 (functions j of block
@@ -2288,13 +2305,14 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_density(DevPlan P, const T
                 }
             }
             if (ok) tiles_end(S, lt, P.status);
-            ring_drain(S, n, P.status);
+            ring_drain(S, n);
         }
         __syncwarp();
     } else if (warp == kWarpMma) {
         uint32_t n = 0;
+        uint32_t lt = 0;
         bool ok = true;
-        for (uint32_t lt = 0; ok && __all_sync(0xffffffffu, tile_wait_full(S, lt, P.status)); lt++) {
+        for (; ok && __all_sync(0xffffffffu, tile_wait_full(S, lt, P.status)); lt++) {
             const int e = (int)(lt % kTiles);
             const int m = S->tile[e].ti, J = S->tile[e].tj, nfn = S->tile[e].nfn, nkc = S->tile[e].nkc;
             if (m < 0) break;
@@ -2320,6 +2338,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_density(DevPlan P, const T
             }
             if (elect_one()) tc_commit(&S->tfull[buf]);
         }
+        // the last commit covers every MMA before it
+        if (lt > 0) mbar_drain(&S->tfull[(lt - 1) & 1], ((lt - 1) >> 1) & 1);
         __syncwarp();
     } else {
         // Warp w of a group: TMEM lanes 32 (w % 4) .. + 31 (points of the tile),
@@ -3103,17 +3123,28 @@ cudaError_t tc_launch_adjoint(const TcPlan &t, const DevPlan &P, const TcWave &w
 // Self-test of the failure path: one CTA waits on an mbarrier that nothing
 // completes.  The bounded wait gives up after kWaitLimitNs and records the
 // time-out in the status word, as a stalled pipeline would; no fault, no hang.
+// Then a copy is started and drained with the abort flag set, as a role does that leaves
+// after a time-out; if the drain gives up, the status becomes another error.
+__device__ __align__(128) unsigned char g_selftest_src[kChunkBytes];
+
 __global__ void k_wait_selftest(int *status)
 {
-    __shared__ uint64_t bar;
+    __shared__ __align__(128) unsigned char dst[kChunkBytes];
+    __shared__ uint64_t bar, copied;
     __shared__ int abort_flag;
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
+        mbar_init(&copied, 1);
         abort_flag = 0;
         fence_mbar_init();
     }
     __syncthreads();
-    if (threadIdx.x == 0) mbar_wait_a(&bar, 0, status, &abort_flag);
+    if (threadIdx.x == 0) {
+        mbar_wait_a(&bar, 0, status, &abort_flag);
+        mbar_expect_tx(&copied, kChunkBytes);
+        bulk_g2s(dst, g_selftest_src, kChunkBytes, &copied);
+        if (!mbar_drain(&copied, 0)) atomicExch(status, kStatusBadIndex);
+    }
 }
 
 cudaError_t tc_launch_wait_selftest(int *status, cudaStream_t s)
