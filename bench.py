@@ -269,25 +269,31 @@ def compare_on_sample(sample, precision, device, dev, torch, Context):
 
 
 def executed_tensor_flops(ctx, products):
-    """BF16 tensor-core FLOPs one step (H + density) executes, from the
-    plan's schedules: 128 x 128 output tiles, contraction depth in chunks
-    of 64, padding included; H over the upper tile triangle, the density
-    over the upper block triangle of D."""
+    """BF16 tensor-core FLOPs one step (H + density) issues, from the plan's
+    schedules: 128 rows a tile; its columns (functions of block I in H, J in the
+    density) and its depth (points in H, functions from 128 J on in the density)
+    end at the next multiple of 16.  H over the upper tile triangle, the
+    density over the upper block triangle of D."""
+    def up16(x):
+        return -(-x // 16) * 16
+
     tot = 0.0
     sh = ctx.schedule("h")
     for P_, n_, rank in zip(sh["sb_points"], sh["sb_fns"], sh["sb_rank"]):
         if rank < 0:
             continue
-        nrb, nc = -(-int(n_) // 128), -(-int(P_) // 64)
-        tot += nrb * (nrb + 1) / 2 * 2.0 * 128 * 128 * nc * 64
+        P, n = int(P_), int(n_)
+        nrb = -(-n // 128)
+        for I in range(nrb):                                      # tiles (I, J), J >= I
+            tot += (nrb - I) * 2.0 * 128 * min(128, up16(n - 128 * I)) * up16(P)
     sd = ctx.schedule("density")
     for P_, n_, rank in zip(sd["sb_points"], sd["sb_fns"], sd["sb_rank"]):
         if rank < 0:
             continue
-        nrb, nkc, nc = -(-int(n_) // 128), -(-int(n_) // 64), -(-int(P_) // 64)
-        tiles = (nc + 1) // 2
-        for J in range(nrb):
-            tot += tiles * 2.0 * 128 * 128 * (nkc - 2 * J) * 64
+        P, n = int(P_), int(n_)
+        for J in range(-(-n // 128)):
+            deep = up16(n - 128 * J)
+            tot += -(-P // 128) * 2.0 * 128 * min(128, deep) * deep
     return tot * products
 
 
