@@ -35,18 +35,6 @@ __device__ __forceinline__ df df_two_prod(float a, float b)
     return {p, fmaf(a, b, -p)};
 }
 
-__device__ __forceinline__ df df_add(df a, df b)
-{
-    df s = df_two_sum(a.hi, b.hi);
-    const df t = df_two_sum(a.lo, b.lo);
-    s.lo += t.hi;
-    s = df_fast_two_sum(s.hi, s.lo);
-    s.lo += t.lo;
-    return df_fast_two_sum(s.hi, s.lo);
-}
-
-__device__ __forceinline__ df df_sub(df a, df b) { return df_add(a, df{-b.hi, -b.lo}); }
-
 // Sum with one error-free transformation (the high parts) and a rounded sum
 // of the low parts: error within about 2^-48 (|a| + |b|) instead of
 // 2^-48 |a + b|.  Exact enough for sums of one sign, and for differences of

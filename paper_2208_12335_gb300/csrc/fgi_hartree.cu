@@ -9,7 +9,7 @@
 //       rho~_a,lm(r_k) = sum_p (w_p / (r_k^3 ln q)) n_p A_lm(rhat_p)
 //     (w_p / (r_k^3 ln q) is the partitioned angular weight; A_lm = Y_lm / K_lm
 //     the unnormalised harmonics).  Harmonics and sums of l >= 1 are double-float
-//     (about 2^-45 relative), w_p n_p, the sum for l = 0 and the final scale FP64:
+//     (about 2^-45 relative), offsets, w_p n_p, the sum for l = 0 and the final scale FP64:
 //     GB300's FP64 pipe has 1/64 of the FP32 rate.
 //  2. k_hartree_radial (FP64): a warp per (atom, l, m), lanes along the shells, the
 //     radial Poisson equation
@@ -650,7 +650,7 @@ size_t hartree_ws_bytes(const HartreeDev &H)
            al256(sizeof(float) * kLf * (size_t)H.n_atoms);
 }
 
-cudaError_t launch_hartree(const DevPlan &P, const HartreeDev &H, int n_batch, long long n_pts, int l_max,
+cudaError_t launch_hartree(const DevPlan &P, const HartreeDev &H, int n_batch, int l_max,
                            const double *n, double *vh, double *ws, cudaStream_t s)
 {
     const HartreeTabs T = carve(H, ws);

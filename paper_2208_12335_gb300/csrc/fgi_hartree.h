@@ -41,7 +41,7 @@ HartreeRad hartree_rad(double r_min, double ln_q, int n_rad);
 size_t hartree_ws_bytes(const HartreeDev &H);
 
 // v_H at every point of the grid from n (both device, caller's point order)
-cudaError_t launch_hartree(const DevPlan &P, const HartreeDev &H, int n_batch, long long n_pts, int l_max,
+cudaError_t launch_hartree(const DevPlan &P, const HartreeDev &H, int n_batch, int l_max,
                            const double *n, double *vh, double *ws, cudaStream_t s);
 
 }  // namespace fgi

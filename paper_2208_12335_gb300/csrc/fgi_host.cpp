@@ -596,7 +596,7 @@ int build_plan(fgi_ctx *c, const char *tune_path)
         }
     // the same with every coefficient times the first normalisation constant
     // of the radial's l (real harmonics, no Condon-Shortley phase): the
-    // lane-per-point basis kernels evaluate C_l u(r) directly
+    // tensor-core basis kernels evaluate C_l u(r) directly
     static const double kFirstYlmC[4] = {0.28209479177387814,   // 1/(2 sqrt pi)
                                          0.4886025119029199,    // sqrt(3/(4 pi))
                                          1.0925484305920792,    // (1/2) sqrt(15/pi), xy
@@ -1571,7 +1571,7 @@ int fgi_hartree(fgi_ctx *c, const double *n, double *vh, int l_max, void *ws, si
     DevPlan P = c->dp;
     P.batches = c->d_batches_f64;
     ProfScope ps(c, s, 4, 0.0, 8.0 * (double)c->n_pts, 3);
-    CUDA_TRY(c, launch_hartree(P, c->hd, (int)c->batch_sys.size(), c->n_pts, l_max, n, vh, (double *)ws, s));
+    CUDA_TRY(c, launch_hartree(P, c->hd, (int)c->batch_sys.size(), l_max, n, vh, (double *)ws, s));
     return FGI_OK;
 }
 

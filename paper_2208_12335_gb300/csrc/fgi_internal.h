@@ -99,7 +99,7 @@ struct DevPlan {
     // the same two tables with every coefficient times the first
     // normalisation constant of the radial's l (C_0 = 1/(2 sqrt pi), C_1, the
     // xy constant of l = 2, the y(3x^2 - y^2) constant of l = 3), rounded
-    // from FP64: the lane-per-point basis kernels.  scoefn interleaves the
+    // from FP64: the tensor-core basis kernels.  scoefn interleaves the
     // shells in the order of DevPlan::shells (grouped by l).
     const float4 *coef_ddn;
     const float4 *scoefn;

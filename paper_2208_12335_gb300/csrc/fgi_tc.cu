@@ -425,7 +425,7 @@ __device__ __forceinline__ void store_zero(uint8_t *dst)
 }
 
 // Ratios of the other normalisation constants of an l shell to its first
-// (the spline tables of the lane kernels hold u times the first constant):
+// (the spline tables of the basis kernels hold u times the first constant):
 // l = 2: C(2z^2-x^2-y^2)/C(xy) = 1/(2 sqrt 3); l = 3: C(z(x^2-y^2))/C(y(3x^2-y^2))
 // = sqrt 6 (C(xyz) is twice that), sqrt(3/5) and sqrt(2/5).
 #define FGI_DF_CONST(c) {(float)(c), (float)((c) - (double)(float)(c))}
@@ -1284,7 +1284,8 @@ __global__ void __launch_bounds__(kPhiThreads, 4) k_h_prep(DevPlan P, const TcBa
 // coordinates; only the angular polynomial Q_lm(x, y, z) is FP32 (its
 // rounding varies from point to point).
 //
-// Three CTAs an SM: two take 2.28 ms where three take 2.06 (four 2.08: spills).
+// Three CTAs an SM (80 registers, of which 96 bytes a thread spill): two take 2.28 ms
+// where three take 2.06 and four (64 registers, more spilled) 2.08.
 __global__ void __launch_bounds__(kPhiThreads, 3) k_tc_phi(DevPlan P, const TcBatch *tb, const WorkItem *items,
                                                 uint8_t *ws, int fixed, const int *bsign)
 {
@@ -2390,9 +2391,11 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_tc_density(DevPlan P, const T
                     for (int q = 0; q < 8; q++)
                         if (8 * piece + q < nj) dst[(long long)q * T.nc_alloc * 64] = hi[q] + lo[q];
                 }
-                // E phi in double-float: e = acc0 + acc1, phi = f0 + (f1 + f2), whose
-                // inner sum is exact and never larger than a non-zero f0.  Rows past
-                // n_b up to the next 16 are zero in both images.
+                // E phi in double-float: e = acc0 + acc1, phi = f0 + (f1 + f2).  The inner
+                // sum is never larger than a non-zero f0; its rounding, 2^-25 of f1, is
+                // far below what f2 itself leaves out (2^-18 of f1).  The products are
+                // summed with their errors, the low parts in FP32: about 2^-42 of the
+                // terms.  Rows past n_b up to the next 16 are zero in both images.
 #pragma unroll
                 for (int q = 0; q < 8; q += 2) {
                     auto term = [&](int sp) {
@@ -2613,7 +2616,8 @@ __device__ __forceinline__ float adj_dist(const float3 &o)
 // atoms and shells staged in shared memory and two points a lane take 1.26
 // (64-atom Si cluster, 1.11 M points; 3.1 GB of E, 0.45 ms at the measured
 // copy rate); 0.38 -> 0.17 ms for a molecule of 30 atoms.  Four CTAs an SM: two
-// and three are slower (1.9, 1.6 ms), six spill.
+// and three are slower (1.9, 1.6 ms), and so are six (1.55); four keep 64 registers a
+// thread and spill 124 bytes.
 __global__ void __launch_bounds__(256, 4) k_tc_adj_grad(DevPlan P, const TcBatch *tb, const WorkItem *items,
                                                      const uint8_t *ws, const double *v, double *dR)
 {
