@@ -178,13 +178,14 @@ __device__ __forceinline__ df df_scaled(double x, int e)
 
 // One warp per (atom, shell).  (A thread per point with FP64 harmonics and
 // (l_max + 1)^2 FP64 atomics was bound by the FP64 pipe: 250-atom cluster, 7.3 M
-// points, l_max 6, 3.30 ms; now 0.51 ms.)  The monopole's sum stays FP64: the
+// points, l_max 6, 3.30 ms; now 0.62 ms.)  The monopole's sum stays FP64: the
 // l = 0 terms are all there is at l_max 0, and the others end in FP32.
 //
 // The offsets are differences in FP64 and w n a product in FP64; both become
 // double-floats relative to a power of two (the largest component's; that of the
 // warp's largest |w n| so far), so that neither an atom far from the origin nor
-// the range of FP32 costs any of the 48 bits.
+// the range of FP32 costs any of the 48 bits.  (Offsets from double-float positions and
+// w n as a pair of FP32 numbers: 0.52 ms.)
 template <int LMAX>
 __global__ void __launch_bounds__(128) k_hartree_moments(DevPlan P, HartreeDev H, const double *n, double *rho)
 {
